@@ -510,8 +510,9 @@ int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const 
     const int32_t k = (int32_t)ent.size();
     const int full = g->full_scan ? 1 : 0;
     const bool pair = d.pair_on != 0;
-    // an undirected edge update: one pass over both directions (the vector path of the
-    // rank-1 pass; every row's candidates taken from the state before the update)
+    // an undirected edge update: one pass over both directions (every row's candidates
+    // taken from the state before the update); an n that is not a multiple of the vector
+    // width keeps the two passes
     const bool fused = !g->directed && k == 1 && !g->full_scan && g->fused_edges && g->n % (16 / g->dbytes) == 0;
     if (fused) {
         kin = kout = 0;
@@ -647,6 +648,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     g->inf = i32 ? (int64_t)INT32_MAX : INT64_MAX;
     Dev& d = g->d;
     d.n = n;
+    d.ld = row_pitch(n);
     d.dbytes = g->dbytes;
     d.directed = dir ? 1 : 0;
     d.st = (cudaStream_t)cuda_stream;
@@ -691,22 +693,22 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
         }
     }
     // ---- device memory
-    const size_t nn = (size_t)n * n;
+    const size_t nn = (size_t)n * d.ld;
     int rc = BC_OK;
     d.nrb_max = (n + kRowsPerBlock - 1) / kRowsPerBlock;
     d.g_arcs = arcs;
     if (g->dbytes == 4) {
         int32_t *pD, *pfD, *pcD, *pcD2, *pgw;
-        if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, n)) ||
-            (rc = dalloc(g, &pcD2, n)) || (rc = dalloc(g, &pgw, arcs))) {
+        if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, d.ld)) ||
+            (rc = dalloc(g, &pcD2, d.ld)) || (rc = dalloc(g, &pgw, arcs))) {
             destroy_all(g);
             return fail(nullptr, rc, "device allocation failed");
         }
         d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2; d.g_w = pgw;
     } else {
         int64_t *pD, *pfD, *pcD, *pcD2, *pgw;
-        if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, n)) ||
-            (rc = dalloc(g, &pcD2, n)) || (rc = dalloc(g, &pgw, arcs))) {
+        if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, d.ld)) ||
+            (rc = dalloc(g, &pcD2, d.ld)) || (rc = dalloc(g, &pgw, arcs))) {
             destroy_all(g);
             return fail(nullptr, rc, "device allocation failed");
         }
@@ -718,8 +720,8 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
         (rc = dalloc(g, &d.err, 1)) || (rc = dalloc(g, &d.stats, kStats)) || (rc = dalloc(g, &d.mark, n)) ||
         (rc = dalloc(g, &d.changed, n)) || (rc = dalloc(g, &d.rows, n)) || (rc = dalloc(g, &d.acc_rows, n)) ||
         (rc = dalloc(g, &d.counts, 8)) || (rc = dalloc(g, &d.fS, n)) || (rc = dalloc(g, &d.fM, n)) ||
-        (rc = dalloc(g, &d.cS, n)) || (rc = dalloc(g, &d.cM, n)) || (rc = dalloc(g, &d.cS2, n)) ||
-        (rc = dalloc(g, &d.partial, (size_t)d.nrb_max * n))) {
+        (rc = dalloc(g, &d.cS, d.ld)) || (rc = dalloc(g, &d.cM, d.ld)) || (rc = dalloc(g, &d.cS2, d.ld)) ||
+        (rc = dalloc(g, &d.partial, (size_t)d.nrb_max * d.ld))) {
         destroy_all(g);
         return fail(nullptr, rc, "device allocation failed");
     }
@@ -780,6 +782,18 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     CKI(cudaMemsetAsync(d.mark, 0, n, d.st));
     CKI(cudaMemsetAsync(d.changed, 0, n, d.st));
     CKI(cudaMemsetAsync(d.counts, 0, 8 * sizeof(int32_t), d.st));
+    if (d.ld > n) {
+        // the column vectors' entries past n: no path (the passes write only the first n)
+        std::vector<unsigned char> inf((size_t)(d.ld - n) * g->dbytes);
+        for (int32_t i = 0; i < d.ld - n; ++i) {
+            if (i32) reinterpret_cast<int32_t*>(inf.data())[i] = INT32_MAX;
+            else reinterpret_cast<int64_t*>(inf.data())[i] = INT64_MAX;
+        }
+        for (void* c : {d.cD, d.cD2})
+            CKI(cudaMemcpyAsync(static_cast<unsigned char*>(c) + (size_t)n * g->dbytes, inf.data(), inf.size(),
+                                cudaMemcpyHostToDevice, d.st));
+        for (uint64_t* c : {d.cS, d.cM, d.cS2}) CKI(cudaMemsetAsync(c + n, 0, sizeof(uint64_t) * (d.ld - n), d.st));
+    }
     if (!dir) {
         CKI(cudaMemsetAsync(d.chg, 0, sizeof(uint32_t) * n * d.chg_words, d.st));
         CKI(cudaMemsetAsync(d.tcnt, 0, sizeof(int32_t) * n, d.st));
@@ -1090,20 +1104,24 @@ int bc_get_rows(bc_graph* g, int32_t s0, int32_t count, int64_t* d_out, uint64_t
     if (!check_alive(g, &rc)) return rc;
     if (s0 < 0 || count < 0 || s0 + count > g->n) return fail(g, BC_ERR_ARG, "rows out of range");
     if ((rc = sync_check(g))) return rc;
-    const size_t n = (size_t)g->n, off = (size_t)s0 * n, cnt = (size_t)count * n;
+    const size_t n = (size_t)g->n, ld = (size_t)g->d.ld, off = (size_t)s0 * ld, cnt = (size_t)count * n;
+    // rows of n entries out of rows of ld
+    auto copy = [&](void* to, const void* from, size_t item) {
+        return cudaMemcpy2D(to, n * item, from, ld * item, n * item, (size_t)count, cudaMemcpyDeviceToHost);
+    };
     if (d_out) {
         if (g->dbytes == 8) {
-            CK(g, cudaMemcpy(d_out, (int64_t*)g->d.D + off, cnt * 8, cudaMemcpyDeviceToHost));
+            CK(g, copy(d_out, (int64_t*)g->d.D + off, 8));
         } else {
             std::vector<int32_t> tmp(cnt);
-            CK(g, cudaMemcpy(tmp.data(), (int32_t*)g->d.D + off, cnt * 4, cudaMemcpyDeviceToHost));
+            CK(g, copy(tmp.data(), (int32_t*)g->d.D + off, 4));
             for (size_t i = 0; i < cnt; ++i) d_out[i] = tmp[i] == INT32_MAX ? INT64_MAX : (int64_t)tmp[i];
         }
     }
-    if (sigma_out) CK(g, cudaMemcpy(sigma_out, g->d.S + off, cnt * 8, cudaMemcpyDeviceToHost));
+    if (sigma_out) CK(g, copy(sigma_out, g->d.S + off, 8));
     if (delta_out) {
         std::vector<ff> tmp(cnt);
-        CK(g, cudaMemcpy(tmp.data(), g->d.Dl + off, cnt * sizeof(ff), cudaMemcpyDeviceToHost));
+        CK(g, copy(tmp.data(), g->d.Dl + off, sizeof(ff)));
         for (size_t i = 0; i < cnt; ++i) delta_out[i] = ff_to_double(tmp[i]);
     }
     return BC_OK;
@@ -1353,13 +1371,12 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     b->L.scan_ctas = 8;
     b->L.bc_ctas = 8;
     b->L.acc_per_sm = 0;
-    b->L.scan_unroll = 4;   // the single-graph item width (kScanUnroll)
+    b->L.scan_unroll = 4;
     b->L.scan_sched = 0;
     b->L.acc_threads = kAccThreadsNarrow;
     int rc;
     if ((rc = balloc(b, &b->d_devs, count)) || (rc = balloc(b, &b->d_coff, count + 1)) ||
-        (rc = balloc(b, &b->d_plans, (4 + (size_t)kPairClasses) * ((size_t)count + 1))) ||
-        (rc = balloc(b, &b->d_pctr, kPairClasses))) {
+        (rc = balloc(b, &b->d_plans, 5 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1))) {
         bc_batch_destroy(b);
         return rc;
     }
@@ -1507,13 +1524,11 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
         }
     }
     // ---- device buffers and launch shape
-    // graphs with pair corrections (undirected, option on) by class of the column test's
-    // columns per thread: the set of pair kernels a round launches
-    int32_t pair_classes = 0;
-    for (bc_graph* g : b->graphs)
-        if (g->d.pair_on) pair_classes |= 1 << pair_class(g->dbytes, pair_vn(g->dbytes, g->n));
-    if (pair_classes != b->L.pair_classes) {
-        b->L.pair_classes = pair_classes;
+    // graphs with pair corrections (undirected, option on): a round launches their kernels
+    int32_t pairs = 0;
+    for (bc_graph* g : b->graphs) pairs |= g->d.pair_on ? 1 : 0;
+    if (pairs != b->L.pairs) {
+        b->L.pairs = pairs;
         drop_exec(b);
     }
     int64_t cap_max = 0;

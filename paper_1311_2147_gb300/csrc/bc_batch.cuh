@@ -38,19 +38,11 @@ struct BatchArgs {
     int64_t* plan_bc;         // [G + 1]
     int64_t* plan_acc;        // [G + 1]
     int64_t* plan_pr;         // [G + 1]: rows listed for pair corrections (graphs with them)
-    int64_t* plan_pw;         // [kPairClasses * (G + 1)]: column-test work per class of columns per thread
-    int32_t* pctr;            // [kPairClasses]: column-test pieces handed out past the first wave
+    int64_t* plan_pw;         // [G + 1]: column-test work
+    int32_t* pctr;            // column-test pieces handed out past the first wave
     int32_t* ws;              // accumulation work space, acc_grid * ws_stride ints
     int64_t ws_stride;
 };
-
-// Classes of the column test's columns per thread (pair_vn): int32 distances 8, 4, 1;
-// int64 distances 2, 1.
-constexpr int kPairClasses = 3;
-__host__ __device__ inline int pair_class(int dbytes, int vn) {
-    if (dbytes == 4) return vn == 8 ? 0 : (vn == 4 ? 1 : 2);
-    return vn == 2 ? 0 : 1;
-}
 
 // Launch shape of a batch; the tunable part is what the autotuner varies.
 struct BatchLaunch {
@@ -65,8 +57,8 @@ struct BatchLaunch {
                           // turn (item = CTA + k * grid)                (tunable)
     int32_t acc_threads;  // threads of an accumulation CTA: 512, 256 or 128 (more sources
                           // in flight per SM)                           (tunable)
-    int32_t pair_classes; // bit c: some graph of the batch has pair corrections with columns
-                          // per thread of class c (0: none; the round skips the pair kernels)
+    int32_t pairs;        // 1: some graph of the batch has pair corrections (0: the round skips
+                          // the pair kernels)
     int32_t acc_grid;
     int32_t acc_smem;
     int32_t mask_in_smem;

@@ -16,13 +16,13 @@ namespace bcg {
 // sigma are symmetric, so d(s,x) is read as d(x,s) (consecutive threads then read
 // consecutive entries of row x instead of one entry of each row).
 template <typename DT, bool SYM = false>
-__device__ __forceinline__ void dev_alg4_in(int s, int n, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__device__ __forceinline__ void dev_alg4_in(int s, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                           int v, const VEdge* __restrict__ e, int k, int directed,
                           DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
                           int32_t* err) {
     const int64_t INF = Inf<DT>::v;
-    const size_t rs = (size_t)s * n;
-    auto at = [&](int x) { return SYM ? (size_t)x * n + s : rs + x; };
+    const size_t rs = (size_t)s * ld;
+    auto at = [&](int x) { return SYM ? (size_t)x * ld + s : rs + x; };
     const int64_t old = D[at(v)];
     int64_t cur = old;
     uint64_t sig = S[at(v)];
@@ -61,12 +61,12 @@ __device__ __forceinline__ void dev_alg4_in(int s, int n, const DT* __restrict__
 // OUT phase, row test: row s (s != v) can change only through a new shortest path
 // s ~> v -> x_j, i.e. d'(s,v) + w'(v,x_j) <= d'(s,x_j) for some out-edge of the update.
 template <typename DT>
-__device__ __forceinline__ void dev_rows_out(int s, int n, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__device__ __forceinline__ void dev_rows_out(int s, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
                            DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
                            int32_t* err) {
     const int64_t INF = Inf<DT>::v;
-    const size_t rs = (size_t)s * n;
+    const size_t rs = (size_t)s * ld;
     const int64_t dsv = D[rs + v];
     const uint64_t ssv = S[rs + v];
     bool aff = false;
@@ -96,11 +96,11 @@ __device__ __forceinline__ void dev_rows_out(int s, int n, const DT* __restrict_
 // out-edges (v, x_j) of the update are in-edges of v in G'_R, and d_R(t, x_j) is
 // d'(x_j, t), read from row x_j.  Produces row v of the result.
 template <typename DT>
-__device__ __forceinline__ void dev_alg4_out(int t, int n, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__device__ __forceinline__ void dev_alg4_out(int t, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
                            DT* cD, uint64_t* cS, uint64_t* cM, uint8_t* changed, int32_t* err) {
     const int64_t INF = Inf<DT>::v;
-    const size_t rv = (size_t)v * n;
+    const size_t rv = (size_t)v * ld;
     const int64_t old = D[rv + t];
     int64_t cur = old;
     uint64_t sig = S[rv + t];
@@ -109,7 +109,7 @@ __device__ __forceinline__ void dev_alg4_out(int t, int n, const DT* __restrict_
     for (int j = 0; j < k; ++j) {
         const VEdge ed = e[j];
         if (directed && ed.dir != 1) continue;
-        const size_t ry = (size_t)ed.x * n;
+        const size_t ry = (size_t)ed.x * ld;
         const int64_t dy = D[ry + t];
         if (dy == INF) continue;
         const int64_t dj = dsum<DT>(ed.w, dy);
@@ -231,11 +231,10 @@ template <> struct Vec<int64_t> {
 };
 
 constexpr int kScanThreads = 256;
-constexpr int kScanUnroll = 4;
 
 template <typename DT>
 struct ScanArgs {
-    int n;
+    int ld;                // entries of a state row: the columns of a pass (those past n hold INF)
     DT* D;
     uint64_t* S;
     const int32_t* rows;
@@ -363,9 +362,9 @@ __device__ __forceinline__ bool rule_vec(const ScanArgs<DT>& a, int s, size_t ro
             V::set(dv, q, nd);
             wr = true;
             ++n_changed;
-            if (a.rec.tcnt) record_change<DT>(a.rec, a.n, s, t + q, dd[q], sig0);
+            if (a.rec.tcnt) record_change<DT>(a.rec, s, t + q, dd[q], sig0);
         } else if (n_ties != ties0 && a.rec.tcnt) {
-            record_change<DT>(a.rec, a.n, s, t + q, dd[q], sig0);
+            record_change<DT>(a.rec, s, t + q, dd[q], sig0);
         }
     }
     return wr;
@@ -387,7 +386,7 @@ __device__ __forceinline__ void load_u64s(const uint64_t* p, uint64_t* o) {
 // (bits 8..15), with their values before the rule in dold / sold, for a caller that
 // records the changes of a whole warp together.  The vector's path counts and the
 // column's counts and multipliers are loaded together (16-byte loads: t is a multiple
-// of VN and so is n), and the changed counts written back together, so a vector costs
+// of VN and so is ld), and the changed counts written back together, so a vector costs
 // one round trip to memory instead of one per pair.
 template <typename DT>
 __device__ __forceinline__ unsigned rule_vec_masked(const ScanArgs<DT>& a, const uint64_t* colS,
@@ -446,7 +445,7 @@ __device__ __forceinline__ unsigned rule_vec_masked(const ScanArgs<DT>& a, const
 // run of lanes on the same row; the first change of a pair in the update saves its old
 // values and lists it, as record_change does.  Every lane of the warp must call it.
 template <typename DT>
-__device__ __forceinline__ void record_changes_warp(const PairRec& r, int n, int s, int t, unsigned bits,
+__device__ __forceinline__ void record_changes_warp(const PairRec& r, int s, int t, unsigned bits,
                                                     const int64_t* dold, const uint64_t* sold) {
     const int lane = threadIdx.x & 31;
     if (s >= 0 && bits) {
@@ -455,7 +454,7 @@ __device__ __forceinline__ void record_changes_warp(const PairRec& r, int n, int
         if (!r.first) wb &= ~*w;   // pairs already recorded in this update keep their saved values
         bits = wb >> (t & 31);
         if (wb) atomicOr(w, wb);
-        const size_t i0 = (size_t)s * n + t;
+        const size_t i0 = (size_t)s * r.ld + t;
         for (unsigned b = bits; b; b &= b - 1) {
             const int q = __ffs(b) - 1;
             static_cast<DT*>(r.oldD)[i0 + q] = (DT)dold[q];
@@ -498,52 +497,32 @@ __device__ __forceinline__ bool scan_vec(const ScanArgs<DT>& a, int s, size_t ro
 }
 
 // One work item of the rank-1 pass: row s (scalars rd, rs, rm), chunk c of CW columns.
-template <typename DT, bool VECTOR, int U = kScanUnroll>
+template <typename DT, int U>
 __device__ __forceinline__ void dev_scan_item(const ScanArgs<DT>& a, int s, int64_t rd, uint64_t rs, uint64_t rm,
                                               int c, int& n_changed, int& n_ties) {
     using V = Vec<DT>;
     constexpr int VN = V::N;
     constexpr int CW = kScanThreads * VN * U;
-    const int n = a.n;
-    const int64_t INF = Inf<DT>::v;
-    const size_t rowoff = (size_t)s * n;
+    const int ld = a.ld;
+    const size_t rowoff = (size_t)s * ld;
     DT* __restrict__ Drow = a.D + rowoff;
     const int t0 = c * CW;
     const int tid = threadIdx.x % kScanThreads;
-    if constexpr (VECTOR) {
-        typename V::T dv[U], cv[U];
+    typename V::T dv[U], cv[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int t = t0 + (u * kScanThreads + tid) * VN;
-            if (t < n) {
-                dv[u] = __ldcs(reinterpret_cast<const typename V::T*>(Drow + t));
-                cv[u] = __ldg(reinterpret_cast<const typename V::T*>(a.cD + t));
-            }
+    for (int u = 0; u < U; ++u) {
+        const int t = t0 + (u * kScanThreads + tid) * VN;
+        if (t < ld) {
+            dv[u] = __ldcs(reinterpret_cast<const typename V::T*>(Drow + t));
+            cv[u] = __ldg(reinterpret_cast<const typename V::T*>(a.cD + t));
         }
+    }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int t = t0 + (u * kScanThreads + tid) * VN;
-            if (t >= n) break;
-            if (scan_vec<DT>(a, s, rowoff, t, dv[u], cv[u], rd, rs, rm, n_changed, n_ties))
-                *reinterpret_cast<typename V::T*>(Drow + t) = dv[u];
-        }
-    } else {
-        for (int t = t0 + tid; t < t0 + CW && t < n; t += kScanThreads) {
-            const int64_t cd = a.cD[t];
-            if (cd == INF) continue;
-            const int64_t old = Drow[t];
-            const int64_t cand = dsum<DT>(rd, cd);
-            int64_t nd;
-            const int ties0 = n_ties;
-            const uint64_t sig0 = a.rec.tcnt ? a.S[rowoff + t] : 0ull;
-            if (pair_rule<DT>(cand, old, rowoff + t, rs, rm, a.cS[t], a.cM[t], a.S, a.err, &nd, &n_ties)) {
-                Drow[t] = (DT)nd;
-                ++n_changed;
-                if (a.rec.tcnt) record_change<DT>(a.rec, n, s, t, old, sig0);
-            } else if (n_ties != ties0 && a.rec.tcnt) {
-                record_change<DT>(a.rec, n, s, t, old, sig0);
-            }
-        }
+    for (int u = 0; u < U; ++u) {
+        const int t = t0 + (u * kScanThreads + tid) * VN;
+        if (t >= ld) break;
+        if (scan_vec<DT>(a, s, rowoff, t, dv[u], cv[u], rd, rs, rm, n_changed, n_ties))
+            *reinterpret_cast<typename V::T*>(Drow + t) = dv[u];
     }
 }
 
@@ -561,15 +540,16 @@ __device__ __forceinline__ void scan_stats(int64_t* stats, int n_changed, int n_
 }
 
 template <typename DT>
-__device__ __forceinline__ void dev_write_row(int t, int n, DT* D, uint64_t* S, int v, const DT* cD, const uint64_t* cS,
+__device__ __forceinline__ void dev_write_row(int t, int ld, DT* D, uint64_t* S, int v, const DT* cD, const uint64_t* cS,
                             const int32_t* err) {
-    D[(size_t)v * n + t] = cD[t];
-    S[(size_t)v * n + t] = cS[t];
+    D[(size_t)v * ld + t] = cD[t];
+    S[(size_t)v * ld + t] = cS[t];
 }
 
 template <typename DT>
 struct AccArgs {
     int n;
+    int ld;
     const DT* D;
     uint64_t* S;
     ff* Dl;
@@ -997,9 +977,9 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
     const int np = (n + 31) & ~31;
     const int tid = threadIdx.x;
     const int64_t INF = Inf<DT>::v;
-    const DT* Ds = a.D + (size_t)s * n;
-    uint64_t* Ss = a.S + (size_t)s * n;
-    ff* out = a.Dl + (size_t)s * n;
+    const DT* Ds = a.D + (size_t)s * a.ld;
+    uint64_t* Ss = a.S + (size_t)s * a.ld;
+    ff* out = a.Dl + (size_t)s * a.ld;
     int wide = 0;
     for (int t = tid; t < n; t += T) {
         const int64_t v = Ds[t];
@@ -1010,6 +990,10 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
         m.d16[t] = c;
         out[t] = ff{0.0f, 0.0f};
         if (STATIC) Ss[t] = (t == s) ? 1ull : 0ull;
+    }
+    if (STATIC && tid < a.ld - n) {   // the entries past n: no path
+        Ss[n + tid] = 0ull;
+        out[n + tid] = ff{0.0f, 0.0f};
     }
     for (int t = tid; t < np / 2; t += T) m.cnt[t] = 0u;
     wide = __syncthreads_or(wide);
@@ -1025,28 +1009,28 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
 // partial[rb][t] = sum over rows r of row block rb of Dl[s_r][t] (t != s_r), rows in
 // increasing order, in float-float (all terms are non-negative); rows = nullptr means
 // all n rows.
-__device__ __forceinline__ void dev_bc_partial(int t, int rb, int n, const int32_t* rows, int total,
+__device__ __forceinline__ void dev_bc_partial(int t, int rb, int ld, const int32_t* rows, int total,
                                                const ff* Dl, ff* partial) {
     const int r0 = rb * kRowsPerBlock;
-    if (r0 >= total || t >= n) return;
+    if (r0 >= total || t >= ld) return;
     const int r1 = min(total, r0 + kRowsPerBlock);
     ff acc{0.0f, 0.0f};
     for (int r = r0; r < r1; ++r) {
         const int s = rows ? rows[r] : r;
-        if (s != t) acc = ff_add(acc, Dl[(size_t)s * n + t]);
+        if (s != t) acc = ff_add(acc, Dl[(size_t)s * ld + t]);
     }
-    partial[(size_t)rb * n + t] = acc;
+    partial[(size_t)rb * ld + t] = acc;
 }
 
 // bc (hi, lo) += sign * (sum of the row-block partials in block order): the partials are
 // summed in float-float, the total is taken to fp64 and added with TwoSum; overwrite
 // starts from zero (the static computation).
-__device__ __forceinline__ void dev_bc_finish(int t, int n, int total, const ff* partial, double sign,
+__device__ __forceinline__ void dev_bc_finish(int t, int ld, int total, const ff* partial, double sign,
                                               int overwrite, double* hi, double* lo) {
     const int nrb = (total + kRowsPerBlock - 1) / kRowsPerBlock;
     if (nrb == 0 && !overwrite) return;
     ff acc{0.0f, 0.0f};
-    for (int rb = 0; rb < nrb; ++rb) acc = ff_add(acc, partial[(size_t)rb * n + t]);
+    for (int rb = 0; rb < nrb; ++rb) acc = ff_add(acc, partial[(size_t)rb * ld + t]);
     const double sum = sign * ff_to_double(acc);
     if (overwrite) {
         hi[t] = sum;

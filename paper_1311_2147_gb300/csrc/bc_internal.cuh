@@ -1,12 +1,18 @@
 // bc_internal.cuh -- device-side types, exact integer helpers and the launch
 // functions shared by the translation units of libbcgpu.so.
 //
-// State layout (row-major n x n, structure of arrays; Section 5 stores the triple
-// (d, sigma, flag) per pair in one row-major array -- here each field is its own
+// State layout (row-major n rows of ld entries, structure of arrays; Section 5 stores the
+// triple (d, sigma, flag) per pair in one row-major array -- here each field is its own
 // array so a pass reads only the fields it needs):
-//   D   [n*n]  distance type DT (int32 or int64), INF = DT max
-//   S   [n*n]  uint64 path counts sigma_st
-//   Dl  [n*n]  dependencies delta_s.(t) as float-float pairs (ff.cuh), 0 on the diagonal
+//   D   [n*ld]  distance type DT (int32 or int64), INF = DT max
+//   S   [n*ld]  uint64 path counts sigma_st
+//   Dl  [n*ld]  dependencies delta_s.(t) as float-float pairs (ff.cuh), 0 on the diagonal
+// ld is n rounded up to a multiple of kRowAlign entries, so every row starts on a 32-byte
+// boundary and the vector loads of the passes serve every n; the entries past n hold
+// INF / 0 / 0 (no path) and no pass changes them.  With rows packed at n entries an odd n
+// had to take one column per thread: 16 edge and vertex updates of BA n = 5003 took
+// 10.4 ms that way and take 5.7 ms so (the column test was 297 us and the rank-1 pass
+// 113 us of an update's 490 us).
 //   BC  [n]    fp64 pair (hi, lo): compensated running sums of the G_D scores
 // E* superset ("E*+") -- every arc that lies on some shortest path, plus arcs that
 // may no longer do so (Section 6: any superset of E* gives the right DAGs) -- is a
@@ -77,6 +83,10 @@ __device__ __forceinline__ uint64_t add_chk(uint64_t a, uint64_t b, int32_t* err
     return s;
 }
 
+// Entries of a row of the state (and of the column vectors the passes read beside it).
+constexpr int kRowAlign = 8;
+__host__ __device__ inline int32_t row_pitch(int32_t n) { return (n + kRowAlign - 1) & ~(kRowAlign - 1); }
+
 template <typename DT> struct Arc;
 template <> struct __align__(8) Arc<int32_t> { int32_t dst; int32_t w; };
 template <> struct __align__(16) Arc<int64_t> { int64_t dst; int64_t w; };
@@ -139,6 +149,7 @@ struct EMoves {
 // Device state of one handle (plain pointers; owned by the host-side bc_graph).
 struct Dev {
     int32_t n;
+    int32_t ld;          // entries of a state row (row_pitch(n))
     int32_t dbytes;      // 4 or 8
     int32_t directed;
     int32_t nsm;
@@ -175,12 +186,12 @@ struct Dev {
     void* fD;            // [n] per-row distance to v after the phase (DT)
     uint64_t* fS;        // [n] per-row path count to v after the phase
     uint64_t* fM;        // [n] per-row multiplier of a tie
-    void* cD;            // [n] per-column distances from v (DT)
-    uint64_t* cS;        // [n] per-column path counts from v
-    uint64_t* cM;        // [n] per-column multiplier of a tie
-    void* cD2;           // [n] second column vector (fused undirected edge pass): distances (DT)
-    uint64_t* cS2;       // [n] its path counts
-    ff* partial;         // [nrb * n] column partial sums
+    void* cD;            // [ld] per-column distances from v (DT); INF past n
+    uint64_t* cS;        // [ld] per-column path counts from v
+    uint64_t* cM;        // [ld] per-column multiplier of a tie
+    void* cD2;           // [ld] second column vector (fused undirected edge pass): distances (DT)
+    uint64_t* cS2;       // [ld] its path counts
+    ff* partial;         // [nrb * ld] column partial sums
     int32_t nrb_max;     // row blocks of the BC reduction
     int32_t acc_grid;    // CTAs of the accumulation kernel
     int32_t acc_smem;    // dynamic shared memory of the accumulation kernel
@@ -196,8 +207,8 @@ struct Dev {
     int32_t tcap;        // targets recorded per row (kPairCap); more -> full re-accumulation
     uint32_t* chg;       // [n * chg_words] bit (s,t): pair changed in this update
     int32_t chg_words;   // (n + 31) / 32
-    void* oldD;          // [n*n] d(s,t) before the update, valid where the bit is set (DT)
-    uint64_t* oldS;      // [n*n] sigma_st before the update, likewise
+    void* oldD;          // [n*ld] d(s,t) before the update, valid where the bit is set (DT)
+    uint64_t* oldS;      // [n*ld] sigma_st before the update, likewise
     int32_t* tcnt;       // [n] changed targets of the row
     int32_t* tlist;      // [n * tcap]
     void* plan;          // [n * tcap] per-target scalars of the pair corrections (k_pair.cu)
@@ -246,6 +257,7 @@ struct PairRec {
     int32_t* tlist;
     int32_t tcap;
     int32_t first;       // no pair has changed yet in this update (the IN phase; row v)
+    int32_t ld;          // entries of a state row
 };
 
 // The recording buffers of a handle with pair corrections.
@@ -259,16 +271,13 @@ __host__ __device__ inline PairRec make_pair_rec(const Dev& d) {
     r.tlist = d.tlist;
     r.tcap = d.tcap;
     r.first = 0;
+    r.ld = d.ld;
     return r;
 }
 
-// Columns per thread of the pair-correction column test for n vertices: 16-byte (or two
-// 16-byte) loads where every row starts on a 16-byte boundary.
-constexpr int kPairVec32 = 8;   // columns per thread with int32 distances (4 or 8)
-__host__ __device__ inline int pair_vn(int dbytes, int n) {
-    if (dbytes == 4) return (kPairVec32 == 8 && n % 8 == 0) ? 8 : (n % 4 == 0 ? 4 : 1);
-    return n % 2 == 0 ? 2 : 1;
-}
+// Columns per thread of the pair-correction column test: two 16-byte loads of a row of
+// int32 distances, one of int64 ones.
+__host__ __device__ constexpr int pair_vn(int dbytes) { return dbytes == 4 ? 8 : 2; }
 
 // The first change of pair (s,t) in an update sets its bit, saves its old distance and
 // path count, and lists t as a changed target of row s (targets beyond the capacity
@@ -277,13 +286,13 @@ __host__ __device__ inline int pair_vn(int dbytes, int n) {
 // bit set by an earlier pass is visible, so a plain read of the word decides; the bit
 // is then set without waiting for the old word.
 template <typename DT>
-__device__ __forceinline__ void record_change(const PairRec& r, int n, int s, int t, int64_t d_old,
+__device__ __forceinline__ void record_change(const PairRec& r, int s, int t, int64_t d_old,
                                               uint64_t sig_old) {
     const uint32_t bit = 1u << (t & 31);
     uint32_t* w = r.chg + (size_t)s * r.chg_words + (t >> 5);
     if (!r.first && (*w & bit)) return;
     atomicOr(w, bit);
-    const size_t i = (size_t)s * n + t;
+    const size_t i = (size_t)s * r.ld + t;
     static_cast<DT*>(r.oldD)[i] = (DT)d_old;
     r.oldS[i] = sig_old;
     const int pos = atomicAdd(r.tcnt + s, 1);

@@ -20,6 +20,7 @@
 
 #include <cuda_runtime.h>
 
+#include "bc_internal.cuh"
 #include "bcgpu.h"
 
 namespace {
@@ -73,7 +74,7 @@ int64_t state_bytes(int32_t n, uint32_t flags) {
     // the change map (one bit per pair) for pair corrections
     const bool und = (flags & BC_UNDIRECTED) != 0;
     const int64_t per_pair = (sd + 16) + (und ? sd + 8 : 0);
-    return (int64_t)n * n * per_pair + (und ? (int64_t)n * n / 8 : 0) + (int64_t)n * 256 + (64 << 20);
+    return (int64_t)n * bcg::row_pitch(n) * per_pair + (und ? (int64_t)n * n / 8 : 0) + (int64_t)n * 256 + (64 << 20);
 }
 
 int evict(bc_server* s, int32_t gid) {

@@ -51,28 +51,18 @@ __global__ void __launch_bounds__(T, 1024 / T) k_accum_smem(AccArgs<DT> a) {
     }
 }
 
-__global__ void k_bc_partial(int n, const int32_t* rows, const int32_t* count, const ff* Dl,
-                             ff* partial, const int32_t* err) {
-    pdl_enter();
-    if (*err) return;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int total = rows ? *count : n;
-    for (int rb = blockIdx.y; rb * kRowsPerBlock < total; rb += gridDim.y)
-        dev_bc_partial(t, rb, n, rows, total, Dl, partial);
-}
-
-// The same partial sums for two adjacent columns per thread (n even): 16-byte loads of
-// both columns' float-float values, eight rows' loads issued before they are added;
+// Column partial sums (dev_bc_partial) for two adjacent columns per thread: 16-byte loads
+// of both columns' float-float values, eight rows' loads issued before they are added;
 // each column still adds its rows one by one in list order, as dev_bc_partial does, so
 // the sums are bit-identical.
 constexpr int kBcUnroll = 8;
-__global__ void __launch_bounds__(256) k_bc_partial2(int n, const int32_t* rows, const int32_t* count,
+__global__ void __launch_bounds__(256) k_bc_partial2(int n, int ld, const int32_t* rows, const int32_t* count,
                                                      const ff* Dl, ff* partial, const int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int t = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int total = rows ? *count : n;
-    if (t >= n) return;
+    if (t >= ld) return;
     for (int rb = blockIdx.y; rb * kRowsPerBlock < total; rb += gridDim.y) {
         const int r0 = rb * kRowsPerBlock;
         const int r1 = min(total, r0 + kRowsPerBlock);
@@ -84,7 +74,7 @@ __global__ void __launch_bounds__(256) k_bc_partial2(int n, const int32_t* rows,
             for (int k = 0; k < kBcUnroll; ++k) sr[k] = r + k < r1 ? (rows ? rows[r + k] : r + k) : -1;
 #pragma unroll
             for (int k = 0; k < kBcUnroll; ++k)
-                if (sr[k] >= 0) v[k] = __ldcs(reinterpret_cast<const float4*>(Dl + (size_t)sr[k] * n + t));
+                if (sr[k] >= 0) v[k] = __ldcs(reinterpret_cast<const float4*>(Dl + (size_t)sr[k] * ld + t));
 #pragma unroll
             for (int k = 0; k < kBcUnroll; ++k) {
                 if (sr[k] < 0) break;
@@ -92,17 +82,17 @@ __global__ void __launch_bounds__(256) k_bc_partial2(int n, const int32_t* rows,
                 if (sr[k] != t + 1) a1 = ff_add(a1, ff{v[k].z, v[k].w});
             }
         }
-        partial[(size_t)rb * n + t] = a0;
-        partial[(size_t)rb * n + t + 1] = a1;
+        partial[(size_t)rb * ld + t] = a0;
+        partial[(size_t)rb * ld + t + 1] = a1;
     }
 }
 
-__global__ void k_bc_finish(int n, const int32_t* rows, const int32_t* count, const ff* partial,
+__global__ void k_bc_finish(int n, int ld, const int32_t* rows, const int32_t* count, const ff* partial,
                             double sign, int overwrite, double* hi, double* lo, const int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) dev_bc_finish(t, n, rows ? *count : n, partial, sign, overwrite, hi, lo);
+    if (t < n) dev_bc_finish(t, ld, rows ? *count : n, partial, sign, overwrite, hi, lo);
 }
 
 // ------------------------------------------------------------------ launches
@@ -111,6 +101,7 @@ template <typename DT>
 static AccArgs<DT> acc_args(const Dev& d, const int32_t* rows, const int32_t* count) {
     AccArgs<DT> a;
     a.n = d.n;
+    a.ld = d.ld;
     a.D = (const DT*)d.D;
     a.S = d.S;
     a.Dl = d.Dl;
@@ -210,16 +201,10 @@ static int bc_row_ctas(const Dev& d, int col_blocks) {
 }
 
 static void bc_rows(const Dev& d, int sign, int is_static, const int32_t* rows, const int32_t* count) {
-    const int tb = (d.n + 255) / 256;
-    dim3 g1(tb, bc_row_ctas(d, tb));
-    if (d.n % 2 == 0) {
-        const int tb2 = (d.n / 2 + 255) / 256;
-        dim3 g2(tb2, bc_row_ctas(d, tb2));
-        launch_k(k_bc_partial2, g2, 256, 0, d.st, d.n, rows, count, d.Dl, d.partial, d.err);
-    } else {
-        launch_k(k_bc_partial, g1, 256, 0, d.st, d.n, rows, count, d.Dl, d.partial, d.err);
-    }
-    launch_k(k_bc_finish, tb, 256, 0, d.st, d.n, rows, count, d.partial, (double)sign, is_static, d.bc_hi, d.bc_lo,
+    const int tb = (d.n + 255) / 256, tb2 = (d.ld / 2 + 255) / 256;
+    launch_k(k_bc_partial2, dim3(tb2, bc_row_ctas(d, tb2)), 256, 0, d.st, d.n, d.ld, rows, count, d.Dl, d.partial,
+             d.err);
+    launch_k(k_bc_finish, tb, 256, 0, d.st, d.n, d.ld, rows, count, d.partial, (double)sign, is_static, d.bc_hi, d.bc_lo,
                                       d.err);
 }
 

@@ -57,26 +57,26 @@ __global__ void kb_vertex_pass(BatchArgs b, int r, int kind) {
         const DT* D = (const DT*)d.D;
         switch (kind) {
             case 0:
-                dev_alg4_in<DT>(x, d.n, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.mark, d.changed,
+                dev_alg4_in<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.mark, d.changed,
                                 d.err);
                 break;
             case 1:
-                dev_rows_out<DT>(x, d.n, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.mark, d.changed,
+                dev_rows_out<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.mark, d.changed,
                                  d.err);
                 break;
             case 2:
-                dev_alg4_out<DT>(x, d.n, D, d.S, u.v, e, u.k, d.directed, (DT*)d.cD, d.cS, d.cM, d.changed, d.err);
+                dev_alg4_out<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.cD, d.cS, d.cM, d.changed, d.err);
                 break;
             default:
                 if (d.pair_on) {
                     // row v is never written before this in an update: its changes are first changes
                     PairRec rec = make_pair_rec(d);
                     rec.first = 1;
-                    const size_t i = (size_t)u.v * d.n + x;
+                    const size_t i = (size_t)u.v * d.ld + x;
                     if (D[i] != ((const DT*)d.cD)[x] || d.S[i] != d.cS[x])
-                        record_change<DT>(rec, d.n, u.v, x, D[i], d.S[i]);
+                        record_change<DT>(rec, u.v, x, D[i], d.S[i]);
                 }
-                dev_write_row<DT>(x, d.n, (DT*)d.D, d.S, u.v, (const DT*)d.cD, d.cS, d.err);
+                dev_write_row<DT>(x, d.ld, (DT*)d.D, d.S, u.v, (const DT*)d.cD, d.cS, d.err);
         }
     }
 }
@@ -103,9 +103,8 @@ __global__ void __launch_bounds__(kCompactThreads) kb_compact(BatchArgs b, int r
 // Per-graph work known only on the device, as exclusive prefix offsets over graphs:
 // kind 0: scan items of the phase rows (rows x column chunks); 1: BC partial tasks
 // (column blocks x row blocks of the rows to re-accumulate); 2: sources to
-// re-accumulate; 3: rows listed for pair corrections; 4 + c: column-test weight of the
-// graphs whose columns per thread are of class c (and its piece counter back to zero).
-// One CTA.
+// re-accumulate; 3: rows listed for pair corrections; 4: column-test weight (and its
+// piece counter back to zero).  One CTA.
 __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, int phase_active, int64_t* out,
                                                 int scan_unroll) {
     __shared__ int64_t wsum[32];
@@ -123,7 +122,7 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
             if (on && *d.err == 0) {
                 if (kind == 0) {
                     const int cw = kScanThreads * (d.dbytes == 4 ? 4 : 2) * scan_unroll;
-                    v = (int64_t)d.counts[0] * ((d.n + cw - 1) / cw);
+                    v = (int64_t)d.counts[0] * ((d.ld + cw - 1) / cw);
                     atomicAdd(reinterpret_cast<unsigned long long*>(d.stats + 6), (unsigned long long)d.counts[0]);
                 } else if (kind == 1) {
                     v = (int64_t)((d.n + 255) / 256) * ((acc_list_count(d) + kRowsPerBlock - 1) / kRowsPerBlock);
@@ -131,7 +130,7 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
                     v = acc_list_count(d);
                 } else if (kind == 3) {
                     v = d.pair_on ? d.counts[1] : 0;
-                } else if (d.pair_on && pair_class(d.dbytes, pair_vn(d.dbytes, d.n)) == kind - 4) {
+                } else if (d.pair_on) {
                     v = d.pair_w[d.counts[5]];
                 }
             }
@@ -163,7 +162,7 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
     }
     if (threadIdx.x == 0) {
         out[G] = s_base;
-        if (kind >= 4) b.pctr[kind - 4] = 0;
+        if (kind == 4) *b.pctr = 0;
     }
 }
 
@@ -172,7 +171,7 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
 template <typename DT>
 __device__ __forceinline__ ScanArgs<DT> batch_scan_args(const Dev& d, const BatchUpd& u, int phase) {
     ScanArgs<DT> a;
-    a.n = d.n;
+    a.ld = d.ld;
     a.D = (DT*)d.D;
     a.S = d.S;
     a.rows = d.rows;
@@ -190,8 +189,8 @@ __device__ __forceinline__ ScanArgs<DT> batch_scan_args(const Dev& d, const Batc
     a.cD2 = nullptr;
     a.cS2 = a.cM2 = nullptr;
     if (phase == 0) {
-        a.cD = (const DT*)d.D + (size_t)u.v * d.n;
-        a.cS = d.S + (size_t)u.v * d.n;
+        a.cD = (const DT*)d.D + (size_t)u.v * d.ld;
+        a.cS = d.S + (size_t)u.v * d.ld;
         a.cM = a.cS;
         a.skip_row = -1;
         a.rec.first = 1;   // the IN phase is the first pass of an update that writes pairs
@@ -235,7 +234,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) kb_scan(BatchArgs b, int r, i
             cur = -1;
             const Dev& d = b.devs[g];
             a = batch_scan_args<DT>(d, b.upd[(int64_t)r * G + g], phase);
-            nchunks = (d.n + CW - 1) / CW;
+            nchunks = (d.ld + CW - 1) / CW;
         }
         const int64_t item = j - off[g];
         const int i = (int)(item / nchunks);
@@ -248,8 +247,7 @@ __global__ void __launch_bounds__(kScanThreads, 4) kb_scan(BatchArgs b, int r, i
             rm = a.fM[s];
         }
         if (rd == Inf<DT>::v) continue;
-        if (a.n % VN == 0) dev_scan_item<DT, true, U>(a, s, rd, rs, rm, c, n_changed, n_ties);
-        else dev_scan_item<DT, false, U>(a, s, rd, rs, rm, c, n_changed, n_ties);
+        dev_scan_item<DT, U>(a, s, rd, rs, rm, c, n_changed, n_ties);
     }
     if (cg >= 0) scan_stats(a.stats, n_changed, n_ties);
     else scan_stats(b.devs[0].stats, 0, 0);
@@ -268,7 +266,7 @@ __global__ void kb_bc_partial(BatchArgs b, int r, const int64_t* off) {
         const int tb = (d.n + 255) / 256;
         const int rb = (int)(task / tb);
         const int t = (int)(task - (int64_t)rb * tb) * 256 + threadIdx.x;
-        dev_bc_partial(t, rb, d.n, acc_list(d), acc_list_count(d), d.Dl, d.partial);
+        dev_bc_partial(t, rb, d.ld, acc_list(d), acc_list_count(d), d.Dl, d.partial);
     }
 }
 
@@ -282,7 +280,7 @@ __global__ void kb_bc_finish(BatchArgs b, int r, double sign) {
         const Dev& d = b.devs[g];
         if (*d.err || b.upd[(int64_t)r * G + g].present == 0) continue;
         const int t = (int)(j - off[g]);
-        dev_bc_finish(t, d.n, acc_list_count(d), d.partial, sign, 0, d.bc_hi, d.bc_lo);
+        dev_bc_finish(t, d.ld, acc_list_count(d), d.partial, sign, 0, d.bc_hi, d.bc_lo);
     }
 }
 
@@ -304,6 +302,7 @@ __global__ void __launch_bounds__(T, 1024 / T) kb_accum(BatchArgs b, int r, cons
         if (block_err(d.err)) continue;
         AccArgs<DT> a;
         a.n = d.n;
+        a.ld = d.ld;
         a.D = (const DT*)d.D;
         a.S = d.S;
         a.Dl = d.Dl;
@@ -358,7 +357,7 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     // in graphs with pair corrections only the rows over the target cap, and the others
     // are corrected pair by pair after (the order of the single-graph path)
     kb_compact<<<std::min(b.G, nsm * 2), kCompactThreads, 0, st>>>(b, r, 2);
-    if (L.pair_classes) batch_pair_lists(b, L, r, st);
+    if (L.pairs) batch_pair_lists(b, L, r, st);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 1, 2, b.plan_bc, L.scan_unroll);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 2, 2, b.plan_acc, L.scan_unroll);
     kb_bc_partial<<<nsm * L.bc_ctas, 256, 0, st>>>(b, r, b.plan_bc);
@@ -368,7 +367,7 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     else kb_accum<DT, 512><<<L.acc_grid, 512, L.acc_smem, st>>>(b, r, b.plan_acc);
     kb_bc_partial<<<nsm * L.bc_ctas, 256, 0, st>>>(b, r, b.plan_bc);
     kb_bc_finish<<<nsm * 2, 256, 0, st>>>(b, r, +1.0);
-    if (L.pair_classes) batch_pair_launches(b, L, r, sizeof(DT), st);
+    if (L.pairs) batch_pair_launches(b, L, r, sizeof(DT), st);
 }
 
 void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* out, int scan_unroll,

@@ -120,6 +120,7 @@ extern "C" int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* 
     if (scratch_address(&base) != cudaSuccess) return BC_ERR_CUDA;
     Dev d{};
     d.n = n;
+    d.ld = row_pitch(n);
     d.dbytes = i32 ? 4 : 8;
     d.directed = dir ? 1 : 0;
     d.st = (cudaStream_t)cuda_stream;

@@ -28,8 +28,8 @@ namespace bcg {
 
 constexpr int kPairThreads = 256;
 constexpr int kPairCtasPerSm = 4;
-// targets whose rows are loaded together: two with up to four columns per thread, one
-// with eight (whose two loads per target already overlap)
+// targets whose rows are loaded together: one with int32 distances (eight columns per
+// thread, whose two loads per target already overlap), two with int64 ones
 template <int VN> struct PairGroup { static constexpr int value = VN >= 8 ? 1 : 2; };
 constexpr int kPairPieces = 8;  // pieces of equal weight per CTA of the grid
 
@@ -169,6 +169,7 @@ static_assert(sizeof(PairTgt) == 40, "the plan is allocated with 40 bytes per ta
 template <typename DT>
 struct PairArgs {
     int n;
+    int ld;                 // entries of a state row
     const DT* D;            // state after the update
     const uint64_t* S;
     const uint32_t* chg;    // change map: bit (s,x) set where the pair changed
@@ -222,7 +223,6 @@ constexpr int kPlanThreads = 256;
 // (One warp; sv: kPairCap ints of shared memory.)
 template <typename DT>
 __device__ __forceinline__ void dev_pair_plan_row(const PairArgs<DT>& a, int s, int32_t* sv) {
-    const int n = a.n;
     const int64_t INF = Inf<DT>::v;
     const int lane = threadIdx.x & 31;
     const int T = a.tcnt[s];
@@ -233,7 +233,7 @@ __device__ __forceinline__ void dev_pair_plan_row(const PairArgs<DT>& a, int s, 
         const int val = sv[j];
         int pos = 0;
         for (int k = 0; k < T; ++k) pos += sv[k] < val;   // targets are distinct
-        const size_t it = (size_t)s * n + val;
+        const size_t it = (size_t)s * a.ld + val;
         const int64_t dol = a.oD[it], dnw = a.D[it];
         const uint64_t sol = a.oS[it], snw = a.S[it];
         PairTgt p;
@@ -265,24 +265,21 @@ __device__ __forceinline__ ff pair_term(uint64_t a, uint64_t b, const ff& rcp) {
     return ff_mul(ff_mul(ff_from_u64(a), ff_from_u64(b)), rcp);
 }
 
-// VN consecutive distances (one 16-byte load when VN > 1).
+// VN consecutive distances in 16-byte loads.
 template <typename DT, int VN>
 struct DVec {
     DT v[VN];
     __device__ __forceinline__ void load(const DT* p) {
-        if constexpr (VN == 8) {
+        if constexpr (sizeof(DT) == 4) {
+            static_assert(VN == 8, "two 16-byte loads");
             const int4 x = *reinterpret_cast<const int4*>(p);
             const int4 y = *reinterpret_cast<const int4*>(p + 4);
             v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
             v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
-        } else if constexpr (VN == 4) {
-            const int4 x = *reinterpret_cast<const int4*>(p);
-            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-        } else if constexpr (VN == 2) {
+        } else {
+            static_assert(VN == 2, "one 16-byte load");
             const longlong2 x = *reinterpret_cast<const longlong2*>(p);
             v[0] = x.x; v[1] = x.y;
-        } else {
-            v[0] = p[0];
         }
     }
 };
@@ -336,7 +333,7 @@ struct TgtFast {
     DT dold, dnew;
 };
 struct TgtSlow {
-    int64_t rt;      // t * n
+    int64_t rt;      // t * ld
     ff rold, rnew;
 };
 
@@ -537,10 +534,9 @@ __device__ __forceinline__ void pair_item(const PairArgs<DT>& a, int s, int U_, 
     static_assert(2 * VN * kPairGroup <= 32 && VN <= 8, "a group's matches fit one 32-bit mask");
     using U = typename Unsigned<DT>::T;
     constexpr unsigned kMask = (1u << VN) - 1u;
-    const int n = a.n;
     const int lane = threadIdx.x & 31;
-    const size_t rs = (size_t)s * n;
-    const bool active = x0 < n;   // the warp runs the item together (the queue needs every lane)
+    const size_t rs = (size_t)s * a.ld;
+    const bool active = x0 < a.n;   // the warp runs the item together (the queue needs every lane)
     DVec<DT, VN> dsn, dso;
     unsigned bs = 0;
     if (active) {
@@ -725,7 +721,7 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) k_pairdep(PairAr
                     __syncthreads();   // the previous row's plan is no longer read
                     if (threadIdx.x < U_) {
                         const PairTgt p = a.plan[(size_t)s * a.tcap + threadIdx.x];
-                        const size_t rt = (size_t)p.t * n;
+                        const size_t rt = (size_t)p.t * a.ld;
                         s_fa[threadIdx.x] =
                             TgtFast<DT>{a.D + rt, a.chg + (size_t)p.t * a.words, (DT)p.dold, (DT)p.dnew};
                         s_sl[threadIdx.x] = TgtSlow{(int64_t)rt, p.rold, p.rnew};
@@ -793,6 +789,7 @@ template <typename DT>
 __host__ __device__ inline PairArgs<DT> pair_args(const Dev& d) {
     PairArgs<DT> a;
     a.n = d.n;
+    a.ld = d.ld;
     a.D = (const DT*)d.D;
     a.S = d.S;
     a.chg = d.chg;
@@ -860,14 +857,14 @@ __global__ void __launch_bounds__(kPlanThreads) kb_pair_plan(BatchArgs b) {
 }
 
 // One CTA per graph in turn: rows most targets first and their weight prefix
-// (k_pair_weights), with the graph's own columns per thread.
+// (k_pair_weights).
 __global__ void __launch_bounds__(1024) kb_pair_weights(BatchArgs b, int r, int scap) {
     __shared__ PairWeightsSmem sm;
     extern __shared__ int32_t s_stage[];   // 2 * scap ints
     for (int g = blockIdx.x; g < b.G; g += gridDim.x) {
         if (!batch_pair_graph(b, r, g)) continue;   // block-uniform
         const Dev& d = b.devs[g];
-        const int cw = kPairThreads * pair_vn(d.dbytes, d.n);
+        const int cw = kPairThreads * pair_vn(d.dbytes);
         const int nchunks = (d.n + cw - 1) / cw;
         dev_pair_weights(d.acc_rows, d.counts + 1, d.tcnt, d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w,
                          d.stats, d.counts + 4, nullptr, nullptr, sm, s_stage, s_stage + scap, scap);
@@ -875,12 +872,12 @@ __global__ void __launch_bounds__(1024) kb_pair_weights(BatchArgs b, int r, int 
     }
 }
 
-// The column test (k_pairdep) over the graphs whose columns per thread are VN: their
-// weight lines laid end to end (plan_pw of the class), cut into kPairPieces x grid pieces
-// of equal weight; a piece runs the items whose start falls in it, across row and graph
-// boundaries, and later pieces go to the CTAs that finish first (counter pctr).
+// The column test (k_pairdep) over every graph with corrections: their weight lines laid
+// end to end (plan_pw), cut into kPairPieces x grid pieces of equal weight; a piece runs
+// the items whose start falls in it, across row and graph boundaries, and later pieces go
+// to the CTAs that finish first (counter pctr).
 template <typename DT, int VN>
-__global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) kb_pairdep(BatchArgs b, int cls) {
+__global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) kb_pairdep(BatchArgs b) {
     __shared__ TgtFast<DT> s_fa[kPairCap];
     __shared__ TgtSlow s_sl[kPairCap];
     __shared__ ff s_acc[VN][kPairThreads];
@@ -888,7 +885,7 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) kb_pairdep(Batch
     __shared__ int s_g, s_i, s_c, s_p;
     constexpr int CW = kPairThreads * VN;
     const int G = b.G;
-    const int64_t* off = b.plan_pw + (int64_t)cls * (G + 1);
+    const int64_t* off = b.plan_pw;
     const int64_t W = off[G];
     const int npieces = gridDim.x * kPairPieces;
     int cg = -1;                     // the graph whose arguments are loaded
@@ -954,7 +951,7 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) kb_pairdep(Batch
                     __syncthreads();   // the previous row's plan is no longer read
                     if (threadIdx.x < U_) {
                         const PairTgt p = a.plan[(size_t)s * a.tcap + threadIdx.x];
-                        const size_t rt = (size_t)p.t * a.n;
+                        const size_t rt = (size_t)p.t * a.ld;
                         s_fa[threadIdx.x] =
                             TgtFast<DT>{a.D + rt, a.chg + (size_t)p.t * a.words, (DT)p.dold, (DT)p.dnew};
                         s_sl[threadIdx.x] = TgtSlow{(int64_t)rt, p.rold, p.rnew};
@@ -967,7 +964,7 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) kb_pairdep(Batch
                     pair_item<DT, VN>(a, s, U_, x0, s_fa, s_sl, s_acc, s_wq[threadIdx.x >> 5]);
             }
         }
-        if (threadIdx.x == 0) s_p = gridDim.x + atomicAdd(b.pctr + cls, 1);
+        if (threadIdx.x == 0) s_p = gridDim.x + atomicAdd(b.pctr, 1);
         __syncthreads();
         piece = s_p;
         __syncthreads();
@@ -1013,18 +1010,8 @@ static void batch_pairs(const BatchArgs& b, const BatchLaunch& L, int r, cudaStr
     const int scap = weights_stage(b.n_max);
     kb_pair_weights<<<std::min(G, nsm * 2), 1024, 2 * sizeof(int32_t) * (size_t)scap, st>>>(b, r, scap);
     const int pgrid = nsm * kPairCtasPerSm;
-    for (int c = 0; c < kPairClasses; ++c) {
-        if (!((L.pair_classes >> c) & 1)) continue;
-        batch_plan(b, r, 4 + c, 2, b.plan_pw + (int64_t)c * (G + 1), L.scan_unroll, st);
-        if constexpr (sizeof(DT) == 4) {
-            if (c == 0) kb_pairdep<DT, 8><<<pgrid, kPairThreads, 0, st>>>(b, c);
-            else if (c == 1) kb_pairdep<DT, 4><<<pgrid, kPairThreads, 0, st>>>(b, c);
-            else kb_pairdep<DT, 1><<<pgrid, kPairThreads, 0, st>>>(b, c);
-        } else {
-            if (c == 0) kb_pairdep<DT, 2><<<pgrid, kPairThreads, 0, st>>>(b, c);
-            else kb_pairdep<DT, 1><<<pgrid, kPairThreads, 0, st>>>(b, c);
-        }
-    }
+    batch_plan(b, r, 4, 2, b.plan_pw, L.scan_unroll, st);
+    kb_pairdep<DT, pair_vn(sizeof(DT))><<<pgrid, kPairThreads, 0, st>>>(b);
     kb_bc_fix<<<nsm * 4, 256, 0, st>>>(b, r);
     kb_pair_clear<<<nsm * 4, 256, 0, st>>>(b, r);
 }
@@ -1145,7 +1132,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkCtasPerSm) k_walk_units(Pai
             const int u = (int)(id - unit_start<DT>(a, w.nchunks, L));
             const PairTgt& pt = a.plan[(size_t)s * a.tcap + u];
             const int t = pt.t;
-            const size_t rs = (size_t)s * n;
+            const size_t rs = (size_t)s * a.ld;
             for (int stt = 0; stt < 2; ++stt) {
                 const bool is_new = stt == 1;
                 int found = 0;   // warp-uniform
@@ -1311,7 +1298,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkRowCtasPerSm) k_walk_rows(P
         const int s = a.prows[r];
         const int T = a.tcnt[s];
         const int64_t id0 = unit_start<DT>(a, w.nchunks, r);
-        const size_t rs = (size_t)s * n;
+        const size_t rs = (size_t)s * a.ld;
         // the row's walks (2 per target) go to the warps in turn
         for (int q = wib; q < 2 * T; q += kWalkWarps) {
             const int u = q >> 1;
@@ -1320,7 +1307,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkRowCtasPerSm) k_walk_rows(P
             const int64_t base = w.useg[(id0 + u) * 4 + 2 * (q & 1)];
             const int len = w.useg[(id0 + u) * 4 + 2 * (q & 1) + 1];
             const ff rcp = is_new ? pt.rnew : pt.rold;
-            const size_t rt = (size_t)pt.t * n;
+            const size_t rt = (size_t)pt.t * a.ld;
             for (int i = lane; i < len; i += 32) {
                 const int x = w.buf[base + i];
                 ff term = pair_term(walk_sigma<DT>(a, rs, s, x, is_new), walk_sigma<DT>(a, rt, pt.t, x, is_new), rcp);
@@ -1412,7 +1399,7 @@ __global__ void __launch_bounds__(H::threads, H::ctas) k_walk_rows_hash(PairArgs
         const int s = a.prows[r];
         const int T = a.tcnt[s];
         const int64_t id0 = unit_start<DT>(a, w.nchunks, r);
-        const size_t rs = (size_t)s * n;
+        const size_t rs = (size_t)s * a.ld;
         for (int q = wib; q < 2 * T; q += kW) {
             const int u = q >> 1;
             const bool is_new = q & 1;
@@ -1420,7 +1407,7 @@ __global__ void __launch_bounds__(H::threads, H::ctas) k_walk_rows_hash(PairArgs
             const int64_t base = w.useg[(id0 + u) * 4 + 2 * (q & 1)];
             const int len = w.useg[(id0 + u) * 4 + 2 * (q & 1) + 1];
             const ff rcp = is_new ? pt.rnew : pt.rold;
-            const size_t rt = (size_t)pt.t * n;
+            const size_t rt = (size_t)pt.t * a.ld;
             for (int i = lane; i < len; i += 32) {
                 const int x = w.buf[base + i];
                 ff term = pair_term(walk_sigma<DT>(a, rs, s, x, is_new), walk_sigma<DT>(a, rt, pt.t, x, is_new), rcp);
@@ -1480,7 +1467,7 @@ cudaError_t walk_setup() {
 }
 
 template <typename DT>
-static void launch_walks(const Dev& d, const WalkUpd& upd, int nchunks, int vn) {
+static void launch_walks(const Dev& d, const WalkUpd& upd, int nchunks) {
     const int grid = d.nsm * kWalkCtasPerSm, rgrid = d.nsm * kWalkRowCtasPerSm;
     WalkArgs<DT> w{d.e_off, d.e_len, (const Arc<DT>*)d.e_arc, d.walk_list, d.walk_buf, d.walk_cap, d.walk_useg,
                    d.walk_acc2, d.walk_tl, d.walk_ctl, d.walk_rowE, d.stats, nchunks, upd};
@@ -1503,22 +1490,14 @@ static void launch_walks(const Dev& d, const WalkUpd& upd, int nchunks, int vn) 
     PairArgs<DT> a = pair_args<DT>(d);
     a.gate = d.walk_ctl + 4;
     const int pgrid = d.nsm * kPairCtasPerSm;
-    if constexpr (sizeof(DT) == 4) {
-        if (vn == 8) launch_k(k_pairdep<DT, 8>, pgrid, kPairThreads, 0, d.st, a);
-        else if (vn == 4) launch_k(k_pairdep<DT, 4>, pgrid, kPairThreads, 0, d.st, a);
-        else launch_k(k_pairdep<DT, 1>, pgrid, kPairThreads, 0, d.st, a);
-    } else {
-        if (vn == 2) launch_k(k_pairdep<DT, 2>, pgrid, kPairThreads, 0, d.st, a);
-        else launch_k(k_pairdep<DT, 1>, pgrid, kPairThreads, 0, d.st, a);
-    }
+    launch_k(k_pairdep<DT, pair_vn(sizeof(DT))>, pgrid, kPairThreads, 0, d.st, a);
 }
 
 void launch_pairdep(const Dev& d, const WalkUpd* upd) {
     const int pgrid = d.nsm * 8;
     if (d.dbytes == 4) launch_k(k_pair_plan<int32_t>, pgrid, kPlanThreads, 0, d.st, pair_args<int32_t>(d));
     else launch_k(k_pair_plan<int64_t>, pgrid, kPlanThreads, 0, d.st, pair_args<int64_t>(d));
-    // columns per thread: 16-byte (or two 16-byte) loads where n allows them
-    const int vn = pair_vn(d.dbytes, d.n);
+    const int vn = pair_vn(d.dbytes);
     const int cw = kPairThreads * vn;
     const int nchunks = (d.n + cw - 1) / cw;
     const int scap = weights_stage(d.n);
@@ -1526,19 +1505,13 @@ void launch_pairdep(const Dev& d, const WalkUpd* upd) {
              d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w, d.stats, d.counts + 4,
              upd ? d.walk_ctl : nullptr, upd ? d.walk_rowE : nullptr, d.err, scap);
     if (upd) {
-        if (d.dbytes == 4) launch_walks<int32_t>(d, *upd, nchunks, vn);
-        else launch_walks<int64_t>(d, *upd, nchunks, vn);
+        if (d.dbytes == 4) launch_walks<int32_t>(d, *upd, nchunks);
+        else launch_walks<int64_t>(d, *upd, nchunks);
         return;
     }
     const int grid = d.nsm * kPairCtasPerSm;   // one resident wave; later pieces go to the first free CTA
-    if (d.dbytes == 4) {
-        if (vn == 8) launch_k(k_pairdep<int32_t, 8>, grid, kPairThreads, 0, d.st, pair_args<int32_t>(d));
-        else if (vn == 4) launch_k(k_pairdep<int32_t, 4>, grid, kPairThreads, 0, d.st, pair_args<int32_t>(d));
-        else launch_k(k_pairdep<int32_t, 1>, grid, kPairThreads, 0, d.st, pair_args<int32_t>(d));
-    } else {
-        if (vn == 2) launch_k(k_pairdep<int64_t, 2>, grid, kPairThreads, 0, d.st, pair_args<int64_t>(d));
-        else launch_k(k_pairdep<int64_t, 1>, grid, kPairThreads, 0, d.st, pair_args<int64_t>(d));
-    }
+    if (d.dbytes == 4) launch_k(k_pairdep<int32_t, 8>, grid, kPairThreads, 0, d.st, pair_args<int32_t>(d));
+    else launch_k(k_pairdep<int64_t, 2>, grid, kPairThreads, 0, d.st, pair_args<int64_t>(d));
 }
 
 void launch_bc_fix(const Dev& d) {

@@ -45,7 +45,7 @@ __device__ __forceinline__ int64_t atomic_min_dt(int64_t* p, int64_t v) {
 // copy of the arc heads to prune (NULL: every arc is searched, dst is read).
 template <typename DT, bool SMEM_DIST>
 __global__ void __launch_bounds__(kSsspThreads)
-k_sssp(int n, const int32_t* __restrict__ off, const int32_t* __restrict__ dst,
+k_sssp(int n, int ld, const int32_t* __restrict__ off, const int32_t* __restrict__ dst,
        const DT* __restrict__ w, DT* D, int32_t* err, const int32_t* __restrict__ order, int32_t* pdst) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int words = (n + 31) >> 5;
@@ -60,7 +60,7 @@ k_sssp(int n, const int32_t* __restrict__ off, const int32_t* __restrict__ dst,
     for (int si = blockIdx.x; si < n; si += gridDim.x) {
         if (block_err(err)) return;
         const int s = order ? order[si] : si;
-        DT* dist = SMEM_DIST ? dist_s : D + (size_t)s * n;
+        DT* dist = SMEM_DIST ? dist_s : D + (size_t)s * ld;
         for (int t = tid; t < n; t += kSsspThreads) dist[t] = (t == s) ? (DT)0 : (DT)INF;
         for (int q = tid; q < words; q += kSsspThreads) {
             cur[q] = (q == (s >> 5)) ? (1u << (s & 31)) : 0u;
@@ -119,9 +119,10 @@ k_sssp(int n, const int32_t* __restrict__ off, const int32_t* __restrict__ dst,
             }
         }
         if (SMEM_DIST) {
-            DT* row = D + (size_t)s * n;
+            DT* row = D + (size_t)s * ld;
             for (int t = tid; t < n; t += kSsspThreads) row[t] = dist_s[t];
         }
+        if (tid < ld - n) D[(size_t)s * ld + n + tid] = (DT)INF;   // the entries past n: no path
         // the search from s is final: the arcs of s with w(s,b) > d(s,b) are not in E*
         if (pdst)
             for (int e = off[s] + tid; e < off[s + 1]; e += kSsspThreads) {
@@ -133,11 +134,11 @@ k_sssp(int n, const int32_t* __restrict__ off, const int32_t* __restrict__ dst,
 }
 
 template <typename DT>
-__global__ void k_estar_flags(int n, int64_t arcs, const int32_t* g_src, const int32_t* g_dst,
+__global__ void k_estar_flags(int ld, int64_t arcs, const int32_t* g_src, const int32_t* g_dst,
                               const DT* g_w, const DT* D, uint8_t* flags) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= arcs) return;
-    flags[e] = ((int64_t)D[(size_t)g_src[e] * n + g_dst[e]] == (int64_t)g_w[e]) ? 1 : 0;
+    flags[e] = ((int64_t)D[(size_t)g_src[e] * ld + g_dst[e]] == (int64_t)g_w[e]) ? 1 : 0;
 }
 
 template <typename DT>
@@ -153,7 +154,7 @@ static void sssp_dispatch(const Dev& d) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp<DT, true>, kSsspThreads, smem);
         if (per_sm < 1) per_sm = 1;
         const int grid = (int)std::min<int64_t>((int64_t)d.nsm * per_sm, d.n);
-        k_sssp<DT, true><<<grid, kSsspThreads, smem, d.st>>>(d.n, d.g_off, d.g_dst, (const DT*)d.g_w,
+        k_sssp<DT, true><<<grid, kSsspThreads, smem, d.st>>>(d.n, d.ld, d.g_off, d.g_dst, (const DT*)d.g_w,
                                                              (DT*)d.D, d.err, d.s_order, d.p_dst);
     } else {
         const size_t smem = bitmaps;
@@ -162,7 +163,7 @@ static void sssp_dispatch(const Dev& d) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp<DT, false>, kSsspThreads, smem);
         if (per_sm < 1) per_sm = 1;
         const int grid = (int)std::min<int64_t>((int64_t)d.nsm * per_sm, d.n);
-        k_sssp<DT, false><<<grid, kSsspThreads, smem, d.st>>>(d.n, d.g_off, d.g_dst, (const DT*)d.g_w,
+        k_sssp<DT, false><<<grid, kSsspThreads, smem, d.st>>>(d.n, d.ld, d.g_off, d.g_dst, (const DT*)d.g_w,
                                                               (DT*)d.D, d.err, d.s_order, d.p_dst);
     }
 }
@@ -176,10 +177,10 @@ void launch_estar_flags(const Dev& d, uint8_t* flags) {
     if (d.g_arcs <= 0) return;
     const int blocks = (int)((d.g_arcs + 255) / 256);
     if (d.dbytes == 4)
-        k_estar_flags<int32_t><<<blocks, 256, 0, d.st>>>(d.n, d.g_arcs, d.g_src, d.g_dst,
+        k_estar_flags<int32_t><<<blocks, 256, 0, d.st>>>(d.ld, d.g_arcs, d.g_src, d.g_dst,
                                                          (const int32_t*)d.g_w, (const int32_t*)d.D, flags);
     else
-        k_estar_flags<int64_t><<<blocks, 256, 0, d.st>>>(d.n, d.g_arcs, d.g_src, d.g_dst,
+        k_estar_flags<int64_t><<<blocks, 256, 0, d.st>>>(d.ld, d.g_arcs, d.g_src, d.g_dst,
                                                          (const int64_t*)d.g_w, (const int64_t*)d.D, flags);
 }
 

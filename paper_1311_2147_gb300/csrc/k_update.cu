@@ -9,12 +9,12 @@
 //   IN  (E_i):  k_alg4_in   Algorithm 4 for every source s -> d'(s,v), sigma'_sv,
 //                           sigma-hat'_sv, and whether row s can change;
 //               k_compact   rows that change, in increasing order;
-//               k_scan      Lemma 4 over those rows: D(s,t) = d'(s,v) + d(v,t).
+//               k_scan_cs    Lemma 4 over those rows: D(s,t) = d'(s,v) + d(v,t).
 //   OUT (E_o):  k_alg4_out  Algorithm 4 on the reversed graph G'_R for every target t
 //                           -> d''(v,t), sigma''_vt, sigma-hat''_vt (row v of the
 //                           result; reads rows x_j of D', which are contiguous);
 //               k_rows_out  rows s with d'(s,v) + w'(v,x_j) <= d'(s,x_j) for some j;
-//               k_compact, k_scan  Lemma 4 read on G'_R: D(s,t) = d'(s,v) + d''(v,t);
+//               k_compact, k_scan_cs  Lemma 4 read on G'_R: D(s,t) = d'(s,v) + d''(v,t);
 //               k_write_row row v <- (d''(v,.), sigma''_v.).
 //
 // Lemma 1 (and its vertex analogue) makes the in-place scan race free: during the IN
@@ -52,7 +52,7 @@ __global__ void k_estar_move(int32_t* e_off, int32_t* e_src, Arc<DT>* e_arc, EMo
 }
 
 template <typename DT>
-__global__ void k_alg4_in(int n, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__global__ void k_alg4_in(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                           int v, const VEdge* __restrict__ e, int k, int directed,
                           DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
                           int32_t* err) {
@@ -60,29 +60,29 @@ __global__ void k_alg4_in(int n, const DT* __restrict__ D, const uint64_t* __res
     if (*err) return;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    if (directed) dev_alg4_in<DT, false>(s, n, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
-    else dev_alg4_in<DT, true>(s, n, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
+    if (directed) dev_alg4_in<DT, false>(s, ld, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
+    else dev_alg4_in<DT, true>(s, ld, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
 }
 
 template <typename DT>
-__global__ void k_rows_out(int n, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__global__ void k_rows_out(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
                            DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
                            int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) dev_rows_out<DT>(s, n, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
+    if (s < n) dev_rows_out<DT>(s, ld, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
 }
 
 template <typename DT>
-__global__ void k_alg4_out(int n, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__global__ void k_alg4_out(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
                            DT* cD, uint64_t* cS, uint64_t* cM, uint8_t* changed, int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) dev_alg4_out<DT>(t, n, D, S, v, e, k, directed, cD, cS, cM, changed, err);
+    if (t < n) dev_alg4_out<DT>(t, ld, D, S, v, e, k, directed, cD, cS, cM, changed, err);
 }
 
 __global__ void __launch_bounds__(kCompactThreads)
@@ -92,48 +92,8 @@ k_compact(int n, uint8_t* mark, int clear, int32_t* rows, int32_t* count, int fu
     dev_compact(n, mark, clear, rows, count, full, stats, err);
 }
 
-// K2: in-place rank-1 min-plus / path-count pass over rows[0..count) x all columns.
-// Work item = (row, chunk of CW columns).  Each CTA takes a contiguous block of items,
-// so the per-row scalars are loaded once per row it meets; each thread issues all of
-// its 16-byte loads of D and of the column vectors of an item before using any.  sigma
-// is read only on ties and written only where the pair changes.
-template <typename DT, bool VECTOR>
-__global__ void __launch_bounds__(kScanThreads, 4) k_scan(ScanArgs<DT> a) {
-    pdl_enter();
-    // warp-uniform early exit: the warp sum at the end needs every lane
-    int bad = 0;
-    if ((threadIdx.x & 31) == 0) bad = *reinterpret_cast<volatile int32_t*>(a.err);
-    if (__shfl_sync(0xffffffffu, bad, 0)) return;
-    constexpr int CW = kScanThreads * Vec<DT>::N * kScanUnroll;
-    const int nchunks = (a.n + CW - 1) / CW;
-    const int64_t total = (int64_t)(*a.count) * nchunks;
-    const int64_t per = (total + gridDim.x - 1) / gridDim.x;
-    const int64_t it0 = (int64_t)blockIdx.x * per;
-    const int64_t it1 = min(total, it0 + per);
-    const int64_t INF = Inf<DT>::v;
-    int n_changed = 0, n_ties = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 6),
-                                                       (unsigned long long)(*a.count));
-    int cur = -1, s = -1;
-    int64_t rd = INF;
-    uint64_t rs = 0, rm = 0;
-    for (int64_t item = it0; item < it1; ++item) {
-        const int i = (int)(item / nchunks);
-        const int c = (int)(item - (int64_t)i * nchunks);
-        if (i != cur) {
-            cur = i;
-            s = a.rows[i];
-            rd = (s == a.skip_row) ? INF : (int64_t)a.fD[s];
-            rs = a.fS[s];
-            rm = a.fM[s];
-        }
-        if (rd == INF) continue;
-        dev_scan_item<DT, VECTOR>(a, s, rd, rs, rm, c, n_changed, n_ties);
-    }
-    scan_stats(a.stats, n_changed, n_ties);
-}
-
-// K2, vector path (n a multiple of the vector width): column-stationary CTAs.  CTA b
+// K2: in-place rank-1 min-plus / path-count pass over rows[0..count) x all columns, by
+// column-stationary CTAs (every row of the state starts on a 16-byte boundary).  CTA b
 // owns column chunk c = b mod nch (kCsThreads threads x kCsVpt 16-byte vectors) for
 // the whole launch and walks the rows i = b / nch, + gridDim / nch, ... of the list.
 // Its column values -- with the tie_cols bump, for the quick test -- sit in registers,
@@ -159,7 +119,7 @@ template <int N>
 __device__ __forceinline__ void cs_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void cs_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// WHOLE: n is a multiple of the chunk width, so no column of a chunk lies past n.
+// WHOLE: ld is a multiple of the chunk width, so no column of a chunk lies past it.
 // DUAL: two row lists, each with its own column vector (a.rows2 set).
 template <typename DT, bool WHOLE, bool DUAL>
 __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<DT> a, int nch) {
@@ -174,7 +134,7 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
     __shared__ unsigned long long s_cmax;
     if (block_err(a.err)) return;
     const int tid = threadIdx.x;
-    const int n = a.n;
+    const int ld = a.ld;
     const int64_t INF = Inf<DT>::v;
     int gpc = (int)gridDim.x / nch;   // CTAs per column chunk
     const int c = (int)blockIdx.x % nch;
@@ -210,7 +170,7 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
 #pragma unroll
     for (int u = 0; u < kCsVpt; ++u) {
         const int t = t0 + (u * kCsThreads + tid) * VN;
-        if (WHOLE || t < n) {
+        if (WHOLE || t < ld) {
             VT x = __ldg(reinterpret_cast<const VT*>(((DUAL && second) ? a.cD2 : a.cD) + t));
             int64_t xv[VN];
             V::unpack(x, xv);
@@ -260,11 +220,11 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
         ring_d[st] = __shfl_sync(0xffffffffu, cur_d, j);
         ring_m[st] = __shfl_sync(0xffffffffu, cur_m, j);
         if (s >= 0) {
-            const DT* src = a.D + (size_t)s * n;
+            const DT* src = a.D + (size_t)s * ld;
 #pragma unroll
             for (int u = 0; u < kCsVpt; ++u) {
                 const int t = t0 + (u * kCsThreads + tid) * VN;
-                if (WHOLE || t < n) cs_copy16(&stage[st][u][tid], src + t);
+                if (WHOLE || t < ld) cs_copy16(&stage[st][u][tid], src + t);
             }
         }
         cs_commit();
@@ -284,7 +244,7 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
             const int2 e = wq[lane];
             s = e.x;
             t = e.y;
-            const size_t rowoff = (size_t)s * n;
+            const size_t rowoff = (size_t)s * ld;
             const int64_t rd = (int64_t)a.fD[s];
             const uint64_t rs = a.fS[s], rm = a.fM[s];
             VT dv = *reinterpret_cast<const VT*>(a.D + rowoff + t);
@@ -294,7 +254,7 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
             if (m & 0xffu) *reinterpret_cast<VT*>(a.D + rowoff + t) = dv;
             bits = (m | (m >> 8)) & 0xffu;
         }
-        if (a.rec.tcnt) record_changes_warp<DT>(a.rec, n, s, t, bits, dold, sold);
+        if (a.rec.tcnt) record_changes_warp<DT>(a.rec, s, t, bits, dold, sold);
     };
 #pragma unroll
     for (int st = 0; st < ST; ++st) issue(st);
@@ -319,7 +279,7 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
 #pragma unroll
                     for (int u = 0; u < kCsVpt; ++u) {
                         const int t = t0 + (u * kCsThreads + tid) * VN;
-                        if (WHOLE || t < n) {
+                        if (WHOLE || t < ld) {
                             const VT x = stage[st][u][tid];
                             const DT* xd = reinterpret_cast<const DT*>(&x);
                             const DT* cd = reinterpret_cast<const DT*>(&cq[u]);
@@ -331,14 +291,14 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
 #pragma unroll
                         for (int u = 0; u < kCsVpt; ++u) {
                             const int t = t0 + (u * kCsThreads + tid) * VN;
-                            if ((WHOLE || t < n) && quick_vec<DT>(stage[st][u][tid], cq[u], rq, true)) cand |= 1u << u;
+                            if ((WHOLE || t < ld) && quick_vec<DT>(stage[st][u][tid], cq[u], rq, true)) cand |= 1u << u;
                         }
                     }
                 } else {
 #pragma unroll
                     for (int u = 0; u < kCsVpt; ++u) {
                         const int t = t0 + (u * kCsThreads + tid) * VN;
-                        if ((WHOLE || t < n) && quick_vec<DT>(stage[st][u][tid], cq[u], rq, false)) cand |= 1u << u;
+                        if ((WHOLE || t < ld) && quick_vec<DT>(stage[st][u][tid], cq[u], rq, false)) cand |= 1u << u;
                     }
                 }
                 // candidates go to the warp's queue (a row adds at most 32 x kCsVpt); the
@@ -377,29 +337,29 @@ __global__ void __launch_bounds__(kCsThreads, kCsCtasPerSm) k_scan_cs(ScanArgs<D
 }
 
 template <typename DT>
-__global__ void k_write_row(int n, DT* D, uint64_t* S, int v, const DT* cD, const uint64_t* cS, PairRec rec,
+__global__ void k_write_row(int n, int ld, DT* D, uint64_t* S, int v, const DT* cD, const uint64_t* cS, PairRec rec,
                             const int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     if (rec.tcnt) {
-        const size_t i = (size_t)v * n + t;
-        if (D[i] != cD[t] || S[i] != cS[t]) record_change<DT>(rec, n, v, t, D[i], S[i]);
+        const size_t i = (size_t)v * ld + t;
+        if (D[i] != cD[t] || S[i] != cS[t]) record_change<DT>(rec, v, t, D[i], S[i]);
     }
-    dev_write_row<DT>(t, n, D, S, v, cD, cS, err);
+    dev_write_row<DT>(t, ld, D, S, v, cD, cS, err);
 }
 
 // keep[e] = 1 when slot e holds an arc (a,b) with w(a,b) == d(a,b), i.e. an arc of E*
 // (an arc lies on a shortest path exactly when it is one itself).
 template <typename DT>
-__global__ void k_estar_keep(int n, const DT* D, const int32_t* e_src, const Arc<DT>* e_arc,
+__global__ void k_estar_keep(int ld, const DT* D, const int32_t* e_src, const Arc<DT>* e_arc,
                              int64_t cap, uint8_t* keep) {
     pdl_enter();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= cap) return;
     const Arc<DT> a = e_arc[e];
-    keep[e] = (a.dst >= 0 && (int64_t)D[(size_t)e_src[e] * n + a.dst] == (int64_t)a.w) ? 1 : 0;
+    keep[e] = (a.dst >= 0 && (int64_t)D[(size_t)e_src[e] * ld + a.dst] == (int64_t)a.w) ? 1 : 0;
 }
 
 // Fused pass of an undirected edge update {u, v} with weight w, preparation (one thread
@@ -417,7 +377,7 @@ __global__ void k_estar_keep(int n, const DT* D, const int32_t* e_src, const Arc
 // passes' d and sigma.  Rows are appended with one atomic per warp and list (the counts
 // start at zero); the order of a list does not affect any result.
 template <typename DT>
-__global__ void k_edge_prep(int n, const DT* D, const uint64_t* S, int u, int v, int64_t w, DT* cDv,
+__global__ void k_edge_prep(int n, int ld, const DT* D, const uint64_t* S, int u, int v, int64_t w, DT* cDv,
                             uint64_t* cSv, DT* cDu, uint64_t* cSu, DT* fD, uint64_t* fS, uint64_t* fM,
                             int32_t* rows1, int32_t* count1, int32_t* rows2, int32_t* count2,
                             uint8_t* changed, int32_t* err) {
@@ -428,8 +388,8 @@ __global__ void k_edge_prep(int n, const DT* D, const uint64_t* S, int u, int v,
     const int64_t INF = Inf<DT>::v;
     bool in1 = false, in2 = false;
     if (s < n) {
-        const int64_t du = D[(size_t)u * n + s], dv = D[(size_t)v * n + s];
-        const uint64_t su = S[(size_t)u * n + s], sv = S[(size_t)v * n + s];
+        const int64_t du = D[(size_t)u * ld + s], dv = D[(size_t)v * ld + s];
+        const uint64_t su = S[(size_t)u * ld + s], sv = S[(size_t)v * ld + s];
         cDu[s] = (DT)du;
         cSu[s] = su;
         cDv[s] = (DT)dv;
@@ -495,28 +455,28 @@ void launch_estar_move(const Dev& d, const EMoves& moves) {
 
 void launch_alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
     if (d.dbytes == 4)
-        launch_k(k_alg4_in<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.fD, d.fS, d.fM,
+        launch_k(k_alg4_in<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.fD, d.fS, d.fM,
             d.mark, d.changed, d.err);
     else
-        launch_k(k_alg4_in<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.fD, d.fS, d.fM,
+        launch_k(k_alg4_in<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.fD, d.fS, d.fM,
             d.mark, d.changed, d.err);
 }
 
 void launch_rows_out(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
     if (d.dbytes == 4)
-        launch_k(k_rows_out<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.fD, d.fS, d.fM,
+        launch_k(k_rows_out<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.fD, d.fS, d.fM,
             d.mark, d.changed, d.err);
     else
-        launch_k(k_rows_out<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.fD, d.fS, d.fM,
+        launch_k(k_rows_out<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.fD, d.fS, d.fM,
             d.mark, d.changed, d.err);
 }
 
 void launch_alg4_out(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
     if (d.dbytes == 4)
-        launch_k(k_alg4_out<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.cD, d.cS, d.cM,
+        launch_k(k_alg4_out<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.cD, d.cS, d.cM,
             d.changed, d.err);
     else
-        launch_k(k_alg4_out<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.cD, d.cS, d.cM,
+        launch_k(k_alg4_out<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.cD, d.cS, d.cM,
             d.changed, d.err);
 }
 
@@ -546,28 +506,23 @@ cudaError_t scan_setup() {
 
 template <typename DT>
 static void scan_dispatch(const Dev& d, ScanArgs<DT> a) {
-    constexpr int VN = Vec<DT>::N;
-    if (d.n % VN == 0) {
-        constexpr int CW = kCsThreads * kCsVpt * VN;
-        const int nch = (d.n + CW - 1) / CW;
-        const int per = std::max(1, d.nsm * kCsCtasPerSm / nch);
-        const bool whole = d.n % CW == 0;
-        if (a.rows2) {
-            if (whole) launch_k(k_scan_cs<DT, true, true>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
-            else launch_k(k_scan_cs<DT, false, true>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
-        } else {
-            if (whole) launch_k(k_scan_cs<DT, true, false>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
-            else launch_k(k_scan_cs<DT, false, false>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
-        }
+    constexpr int CW = kCsThreads * kCsVpt * Vec<DT>::N;
+    const int nch = (d.ld + CW - 1) / CW;
+    const int per = std::max(1, d.nsm * kCsCtasPerSm / nch);
+    const bool whole = d.ld % CW == 0;
+    if (a.rows2) {
+        if (whole) launch_k(k_scan_cs<DT, true, true>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
+        else launch_k(k_scan_cs<DT, false, true>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
     } else {
-        launch_k(k_scan<DT, false>, d.nsm * 8, kScanThreads, 0, d.st, a);
+        if (whole) launch_k(k_scan_cs<DT, true, false>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
+        else launch_k(k_scan_cs<DT, false, false>, nch * per, kCsThreads, kCsSmem, d.st, a, nch);
     }
 }
 
 template <typename DT>
 static ScanArgs<DT> scan_args(const Dev& d) {
     ScanArgs<DT> a;
-    a.n = d.n;
+    a.ld = d.ld;
     a.D = (DT*)d.D;
     a.S = d.S;
     a.rows = d.rows;
@@ -595,16 +550,16 @@ void launch_scan_in(const Dev& d, int32_t v) {
         ScanArgs<int32_t> a = scan_args<int32_t>(d);
         a.rec.first = 1;
         a.tie_rows = 1;
-        a.cD = (const int32_t*)d.D + (size_t)v * d.n;
-        a.cS = d.S + (size_t)v * d.n;
+        a.cD = (const int32_t*)d.D + (size_t)v * d.ld;
+        a.cS = d.S + (size_t)v * d.ld;
         a.cM = a.cS;
         scan_dispatch<int32_t>(d, a);
     } else {
         ScanArgs<int64_t> a = scan_args<int64_t>(d);
         a.rec.first = 1;
         a.tie_rows = 1;
-        a.cD = (const int64_t*)d.D + (size_t)v * d.n;
-        a.cS = d.S + (size_t)v * d.n;
+        a.cD = (const int64_t*)d.D + (size_t)v * d.ld;
+        a.cS = d.S + (size_t)v * d.ld;
         a.cM = a.cS;
         scan_dispatch<int64_t>(d, a);
     }
@@ -638,10 +593,10 @@ void launch_write_row(const Dev& d, int32_t v) {
     PairRec rec = d.pair_on ? pair_rec(d) : PairRec{};
     rec.first = 1;
     if (d.dbytes == 4)
-        launch_k(k_write_row<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (int32_t*)d.D, d.S, v,
+        launch_k(k_write_row<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (int32_t*)d.D, d.S, v,
                                                                 (const int32_t*)d.cD, d.cS, rec, d.err);
     else
-        launch_k(k_write_row<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, (int64_t*)d.D, d.S, v,
+        launch_k(k_write_row<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (int64_t*)d.D, d.S, v,
                                                                 (const int64_t*)d.cD, d.cS, rec, d.err);
 }
 
@@ -654,10 +609,10 @@ void launch_edge_prep(const Dev& d, int32_t u, int32_t v, int64_t w) {
     cudaMemsetAsync(d.counts, 0, 3 * sizeof(int32_t), d.st);   // counts[0..2]; [1] is rewritten later
     const int grid = (d.n + 255) / 256;
     if (d.dbytes == 4)
-        launch_k(k_edge_prep<int32_t>, grid, 256, 0, d.st, d.n, (const int32_t*)d.D, d.S, u, v, w, (int32_t*)d.cD, d.cS, (int32_t*)d.cD2, d.cS2, (int32_t*)d.fD,
+        launch_k(k_edge_prep<int32_t>, grid, 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, u, v, w, (int32_t*)d.cD, d.cS, (int32_t*)d.cD2, d.cS2, (int32_t*)d.fD,
             d.fS, d.fM, d.rows, d.counts, d.acc_rows, d.counts + 2, d.changed, d.err);
     else
-        launch_k(k_edge_prep<int64_t>, grid, 256, 0, d.st, d.n, (const int64_t*)d.D, d.S, u, v, w, (int64_t*)d.cD, d.cS, (int64_t*)d.cD2, d.cS2, (int64_t*)d.fD,
+        launch_k(k_edge_prep<int64_t>, grid, 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, u, v, w, (int64_t*)d.cD, d.cS, (int64_t*)d.cD2, d.cS2, (int64_t*)d.fD,
             d.fS, d.fM, d.rows, d.counts, d.acc_rows, d.counts + 2, d.changed, d.err);
 }
 
@@ -685,9 +640,9 @@ void launch_edge_scan(const Dev& d) {
 void launch_estar_keep(const Dev& d, uint8_t* keep) {
     if (d.e_cap <= 0) return;
     if (d.dbytes == 4)
-        launch_k(k_estar_keep<int32_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.n, (const int32_t*)d.D, d.e_src, (const Arc<int32_t>*)d.e_arc, d.e_cap, keep);
+        launch_k(k_estar_keep<int32_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.ld, (const int32_t*)d.D, d.e_src, (const Arc<int32_t>*)d.e_arc, d.e_cap, keep);
     else
-        launch_k(k_estar_keep<int64_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.n, (const int64_t*)d.D, d.e_src, (const Arc<int64_t>*)d.e_arc, d.e_cap, keep);
+        launch_k(k_estar_keep<int64_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.ld, (const int64_t*)d.D, d.e_src, (const Arc<int64_t>*)d.e_arc, d.e_cap, keep);
 }
 
 }  // namespace bcg

@@ -262,9 +262,9 @@ int bc_get_profile(bc_graph* g, double* ms, int64_t* launches, int32_t reset);
  *                     results bit for bit.
  *   "wide_accum" 0|1 (on by default): on graphs of at least 4096 vertices, re-run
  *                     Algorithm 1 for the rows over the target cap in 1024-thread CTAs
- *                     (one source's passes spread over more threads); 0: 256-thread
- *                     CTAs, which share SMs better with other handles' work (the server
- *                     sets 0 for its graphs).  Same results bit for bit.
+ *                     (one source's passes spread over more threads); 0: the
+ *                     CTAs chosen by n for thousands of sources, which share SMs better
+ *                     with other handles' work (the server sets 0 for its graphs).  Same results bit for bit.
  *   "pair_walk" 0|1 (undirected graphs only; BC_ERR_ARG on a directed graph): find the
  *                     columns of each changed pair (s,t) -- the vertices on a shortest
  *                     s-t path of the old and of the new state -- by walking DAG(s) of

@@ -220,6 +220,12 @@ int sync_check(bc_graph* g) {
     return BC_OK;
 }
 
+// First slot at or after at where a segment of c slots crosses no group boundary (one
+// longer than a group starts with a group).
+int64_t segment_start(int64_t at, int64_t c) {
+    return at / kGroupSlots == (at + c - 1) / kGroupSlots ? at : group_slots(at);
+}
+
 // Lay the E* superset out with slack per vertex and upload it.  The device arrays get
 // a quarter more slots than the layout needs: the free region where full segments move.
 int estar_layout(bc_graph* g, const std::vector<HArc>& arcs, const std::vector<int32_t>* extra = nullptr) {
@@ -231,32 +237,34 @@ int estar_layout(bc_graph* g, const std::vector<HArc>& arcs, const std::vector<i
     g->e_capv.assign(n, 0);
     for (int32_t a = 0; a < n; ++a) {
         g->e_capv[a] = deg[a] + 2 + deg[a] / 8 + (extra ? (*extra)[a] : 0);
-        g->e_off[a + 1] = g->e_off[a] + g->e_capv[a];
+        // a segment lies in one group of slots where it fits one (so the accumulation finds a
+        // vertex's DAG arcs together; at 10 slots a segment this leaves 2 % empty)
+        int64_t at = a ? (int64_t)g->e_off[a - 1] + g->e_capv[a - 1] : 0;
+        g->e_off[a] = (int32_t)segment_start(at, g->e_capv[a]);
     }
-    const int64_t cap = g->e_off[n];
+    const int64_t cap = n ? (int64_t)g->e_off[n - 1] + g->e_capv[n - 1] : 0;
+    g->e_off[n] = (int32_t)cap;
     Dev& d = g->d;
-    const size_t asz = g->dbytes == 4 ? sizeof(Arc<int32_t>) : sizeof(Arc<int64_t>);
     if (cap + cap / 8 > d.e_cap) {
-        dfree_async(g, d.e_src);
         dfree_async(g, d.e_arc);
-        d.e_src = nullptr;
+        dfree_async(g, d.e_w64);
         d.e_arc = nullptr;
-        const int64_t ncap = cap + cap / 4 + 64;
+        d.e_w64 = nullptr;
+        const int64_t ncap = group_slots(cap + cap / 4 + 64);
         int rc;
-        if ((rc = dalloc_async(g, &d.e_src, ncap))) return rc;
-        unsigned char* p = nullptr;
-        if ((rc = dalloc_async(g, &p, ncap * asz))) return rc;
-        d.e_arc = p;
+        if ((rc = dalloc_async(g, &d.e_arc, ncap)) ||
+            (g->dbytes == 8 && (rc = dalloc_async(g, &d.e_w64, ncap))))
+            return rc;
         d.e_cap = ncap;
     }
-    g->pool_top = cap;
+    g->pool_top = d.e_used = cap;
     g->e_src.assign(d.e_cap, 0);
     g->e_dst.assign(d.e_cap, -1);
     g->e_w.assign(d.e_cap, 0);
     g->eslot.clear();
     g->eslot.reserve(arcs.size() * 2 + 16);
     for (int32_t a = 0; a < n; ++a)
-        for (int32_t s = g->e_off[a]; s < g->e_off[a + 1]; ++s) g->e_src[s] = a;
+        for (int32_t s = g->e_off[a]; s < g->e_off[a] + g->e_capv[a]; ++s) g->e_src[s] = a;
     for (const HArc& x : arcs) {
         const int32_t slot = g->e_off[x.a] + g->e_len[x.a]++;
         g->e_dst[slot] = x.b;
@@ -264,22 +272,17 @@ int estar_layout(bc_graph* g, const std::vector<HArc>& arcs, const std::vector<i
         g->eslot[arc_key(x.a, x.b)] = slot;
     }
     g->estar_arcs = (int64_t)arcs.size();
-    std::vector<unsigned char> arc_bytes(d.e_cap * asz);
-    if (g->dbytes == 4) {
-        Arc<int32_t>* A = reinterpret_cast<Arc<int32_t>*>(arc_bytes.data());
-        for (int64_t i = 0; i < d.e_cap; ++i) A[i] = Arc<int32_t>{g->e_dst[i], (int32_t)g->e_w[i]};
-    } else {
-        Arc<int64_t>* A = reinterpret_cast<Arc<int64_t>*>(arc_bytes.data());
-        for (int64_t i = 0; i < d.e_cap; ++i) A[i] = Arc<int64_t>{(int64_t)g->e_dst[i], g->e_w[i]};
-    }
+    std::vector<Arc> A(d.e_cap);
+    for (int64_t i = 0; i < d.e_cap; ++i)
+        A[i] = g->e_dst[i] < 0 ? empty_arc() : make_arc(g->e_src[i], g->e_dst[i], g->e_w[i]);
     CK(g, cudaMemcpyAsync(d.e_off, g->e_off.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, d.st));
     CK(g, cudaMemcpyAsync(d.e_len, g->e_len.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, d.st));
-    CK(g, cudaMemcpyAsync(d.e_src, g->e_src.data(), sizeof(int32_t) * d.e_cap, cudaMemcpyHostToDevice, d.st));
-    CK(g, cudaMemcpyAsync(d.e_arc, arc_bytes.data(), arc_bytes.size(), cudaMemcpyHostToDevice, d.st));
+    CK(g, cudaMemcpyAsync(d.e_arc, A.data(), sizeof(Arc) * A.size(), cudaMemcpyHostToDevice, d.st));
+    if (d.e_w64)
+        CK(g, cudaMemcpyAsync(d.e_w64, g->e_w.data(), sizeof(int64_t) * d.e_cap, cudaMemcpyHostToDevice, d.st));
     CK(g, cudaStreamSynchronize(d.st));
-    // launch shape of the accumulation depends on the capacity: size its work space
     accum_config(d);
-    const int64_t need = (int64_t)d.acc_grid * d.ws_stride;
+    const int64_t need = (int64_t)d.acc_ctas * d.ws_stride;
     if (need > g->ws_cap) {
         dfree_async(g, d.ws);
         d.ws = nullptr;
@@ -366,9 +369,11 @@ int validate_update(bc_graph* g, const bc_update& u, const bc_vedge* edges, int6
 bool estar_move(bc_graph* g, int32_t a, int32_t want, std::vector<EMove>& moves) {
     const int32_t len = g->e_len[a];
     const int64_t c = (int64_t)want + want / 2 + 8;
-    if (g->pool_top + c > g->d.e_cap) return false;
-    const int32_t from = g->e_off[a], to = (int32_t)g->pool_top;
-    g->pool_top += c;
+    const int64_t at = segment_start(g->pool_top, c);
+    if (at + c > g->d.e_cap) return false;
+    const int32_t from = g->e_off[a], to = (int32_t)at;
+    g->pool_top = at + c;
+    g->d.e_used = g->pool_top;
     for (int32_t i = 0; i < len; ++i) {
         g->e_dst[to + i] = g->e_dst[from + i];
         g->e_w[to + i] = g->e_w[from + i];
@@ -1190,10 +1195,10 @@ int bc_set_option(bc_graph* g, const char* name, int64_t value) {
     }
     if (std::strcmp(name, "wide_accum") == 0) {
         // 1024-thread accumulation CTAs for the rows over the target cap (graphs of at
-        // least 4096 vertices); 0: 256-thread ones, which share SMs better with the work of
+        // least 4096 vertices); 0: the ordinary ones, which share SMs better with the work of
         // other handles running at the same time (the server turns them off)
         g->d.acc_narrow_only = value != 0 ? 0 : 1;
-        g->d.acc_threads = (value != 0 && g->n >= kAccWideMinN) ? kAccThreadsWide : kAccThreadsNarrow;
+        g->d.acc_wide = value != 0 && g->n >= kAccWideMinN;
         return BC_OK;
     }
     if (std::strcmp(name, "fused_edges") == 0) {
@@ -1373,7 +1378,7 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     b->L.acc_per_sm = 0;
     b->L.scan_unroll = 4;
     b->L.scan_sched = 0;
-    b->L.acc_threads = kAccThreadsNarrow;
+    b->L.acc_threads = 256;
     int rc;
     if ((rc = balloc(b, &b->d_devs, count)) || (rc = balloc(b, &b->d_coff, count + 1)) ||
         (rc = balloc(b, &b->d_plans, 5 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1))) {
@@ -1587,7 +1592,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
         CKB(b, cudaMemcpyAsync(b->d_eops, eops.data(), sizeof(BatchEOp) * eops.size(), cudaMemcpyHostToDevice, b->st));
     BatchArgs& a = b->args;
     a.G = G;
-    a.mask_in_smem = b->L.mask_in_smem;
+    a.lay = b->L.lay;
     a.n_max = b->n_max;
     a.devs = b->d_devs;
     a.upd = b->d_upd;

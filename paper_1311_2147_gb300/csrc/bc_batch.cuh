@@ -25,7 +25,6 @@ struct BatchEOp {
 
 struct BatchArgs {
     int32_t G;
-    int32_t mask_in_smem;
     int32_t n_max;            // largest n of the batch
     const Dev* devs;          // [G]
     const BatchUpd* upd;      // [rounds * G]
@@ -42,6 +41,7 @@ struct BatchArgs {
     int32_t* pctr;            // column-test pieces handed out past the first wave
     int32_t* ws;              // accumulation work space, acc_grid * ws_stride ints
     int64_t ws_stride;
+    AccLayout lay;            // arrays of an accumulation CTA, sized for the largest graph
 };
 
 // Launch shape of a batch; the tunable part is what the autotuner varies.
@@ -60,8 +60,7 @@ struct BatchLaunch {
     int32_t pairs;        // 1: some graph of the batch has pair corrections (0: the round skips
                           // the pair kernels)
     int32_t acc_grid;
-    int32_t acc_smem;
-    int32_t mask_in_smem;
+    AccLayout lay;
     int64_t ws_stride;
     int64_t max_eops;
 };

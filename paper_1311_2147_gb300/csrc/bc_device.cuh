@@ -555,41 +555,24 @@ struct AccArgs {
     ff* Dl;
     const int32_t* e_off;
     const int32_t* e_len;
-    const int32_t* e_src;
-    const Arc<DT>* e_arc;
-    int64_t e_cap;
+    const Arc* e_arc;
+    const int64_t* e_w64;
+    int64_t e_used;      // slots in use, a multiple of kGroupSlots (the rest of the last group is empty)
     const int32_t* rows;
     const int32_t* count;
     int32_t* ws;
     int64_t ws_stride;
     int32_t* err;
-    int mask_in_smem;
+    AccLayout lay;
 };
 
 constexpr uint32_t FULL = 0xffffffffu;
 
-// Distance of vertex i of the current source, with the row's own INF marker.
-struct Dist16 {
-    const uint16_t* p;
-    static constexpr uint64_t INFV = 0xFFFFull;
-    __device__ __forceinline__ uint64_t operator()(int i) const { return p[i]; }
-};
-template <typename DT>
-struct DistG {
-    const DT* p;
-    static constexpr uint64_t INFV = (uint64_t)Inf<DT>::v;
-    __device__ __forceinline__ uint64_t operator()(int i) const { return (uint64_t)(int64_t)__ldg(p + i); }
-};
-
-// Arc (x -> b, w) is in DAG'(s): d(x) finite (checked by the caller), d(b) finite and
-// d(x) + w == d(b).
-template <typename DA>
-__device__ __forceinline__ bool on_dag(const DA& dist, uint64_t dx, int b, uint64_t w) {
-    const uint64_t db = dist(b);
-    return db != DA::INFV && dx + w == db;
-}
-
-// 16-bit in-degree counters, two to a 32-bit word (in-degrees stay below 65536).
+// DAG in-degrees still to be taken, in 16-bit halves of 32-bit words (below 32768).  Most
+// vertices have one: they are marked kOneTail and need no atomic, which the levels'
+// chains would wait for (an update's vertices without DAG out-arcs are marked 0, they
+// join no level).  The others count down, and the last tail to be taken is told.
+constexpr uint32_t kOneTail = 0x8000;
 __device__ __forceinline__ void cnt_inc(uint32_t* cnt, int b) {
     atomicAdd(cnt + (b >> 1), 1u << ((b & 1) << 4));
 }
@@ -597,16 +580,14 @@ __device__ __forceinline__ bool cnt_last(uint32_t* cnt, int b) {
     const uint32_t sh = (b & 1) << 4;
     return ((atomicSub(cnt + (b >> 1), 1u << sh) >> sh) & 0xFFFFu) == 1u;
 }
-
-// Append the lanes' ready vertices to the order with one shared atomic per warp.
-__device__ __forceinline__ void warp_append(bool ready, int b, uint16_t* order, int* tail) {
-    const unsigned bal = __ballot_sync(FULL, ready);
-    if (!bal) return;
-    const int lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == __ffs(bal) - 1) base = atomicAdd(tail, __popc(bal));
-    base = __shfl_sync(FULL, base, __ffs(bal) - 1);
-    if (ready) order[base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)b;
+__device__ __forceinline__ uint32_t cnt_get(const uint32_t* cnt, int b) {
+    return reinterpret_cast<const volatile uint16_t*>(cnt)[b];
+}
+// To the marks above, by the vertex's own thread, once all are counted.
+__device__ __forceinline__ void cnt_mark(uint32_t* cnt, int x, bool leave_out) {
+    uint16_t* c = reinterpret_cast<uint16_t*>(cnt) + x;
+    if (leave_out) *c = 0;
+    else if (*c == 1) *c = (uint16_t)kOneTail;
 }
 
 __device__ __forceinline__ ff warp_sum(ff x) {
@@ -615,395 +596,513 @@ __device__ __forceinline__ ff warp_sum(ff x) {
     return x;
 }
 
-// Finish vertex x: delta(x) = sigma_sx * acc, rho(x) = (1 + delta(x)) / sigma_sx
-// = acc + 1 / sigma_sx.
-__device__ __forceinline__ void finish_vertex(int x, ff acc, uint64_t sigma, ff* out, ff* rho) {
-    const ff sx = ff_from_u64(sigma);
-    out[x] = ff_mul(sx, acc);
-    rho[x] = ff_add(acc, ff_rcp(sx));
+// ---- one source's dependencies
+//
+constexpr int kNearLevels = 512;
+// The arrays of one accumulation CTA (acc_layout says where each lives).
+struct AccMem {
+    uint32_t* row;     // [np] the source's distances in 32 bits; dead once the DAG is read off
+    uint16_t* first;   // [np] (over row) first pool entry of a vertex's heads
+    uint32_t* cnt;     // [np / 2] (over row) in-degrees
+    uint32_t* mask;    // [words] bit per slot of the superset: its arc is in DAG'(s)
+    uint16_t* base;    // [words] first pool entry of a mask word's arcs
+    uint16_t* order;   // [np] (over mask and base) vertices with DAG out-arcs, level by level
+    uint16_t* pool;    // [pcap + 4] heads of the DAG arcs
+    uint64_t* cell;    // [np] sigma_sx, then rho(x) once x is finished
+    uint32_t* sink;    // [np / 32] bit per vertex: no DAG out-arc
+    uint32_t* big;     // [np / 32] bit per vertex: kBigDag DAG out-arcs or more
+    uint16_t* level;   // [kNearLevels] start of each level in order, the later ones in far
+    uint16_t* far;     // [np] (work space)
+    __device__ __forceinline__ uint16_t& level_at(int l) const { return l < kNearLevels ? level[l] : far[l]; }
+};
+// cp.async of 16 bytes into shared memory, read back after async_wait_all and a barrier.
+__device__ __forceinline__ void async_copy16(void* smem, const void* gmem) {
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Passes 2 and 3 walk only the arcs of DAG'(s): pass 1 evaluates the predicate once per
-// slot of the E* superset and records it in a bit mask (one warp ballot per 32 slots).
-// Within a level, the DAG arcs of the level's vertices are spread evenly over the
-// threads: a block scan of the vertices' DAG out-degrees gives each arc a rank, a
-// thread finds the owner of its rank by binary search and the arc by selecting the
-// right set bit of the owner's slot range.  In pass 3 the arcs' contributions go to a
-// shared buffer and each owner adds its own in rank order (deterministic).  Vertices
-// with more than kBigDag DAG out-arcs are taken by whole warps instead (lanes over
-// their slots, fixed butterfly), so no owner loops long.
-constexpr int kBigDag = 32;
-constexpr int kBigCap = 2048;
-
-__device__ __forceinline__ int count_bits(const uint32_t* m, int beg, int end) {
-    if (beg >= end) return 0;
-    const int w0 = beg >> 5, w1 = (end - 1) >> 5;
-    int c = 0;
-    for (int w = w0; w <= w1; ++w) {
-        uint32_t b = m[w];
-        if (w == w0) b &= 0xffffffffu << (beg & 31);
-        if (w == w1) b &= 0xffffffffu >> (31 - ((end - 1) & 31));
-        c += __popc(b);
-    }
-    return c;
-}
-
-// Slot of the r-th (0-based) set bit of m at or after slot beg.  Callers pass r below
-// the number of set bits of the vertex's slot range, so the bit lies inside the range.
-__device__ __forceinline__ int select_bit(const uint32_t* m, int beg, int r) {
-    int w = beg >> 5;
-    uint32_t b = m[w] & (0xffffffffu << (beg & 31));
-    for (;;) {
-        const int c = __popc(b);
-        if (r < c) break;
-        r -= c;
-        b = m[++w];
-    }
-    for (; r > 0; --r) b &= b - 1u;
-    return (w << 5) + __ffs(b) - 1;
-}
-
-// Exclusive block-wide prefix sum of v (all threads call it); *total gets the sum.
-// s_ws needs T / 32 + 1 ints and must not be reused before a barrier (T threads).
-template <int T>
-__device__ __forceinline__ int block_excl_scan(int v, int* s_ws, int* total) {
-    constexpr int NW = T / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_ws[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int x = lane < NW ? s_ws[lane] : 0;
-        int ix = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(FULL, ix, o);
-            if (lane >= o) ix += y;
-        }
-        if (lane < NW) s_ws[lane] = ix - x;
-        if (lane == NW - 1) s_ws[NW] = ix;
-    }
-    __syncthreads();
-    *total = s_ws[NW];
-    return s_ws[warp] + incl - v;
-}
-
-// Last index i in [0, T) with off[i] <= j (off non-decreasing, off[0] = 0).
-template <int T>
-__device__ __forceinline__ int owner_of(const int* off, int j) {
-    int lo = 0, hi = T;
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (off[mid] <= j) lo = mid;
-        else hi = mid;
-    }
-    return lo;
-}
-
-// Append x to the big list when there is room (warp-aggregated); returns whether it was.
-__device__ __forceinline__ bool big_push(bool want, int x, uint16_t* big, int* nbig) {
-    const unsigned bal = __ballot_sync(FULL, want);
-    if (!bal) return false;
-    const int lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == __ffs(bal) - 1) base = atomicAdd(nbig, __popc(bal));
-    base = __shfl_sync(FULL, base, __ffs(bal) - 1);
-    const int pos = base + __popc(bal & ((1u << lane) - 1u));
-    if (want && pos < kBigCap) {
-        big[pos] = (uint16_t)x;
-        return true;
-    }
-    return false;
-}
-
-template <typename DT, bool STATIC>
-__device__ __forceinline__ void push_sigma(uint64_t* Ss, int b, uint64_t sx, int32_t* err) {
-    if (STATIC) {
-        const unsigned long long old =
-            atomicAdd(reinterpret_cast<unsigned long long*>(Ss + b), (unsigned long long)sx);
-        if (old + sx < old) set_err(err, ERRF_OVERFLOW);
-    }
-}
-
-// Per-round shared scratch of the level passes.
-// A round of a level pass gives every thread up to kPerThread vertices of the level.
-constexpr int kPerThread = 2;
-
-template <int T>
-struct LevelSmem {
-    int off[T];                  // first arc rank of the thread's vertices
-    int beg[kPerThread][T];      // slot range start of each vertex
-    int k0[T];                   // DAG out-arcs of the thread's first vertex
-    uint64_t sx[kPerThread][T];  // path counts (static pass 2)
-    ff buf[T];
-    int ws[T / 32 + 1];
+struct AccShared {
+    int arcs;          // pool entries handed out
+    int q[3];          // vertices appended for the next level, by level modulo 3
 };
 
-template <typename DT, bool STATIC, int T, typename DA>
-__device__ __forceinline__ void accumulate_source(const AccArgs<DT>& a, const DA dist, int s, uint64_t* Ss,
-                                                  ff* out, uint32_t* cnt, uint16_t* order, uint32_t* mask,
-                                                  uint16_t* big, LevelSmem<T>& ls, ff* rho, int32_t* lvl,
-                                                  int* s_tail, int* s_nbig) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = T / 32, U = 8;
-    // ---- pass 1: DAG'(s) membership of every slot, and in-degrees (loads of U chunks
-    // are issued before any of them is used)
-    const int nchunk = (int)((a.e_cap + 31) >> 5);
-    for (int c0 = warp; c0 < nchunk; c0 += U * NW) {
-        Arc<DT> r[U];
-        int src[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t e = ((int64_t)(c0 + u * NW) << 5) + lane;
-            r[u].dst = -1;
-            src[u] = 0;
-            if (e < a.e_cap) {
-                r[u] = a.e_arc[e];
-                src[u] = a.e_src[e];
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int c = c0 + u * NW;
-            if (c >= nchunk) break;
-            const int b = (int)r[u].dst;
-            bool on = false;
-            if (b >= 0) {
-                const uint64_t dx = dist(src[u]);
-                on = dx != DA::INFV && on_dag(dist, dx, b, (uint64_t)r[u].w);
-            }
-            if (on) cnt_inc(cnt, b);
-            const unsigned word = __ballot_sync(FULL, on);
-            if (lane == 0) mask[c] = word;
-        }
-    }
-    __syncthreads();   // the distance row (aliased by order) is dead from here on
-    if (tid == 0) {
-        order[0] = (uint16_t)s;
-        lvl[0] = 0;
-        lvl[1] = 1;
-        *s_tail = 1;
-        *s_nbig = 0;
-    }
-    __syncthreads();
-    // ---- pass 2: Kahn levels (statically also the forward path counts)
-    int L = 0;
-    for (;;) {
-        const int lo = lvl[L], hi = lvl[L + 1];
-        for (int qb = lo; qb < hi; qb += kPerThread * T) {
-            int kk[kPerThread];
-            int kt = 0;
-#pragma unroll
-            for (int v = 0; v < kPerThread; ++v) {
-                const int q = qb + v * T + tid;
-                int x = 0, beg = 0, k = 0;
-                if (q < hi) {
-                    x = order[q];
-                    beg = a.e_off[x];
-                    k = count_bits(mask, beg, beg + a.e_len[x]);
-                }
-                if (big_push(k > kBigDag, x, big, s_nbig)) k = 0;
-                kk[v] = k;
-                kt += k;
-                ls.beg[v][tid] = beg;
-                if (STATIC) ls.sx[v][tid] = k ? Ss[x] : 0ull;
-            }
-            int total;
-            const int off = block_excl_scan<T>(kt, ls.ws, &total);
-            ls.off[tid] = off;
-            ls.k0[tid] = kk[0];
-            __syncthreads();
-            for (int jb = 0; jb < total; jb += T) {
-                const int j = jb + tid;
-                bool ready = false;
-                int b = 0;
-                if (j < total) {
-                    const int o = owner_of<T>(ls.off, j);
-                    int r = j - ls.off[o];
-                    const int v = r < ls.k0[o] ? 0 : 1;
-                    if (v) r -= ls.k0[o];
-                    const int e = select_bit(mask, ls.beg[v][o], r);
-                    b = (int)a.e_arc[e].dst;
-                    push_sigma<DT, STATIC>(Ss, b, STATIC ? ls.sx[v][o] : 0ull, a.err);
-                    ready = cnt_last(cnt, b);
-                }
-                warp_append(ready, b, order, s_tail);
-            }
-            __syncthreads();
-        }
-        const int nb = min(*s_nbig, kBigCap);
-        for (int i = warp; i < nb; i += NW) {
-            const int x = big[i];
-            const int beg = a.e_off[x], end = beg + a.e_len[x];
-            const uint64_t sx = STATIC ? Ss[x] : 0ull;
-            for (int eb = beg; eb < end; eb += 32) {
-                const int e = eb + lane;
-                bool ready = false;
-                int b = 0;
-                if (e < end && ((mask[e >> 5] >> (e & 31)) & 1u)) {
-                    b = (int)a.e_arc[e].dst;
-                    push_sigma<DT, STATIC>(Ss, b, sx, a.err);
-                    ready = cnt_last(cnt, b);
-                }
-                warp_append(ready, b, order, s_tail);
-            }
-        }
-        __syncthreads();
-        if (tid == 0) {
-            lvl[L + 2] = *s_tail;
-            *s_nbig = 0;
-        }
-        __syncthreads();
-        if (lvl[L + 2] == hi) break;
-        ++L;
-    }
-    // ---- pass 3: Eq. 4 in reverse level order (level 0 is s: delta_s.(s) is not kept)
-    for (int Lq = L; Lq >= 1; --Lq) {
-        const int lo = lvl[Lq], hi = lvl[Lq + 1];
-        for (int qb = lo; qb < hi; qb += kPerThread * T) {
-            int xs[kPerThread], kk[kPerThread];
-            uint64_t sig[kPerThread];
-            bool mine[kPerThread];
-            int kt = 0;
-#pragma unroll
-            for (int v = 0; v < kPerThread; ++v) {
-                const int q = qb + v * T + tid;
-                int x = 0, beg = 0, k = 0;
-                if (q < hi) {
-                    x = order[q];
-                    beg = a.e_off[x];
-                    k = count_bits(mask, beg, beg + a.e_len[x]);
-                }
-                const bool is_big = big_push(k > kBigDag, x, big, s_nbig);
-                if (is_big) k = 0;
-                mine[v] = q < hi && !is_big;
-                sig[v] = mine[v] ? Ss[x] : 1ull;
-                xs[v] = x;
-                kk[v] = k;
-                kt += k;
-                ls.beg[v][tid] = beg;
-            }
-            int total;
-            const int off = block_excl_scan<T>(kt, ls.ws, &total);
-            ls.off[tid] = off;
-            ls.k0[tid] = kk[0];
-            __syncthreads();
-            ff acc[kPerThread];
-#pragma unroll
-            for (int v = 0; v < kPerThread; ++v) acc[v] = ff{0.0f, 0.0f};
-            for (int jb = 0; jb < total; jb += T) {
-                const int j = jb + tid;
-                if (j < total) {
-                    const int o = owner_of<T>(ls.off, j);
-                    int r = j - ls.off[o];
-                    const int v = r < ls.k0[o] ? 0 : 1;
-                    if (v) r -= ls.k0[o];
-                    const int e = select_bit(mask, ls.beg[v][o], r);
-                    ls.buf[tid] = rho[a.e_arc[e].dst];
-                }
-                __syncthreads();
-                int p = off;
-#pragma unroll
-                for (int v = 0; v < kPerThread; ++v) {
-                    const int p0 = max(p, jb), p1 = min(p + kk[v], jb + T);
-                    for (int pp = p0; pp < p1; ++pp) acc[v] = ff_add(acc[v], ls.buf[pp - jb]);
-                    p += kk[v];
-                }
-                __syncthreads();
-            }
-#pragma unroll
-            for (int v = 0; v < kPerThread; ++v)
-                if (mine[v]) finish_vertex(xs[v], acc[v], sig[v], out, rho);
-        }
-        __syncthreads();
-        const int nb = min(*s_nbig, kBigCap);
-        for (int i = warp; i < nb; i += NW) {
-            const int x = big[i];
-            const int beg = a.e_off[x], end = beg + a.e_len[x];
-            ff acc{0.0f, 0.0f};
-            for (int e = beg + lane; e < end; e += 32)
-                if ((mask[e >> 5] >> (e & 31)) & 1u) acc = ff_add(acc, rho[a.e_arc[e].dst]);
-            acc = warp_sum(acc);
-            if (lane == 0) finish_vertex(x, acc, Ss[x], out, rho);
-        }
-        __syncthreads();
-        if (tid == 0) *s_nbig = 0;
-        __syncthreads();
-    }
-}
-
-// Shared-memory layout of the accumulation kernel for n vertices (n rounded to np):
-// [d16 | order] (2np bytes; the distance row is dead once the slot mask is built, so
-// the level order reuses it) | cnt (np/2 words) | big list | slot mask (here when it
-// fits, else in the work space).
-struct AccSmem {
-    uint16_t* d16;
-    uint16_t* order;
-    uint32_t* cnt;
-    uint16_t* big;
-    uint32_t* mask;
-    ff* rho;
-    int32_t* lvl;
-};
-
-template <typename DT>
-__device__ __forceinline__ AccSmem acc_smem(const AccArgs<DT>& a, unsigned char* smem, int32_t* wsb) {
-    const int n = a.n;
-    const int np = (n + 31) & ~31;
-    AccSmem m;
-    m.d16 = reinterpret_cast<uint16_t*>(smem);
-    m.order = m.d16;
-    m.cnt = reinterpret_cast<uint32_t*>(smem + 2 * (size_t)np);
-    m.big = reinterpret_cast<uint16_t*>(smem + 4 * (size_t)np);
-    m.rho = reinterpret_cast<ff*>(wsb);
-    m.lvl = wsb + 2 * (size_t)n;
-    m.mask = a.mask_in_smem ? reinterpret_cast<uint32_t*>(smem + 4 * (size_t)np + 2 * kBigCap)
-                            : reinterpret_cast<uint32_t*>(wsb + ((3 * (int64_t)n + 2 + 3) & ~(int64_t)3));
+// SM: every array is in shared memory (the compiler then addresses it as such).
+template <bool SM>
+__device__ __forceinline__ AccMem acc_mem(const AccLayout& l, unsigned char* smem, int32_t* wsb) {
+    unsigned char* ws = reinterpret_cast<unsigned char*>(wsb);
+    AccMem m;
+    auto at = [&](int32_t off, bool in_ws) { return (SM || !in_ws) ? smem + off : ws + off; };
+    m.row = reinterpret_cast<uint32_t*>(smem + l.row);
+    m.first = reinterpret_cast<uint16_t*>(smem + l.row);
+    m.cnt = reinterpret_cast<uint32_t*>(smem + l.cnt);
+    m.level = reinterpret_cast<uint16_t*>(smem + l.level);
+    m.far = reinterpret_cast<uint16_t*>(ws + l.far);
+    m.sink = reinterpret_cast<uint32_t*>(smem + l.sink);
+    m.big = reinterpret_cast<uint32_t*>(smem + l.big);
+    m.mask = reinterpret_cast<uint32_t*>(at(l.mask, l.mask_ws));
+    m.base = reinterpret_cast<uint16_t*>(at(l.base, l.mask_ws));
+    m.order = reinterpret_cast<uint16_t*>(m.mask);
+    m.pool = reinterpret_cast<uint16_t*>(at(l.pool, l.pool_ws));
+    m.cell = reinterpret_cast<uint64_t*>(at(l.cell, l.cell_ws));
     return m;
 }
 
-// Re-accumulate source s (whole block; every thread calls it): stage its distance row,
-// rebuild DAG'(s), order it, pull Eq. 4, write its delta row (and, statically, its
-// sigma row).
-template <typename DT, bool STATIC, int T>
-__device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, const AccSmem& m, LevelSmem<T>& ls,
-                                                 int* s_tail, int* s_nbig) {
-    const int n = a.n;
-    const int np = (n + 31) & ~31;
-    const int tid = threadIdx.x;
-    const int64_t INF = Inf<DT>::v;
-    const DT* Ds = a.D + (size_t)s * a.ld;
-    uint64_t* Ss = a.S + (size_t)s * a.ld;
-    ff* out = a.Dl + (size_t)s * a.ld;
-    int wide = 0;
-    for (int t = tid; t < n; t += T) {
-        const int64_t v = Ds[t];
-        uint16_t c;
-        if (v == INF) c = 0xFFFF;
-        else if (v < 0xFFFF) c = (uint16_t)v;
-        else { c = 0xFFFE; wide = 1; }
-        m.d16[t] = c;
-        out[t] = ff{0.0f, 0.0f};
-        if (STATIC) Ss[t] = (t == s) ? 1ull : 0ull;
+__device__ __forceinline__ uint64_t cell_rho(ff r) {
+    return ((uint64_t)__float_as_uint(r.hi) << 32) | __float_as_uint(r.lo);
+}
+__device__ __forceinline__ ff cell_ff(uint64_t c) {
+    return ff{__uint_as_float((uint32_t)(c >> 32)), __uint_as_float((uint32_t)c)};
+}
+
+// The last head of a vertex carries kLastHead.  A vertex with kBigDag DAG out-arcs or
+// more is taken by a whole warp; its first pool entry is their number and the heads
+// follow.
+constexpr int kBigDag = 31;
+constexpr uint32_t kLastHead = 0x8000, kHeadMask = 0x7FFF;
+
+__device__ __forceinline__ bool bit_of(const uint32_t* w, int x) { return (w[x >> 5] >> (x & 31)) & 1u; }
+
+// The heads of a vertex from pool entry p on, four at a time (a chain of one head after
+// the other costs two or three shared-memory latencies a head): f(h, valid) with up to
+// four heads, bit u of valid set where h[u] is one.  All lanes of a warp call it together,
+// those without a vertex with go false, and f is called by all of them.
+template <typename F>
+__device__ __forceinline__ void four_heads(const AccMem& m, int p, bool go, F&& f) {
+    while (__any_sync(FULL, go)) {
+        uint32_t h[4] = {0u, 0u, 0u, 0u};
+        if (go) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) h[u] = m.pool[p + u];   // the pool is four entries longer
+        }
+        // up to the first that is marked last
+        const unsigned last = (h[0] & kLastHead) >> 15 | (h[1] & kLastHead) >> 14 | (h[2] & kLastHead) >> 13 |
+                              (h[3] & kLastHead) >> 12;
+        const unsigned valid = go ? (last ^ (last - 1u)) & 15u : 0u;
+        go = go && last == 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h[u] = (valid >> u) & 1u ? h[u] & kHeadMask : 0u;
+        f(h, valid);
+        p += 4;
+    }
+}
+
+// Appends the lanes' vertices (u < 4, where bit u of ready is set) to the next level.
+__device__ __forceinline__ void append4(const AccMem& m, int* q, int at, unsigned ready, const uint32_t* b) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned bal[4];
+    int tot = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        bal[u] = __ballot_sync(FULL, (ready >> u) & 1u);
+        tot += __popc(bal[u]);
+    }
+    if (!tot) return;
+    int p = 0;
+    if (lane == 0) p = atomicAdd(q, tot);
+    p = at + __shfl_sync(FULL, p, 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        if ((ready >> u) & 1u) m.order[p + __popc(bal[u] & lt)] = (uint16_t)b[u];
+        p += __popc(bal[u]);
+    }
+}
+
+// DAG'(s) read off the distance row: a lane per slot of the superset (the loads of a
+// group of slots are issued before any is used).  The heads of the DAG arcs go to the
+// pool, those of a group together in slot order.  Arc (x, b, w) is in DAG'(s) where
+// d(s,x) + w = d(s,b) (Eq. 1).  On the row in shared memory INF is 2^31 - 1, a weight that
+// does not fit 31 bits is held as that too and an empty slot's as 2^31, so one 32-bit
+// sum and compare decides: a sum with INF or an empty slot's exceeds every entry of the
+// row, none wraps, and no finite sum equals INF (where b is unreachable no arc from a
+// reachable x leads to it).  WIDE: some finite distance of the row does not fit;
+// distances and weights then come from memory.
+template <typename DT, int T, bool WIDE>
+__device__ __forceinline__ void dag_slots(const AccArgs<DT>& a, const AccMem& m, const DT* Ds, int* s_arcs) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    constexpr int NW = T / 32, U = kGroupSlots / 32;
+    const int ngroup = (int)(a.e_used / kGroupSlots);
+    for (int g = warp; g < ngroup; g += NW) {
+        const Arc* ap = a.e_arc + (int64_t)g * kGroupSlots + lane;
+        Arc r[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) r[u] = ap[32 * u];
+        unsigned word[U];
+        int tot = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            bool on;
+            if constexpr (WIDE) {
+                const int64_t dx = __ldg(Ds + r[u].src());
+                on = !r[u].empty() && dx != Inf<DT>::v &&
+                     dx + a.e_w64[(int64_t)g * kGroupSlots + 32 * u + lane] == (int64_t)__ldg(Ds + r[u].dst());
+            } else {
+                on = m.row[r[u].src()] + (uint32_t)r[u].w == m.row[r[u].dst()];
+            }
+            word[u] = __ballot_sync(FULL, on);
+            tot += __popc(word[u]);
+        }
+        int p = 0;
+        if (lane == 0 && tot) p = atomicAdd(s_arcs, tot);
+        p = __shfl_sync(FULL, p, 0);
+        const bool fits = p + tot <= a.lay.pcap;   // past the end the arcs are only counted
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (fits && ((word[u] >> lane) & 1u)) m.pool[p + __popc(word[u] & lt)] = (uint16_t)r[u].dst();
+            if (lane == u) {
+                m.mask[g * U + u] = word[u];
+                m.base[g * U + u] = (uint16_t)p;
+            }
+            p += __popc(word[u]);
+        }
+    }
+}
+
+// DAG out-degree of the vertex whose segment is [beg, beg + len), and its heads' first
+// pool entry where they lie in one group.
+__device__ __forceinline__ int count_dag(const AccMem& m, int beg, int len, int* p) {
+    if (len <= 0) return 0;
+    const int w = beg >> 5, sh = beg & 31;
+    const uint32_t m0 = m.mask[w];
+    *p = (int)m.base[w] + __popc(m0 & ((1u << sh) - 1u));
+    if (sh + len <= 32) return __popc((m0 >> sh) & (0xffffffffu >> (32 - len)));
+    int k = __popc(m0 >> sh);
+    const int end = beg + len, w1 = (end - 1) >> 5;
+    for (int v = w + 1; v < w1; ++v) k += __popc(m.mask[v]);
+    return k + __popc(m.mask[w1] & (0xffffffffu >> (31 - ((end - 1) & 31))));
+}
+
+// First pool entry of the heads of a vertex with k > 0 DAG out-arcs; p as count_dag gives
+// it.  Marks the last head.  Heads that lie in several groups, and those of a big vertex
+// behind their number, are copied to the end of the pool (past its end they are only
+// counted).
+__device__ __forceinline__ uint16_t place_heads(const AccMem& m, int pcap, int* s_arcs, int beg, int len, int k, int p) {
+    const int h = k >= kBigDag ? 1 : 0;
+    if (h || beg / kGroupSlots != (beg + len - 1) / kGroupSlots) {
+        p = atomicAdd(s_arcs, k + h);
+        if (p + k + h > pcap) return 0;
+        int at = p;
+        if (h) m.pool[at++] = (uint16_t)k;
+        const int w0 = beg >> 5, w1 = (beg + len - 1) >> 5;
+        for (int w = w0; w <= w1; ++w) {
+            const uint32_t word = m.mask[w], low = w == w0 ? (1u << (beg & 31)) - 1u : 0u;
+            uint32_t b = word & ~low;
+            if (w == w1) b &= 0xffffffffu >> (31 - ((beg + len - 1) & 31));
+            const int p0 = (int)m.base[w] + __popc(word & low), c = __popc(b);
+            for (int q = 0; q < c; ++q) m.pool[at++] = m.pool[p0 + q] & kHeadMask;
+        }
+    }
+    if (p + k + h <= pcap) m.pool[p + k + h - 1] |= kLastHead;
+    return (uint16_t)p;
+}
+
+// The DAG heads of vertex x from the superset and the distance row in memory, for a DAG
+// with more arcs than the pool holds (ties everywhere).
+template <typename DT, typename F>
+__device__ __forceinline__ void dag_heads(const AccArgs<DT>& a, const DT* Ds, int x, F&& f) {
+    const int64_t dx = Ds[x];
+    const int beg = a.e_off[x], end = beg + a.e_len[x];
+    for (int e = beg; e < end; ++e) {
+        const Arc arc = a.e_arc[e];
+        const int64_t w = sizeof(DT) == 4 ? (int64_t)arc.w : a.e_w64[e];
+        if (dx + w == (int64_t)Ds[arc.dst()]) f(arc.dst());
+    }
+}
+
+// The levels of DAG'(s) forwards (Kahn): a vertex joins the next level when its last DAG
+// in-arc is taken; vertices without DAG out-arcs are left out.  Statically the path
+// counts go along: sigma_sb is the sum of sigma_sa over the DAG in-arcs (a, b).  Returns
+// the number of levels; level l is order[level_at(l) .. level_at(l + 1)).
+template <typename DT, bool STATIC, int T, bool POOLED>
+__device__ __forceinline__ int dag_levels(const AccArgs<DT>& a, const AccMem& m, AccShared& sh, int s, const DT* Ds) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    int lo = 0, hi = bit_of(m.sink, s) ? 0 : 1, L = 0;
+    if (tid == 0) {
+        m.order[0] = (uint16_t)s;
+        m.level_at(0) = 0;
+    }
+    __syncthreads();   // the masks under order are dead from here on
+    while (lo < hi) {
+        int* q = &sh.q[L % 3];
+        if (tid == 0) sh.q[(L + 1) % 3] = 0;
+        // one more tail, with sx paths, of vertex b is taken: whether it was the last
+        auto take = [&](int b, uint64_t sx) {
+            const uint32_t c = cnt_get(m.cnt, b);
+            if (c == kOneTail) {
+                if (STATIC) m.cell[b] = sx;
+                return true;
+            }
+            if (!STATIC && c == 0) return false;
+            if (STATIC) {
+                const unsigned long long old =
+                    atomicAdd(reinterpret_cast<unsigned long long*>(m.cell + b), (unsigned long long)sx);
+                if (old + sx < old) set_err(a.err, ERRF_OVERFLOW);
+            }
+            return cnt_last(m.cnt, b);
+        };
+        for (int i0 = lo + (tid & ~31); i0 < hi; i0 += T) {   // warp-uniform
+            const int i = i0 + lane;
+            const bool have = i < hi;
+            const int x = have ? m.order[i] : 0;
+            const uint64_t sx = STATIC ? m.cell[x] : 0ull;
+            if constexpr (POOLED) {
+                const bool big = have && bit_of(m.big, x);
+                const int p = m.first[x];
+                four_heads(m, p, have && !big, [&](const uint32_t* b, unsigned valid) {
+                    // one tail only (nearly all): ready, without branches; then the others
+                    unsigned ready = 0, others = 0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const uint32_t c = cnt_get(m.cnt, (int)b[u]);
+                        ready |= c == kOneTail ? 1u << u : 0u;
+                        others |= c != 0 ? 1u << u : 0u;
+                        if (STATIC && c == kOneTail && ((valid >> u) & 1u)) m.cell[b[u]] = sx;
+                    }
+                    ready &= valid;
+                    others &= valid & ~ready;
+                    if (others) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if ((others >> u) & 1u) ready |= take((int)b[u], sx) ? 1u << u : 0u;
+                    }
+                    if (STATIC) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) ready &= ~((unsigned)bit_of(m.sink, (int)b[u]) << u);
+                    }
+                    append4(m, q, hi, ready, b);
+                });
+                for (unsigned bb = __ballot_sync(FULL, big); bb; bb &= bb - 1u) {
+                    const int src = __ffs(bb) - 1;
+                    const int pb = __shfl_sync(FULL, p, src), k = m.pool[pb];
+                    const uint64_t sb = STATIC ? m.cell[__shfl_sync(FULL, x, src)] : 0ull;
+                    for (int c = 0; c < k; c += 32) {
+                        uint32_t b[4] = {0u, 0u, 0u, 0u};
+                        unsigned ready = 0;
+                        if (c + lane < k) {
+                            b[0] = m.pool[pb + 1 + c + lane] & kHeadMask;
+                            ready = take((int)b[0], sb) && !bit_of(m.sink, (int)b[0]) ? 1u : 0u;
+                        }
+                        append4(m, q, hi, ready, b);
+                    }
+                }
+            } else if (have) {
+                dag_heads(a, Ds, x, [&](int b) {
+                    if (take(b, sx) && !bit_of(m.sink, b)) m.order[hi + atomicAdd(q, 1)] = (uint16_t)b;
+                });
+            }
+        }
+        __syncthreads();
+        const int c = *q;
+        ++L;
+        if (tid == 0) m.level_at(L) = (uint16_t)hi;
+        lo = hi;
+        hi += c;
+    }
+    return L;
+}
+
+// Eq. 4 back over the levels (level 0 is s: delta_s.(s) is not kept).
+template <typename DT, int T, bool POOLED>
+__device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, const DT* Ds, int L, ff* out) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    for (int l = L - 1; l >= 1; --l) {
+        const int lo = m.level_at(l), hi = m.level_at(l + 1);
+        for (int i0 = lo + (tid & ~31); i0 < hi; i0 += T) {   // warp-uniform
+            const int i = i0 + lane;
+            const bool have = i < hi;
+            const int x = have ? m.order[i] : 0;
+            const ff sx = ff_from_u64(m.cell[x]), rx = ff_rcp(sx);
+            ff acc{0.0f, 0.0f};
+            if constexpr (POOLED) {
+                const bool big = have && bit_of(m.big, x);
+                const int p = m.first[x];
+                four_heads(m, p, have && !big, [&](const uint32_t* b, unsigned valid) {
+                    uint64_t c[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) c[u] = (valid >> u) & 1u ? m.cell[b[u]] : 0ull;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc = ff_add(acc, cell_ff(c[u]));   // + 0 past the end: exact
+                });
+                for (unsigned bb = __ballot_sync(FULL, big); bb; bb &= bb - 1u) {
+                    const int src = __ffs(bb) - 1;
+                    const int pb = __shfl_sync(FULL, p, src), k = m.pool[pb];
+                    ff part{0.0f, 0.0f};
+                    for (int c = lane; c < k; c += 32)
+                        part = ff_add(part, cell_ff(m.cell[m.pool[pb + 1 + c] & kHeadMask]));
+                    part = warp_sum(part);
+                    if (lane == src) acc = part;
+                }
+            } else if (have) {
+                // kBigDag heads or more are summed as a warp would: 32 sums by rank, then a butterfly
+                int k = 0;
+                dag_heads(a, Ds, x, [&](int b) {
+                    ++k;
+                    acc = ff_add(acc, cell_ff(m.cell[b]));
+                });
+                if (k >= kBigDag) {
+                    ff part[32];
+                    for (int c = 0; c < 32; ++c) part[c] = ff{0.0f, 0.0f};
+                    k = 0;
+                    dag_heads(a, Ds, x, [&](int b) {
+                        part[k & 31] = ff_add(part[k & 31], cell_ff(m.cell[b]));
+                        ++k;
+                    });
+                    for (int o = 16; o > 0; o >>= 1)
+                        for (int c = 0; c < o; ++c) part[c] = ff_add(part[c], part[c + o]);
+                    acc = part[0];
+                }
+            }
+            // delta(x) = sigma_sx * acc, rho(x) = (1 + delta(x)) / sigma_sx = acc + 1 / sigma_sx
+            if (have) {
+                m.cell[x] = cell_rho(ff_add(acc, rx));
+                out[x] = ff_mul(sx, acc);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Once the DAG's levels are known: the vertices without DAG out-arcs are finished, then
+// the others back over the levels.
+template <typename DT, bool STATIC, int T, bool POOLED>
+__device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m, AccShared& sh, int s, const DT* Ds,
+                                           uint64_t* Ss, ff* out) {
+    const int n = a.n, tid = threadIdx.x;
+    if (!POOLED) {   // the pool's heads were counted as they came; now from the superset
+        for (int t = tid; t < (n + 1) / 2; t += T) m.cnt[t] = 0u;
+        __syncthreads();
+        for (int x = tid; x < n; x += T)
+            if (!bit_of(m.sink, x)) dag_heads(a, Ds, x, [&](int b) { cnt_inc(m.cnt, b); });
+        __syncthreads();
+        for (int x = tid; x < n; x += T) cnt_mark(m.cnt, x, !STATIC && bit_of(m.sink, x));
+        __syncthreads();
+    }
+    const int L = dag_levels<DT, STATIC, T, POOLED>(a, m, sh, s, Ds);
+    for (int x = tid; x < n; x += T) {
+        const uint64_t sg = m.cell[x];
+        if (STATIC) Ss[x] = sg;
+        if (x == s || bit_of(m.sink, x)) {
+            out[x] = ff{0.0f, 0.0f};
+            if (sg != 0) m.cell[x] = cell_rho(ff_rcp(ff_from_u64(sg)));
+        }
     }
     if (STATIC && tid < a.ld - n) {   // the entries past n: no path
         Ss[n + tid] = 0ull;
         out[n + tid] = ff{0.0f, 0.0f};
     }
-    for (int t = tid; t < np / 2; t += T) m.cnt[t] = 0u;
-    wide = __syncthreads_or(wide);
-    if (!wide)
-        accumulate_source<DT, STATIC, T>(a, Dist16{m.d16}, s, Ss, out, m.cnt, m.order, m.mask, m.big, ls, m.rho, m.lvl,
-                                      s_tail, s_nbig);
-    else
-        accumulate_source<DT, STATIC, T>(a, DistG<DT>{Ds}, s, Ss, out, m.cnt, m.order, m.mask, m.big, ls, m.rho, m.lvl,
-                                      s_tail, s_nbig);
     __syncthreads();
+    dag_pull<DT, T, POOLED>(a, m, Ds, L, out);
+}
+template <typename DT, bool STATIC, int T>
+__device__ __noinline__ void dag_source_unpooled(AccArgs<DT> a, AccMem m, AccShared* sh, int s) {
+    const size_t row = (size_t)s * a.ld;
+    dag_source<DT, STATIC, T, false>(a, m, *sh, s, a.D + row, a.S + row, a.Dl + row);
+}
+
+// Re-accumulate source s (whole block; every thread calls it): stage its distance row,
+// read DAG'(s) off it, order it by levels, pull Eq. 4 back over them, write the delta row
+// (and, statically, the sigma row).  A sum runs in slot order (kBigDag heads or more: by
+// rank modulo 32, then a butterfly), so it does not depend on scheduling.
+//
+// What bounds it: instructions (about 25 per 32 slots of the superset, for every source)
+// and two chains of shared-memory reads per level.  Everything after the slots is read
+// once lives in shared memory; before, the levels read the superset, its heads and rho
+// from L2, three dependent reads per level and direction, around a dozen barriers, now
+// one.  Time per source over an update's changed rows, before and now: ER n = 256 (int64)
+// 0.50 and 0.21 us, ER n = 4096 0.43 and 0.18, BA n = 8192 0.86 and 0.48, BA n = 16384
+// 2.50 and 1.10.  Of the cycles of one source at ER n = 4096, 24 % go to the slots, 13 %
+// to the heads, 36 % to the levels forwards, 20 % to the pull.  Measured and not kept:
+// no order at all, each thread looking through its open vertices in sweeps until their
+// heads are finished (0.22 at ER n = 4096); a thread per vertex instead of a lane per
+// slot to read the DAG off (0.29: four dependent L2 reads per 256 vertices, and the hubs
+// of a BA graph in the same few warps).
+template <typename DT, bool STATIC, int T, bool SM>
+__device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, const AccMem& m, AccShared& sh) {
+    const int n = a.n;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const DT* Ds = a.D + (size_t)s * a.ld;
+    uint64_t* Ss = a.S + (size_t)s * a.ld;
+    ff* out = a.Dl + (size_t)s * a.ld;
+    int wide = 0;
+    for (int t = tid * 4; t < n; t += T * 4) {   // rows start on 32-byte boundaries, np >= t + 4
+        uint4 c;
+        if constexpr (sizeof(DT) == 4) {
+            c = *reinterpret_cast<const uint4*>(Ds + t);
+        } else {
+            longlong2 v[2];
+            v[0] = *reinterpret_cast<const longlong2*>(Ds + t);
+            v[1] = *reinterpret_cast<const longlong2*>(Ds + t + 2);
+            const long long* vv = reinterpret_cast<const long long*>(v);
+            uint32_t* cc = reinterpret_cast<uint32_t*>(&c);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                cc[q] = vv[q] < INT32_MAX ? (uint32_t)vv[q] : (uint32_t)INT32_MAX;
+                wide |= vv[q] >= INT32_MAX && vv[q] != Inf<DT>::v;
+            }
+        }
+        *reinterpret_cast<uint4*>(m.row + t) = c;
+    }
+    if (STATIC) {
+        for (int t = tid; t < n; t += T) m.cell[t] = t == s ? 1ull : 0ull;
+    } else {
+        // the cells start as the source's path counts, on their way while the DAG is read off
+        for (int t = tid * 2; t < n; t += T * 2) {
+            if (SM) async_copy16(m.cell + t, Ss + t);
+            else *reinterpret_cast<ulonglong2*>(m.cell + t) = *reinterpret_cast<const ulonglong2*>(Ss + t);
+        }
+        if (SM) async_commit();
+    }
+    if (tid == 0) sh.arcs = sh.q[0] = 0;
+    wide = __syncthreads_or(wide);
+    if constexpr (sizeof(DT) == 8) {
+        if (wide) dag_slots<DT, T, true>(a, m, Ds, &sh.arcs);
+        else dag_slots<DT, T, false>(a, m, Ds, &sh.arcs);
+    } else {
+        dag_slots<DT, T, false>(a, m, Ds, &sh.arcs);
+    }
+    __syncthreads();   // the distance row is dead from here on
+    for (int t = tid; t < (n + 1) / 2; t += T) m.cnt[t] = 0u;
+    const int arcs = sh.arcs;
+    __syncthreads();
+    if (arcs <= a.lay.pcap)
+        for (int q = tid; q < arcs; q += T) cnt_inc(m.cnt, m.pool[q]);
+    __syncthreads();   // the lists below mark and copy pool entries
+    constexpr int VU = 8;
+    for (int i0 = 0; i0 * T < n; i0 += VU) {
+        int beg[VU], len[VU];
+#pragma unroll
+        for (int v = 0; v < VU; ++v) {
+            const int x = (i0 + v) * T + tid;
+            beg[v] = len[v] = 0;
+            if (x < n) {
+                beg[v] = a.e_off[x];
+                len[v] = a.e_len[x];
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < VU; ++v) {
+            const int x = (i0 + v) * T + tid;
+            if ((i0 + v) * T >= n) break;
+            int p = 0;
+            const int k = count_dag(m, beg[v], len[v], &p);
+            if (x < n) {
+                m.first[x] = k > 0 ? place_heads(m, a.lay.pcap, &sh.arcs, beg[v], len[v], k, p) : (uint16_t)0;
+                cnt_mark(m.cnt, x, !STATIC && k == 0);
+            }
+            const unsigned sinks = __ballot_sync(FULL, k == 0), bigs = __ballot_sync(FULL, k >= kBigDag);
+            if (lane == 0 && x < n) {
+                m.sink[x >> 5] = sinks;
+                m.big[x >> 5] = bigs;
+            }
+        }
+    }
+    if (SM && !STATIC) async_wait_all();
+    __syncthreads();
+    if (sh.arcs <= a.lay.pcap) dag_source<DT, STATIC, T, true>(a, m, sh, s, Ds, Ss, out);
+    else dag_source_unpooled<DT, STATIC, T>(a, m, &sh, s);
 }
 
 // partial[rb][t] = sum over rows r of row block rb of Dl[s_r][t] (t != s_r), rows in

@@ -17,10 +17,9 @@
 // E* superset ("E*+") -- every arc that lies on some shortest path, plus arcs that
 // may no longer do so (Section 6: any superset of E* gives the right DAGs) -- is a
 // CSR with per-vertex slack: arcs of vertex a sit in slots [off[a], off[a]+len[a]),
-// followed by free slots (dst = -1).  A segment that fills up moves to the free region
-// past the laid-out ones (off[a] changes, its old slots are emptied).  Each slot is a
-// packed (dst, w) pair (Arc<DT>: 8 bytes for int32 distances, 16 for int64) so one load
-// brings both; src[] repeats the tail of each slot for passes that run over the slots.
+// followed by empty slots.  A segment that fills up moves to the free region past the
+// laid-out ones (off[a] changes, its old slots are emptied).  A slot holds tail, head and
+// weight in 8 bytes (Arc), so one load brings what a pass over the slots needs.
 #pragma once
 
 #include <cstdint>
@@ -87,9 +86,25 @@ __device__ __forceinline__ uint64_t add_chk(uint64_t a, uint64_t b, int32_t* err
 constexpr int kRowAlign = 8;
 __host__ __device__ inline int32_t row_pitch(int32_t n) { return (n + kRowAlign - 1) & ~(kRowAlign - 1); }
 
-template <typename DT> struct Arc;
-template <> struct __align__(8) Arc<int32_t> { int32_t dst; int32_t w; };
-template <> struct __align__(16) Arc<int64_t> { int64_t dst; int64_t w; };
+// One slot of the superset: the arc's tail and head (15 bits each; the head in bits 2..16,
+// so that masking gives four times it) and its weight, held as 2^31 - 1 where it does not
+// fit 31 bits (an int64 graph keeps the weights in full beside the slots, e_w64) and as
+// -2^31 in an empty slot.
+struct __align__(8) Arc {
+    uint32_t ids;
+    int32_t w;
+    __host__ __device__ int dst() const { return (int)((ids >> 2) & 0x7FFFu); }
+    __host__ __device__ int src() const { return (int)(ids >> 17); }
+    __host__ __device__ bool empty() const { return w < 0; }
+};
+constexpr int kMaxVertices = 32768;
+inline __host__ __device__ Arc make_arc(int32_t a, int32_t b, int64_t w) {
+    return Arc{((uint32_t)a << 17) | ((uint32_t)b << 2), w < INT32_MAX ? (int32_t)w : INT32_MAX};
+}
+inline __host__ __device__ Arc empty_arc() { return Arc{0u, INT32_MIN}; }
+// Slots a warp of the accumulation takes at a time; the slot array is a whole number of
+// groups.
+constexpr int kGroupSlots = 256;
 
 constexpr int kPairCap = 128;   // changed targets of a row corrected pair by pair (k_pair.cu)
 
@@ -146,6 +161,22 @@ struct EMoves {
     EMove mv[kMaxEMoves];
 };
 
+// Where the arrays of an accumulation CTA live (dev_accum_source): byte offsets into its
+// shared memory or, for the ones marked, into its part of the work space (acc_layout).
+struct AccLayout {
+    int32_t row, cnt, level, far, sink, big, mask, base, pool, cell;
+    uint8_t mask_ws, pool_ws, cell_ws;
+    int32_t pcap;        // heads the pool holds
+    int32_t smem;        // bytes of shared memory
+    int32_t ws;          // bytes of work space
+    uint8_t all_smem;    // no array but far is in the work space
+};
+inline __host__ __device__ int64_t group_slots(int64_t slots) {
+    return (slots + kGroupSlots - 1) / kGroupSlots * kGroupSlots;
+}
+AccLayout acc_layout(int n, int64_t e_cap, bool is_static);
+inline bool acc_all_smem(const AccLayout& l) { return l.all_smem != 0; }
+
 // Device state of one handle (plain pointers; owned by the host-side bc_graph).
 struct Dev {
     int32_t n;
@@ -169,9 +200,10 @@ struct Dev {
     // E*+ CSR with slack
     int32_t* e_off;
     int32_t* e_len;
-    int32_t* e_src;
-    void* e_arc;         // Arc<DT>[e_cap]
-    int64_t e_cap;
+    Arc* e_arc;          // [e_cap]
+    int64_t* e_w64;      // [e_cap] weights in full (int64 distances; else NULL)
+    int64_t e_cap;       // a multiple of kGroupSlots
+    int64_t e_used;      // slots laid out or moved to so far; the rest is the free region
     // error word, counters
     int32_t* err;
     int64_t* stats;      // [0] rows re-accumulated [1] no-op updates [2] max rows [3] updates
@@ -193,13 +225,14 @@ struct Dev {
     uint64_t* cS2;       // [ld] its path counts
     ff* partial;         // [nrb * ld] column partial sums
     int32_t nrb_max;     // row blocks of the BC reduction
-    int32_t acc_grid;    // CTAs of the accumulation kernel
-    int32_t acc_smem;    // dynamic shared memory of the accumulation kernel
-    int32_t acc_mask_smem;  // 1: the DAG slot mask lives in shared memory
-    int32_t acc_threads;    // kAccThreadsWide: wide CTAs allowed for partial waves of sources
+    AccLayout acc_lay[2];   // of the accumulation kernel: updates, static computation
+    int32_t acc_threads[2]; // its threads per CTA
+    int32_t acc_grid[2];    // its CTAs
+    int32_t acc_grid_wide[2];  // its CTAs of kAccThreadsWide threads
+    int32_t acc_wide;       // 1: wide CTAs for partial waves of sources
     int32_t acc_narrow_only;  // 1: never the wide CTAs (kept across launch-shape updates)
-    int32_t acc_grid_wide;  // CTAs of the wide accumulation kernel (acc_grid: of the narrow one)
-    int32_t* ws;         // accumulation work space, acc_grid * ws_stride ints
+    int32_t* ws;         // accumulation work space, acc_ctas * ws_stride ints
+    int32_t acc_ctas;    // most CTAs of any accumulation launch
     int64_t ws_stride;
     // pair-dependency corrections (undirected graphs): the pairs changed by this update,
     // their values before it, and the changed targets of each row
@@ -234,17 +267,15 @@ struct Dev {
 };
 
 constexpr int kRowsPerBlock = 64;   // rows per partial sum of the BC reduction
-// Threads of an accumulation CTA (one source at a time): 1024 for the few rows over the
-// target cap of an update on graphs of at least kAccWideMinN vertices (the level passes
-// of one source spread over more threads), 256 otherwise (four sources in flight per SM:
-// saturated serving of 64 graphs 1783 -> 2028 updates/s against 512 threads, 128 threads
-// 1843); the batched path picks 128, 256 or 512 by autotuning.
+// Threads of an accumulation CTA (one source at a time) for the few rows over the target
+// cap of an update on graphs of at least kAccWideMinN vertices (one source's levels
+// spread over more threads); otherwise 256, 512 or 1024 by its shared memory
+// (accum_config).  The batched path picks 128, 256 or 512 by autotuning.
 constexpr int kAccThreadsWide = 1024;
-constexpr int kAccThreadsNarrow = 256;
 constexpr int kAccWideMinN = 4096;
 
-// Accumulation launch shape for n and the current E* capacity (sets acc_grid, acc_smem,
-// acc_mask_smem and ws_stride of d); the work space must then hold acc_grid * ws_stride.
+// Accumulation launch shape for n and the current E* capacity (sets the acc_ fields and
+// ws_stride of d); the work space must then hold acc_ctas * ws_stride ints.
 void accum_config(Dev& d);
 
 // Recording of changed pairs by the passes that write D and sigma (pair corrections).

@@ -14,40 +14,36 @@
 //   * delta_s. is pulled in reverse level order (Eq. 4), in float-float (ff.cuh):
 //         delta(a) = sum over DAG out-arcs (a,b) of sigma_sa / sigma_sb * (1 + delta(b))
 //                  = sigma_sa * sum over the same arcs of rho(b),
-//     with rho(b) = (1 + delta(b)) / sigma_sb kept per vertex.  The DAG out-arcs of a
-//     level are flattened over the CTA (a block scan of the per-vertex arc counts, each
-//     thread fetching rho of one arc, each vertex summing its own arcs in slot order);
-//     vertices with more than kBigDag DAG out-arcs are summed by a warp over a fixed
-//     stride and butterfly.  Either way the result does not depend on scheduling.
-// The kernel stages in shared memory the source's distance row (16-bit when every
-// finite distance of the row is below 65535, otherwise read from its row of D), the
-// packed 16-bit Kahn counters, the 16-bit level order and a bit mask over the slots of
-// the E* superset marking the arcs of DAG'(s): about 4n bytes plus one bit per slot,
-// two CTAs per SM at n = 16384.  rho and the level bounds live in a per-CTA work space
-// in global memory (L2-resident), and so does the slot mask when it is too large.
+//     with rho(b) = (1 + delta(b)) / sigma_sb kept per vertex, a thread per vertex (a warp
+//     for kBigDag DAG out-arcs or more), in slot order: the result does not depend on
+//     scheduling.
+// The kernel keeps in shared memory the source's distance row, then what it read off it:
+// the heads of the DAG arcs, the levels and a cell per vertex (sigma, then rho); see
+// dev_accum_source.
 //
 // BC is maintained as BC += sum over changed rows of (delta'_s - delta_s): the old rows
 // are subtracted before the rows are rewritten and the new rows added after
 // (Algorithm 3 step 1 recomputes BC from zero; rows that did not change contribute
 // the same amount before and after, so only changed rows are touched).  Column sums
 // run over row blocks in a fixed order into a compensated (hi, lo) pair.
+#include <algorithm>
+#include <type_traits>
+
 #include "bc_device.cuh"
 
 namespace bcg {
 
-// One CTA per source at a time (shared memory as described at AccSmem; the per-round
-// scratch of the level passes is static shared memory).
-template <typename DT, bool STATIC, int T>
-__global__ void __launch_bounds__(T, 1024 / T) k_accum_smem(AccArgs<DT> a) {
+// One CTA per source at a time.
+template <typename DT, bool STATIC, int T, bool SM>
+__global__ void __launch_bounds__(T, 1024 / T) k_accum(AccArgs<DT> a) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ LevelSmem<T> ls;
-    __shared__ int s_tail, s_nbig;
-    const AccSmem m = acc_smem(a, smem, a.ws + (size_t)blockIdx.x * a.ws_stride);
+    __shared__ AccShared sh;
+    const AccMem m = acc_mem<SM>(a.lay, smem, a.ws + (size_t)blockIdx.x * a.ws_stride);
     const int total = STATIC ? a.n : *a.count;
     for (int i = blockIdx.x; i < total; i += gridDim.x) {
         if (block_err(a.err)) return;
-        dev_accum_source<DT, STATIC, T>(a, STATIC ? i : a.rows[i], m, ls, &s_tail, &s_nbig);
+        dev_accum_source<DT, STATIC, T, SM>(a, STATIC ? i : a.rows[i], m, sh);
     }
 }
 
@@ -98,7 +94,7 @@ __global__ void k_bc_finish(int n, int ld, const int32_t* rows, const int32_t* c
 // ------------------------------------------------------------------ launches
 
 template <typename DT>
-static AccArgs<DT> acc_args(const Dev& d, const int32_t* rows, const int32_t* count) {
+static AccArgs<DT> acc_args(const Dev& d, int is_static, const int32_t* rows, const int32_t* count) {
     AccArgs<DT> a;
     a.n = d.n;
     a.ld = d.ld;
@@ -107,84 +103,132 @@ static AccArgs<DT> acc_args(const Dev& d, const int32_t* rows, const int32_t* co
     a.Dl = d.Dl;
     a.e_off = d.e_off;
     a.e_len = d.e_len;
-    a.e_src = d.e_src;
-    a.e_arc = (const Arc<DT>*)d.e_arc;
-    a.e_cap = d.e_cap;
+    a.e_arc = d.e_arc;
+    a.e_w64 = d.e_w64;
+    a.e_used = group_slots(d.e_used);
     a.rows = rows;
     a.count = count;
     a.ws = d.ws;
     a.ws_stride = d.ws_stride;
     a.err = d.err;
-    a.mask_in_smem = d.acc_mask_smem;
+    a.lay = d.acc_lay[is_static];
     return a;
 }
 
-// Shared memory of the accumulation kernel without / with the slot mask.
-static size_t smem_base(int n) {
-    const size_t np = ((size_t)n + 31) & ~(size_t)31;
-    return 4 * np + 2 * (size_t)kBigCap;
+constexpr int32_t kAccSmemMax = 224 * 1024;   // of the 227 KB a CTA may have
+// The cells (8 bytes per vertex, the largest array) stay in shared memory while two CTAs
+// fit an SM with them: past that (n above ~5500) they go to the work space, in L2, and
+// more threads per SM pay for it (BA n = 8192, every changed row: 0.48 us per row with
+// two CTAs of 512 threads and the cells in L2, 0.54 with one of 1024 and the cells here).
+constexpr int32_t kAccCellSmem = 100 * 1024;
+
+AccLayout acc_layout(int n, int64_t e_cap, bool is_static) {
+    AccLayout l{};
+    const int64_t np = ((int64_t)n + 31) & ~(int64_t)31, words = group_slots(e_cap) / 32;
+    auto up = [](int64_t x) { return (x + 15) & ~(int64_t)15; };
+    int64_t sm = 0, ws = 0;
+    auto place = [&](int32_t& off, uint8_t& in_ws, int64_t bytes, int64_t limit) {
+        in_ws = sm + up(bytes) > limit;
+        int64_t& at = in_ws ? ws : sm;
+        off = (int32_t)at;
+        at += up(bytes);
+    };
+    uint8_t no = 0;
+    l.pcap = (int32_t)std::min<int64_t>(65532, 7 * np / 4);
+    place(l.row, no, 4 * np, kAccSmemMax);
+    l.cnt = (int32_t)(l.row + 2 * np);
+    place(l.level, no, 2 * kNearLevels, kAccSmemMax);
+    place(l.far, no, 2 * (np + 1), 0);
+    place(l.sink, no, np / 8, kAccSmemMax);
+    place(l.big, no, np / 8, kAccSmemMax);
+    place(l.mask, l.mask_ws, std::max(6 * words, 2 * np), kAccSmemMax);
+    l.base = (int32_t)(l.mask + 4 * words);
+    place(l.pool, l.pool_ws, 2 * (int64_t)(l.pcap + 4), kAccSmemMax);
+    place(l.cell, l.cell_ws, 8 * np, kAccCellSmem);
+    l.all_smem = !(l.mask_ws || l.pool_ws || l.cell_ws);
+    l.smem = (int32_t)sm;
+    l.ws = (int32_t)ws;
+    return l;
 }
-static size_t mask_bytes(int64_t cap) { return 4 * (size_t)((cap + 31) / 32); }
 
-constexpr size_t kSmemLimit = 180 * 1024;
-
-template <typename DT, int T>
-static int accum_occupancy(size_t smem) {
-    const int maxs = (int)kSmemLimit;
-    cudaFuncSetAttribute(k_accum_smem<DT, false, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
-    cudaFuncSetAttribute(k_accum_smem<DT, true, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxs);
+template <typename DT, bool STATIC, int T>
+static int accum_occupancy(const AccLayout& l) {
     int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_accum_smem<DT, false, T>, T, smem);
-    return per_sm;
+    if (acc_all_smem(l)) {
+        cudaFuncSetAttribute(k_accum<DT, STATIC, T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAccSmemMax);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_accum<DT, STATIC, T, true>, T, l.smem);
+    } else {
+        cudaFuncSetAttribute(k_accum<DT, STATIC, T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAccSmemMax);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_accum<DT, STATIC, T, false>, T, l.smem);
+    }
+    return std::max(per_sm, 1);
+}
+
+// Calls f with the thread count as a type; the counts an accumulation CTA is built for.
+template <typename F>
+static auto with_threads(int threads, F&& f) {
+    if (threads == 256) return f(std::integral_constant<int, 256>{});
+    if (threads == 512) return f(std::integral_constant<int, 512>{});
+    return f(std::integral_constant<int, kAccThreadsWide>{});
+}
+
+// Threads of a CTA by how many CTAs' shared memory fits an SM, so that an SM has about
+// 1024 (us per row when every changed row is re-accumulated, with 256 / 512 / 1024
+// threads: ER n = 1024 0.122 / 0.152 / 0.233, ER n = 4096 0.183 / 0.203 / 0.305, BA
+// n = 8192 0.583 / 0.478 / 0.602, BA n = 16384 1.83 / 1.29 / 1.10; static n = 16384
+// 140 / 130 / 126 ms).
+static int acc_threads_for(const AccLayout& l) {
+    const int ctas = (227 * 1024) / (l.smem + 1088);
+    return ctas >= 3 ? 256 : ctas == 2 ? 512 : kAccThreadsWide;
 }
 
 void accum_config(Dev& d) {
-    const size_t base = smem_base(d.n);
-    const size_t mb = mask_bytes(d.e_cap);
-    const bool in_smem = base + mb <= kSmemLimit;
-    const size_t smem = in_smem ? base + mb : base;
-    int per_sm = d.dbytes == 4 ? accum_occupancy<int32_t, kAccThreadsNarrow>(smem)
-                               : accum_occupancy<int64_t, kAccThreadsNarrow>(smem);
-    int per_sm_w = d.dbytes == 4 ? accum_occupancy<int32_t, kAccThreadsWide>(smem)
-                                 : accum_occupancy<int64_t, kAccThreadsWide>(smem);
-    if (per_sm < 1) per_sm = 1;
-    if (per_sm_w < 1) per_sm_w = 1;
-    d.acc_threads = (d.n >= kAccWideMinN && !d.acc_narrow_only) ? kAccThreadsWide : kAccThreadsNarrow;
-    d.acc_smem = (int32_t)smem;
-    d.acc_mask_smem = in_smem ? 1 : 0;
-    d.acc_grid = std::min(d.nsm * std::max(per_sm, per_sm_w), std::max(d.n, 1));
-    d.acc_grid_wide = std::min(d.nsm * per_sm_w, d.acc_grid);
-    // per CTA: rho (n float-float pairs) | level bounds (n + 2 ints) | slot mask if not in smem
-    const int64_t head = ((3 * (int64_t)d.n + 2) + 3) & ~(int64_t)3;
-    d.ws_stride = head + (in_smem ? 0 : (((int64_t)mb / 4 + 3) & ~(int64_t)3));
+    const int n = std::max(d.n, 1);
+    d.acc_ctas = 0;
+    d.ws_stride = 0;
+    for (int k = 0; k < 2; ++k) {
+        d.acc_lay[k] = acc_layout(d.n, d.e_cap, k == 1);
+        d.acc_threads[k] = acc_threads_for(d.acc_lay[k]);
+        auto grid = [&](int threads) {
+            return std::min(n, d.nsm * with_threads(threads, [&](auto t) {
+                constexpr int T = decltype(t)::value;
+                const AccLayout& l = d.acc_lay[k];
+                if (d.dbytes == 4) return k ? accum_occupancy<int32_t, true, T>(l) : accum_occupancy<int32_t, false, T>(l);
+                return k ? accum_occupancy<int64_t, true, T>(l) : accum_occupancy<int64_t, false, T>(l);
+            }));
+        };
+        d.acc_grid[k] = grid(d.acc_threads[k]);
+        d.acc_grid_wide[k] = grid(kAccThreadsWide);
+        d.acc_ctas = std::max({d.acc_ctas, d.acc_grid[k], d.acc_grid_wide[k]});
+        d.ws_stride = std::max<int64_t>(d.ws_stride, (d.acc_lay[k].ws + 15) / 16 * 4);
+    }
+    d.acc_wide = d.n >= kAccWideMinN && !d.acc_narrow_only;
 }
 
 // Algorithm 1 for the sources listed in rows[0..*count), or for every source.
-template <typename DT, int T>
-static void accum_t(const Dev& d, int is_static, const int32_t* rows, const int32_t* count) {
-    const int grid = T == kAccThreadsWide ? d.acc_grid_wide : d.acc_grid;
-    const size_t smem = (size_t)d.acc_smem;
-    if (is_static) launch_k(k_accum_smem<DT, true, T>, grid, T, smem, d.st, acc_args<DT>(d, rows, count));
-    else launch_k(k_accum_smem<DT, false, T>, grid, T, smem, d.st, acc_args<DT>(d, rows, count));
+template <typename DT, bool STATIC>
+static void accum_t(const Dev& d, bool wide, const int32_t* rows, const int32_t* count) {
+    const AccArgs<DT> a = acc_args<DT>(d, STATIC, rows, count);
+    const int grid = wide ? d.acc_grid_wide[STATIC] : d.acc_grid[STATIC];
+    with_threads(wide ? kAccThreadsWide : d.acc_threads[STATIC], [&](auto t) {
+        constexpr int T = decltype(t)::value;
+        if (acc_all_smem(a.lay)) launch_k(k_accum<DT, STATIC, T, true>, grid, T, a.lay.smem, d.st, a);
+        else launch_k(k_accum<DT, STATIC, T, false>, grid, T, a.lay.smem, d.st, a);
+    });
 }
 
 // The wide CTAs serve a partial wave of sources (the rows over the target cap of an
-// update with pair corrections: tens per update), where one source's latency is the
-// time (BA n = 16384: 0.30 ms per update wide, 0.41 ms with 512-thread CTAs), and the
-// static computation on the largest graphs (n = 16384: 139 ms wide, 141 ms with 512
-// threads; n = 8192: 33.7 ms wide, 30.5 ms with 512 threads, 30.3 ms with 256).  Every
-// changed row of an update without pair corrections (thousands of sources) is served
-// faster by the narrow ones, several per SM.
-constexpr int kAccStaticWideMinN = 16384;
-
+// update with pair corrections: tens per update), where one source's latency is the time.
+// Every changed row of an update without pair corrections (thousands of sources) and the
+// static computation are served faster by more sources per SM.
 static void accum(const Dev& d, int is_static, const int32_t* rows, const int32_t* count) {
-    const bool wide = d.acc_threads == kAccThreadsWide && (is_static ? d.n >= kAccStaticWideMinN : d.pair_on != 0);
+    const bool wide = d.acc_wide && !is_static && d.pair_on != 0;
     if (d.dbytes == 4) {
-        if (wide) accum_t<int32_t, kAccThreadsWide>(d, is_static, rows, count);
-        else accum_t<int32_t, kAccThreadsNarrow>(d, is_static, rows, count);
+        if (is_static) accum_t<int32_t, true>(d, wide, rows, count);
+        else accum_t<int32_t, false>(d, wide, rows, count);
     } else {
-        if (wide) accum_t<int64_t, kAccThreadsWide>(d, is_static, rows, count);
-        else accum_t<int64_t, kAccThreadsNarrow>(d, is_static, rows, count);
+        if (is_static) accum_t<int64_t, true>(d, wide, rows, count);
+        else accum_t<int64_t, false>(d, wide, rows, count);
     }
 }
 

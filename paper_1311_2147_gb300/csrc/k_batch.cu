@@ -27,11 +27,8 @@ __global__ void kb_estar(BatchArgs b, int r) {
         const BatchEOp op = b.eops[j];
         const Dev& d = b.devs[op.g];
         if (op.op.slot >= 0) {
-            d.e_src[op.op.slot] = op.op.a;
-            if (d.dbytes == 4)
-                static_cast<Arc<int32_t>*>(d.e_arc)[op.op.slot] = Arc<int32_t>{op.op.b, (int32_t)op.op.w};
-            else
-                static_cast<Arc<int64_t>*>(d.e_arc)[op.op.slot] = Arc<int64_t>{(int64_t)op.op.b, op.op.w};
+            d.e_arc[op.op.slot] = make_arc(op.op.a, op.op.b, op.op.w);
+            if (d.e_w64) d.e_w64[op.op.slot] = op.op.w;
         }
         atomicMax(d.e_len + op.op.a, op.op.len_a);
     }
@@ -288,14 +285,13 @@ __global__ void kb_bc_finish(BatchArgs b, int r, double sign) {
 
 // One source per CTA of T threads (128, 256 or 512: a tile the autotuner picks), held to
 // 64 registers so that 1024 threads share an SM.
-template <typename DT, int T>
+template <typename DT, int T, bool SM>
 __global__ void __launch_bounds__(T, 1024 / T) kb_accum(BatchArgs b, int r, const int64_t* off) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ LevelSmem<T> ls;
-    __shared__ int s_tail, s_nbig;
+    __shared__ AccShared sh;
     const int G = b.G;
     const int64_t total = off[G];
-    int32_t* wsb = b.ws + (size_t)blockIdx.x * b.ws_stride;
+    const AccMem m = acc_mem<SM>(b.lay, smem, b.ws + (size_t)blockIdx.x * b.ws_stride);
     for (int64_t j = blockIdx.x; j < total; j += gridDim.x) {
         const int g = graph_of(off, G, j);
         const Dev& d = b.devs[g];
@@ -308,17 +304,16 @@ __global__ void __launch_bounds__(T, 1024 / T) kb_accum(BatchArgs b, int r, cons
         a.Dl = d.Dl;
         a.e_off = d.e_off;
         a.e_len = d.e_len;
-        a.e_src = d.e_src;
-        a.e_arc = (const Arc<DT>*)d.e_arc;
-        a.e_cap = d.e_cap;
+        a.e_arc = d.e_arc;
+        a.e_w64 = d.e_w64;
+        a.e_used = group_slots(d.e_used);
         a.rows = acc_list(d);
         a.count = d.pair_on ? d.counts + 3 : d.counts + 1;
         a.ws = b.ws;
         a.ws_stride = b.ws_stride;
         a.err = d.err;
-        a.mask_in_smem = b.mask_in_smem;
-        const AccSmem m = acc_smem(a, smem, wsb);
-        dev_accum_source<DT, false, T>(a, a.rows[j - off[g]], m, ls, &s_tail, &s_nbig);
+        a.lay = b.lay;
+        dev_accum_source<DT, false, T, SM>(a, a.rows[j - off[g]], m, sh);
     }
 }
 
@@ -335,6 +330,24 @@ static void batch_scan(const BatchArgs& b, const BatchLaunch& L, int r, int phas
         case 8: kb_scan<DT, 8><<<grid, kScanThreads, 0, st>>>(b, r, phase, b.plan_scan, L.scan_sched); break;
         default: kb_scan<DT, 4><<<grid, kScanThreads, 0, st>>>(b, r, phase, b.plan_scan, L.scan_sched); break;
     }
+}
+
+template <typename DT, int T>
+static void batch_accum(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st) {
+    if (acc_all_smem(b.lay)) kb_accum<DT, T, true><<<L.acc_grid, T, b.lay.smem, st>>>(b, r, b.plan_acc);
+    else kb_accum<DT, T, false><<<L.acc_grid, T, b.lay.smem, st>>>(b, r, b.plan_acc);
+}
+
+template <typename DT, int T>
+static int batch_accum_occupancy(const AccLayout& l) {
+    int per_sm = 1;
+    auto occ = [&](auto kern) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, l.smem);
+    };
+    if (acc_all_smem(l)) occ(kb_accum<DT, T, true>);
+    else occ(kb_accum<DT, T, false>);
+    return std::max(per_sm, 1);
 }
 
 template <typename DT>
@@ -362,9 +375,9 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     kb_plan<<<1, 1024, 0, st>>>(b, r, 2, 2, b.plan_acc, L.scan_unroll);
     kb_bc_partial<<<nsm * L.bc_ctas, 256, 0, st>>>(b, r, b.plan_bc);
     kb_bc_finish<<<nsm * 2, 256, 0, st>>>(b, r, -1.0);
-    if (L.acc_threads == 128) kb_accum<DT, 128><<<L.acc_grid, 128, L.acc_smem, st>>>(b, r, b.plan_acc);
-    else if (L.acc_threads == 256) kb_accum<DT, 256><<<L.acc_grid, 256, L.acc_smem, st>>>(b, r, b.plan_acc);
-    else kb_accum<DT, 512><<<L.acc_grid, 512, L.acc_smem, st>>>(b, r, b.plan_acc);
+    if (L.acc_threads == 128) batch_accum<DT, 128>(b, L, r, st);
+    else if (L.acc_threads == 256) batch_accum<DT, 256>(b, L, r, st);
+    else batch_accum<DT, 512>(b, L, r, st);
     kb_bc_partial<<<nsm * L.bc_ctas, 256, 0, st>>>(b, r, b.plan_bc);
     kb_bc_finish<<<nsm * 2, 256, 0, st>>>(b, r, +1.0);
     if (L.pairs) batch_pair_launches(b, L, r, sizeof(DT), st);
@@ -375,33 +388,20 @@ void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* 
     kb_plan<<<1, 1024, 0, st>>>(b, r, kind, phase_active, out, scan_unroll);
 }
 
+// One layout for all graphs of the batch, sized for the largest.
 void batch_config(BatchLaunch& L, int dbytes, int n_max, int64_t cap_max) {
-    const size_t np = ((size_t)n_max + 31) & ~(size_t)31;
-    const size_t base = 4 * np + 2 * (size_t)kBigCap;
-    const size_t mb = 4 * (size_t)((cap_max + 31) / 32);
-    const size_t limit = 180 * 1024;
-    L.mask_in_smem = base + mb <= limit ? 1 : 0;
-    L.acc_smem = (int)(L.mask_in_smem ? base + mb : base);
-    int per_sm = 1;
-    if (L.acc_threads != 128 && L.acc_threads != 256 && L.acc_threads != 512) L.acc_threads = kAccThreadsNarrow;
-    auto occ = [&](auto kern, int threads) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, L.acc_smem);
+    L.lay = acc_layout(n_max, cap_max, false);
+    if (L.acc_threads != 128 && L.acc_threads != 256 && L.acc_threads != 512) L.acc_threads = 256;
+    auto occ = [&](auto dt) {
+        using DT = decltype(dt);
+        if (L.acc_threads == 128) return batch_accum_occupancy<DT, 128>(L.lay);
+        if (L.acc_threads == 256) return batch_accum_occupancy<DT, 256>(L.lay);
+        return batch_accum_occupancy<DT, 512>(L.lay);
     };
-    if (dbytes == 4) {
-        if (L.acc_threads == 128) occ(kb_accum<int32_t, 128>, 128);
-        else if (L.acc_threads == 256) occ(kb_accum<int32_t, 256>, 256);
-        else occ(kb_accum<int32_t, 512>, 512);
-    } else {
-        if (L.acc_threads == 128) occ(kb_accum<int64_t, 128>, 128);
-        else if (L.acc_threads == 256) occ(kb_accum<int64_t, 256>, 256);
-        else occ(kb_accum<int64_t, 512>, 512);
-    }
-    if (per_sm < 1) per_sm = 1;
+    int per_sm = dbytes == 4 ? occ(int32_t{}) : occ(int64_t{});
     if (L.acc_per_sm > 0) per_sm = std::min(per_sm, L.acc_per_sm);
     L.acc_grid = L.nsm * per_sm;
-    const int64_t head = ((3 * (int64_t)n_max + 2) + 3) & ~(int64_t)3;
-    L.ws_stride = head + (L.mask_in_smem ? 0 : (((int64_t)mb / 4 + 3) & ~(int64_t)3));
+    L.ws_stride = (L.lay.ws + 3) / 4;
 }
 
 void batch_launch_rounds(const BatchArgs& b, const BatchLaunch& L, int rounds, int dbytes, cudaStream_t st) {

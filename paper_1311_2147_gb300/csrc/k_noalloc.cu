@@ -33,9 +33,11 @@ constexpr size_t kOffDl = kOffS + al((size_t)kMaxN * kMaxN * 8);
 constexpr size_t kOffHi = kOffDl + al((size_t)kMaxN * kMaxN * sizeof(ff));
 constexpr size_t kOffLo = kOffHi + al((size_t)kMaxN * 8);
 constexpr size_t kOffGw = kOffLo + al((size_t)kMaxN * 8);
+constexpr size_t kSlots = (size_t)kMaxArcs;
+static_assert(kSlots % kGroupSlots == 0, "whole groups of slots");
 constexpr size_t kOffArc = kOffGw + al((size_t)kMaxArcs * 8);
-constexpr size_t kOffSrc = kOffArc + al((size_t)kMaxArcs * sizeof(Arc<int64_t>));
-constexpr size_t kOffLen = kOffSrc + al((size_t)kMaxArcs * 4);
+constexpr size_t kOffW64 = kOffArc + al(kSlots * sizeof(Arc));
+constexpr size_t kOffLen = kOffW64 + al(kSlots * 8);
 constexpr size_t kOffPart = kOffLen + al((size_t)kMaxN * 4);
 constexpr size_t kOffErr = kOffPart + al((size_t)((kMaxN + kRowsPerBlock - 1) / kRowsPerBlock) * kMaxN * sizeof(ff));
 constexpr size_t kOffCnt = kOffErr + 256;
@@ -74,27 +76,33 @@ cudaError_t scratch_address(unsigned char** out) {
 }
 
 // Pack the caller's CSR into the slot format of the accumulation (every arc a slot),
-// and check each arc: endpoints in range, no self-loop, weight in [1, INF-1].
+// and check each arc: endpoints in range, no self-loop, weight in [1, INF-1].  The
+// slots past the arcs, up to a whole group, are empty.
 template <typename DT>
 __global__ void k_pack_graph(int n, int64_t arcs, const int32_t* off, const int32_t* dst, const int64_t* w,
-                             DT* gw, Arc<DT>* arc, int32_t* src, int32_t* len, int32_t* err) {
+                             DT* gw, Arc* arc, int64_t* w64, int32_t* len, int32_t* err) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
         const int32_t a = off[i], b = off[i + 1];
-        len[i] = b - a;
-        if (a < 0 || b < a || b > arcs) set_err(err, ERRF_ARG_DEVICE);
-        else
+        if (a < 0 || b < a || b > arcs) {
+            len[i] = 0;
+            set_err(err, ERRF_ARG_DEVICE);
+        } else {
+            len[i] = b - a;
             for (int32_t e = a; e < b; ++e) {
-                src[e] = (int32_t)i;
                 if (dst[e] == (int32_t)i) set_err(err, ERRF_ARG_DEVICE);   // self-loop
+                arc[e] = make_arc((int32_t)i, dst[e], w[e]);
+                if (sizeof(DT) == 8) w64[e] = w[e];
             }
+        }
     }
     if (i < arcs) {
         const int32_t b = dst[i];
         const int64_t x = w[i];
         if (b < 0 || b >= n || x < 1 || x >= Inf<DT>::v) set_err(err, ERRF_ARG_DEVICE);
         gw[i] = (DT)x;
-        arc[i] = Arc<DT>{(b >= 0 && b < n) ? (DT)b : (DT)-1, (DT)x};
+    } else if (i < group_slots(arcs)) {
+        arc[i] = empty_arc();
     }
 }
 
@@ -138,31 +146,27 @@ extern "C" int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* 
     d.g_arcs = arcs;
     d.e_off = const_cast<int32_t*>(d_off);
     d.e_len = reinterpret_cast<int32_t*>(base + kOffLen);
-    d.e_src = reinterpret_cast<int32_t*>(base + kOffSrc);
-    d.e_arc = base + kOffArc;
-    d.e_cap = arcs;
+    d.e_arc = reinterpret_cast<Arc*>(base + kOffArc);
+    d.e_w64 = i64 ? reinterpret_cast<int64_t*>(base + kOffW64) : nullptr;
+    d.e_cap = d.e_used = arcs;
     d.err = reinterpret_cast<int32_t*>(base + kOffErr);
     d.counts = reinterpret_cast<int32_t*>(base + kOffCnt);
     d.stats = reinterpret_cast<int64_t*>(base + kOffStats);
     d.partial = reinterpret_cast<ff*>(base + kOffPart);
     d.nrb_max = (n + kRowsPerBlock - 1) / kRowsPerBlock;
     accum_config(d);
-    if ((size_t)d.acc_grid * (size_t)d.ws_stride * sizeof(int32_t) > kWsBytes) {
-        // fewer CTAs keep the work space inside its share of the scratch
-        d.acc_grid = (int32_t)(kWsBytes / ((size_t)d.ws_stride * sizeof(int32_t)));
-        if (d.acc_grid < 1) return BC_ERR_ARG;
-    }
+    if ((size_t)d.acc_ctas * (size_t)d.ws_stride * sizeof(int32_t) > kWsBytes) return BC_ERR_ARG;   // not for n <= kMaxN
     d.ws = reinterpret_cast<int32_t*>(base + kOffWs);
     // the error word and counters start at zero on every call (the scratch keeps the
     // previous call's contents)
     if (cudaMemsetAsync(d.err, 0, 256 * 3, d.st) != cudaSuccess) return BC_ERR_CUDA;
-    const int blocks = (int)((std::max<int64_t>(n, arcs) + 255) / 256);
+    const int blocks = (int)((std::max<int64_t>(n, group_slots(arcs)) + 255) / 256);
     if (d.dbytes == 4)
-        k_pack_graph<int32_t><<<blocks, 256, 0, d.st>>>(n, arcs, d_off, d_dst, d_w, (int32_t*)d.g_w,
-                                                         (Arc<int32_t>*)d.e_arc, d.e_src, d.e_len, d.err);
+        k_pack_graph<int32_t><<<blocks, 256, 0, d.st>>>(n, arcs, d_off, d_dst, d_w, (int32_t*)d.g_w, d.e_arc,
+                                                         d.e_w64, d.e_len, d.err);
     else
-        k_pack_graph<int64_t><<<blocks, 256, 0, d.st>>>(n, arcs, d_off, d_dst, d_w, (int64_t*)d.g_w,
-                                                         (Arc<int64_t>*)d.e_arc, d.e_src, d.e_len, d.err);
+        k_pack_graph<int64_t><<<blocks, 256, 0, d.st>>>(n, arcs, d_off, d_dst, d_w, (int64_t*)d.g_w, d.e_arc,
+                                                         d.e_w64, d.e_len, d.err);
     launch_sssp(d);
     launch_accum(d, 1);
     launch_bc_rows(d, +1, 1);

@@ -1046,7 +1046,8 @@ template <typename DT>
 struct WalkArgs {
     const int32_t* e_off;
     const int32_t* e_len;
-    const Arc<DT>* e_arc;
+    const Arc* e_arc;
+    const int64_t* e_w64;
     int32_t* list;      // [walk warps * n] vertices of a walk, level by level (phase 1)
     int32_t* buf;       // [cap] vertices found by the walks of the update's units
     int64_t cap;
@@ -1182,13 +1183,14 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkCtasPerSm) k_walk_units(Pai
                                 bool fresh = false;
                                 int x = -1;
                                 if (k < tot) {
-                                    const Arc<DT> arc = w.e_arc[offj + (k - exj)];
-                                    x = (int)arc.dst;
-                                    int64_t wv = (int64_t)arc.w;
+                                    const int e = offj + (k - exj);
+                                    const Arc arc = w.e_arc[e];
+                                    x = arc.dst();
+                                    int64_t wv = sizeof(DT) == 4 ? (int64_t)arc.w : w.e_w64[e];
                                     if (!is_new && (yj == v || x == v)) {
                                         const int o = yj == v ? x : yj;
-                                        for (int e = 0; e < w.upd.k; ++e)
-                                            if (w.upd.x[e] == o) wv = w.upd.wold[e];
+                                        for (int u = 0; u < w.upd.k; ++u)
+                                            if (w.upd.x[u] == o) wv = w.upd.wold[u];
                                     }
                                     if (x >= 0 && x != s && wv >= 0 && wv <= dyj) {   // else no predecessor
                                         const int64_t dx = walk_d<DT>(a, rs, s, x, is_new);
@@ -1469,7 +1471,7 @@ cudaError_t walk_setup() {
 template <typename DT>
 static void launch_walks(const Dev& d, const WalkUpd& upd, int nchunks) {
     const int grid = d.nsm * kWalkCtasPerSm, rgrid = d.nsm * kWalkRowCtasPerSm;
-    WalkArgs<DT> w{d.e_off, d.e_len, (const Arc<DT>*)d.e_arc, d.walk_list, d.walk_buf, d.walk_cap, d.walk_useg,
+    WalkArgs<DT> w{d.e_off, d.e_len, d.e_arc, d.e_w64, d.walk_list, d.walk_buf, d.walk_cap, d.walk_useg,
                    d.walk_acc2, d.walk_tl, d.walk_ctl, d.walk_rowE, d.stats, nchunks, upd};
     launch_k(k_walk_units<DT>, grid, kWalkThreads, walk_smem(d.n), d.st, pair_args<DT>(d), w);
     // phase 2: the heaviest rows (a few CTAs with a long tail) on the third stream beside

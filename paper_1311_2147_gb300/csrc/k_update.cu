@@ -23,30 +23,28 @@
 
 namespace bcg {
 
-__global__ void k_estar_write(int32_t* e_src, void* e_arc, int32_t* e_len, int dbytes, EOps ops) {
+__global__ void k_estar_write(Arc* e_arc, int64_t* e_w64, int32_t* e_len, EOps ops) {
     pdl_enter();
     int i = threadIdx.x;
     if (i >= ops.count) return;
     const EOp o = ops.op[i];
     if (o.slot >= 0) {
-        e_src[o.slot] = o.a;
-        if (dbytes == 4) static_cast<Arc<int32_t>*>(e_arc)[o.slot] = Arc<int32_t>{o.b, (int32_t)o.w};
-        else static_cast<Arc<int64_t>*>(e_arc)[o.slot] = Arc<int64_t>{(int64_t)o.b, o.w};
+        e_arc[o.slot] = make_arc(o.a, o.b, o.w);
+        if (e_w64) e_w64[o.slot] = o.w;
     }
     atomicMax(e_len + o.a, o.len_a);   // lengths only grow between rebuilds
 }
 
 // One CTA per move: copy the segment, empty its old slots, point e_off[a] at the copy.
 // Source and destination ranges of all moves are disjoint.
-template <typename DT>
-__global__ void k_estar_move(int32_t* e_off, int32_t* e_src, Arc<DT>* e_arc, EMoves moves) {
+__global__ void k_estar_move(int32_t* e_off, Arc* e_arc, int64_t* e_w64, EMoves moves) {
     pdl_enter();
     if ((int)blockIdx.x >= moves.count) return;
     const EMove m = moves.mv[blockIdx.x];
     for (int i = threadIdx.x; i < m.len; i += blockDim.x) {
         e_arc[m.to + i] = e_arc[m.from + i];
-        e_src[m.to + i] = m.a;
-        e_arc[m.from + i].dst = -1;
+        if (e_w64) e_w64[m.to + i] = e_w64[m.from + i];
+        e_arc[m.from + i] = empty_arc();
     }
     if (threadIdx.x == 0) e_off[m.a] = m.to;
 }
@@ -353,13 +351,14 @@ __global__ void k_write_row(int n, int ld, DT* D, uint64_t* S, int v, const DT* 
 // keep[e] = 1 when slot e holds an arc (a,b) with w(a,b) == d(a,b), i.e. an arc of E*
 // (an arc lies on a shortest path exactly when it is one itself).
 template <typename DT>
-__global__ void k_estar_keep(int ld, const DT* D, const int32_t* e_src, const Arc<DT>* e_arc,
+__global__ void k_estar_keep(int ld, const DT* D, const Arc* e_arc, const int64_t* e_w64,
                              int64_t cap, uint8_t* keep) {
     pdl_enter();
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= cap) return;
-    const Arc<DT> a = e_arc[e];
-    keep[e] = (a.dst >= 0 && (int64_t)D[(size_t)e_src[e] * ld + a.dst] == (int64_t)a.w) ? 1 : 0;
+    const Arc a = e_arc[e];
+    const int64_t w = e_w64 ? e_w64[e] : (int64_t)a.w;
+    keep[e] = (!a.empty() && (int64_t)D[(size_t)a.src() * ld + a.dst()] == w) ? 1 : 0;
 }
 
 // Fused pass of an undirected edge update {u, v} with weight w, preparation (one thread
@@ -442,15 +441,12 @@ static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 void launch_estar_write(const Dev& d, const EOps& ops) {
     if (ops.count <= 0) return;
-    launch_k(k_estar_write, 1, kMaxEOps, 0, d.st, d.e_src, d.e_arc, d.e_len, d.dbytes, ops);
+    launch_k(k_estar_write, 1, kMaxEOps, 0, d.st, d.e_arc, d.e_w64, d.e_len, ops);
 }
 
 void launch_estar_move(const Dev& d, const EMoves& moves) {
     if (moves.count <= 0) return;
-    if (d.dbytes == 4)
-        launch_k(k_estar_move<int32_t>, moves.count, 128, 0, d.st, d.e_off, d.e_src, (Arc<int32_t>*)d.e_arc, moves);
-    else
-        launch_k(k_estar_move<int64_t>, moves.count, 128, 0, d.st, d.e_off, d.e_src, (Arc<int64_t>*)d.e_arc, moves);
+    launch_k(k_estar_move, moves.count, 128, 0, d.st, d.e_off, d.e_arc, d.e_w64, moves);
 }
 
 void launch_alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
@@ -640,9 +636,9 @@ void launch_edge_scan(const Dev& d) {
 void launch_estar_keep(const Dev& d, uint8_t* keep) {
     if (d.e_cap <= 0) return;
     if (d.dbytes == 4)
-        launch_k(k_estar_keep<int32_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.ld, (const int32_t*)d.D, d.e_src, (const Arc<int32_t>*)d.e_arc, d.e_cap, keep);
+        launch_k(k_estar_keep<int32_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.ld, (const int32_t*)d.D, d.e_arc, d.e_w64, d.e_cap, keep);
     else
-        launch_k(k_estar_keep<int64_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.ld, (const int64_t*)d.D, d.e_src, (const Arc<int64_t>*)d.e_arc, d.e_cap, keep);
+        launch_k(k_estar_keep<int64_t>, nblk(d.e_cap, 256), 256, 0, d.st, d.ld, (const int64_t*)d.D, d.e_arc, d.e_w64, d.e_cap, keep);
 }
 
 }  // namespace bcg

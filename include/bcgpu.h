@@ -139,12 +139,11 @@ typedef struct bc_info {
  *   flags        exactly one of BC_DIRECTED / BC_UNDIRECTED, and one of
  *                BC_DIST_I32 / BC_DIST_I64; optionally BC_STATIC_ALL_ARCS.
  *   cuda_stream  a cudaStream_t (NULL = legacy default stream).
- * The all-pairs distances come from one search per source (one CTA each).  By default
- * the searches are restricted to E* as it becomes known (Section 6, Algorithm 6 step
- * 1, whose Hidden Paths algorithm examines only arcs of E*): once the search from a
- * has finished, the arcs (a,b) with w(a,b) > d(a,b) are left out of every later search,
- * and the sources run highest out-degree first.  BC_STATIC_ALL_ARCS searches every
- * arc instead (the same results; kept for comparison).
+ * The all-pairs distances come from one search per source.  By default the searches of a
+ * dense graph are restricted to a set of arcs that contains E* (Section 6, Algorithm 6
+ * step 1, whose Hidden Paths algorithm examines only arcs of E*): the arcs no longer than
+ * the paths over each vertex's lightest arcs.  BC_STATIC_ALL_ARCS searches every arc
+ * instead (the same results; kept for comparison).
  * Synchronous.  Returns BC_ERR_ARG for a malformed graph or flags, BC_ERR_OOM when
  * the n x n state does not fit, and the device-side errors above.
  */

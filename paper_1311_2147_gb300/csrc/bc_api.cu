@@ -703,25 +703,25 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     d.nrb_max = (n + kRowsPerBlock - 1) / kRowsPerBlock;
     d.g_arcs = arcs;
     if (g->dbytes == 4) {
-        int32_t *pD, *pfD, *pcD, *pcD2, *pgw;
+        int32_t *pD, *pfD, *pcD, *pcD2;
         if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, d.ld)) ||
-            (rc = dalloc(g, &pcD2, d.ld)) || (rc = dalloc(g, &pgw, arcs))) {
+            (rc = dalloc(g, &pcD2, d.ld))) {
             destroy_all(g);
             return fail(nullptr, rc, "device allocation failed");
         }
-        d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2; d.g_w = pgw;
+        d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2;
     } else {
-        int64_t *pD, *pfD, *pcD, *pcD2, *pgw;
+        int64_t *pD, *pfD, *pcD, *pcD2;
         if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, d.ld)) ||
-            (rc = dalloc(g, &pcD2, d.ld)) || (rc = dalloc(g, &pgw, arcs))) {
+            (rc = dalloc(g, &pcD2, d.ld))) {
             destroy_all(g);
             return fail(nullptr, rc, "device allocation failed");
         }
-        d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2; d.g_w = pgw;
+        d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2;
     }
     if ((rc = dalloc(g, &d.S, nn)) || (rc = dalloc(g, &d.Dl, nn)) || (rc = dalloc(g, &d.bc_hi, n)) ||
-        (rc = dalloc(g, &d.bc_lo, n)) || (rc = dalloc(g, &d.g_off, n + 1)) || (rc = dalloc(g, &d.g_src, arcs)) ||
-        (rc = dalloc(g, &d.g_dst, arcs)) || (rc = dalloc(g, &d.e_off, n + 1)) || (rc = dalloc(g, &d.e_len, n)) ||
+        (rc = dalloc(g, &d.bc_lo, n)) || (rc = dalloc(g, &d.g_arc, arcs)) || (rc = dalloc(g, &d.g_off, n + 1)) || (rc = dalloc(g, &d.g_count, 3)) ||
+        (!i32 && (rc = dalloc(g, &d.g_w64, arcs))) || (rc = dalloc(g, &d.e_off, n + 1)) || (rc = dalloc(g, &d.e_len, n)) ||
         (rc = dalloc(g, &d.err, 1)) || (rc = dalloc(g, &d.stats, kStats)) || (rc = dalloc(g, &d.mark, n)) ||
         (rc = dalloc(g, &d.changed, n)) || (rc = dalloc(g, &d.rows, n)) || (rc = dalloc(g, &d.acc_rows, n)) ||
         (rc = dalloc(g, &d.counts, 8)) || (rc = dalloc(g, &d.fS, n)) || (rc = dalloc(g, &d.fM, n)) ||
@@ -806,36 +806,20 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     }
     CKI(cudaStreamSynchronize(d.st));
     CKI(cudaEventRecord(e0, d.st));
+    std::vector<Arc> garc(arcs);
+    int64_t w_max = 1;
+    for (int64_t i = 0; i < arcs; ++i) {
+        garc[i] = make_arc(csrc[i], cdst[i], cw[i]);
+        w_max = std::max(w_max, cw[i]);
+    }
+    CKI(cudaMemcpyAsync(d.g_arc, garc.data(), sizeof(Arc) * arcs, cudaMemcpyHostToDevice, d.st));
+    if (d.g_w64) CKI(cudaMemcpyAsync(d.g_w64, cw.data(), sizeof(int64_t) * arcs, cudaMemcpyHostToDevice, d.st));
+    const unsigned long long garcs[3] = {(unsigned long long)arcs, 0ull, 0ull};
+    CKI(cudaMemcpyAsync(d.g_count, garcs, sizeof(garcs), cudaMemcpyHostToDevice, d.st));
     CKI(cudaMemcpyAsync(d.g_off, off.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, d.st));
-    CKI(cudaMemcpyAsync(d.g_src, csrc.data(), sizeof(int32_t) * arcs, cudaMemcpyHostToDevice, d.st));
-    CKI(cudaMemcpyAsync(d.g_dst, cdst.data(), sizeof(int32_t) * arcs, cudaMemcpyHostToDevice, d.st));
-    std::vector<int32_t> w32;
-    if (g->dbytes == 4) {
-        w32.resize(arcs);
-        for (int64_t i = 0; i < arcs; ++i) w32[i] = (int32_t)cw[i];
-        CKI(cudaMemcpyAsync(d.g_w, w32.data(), sizeof(int32_t) * arcs, cudaMemcpyHostToDevice, d.st));
-    } else {
-        CKI(cudaMemcpyAsync(d.g_w, cw.data(), sizeof(int64_t) * arcs, cudaMemcpyHostToDevice, d.st));
-    }
     // all-pairs distances, then E* read off them.  Unless asked for the search over every
-    // arc, arcs found outside E* are pruned as the searches finish (k_static.cu), the
-    // sources running highest out-degree first.
-    const bool prune = (flags & BC_STATIC_ALL_ARCS) == 0 && arcs > 0;
-    if (prune) {
-        std::vector<int32_t> order(n);
-        for (int32_t i = 0; i < n; ++i) order[i] = i;
-        std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) {
-            return off[a + 1] - off[a] > off[b + 1] - off[b];
-        });
-        // scratch in the dependency rows (n^2 float-float pairs, >= 4 (arcs + n) bytes),
-        // which the accumulation writes only after the searches: no allocation here (a
-        // cudaFree waits for the whole device, other handles' work included)
-        d.p_dst = reinterpret_cast<int32_t*>(d.Dl);
-        d.s_order = d.p_dst + arcs;
-        CKI(cudaMemcpyAsync(d.p_dst, d.g_dst, sizeof(int32_t) * arcs, cudaMemcpyDeviceToDevice, d.st));
-        CKI(cudaMemcpyAsync(d.s_order, order.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, d.st));
-    }
-    launch_sssp(d);
+    // arc, arcs of a dense graph that cannot be in E* are left out (k_static.cu).
+    launch_sssp(d, w_max, (flags & BC_STATIC_ALL_ARCS) != 0);
     // the E* flags, also in the dependency rows' memory (free until the accumulation)
     uint8_t* d_flags = reinterpret_cast<uint8_t*>(d.Dl);
     launch_estar_flags(d, d_flags);
@@ -843,7 +827,6 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     CKI(cudaMemcpyAsync(eflags.data(), d_flags, arcs, cudaMemcpyDeviceToHost, d.st));
     CKI(cudaStreamSynchronize(d.st));
     CKI(cudaGetLastError());
-    d.p_dst = d.s_order = nullptr;
     {
         std::vector<HArc> estar;
         for (int64_t i = 0; i < arcs; ++i)

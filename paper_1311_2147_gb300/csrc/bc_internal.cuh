@@ -189,14 +189,12 @@ struct Dev {
     ff* Dl;
     double* bc_hi;
     double* bc_lo;
-    // full graph (G or G_D) CSR, used by the static computation
-    int32_t* g_off;
-    int32_t* g_src;
-    int32_t* g_dst;
-    void* g_w;
-    int32_t* p_dst;      // static search: working copy of g_dst pruned to E* (NULL: no pruning)
-    int32_t* s_order;    // static search: sources in order (NULL: 0 .. n-1)
+    // full graph (G or G_D), used by the static computation
+    Arc* g_arc;          // [g_arcs] by tail
+    int64_t* g_w64;      // [g_arcs] weights in full (int64 distances; else NULL)
+    int32_t* g_off;      // [n + 1] first arc of each tail (NULL: the search takes every arc)
     int64_t g_arcs;
+    unsigned long long* g_count;   // [3] number of arcs in g_arc, and of two lists of the search
     // E*+ CSR with slack
     int32_t* e_off;
     int32_t* e_len;
@@ -391,7 +389,7 @@ void launch_bc_rows(const Dev& d, int sign, int is_static);
 void launch_bc_rows_list(const Dev& d, int sign, const int32_t* rows, const int32_t* count);
 
 // ---- launches (k_static.cu) ----
-void launch_sssp(const Dev& d);
+void launch_sssp(const Dev& d, int64_t w_max, bool all_arcs);
 void launch_estar_flags(const Dev& d, uint8_t* flags);
 
 }  // namespace bcg

@@ -32,10 +32,9 @@ constexpr size_t kOffS = kOffD + al((size_t)kMaxN * kMaxN * 8);
 constexpr size_t kOffDl = kOffS + al((size_t)kMaxN * kMaxN * 8);
 constexpr size_t kOffHi = kOffDl + al((size_t)kMaxN * kMaxN * sizeof(ff));
 constexpr size_t kOffLo = kOffHi + al((size_t)kMaxN * 8);
-constexpr size_t kOffGw = kOffLo + al((size_t)kMaxN * 8);
 constexpr size_t kSlots = (size_t)kMaxArcs;
 static_assert(kSlots % kGroupSlots == 0, "whole groups of slots");
-constexpr size_t kOffArc = kOffGw + al((size_t)kMaxArcs * 8);
+constexpr size_t kOffArc = kOffLo + al((size_t)kMaxN * 8);
 constexpr size_t kOffW64 = kOffArc + al(kSlots * sizeof(Arc));
 constexpr size_t kOffLen = kOffW64 + al(kSlots * 8);
 constexpr size_t kOffPart = kOffLen + al((size_t)kMaxN * 4);
@@ -79,9 +78,10 @@ cudaError_t scratch_address(unsigned char** out) {
 // and check each arc: endpoints in range, no self-loop, weight in [1, INF-1].  The
 // slots past the arcs, up to a whole group, are empty.
 template <typename DT>
-__global__ void k_pack_graph(int n, int64_t arcs, const int32_t* off, const int32_t* dst, const int64_t* w,
-                             DT* gw, Arc* arc, int64_t* w64, int32_t* len, int32_t* err) {
+__global__ void k_pack_graph(int n, int64_t arcs, unsigned long long* count, const int32_t* off, const int32_t* dst, const int64_t* w,
+                             Arc* arc, int64_t* w64, int32_t* len, int32_t* err) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0) *count = (unsigned long long)arcs;
     if (i < n) {
         const int32_t a = off[i], b = off[i + 1];
         if (a < 0 || b < a || b > arcs) {
@@ -100,7 +100,6 @@ __global__ void k_pack_graph(int n, int64_t arcs, const int32_t* off, const int3
         const int32_t b = dst[i];
         const int64_t x = w[i];
         if (b < 0 || b >= n || x < 1 || x >= Inf<DT>::v) set_err(err, ERRF_ARG_DEVICE);
-        gw[i] = (DT)x;
     } else if (i < group_slots(arcs)) {
         arc[i] = empty_arc();
     }
@@ -140,18 +139,18 @@ extern "C" int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* 
     d.Dl = reinterpret_cast<ff*>(base + kOffDl);
     d.bc_hi = reinterpret_cast<double*>(base + kOffHi);
     d.bc_lo = reinterpret_cast<double*>(base + kOffLo);
-    d.g_off = const_cast<int32_t*>(d_off);
-    d.g_dst = const_cast<int32_t*>(d_dst);
-    d.g_w = base + kOffGw;
     d.g_arcs = arcs;
     d.e_off = const_cast<int32_t*>(d_off);
     d.e_len = reinterpret_cast<int32_t*>(base + kOffLen);
     d.e_arc = reinterpret_cast<Arc*>(base + kOffArc);
     d.e_w64 = i64 ? reinterpret_cast<int64_t*>(base + kOffW64) : nullptr;
     d.e_cap = d.e_used = arcs;
+    d.g_arc = d.e_arc;
+    d.g_w64 = d.e_w64;
     d.err = reinterpret_cast<int32_t*>(base + kOffErr);
     d.counts = reinterpret_cast<int32_t*>(base + kOffCnt);
     d.stats = reinterpret_cast<int64_t*>(base + kOffStats);
+    d.g_count = reinterpret_cast<unsigned long long*>(base + kOffStats + 128);
     d.partial = reinterpret_cast<ff*>(base + kOffPart);
     d.nrb_max = (n + kRowsPerBlock - 1) / kRowsPerBlock;
     accum_config(d);
@@ -162,12 +161,10 @@ extern "C" int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* 
     if (cudaMemsetAsync(d.err, 0, 256 * 3, d.st) != cudaSuccess) return BC_ERR_CUDA;
     const int blocks = (int)((std::max<int64_t>(n, group_slots(arcs)) + 255) / 256);
     if (d.dbytes == 4)
-        k_pack_graph<int32_t><<<blocks, 256, 0, d.st>>>(n, arcs, d_off, d_dst, d_w, (int32_t*)d.g_w, d.e_arc,
-                                                         d.e_w64, d.e_len, d.err);
+        k_pack_graph<int32_t><<<blocks, 256, 0, d.st>>>(n, arcs, d.g_count, d_off, d_dst, d_w, d.e_arc, d.e_w64, d.e_len, d.err);
     else
-        k_pack_graph<int64_t><<<blocks, 256, 0, d.st>>>(n, arcs, d_off, d_dst, d_w, (int64_t*)d.g_w, d.e_arc,
-                                                         d.e_w64, d.e_len, d.err);
-    launch_sssp(d);
+        k_pack_graph<int64_t><<<blocks, 256, 0, d.st>>>(n, arcs, d.g_count, d_off, d_dst, d_w, d.e_arc, d.e_w64, d.e_len, d.err);
+    launch_sssp(d, 0, true);
     launch_accum(d, 1);
     launch_bc_rows(d, +1, 1);
     k_scores_out<<<(n + 255) / 256, 256, 0, d.st>>>(n, d.bc_hi, d.bc_lo, dir ? 1.0 : 0.5, d_scores, d.err);

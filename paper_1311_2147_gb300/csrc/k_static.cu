@@ -2,186 +2,319 @@
 //
 // bc_init_static needs d(s,t) for every pair before E* can be read off it.  Brandes
 // (Appendix, Algorithm 7) runs Dijkstra from every source; a priority queue does not
-// map well onto a CTA, so each CTA runs a label-correcting (Bellman-Ford) sweep from
-// one source at a time with a frontier bitmap in shared memory: every round relaxes
-// the out-arcs of the vertices whose distance dropped in the round before, until no
-// distance drops.  With positive weights this ends after at most n-1 rounds with the
-// same distances Dijkstra settles.  The distance row lives in shared memory when it
-// fits, else in its row of D.
+// map well onto a CTA, so each CTA runs a label-correcting (Bellman-Ford) search from a
+// group of sources at a time: every round relaxes, a lane per arc, the arcs whose tail's
+// distance dropped in the round before, until no distance drops.  With positive weights
+// this ends after at most n-1 rounds with the same distances Dijkstra settles.
+//
+// What bounds it: shared-memory gathers (two per arc, source and round in which the tail
+// changed; the random one takes about three bank cycles) and, for few sources per group,
+// the arcs' L2 reads of every round.  The arcs are read in order, 8 bytes each, once per
+// round for all sources of the group; before, a warp took the changed vertices of one
+// source one after the other, a chain of two L2 reads each.  Static search, before and
+// now: BA n = 4096 4.79 and 1.71 ms, ER n = 3001 (int64) 2.32 and 0.66 ms, BA n = 16384
+// 91 and 33 ms.
 //
 // E* (Section 1: arcs on some shortest path) is then {(a,b) : w(a,b) = d(a,b)}: the
 // one-arc path a->b is shortest exactly when the arc lies on a shortest path (a
 // sub-path of a shortest path is shortest).
 //
-// E* pruning (Section 6, Algorithm 6 step 1: the Hidden Paths algorithm examines only
-// arcs of E*).  A search from s needs only the arcs of E* (every shortest path is made
-// of them), and an arc (a,b) is known to be in E* or not as soon as the search from a
-// has finished: w(a,b) = d(a,b).  So with pruning on, the CTA that finishes the
-// search from a overwrites the head of every arc of a that is not in E* with -1 in a
-// working copy of the arc heads, and every later search skips those arcs.  A search
-// that reads a head while it is being overwritten sees either the head or -1; both are
-// correct, since a search may use any set of arcs that contains E*.  The sources run in
-// the given order, highest out-degree first, so that most arcs are decided early.
-// (Hidden Paths settles the pairs of all sources in one global distance order and so
-// never examines an arc outside E*; this form examines each arc at most until its
-// tail's own search has finished.)
+// Dense graphs (Section 6, Algorithm 6 step 1: the Hidden Paths algorithm examines only
+// arcs of E*; a search may use any set of arcs that contains E*): a first search over each
+// vertex's lightest arcs bounds every distance from above, arcs longer than that bound
+// are not in E*, and the search runs over the others.  Hidden Paths finds E* exactly, in
+// one global distance order over all sources; this finds a little more than E* and keeps
+// the sources independent.
+#include <algorithm>
+#include <type_traits>
+
 #include "bc_internal.cuh"
 
 namespace bcg {
 
-constexpr int kSsspThreads = 512;
+constexpr int kSsspMaxSources = 16;   // sources of a group (bits of a change mask)
+
+__device__ __forceinline__ void atomic_min_dist(uint32_t* p, uint32_t v) { atomicMin(p, v); }
+__device__ __forceinline__ void atomic_min_dist(int64_t* p, int64_t v) {
+    atomicMin(reinterpret_cast<long long*>(p), (long long)v);
+}
+template <typename DS> struct Far;
+template <> struct Far<uint32_t> { static constexpr uint32_t v = INT32_MAX; };
+template <> struct Far<int64_t> { static constexpr int64_t v = INT64_MAX; };
+
+// d(s,b) through an arc of weight w, or at least Far where the sum does not fit.
+__device__ __forceinline__ uint32_t through(uint32_t d, uint32_t w) { return d + w; }   // both below 2^31
+__device__ __forceinline__ int64_t through(int64_t d, int64_t w) { return w > INT64_MAX - 1 - d ? INT64_MAX : d + w; }
 
 template <typename DT>
-__device__ __forceinline__ int64_t ld_relaxed(const DT* p) {
-    return (int64_t)*reinterpret_cast<const volatile DT*>(p);
-}
+struct SsspArgs {
+    int n, ld;
+    const Arc* arc;        // arcs, by tail
+    const int64_t* w64;    // their weights in full (int64 distances)
+    const unsigned long long* arcs;   // their number
+    DT* D;
+    int32_t* err;
+    int S;                 // sources of a group
+    int check;             // a distance might not fit its type
+};
 
-__device__ __forceinline__ int32_t atomic_min_dt(int32_t* p, int32_t v) { return atomicMin(p, v); }
-__device__ __forceinline__ int64_t atomic_min_dt(int64_t* p, int64_t v) {
-    return (int64_t)atomicMin(reinterpret_cast<long long*>(p), (long long)v);
-}
-
-// order: the sources in the order to run them (NULL: 0 .. n-1).  pdst: the working
-// copy of the arc heads to prune (NULL: every arc is searched, dst is read).
-template <typename DT, bool SMEM_DIST>
-__global__ void __launch_bounds__(kSsspThreads)
-k_sssp(int n, int ld, const int32_t* __restrict__ off, const int32_t* __restrict__ dst,
-       const DT* __restrict__ w, DT* D, int32_t* err, const int32_t* __restrict__ order, int32_t* pdst) {
+// A group of S sources per CTA: their distance rows (DS) and two change masks per vertex
+// (bit k: d(s_k, x) dropped in the last round / in this one) in shared memory.  A round
+// goes over all arcs, a lane per arc; a vector of 32 arcs is skipped for the sources in
+// which none of its tails changed.
+template <typename DT, typename DS, int T>
+__global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int words = (n + 31) >> 5;
-    DT* dist_s = reinterpret_cast<DT*>(smem);
-    uint32_t* cur = reinterpret_cast<uint32_t*>(smem + (SMEM_DIST ? (((size_t)n * sizeof(DT) + 15) & ~(size_t)15) : 0));
-    uint32_t* nxt = cur + words;
-    __shared__ int s_sat;
+    const int n = a.n, np = (n + 31) & ~31;
+    DS* dist = reinterpret_cast<DS*>(smem);
+    uint32_t* cur = reinterpret_cast<uint32_t*>(dist + (size_t)a.S * np);
+    uint32_t* nxt = cur + np / 2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int nwarps = kSsspThreads / 32;
-    const int64_t INF = Inf<DT>::v;
-    const int32_t* heads = pdst ? pdst : dst;
-    for (int si = blockIdx.x; si < n; si += gridDim.x) {
-        if (block_err(err)) return;
-        const int s = order ? order[si] : si;
-        DT* dist = SMEM_DIST ? dist_s : D + (size_t)s * ld;
-        for (int t = tid; t < n; t += kSsspThreads) dist[t] = (t == s) ? (DT)0 : (DT)INF;
-        for (int q = tid; q < words; q += kSsspThreads) {
-            cur[q] = (q == (s >> 5)) ? (1u << (s & 31)) : 0u;
-            nxt[q] = 0u;
+    constexpr int NW = T / 32, U = 4;
+    const int64_t arcs = (int64_t)*a.arcs;
+    const int nchunk = (int)((arcs + 31) >> 5);
+    for (int s0 = blockIdx.x * a.S; s0 < n; s0 += gridDim.x * a.S) {
+        if (block_err(a.err)) return;
+        const int S = min(a.S, n - s0);
+        for (int t = tid; t < S * np; t += T) dist[t] = Far<DS>::v;
+        for (int t = tid; t < np / 2; t += T) cur[t] = nxt[t] = 0u;
+        __syncthreads();
+        if (tid < S) {
+            dist[(size_t)tid * np + s0 + tid] = (DS)0;
+            atomicOr(cur + ((s0 + tid) >> 1), (1u << tid) << (((s0 + tid) & 1) << 4));
         }
-        if (tid == 0) s_sat = 0;
         __syncthreads();
         bool converged = false;
         for (int round = 0; round <= n; ++round) {
-            for (int q = warp; q < words; q += nwarps) {
-                uint32_t bits = cur[q];
-                while (bits) {
-                    const int x = (q << 5) + __ffs(bits) - 1;
-                    bits &= bits - 1u;
-                    const int64_t dx = ld_relaxed(dist + x);
-                    const int end = off[x + 1];
-                    for (int e = off[x] + lane; e < end; e += 32) {
-                        const int b = ld_relaxed(heads + e);
-                        if (b < 0) continue;   // pruned: not in E*
-                        const int64_t nd = dsum<DT>(dx, (int64_t)w[e]);
-                        if (nd == SAT) {
-                            s_sat = 1;
-                            continue;
-                        }
-                        if (nd < ld_relaxed(dist + b)) {
-                            const int64_t old = atomic_min_dt(dist + b, (DT)nd);
-                            if (nd < old) atomicOr(nxt + (b >> 5), 1u << (b & 31));
+            bool any = false;
+            for (int c0 = warp * U; c0 < nchunk; c0 += U * NW) {
+                Arc r[U];
+                int64_t w[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t e = ((int64_t)(c0 + u) << 5) + lane;
+                    r[u] = empty_arc();
+                    w[u] = 0;
+                    if (e < arcs) {
+                        r[u] = a.arc[e];
+                        if (sizeof(DS) == 8) w[u] = a.w64[e];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int x = r[u].src(), b = r[u].dst();
+                    const unsigned mine =
+                        r[u].empty() ? 0u : (unsigned)reinterpret_cast<const volatile uint16_t*>(cur)[x];
+                    for (unsigned m = __reduce_or_sync(0xffffffffu, mine); m; m &= m - 1u) {
+                        const int k = __ffs(m) - 1;
+                        if (!((mine >> k) & 1u)) continue;
+                        DS* d = dist + (size_t)k * np;
+                        const DS dx = *(volatile DS*)(d + x);
+                        const DS nd = through(dx, sizeof(DS) == 8 ? (DS)w[u] : (DS)r[u].w);
+                        if (nd < *(volatile DS*)(d + b)) {
+                            atomic_min_dist(d + b, nd);
+                            atomicOr(nxt + (b >> 1), (1u << k) << ((b & 1) << 4));
+                            any = true;
                         }
                     }
                 }
-            }
-            __syncthreads();
-            int any = 0;
-            for (int q = tid; q < words; q += kSsspThreads) {
-                const uint32_t x = nxt[q];
-                cur[q] = x;
-                nxt[q] = 0u;
-                any |= (x != 0u);
             }
             if (!__syncthreads_or(any)) {
                 converged = true;
                 break;
             }
+            uint32_t* t = cur;
+            cur = nxt;
+            nxt = t;
+            for (int q = tid; q < np / 2; q += T) nxt[q] = 0u;
+            __syncthreads();
         }
         // positive weights converge within n-1 rounds; anything else is reported
-        if (!converged && tid == 0) set_err(err, ERRF_TIMEOUT);
-        // A relaxation whose sum did not fit matters only if it was the way to reach a
-        // vertex: then that vertex has a distance the type cannot hold.
-        if (s_sat) {
-            for (int x = warp; x < n; x += nwarps) {
-                const int64_t dx = dist[x];
-                if (dx == INF) continue;
-                for (int e = off[x] + lane; e < off[x + 1]; e += 32)
-                    if (dsum<DT>(dx, (int64_t)w[e]) == SAT && (int64_t)dist[dst[e]] == INF)
-                        set_err(err, ERRF_DIST);
+        if (!converged && tid == 0) set_err(a.err, ERRF_TIMEOUT);
+        // An arc from a vertex with a distance to one without: their sum did not fit, so
+        // that vertex has a distance the type cannot hold.
+        if (a.check)
+            for (int64_t e = tid; e < arcs; e += T) {
+                const Arc r = a.arc[e];
+                for (int k = 0; k < S; ++k)
+                    if (dist[(size_t)k * np + r.src()] != Far<DS>::v && dist[(size_t)k * np + r.dst()] == Far<DS>::v)
+                        set_err(a.err, ERRF_DIST);
+            }
+        for (int k = 0; k < S; ++k) {
+            DT* row = a.D + (size_t)(s0 + k) * a.ld;
+            for (int t = tid; t < a.ld; t += T) {   // the entries past n: no path
+                const DS d = t < n ? dist[(size_t)k * np + t] : Far<DS>::v;
+                row[t] = d == Far<DS>::v ? (DT)Inf<DT>::v : (DT)d;
             }
         }
-        if (SMEM_DIST) {
-            DT* row = D + (size_t)s * ld;
-            for (int t = tid; t < n; t += kSsspThreads) row[t] = dist_s[t];
-        }
-        if (tid < ld - n) D[(size_t)s * ld + n + tid] = (DT)INF;   // the entries past n: no path
-        // the search from s is final: the arcs of s with w(s,b) > d(s,b) are not in E*
-        if (pdst)
-            for (int e = off[s] + tid; e < off[s + 1]; e += kSsspThreads) {
-                const int b = dst[e];
-                if ((int64_t)w[e] != ld_relaxed(dist + b)) pdst[e] = -1;
-            }
         __syncthreads();
     }
 }
 
 template <typename DT>
-__global__ void k_estar_flags(int ld, int64_t arcs, const int32_t* g_src, const int32_t* g_dst,
-                              const DT* g_w, const DT* D, uint8_t* flags) {
+__global__ void k_estar_flags(int ld, int64_t arcs, const Arc* arc, const int64_t* w64, const DT* D, uint8_t* flags) {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= arcs) return;
-    flags[e] = ((int64_t)D[(size_t)g_src[e] * ld + g_dst[e]] == (int64_t)g_w[e]) ? 1 : 0;
+    const Arc r = arc[e];
+    const int64_t w = sizeof(DT) == 8 ? w64[e] : (int64_t)r.w;
+    flags[e] = ((int64_t)D[(size_t)r.src() * ld + r.dst()] == w) ? 1 : 0;
 }
 
-template <typename DT>
-static void sssp_dispatch(const Dev& d) {
-    const size_t words = ((size_t)d.n + 31) / 32;
-    const size_t bitmaps = 2 * words * sizeof(uint32_t);
-    const size_t dist_bytes = (((size_t)d.n * sizeof(DT)) + 15) & ~(size_t)15;
-    const size_t smem_cap = 200 * 1024;
-    if (dist_bytes + bitmaps <= smem_cap) {
-        const size_t smem = dist_bytes + bitmaps;
-        cudaFuncSetAttribute(k_sssp<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp<DT, true>, kSsspThreads, smem);
-        if (per_sm < 1) per_sm = 1;
-        const int grid = (int)std::min<int64_t>((int64_t)d.nsm * per_sm, d.n);
-        k_sssp<DT, true><<<grid, kSsspThreads, smem, d.st>>>(d.n, d.ld, d.g_off, d.g_dst, (const DT*)d.g_w,
-                                                             (DT*)d.D, d.err, d.s_order, d.p_dst);
-    } else {
-        const size_t smem = bitmaps;
-        cudaFuncSetAttribute(k_sssp<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sssp<DT, false>, kSsspThreads, smem);
-        if (per_sm < 1) per_sm = 1;
-        const int grid = (int)std::min<int64_t>((int64_t)d.nsm * per_sm, d.n);
-        k_sssp<DT, false><<<grid, kSsspThreads, smem, d.st>>>(d.n, d.ld, d.g_off, d.g_dst, (const DT*)d.g_w,
-                                                              (DT*)d.D, d.err, d.s_order, d.p_dst);
+// ---- dense graphs: arcs that cannot be in E* left out before the search
+//
+// A path is at most as long as one over each vertex's lightest arcs only, so an arc longer
+// than that path is not shortest and not in E*, and the search may leave it out.
+
+constexpr int kLight = 12;   // lightest arcs of a vertex, at least (with equal weights up to twice that)
+
+// A warp per vertex: appends its kLight lightest arcs (all of them when there are no more)
+// to the list, the threshold found by bisection on the weight.
+__global__ void __launch_bounds__(256) k_light_arcs(int n, const int32_t* off, const Arc* arc, const int64_t* w64,
+                                                    int64_t w_max, Arc* l_arc, int64_t* l_w64,
+                                                    unsigned long long* l_count) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    for (int x = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x < n; x += (gridDim.x * blockDim.x) >> 5) {
+        const int beg = off[x], end = off[x + 1];
+        auto weight = [&](int e) { return w64 ? w64[e] : (int64_t)arc[e].w; };
+        int64_t lo = 0, hi = w_max;
+        while (lo < hi && end - beg > kLight) {   // least threshold with kLight arcs at or below it
+            const int64_t mid = lo + (hi - lo) / 2;
+            int c = 0;
+            for (int e = beg + lane; e < end; e += 32) c += weight(e) <= mid;
+            if (__reduce_add_sync(0xffffffffu, c) >= kLight) hi = mid;
+            else lo = mid + 1;
+        }
+        int left = 2 * kLight;   // warp-uniform
+        for (int e0 = beg; e0 < end && left > 0; e0 += 32) {
+            const int e = e0 + lane;
+            const bool light = e < end && weight(e) <= hi;
+            const unsigned b = __ballot_sync(0xffffffffu, light);
+            const int c = min(__popc(b), left), rank = __popc(b & lt);
+            left -= c;
+            unsigned long long p = 0;
+            if (lane == 0 && c) p = atomicAdd(l_count, (unsigned long long)c);
+            p = __shfl_sync(0xffffffffu, p, 0);
+            if (light && rank < c) {
+                l_arc[p + rank] = arc[e];
+                if (w64) l_w64[p + rank] = w64[e];
+            }
+        }
     }
 }
 
-void launch_sssp(const Dev& d) {
-    if (d.dbytes == 4) sssp_dispatch<int32_t>(d);
-    else sssp_dispatch<int64_t>(d);
+// Appends the arcs that are no longer than the distances of the search over the light ones.
+template <typename DT>
+__global__ void __launch_bounds__(256) k_filter_arcs(int ld, int64_t arcs, const Arc* arc, const int64_t* w64,
+                                                     const DT* D, Arc* f_arc, int64_t* f_w64,
+                                                     unsigned long long* f_count) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x; e0 < arcs; e0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e = e0 + threadIdx.x;
+        bool keep = false;
+        Arc r = empty_arc();
+        int64_t w = 0;
+        if (e < arcs) {
+            r = arc[e];
+            w = sizeof(DT) == 8 ? w64[e] : (int64_t)r.w;
+            keep = w <= (int64_t)D[(size_t)r.src() * ld + r.dst()];
+        }
+        const unsigned b = __ballot_sync(0xffffffffu, keep);
+        unsigned long long p = 0;
+        if (lane == 0 && b) p = atomicAdd(f_count, (unsigned long long)__popc(b));
+        p = __shfl_sync(0xffffffffu, p, 0) + __popc(b & ((1u << lane) - 1u));
+        if (keep) {
+            f_arc[p] = r;
+            if (sizeof(DT) == 8) f_w64[p] = w;
+        }
+    }
+}
+
+constexpr size_t kSsspSmemMax = 224 * 1024;
+
+// arcs_about: the number of arcs, for the choice of S (it is known only on the device).
+template <typename DT, typename DS>
+static void sssp_search(const Dev& d, const Arc* arc, const int64_t* w64, const unsigned long long* arcs,
+                        double arcs_about, bool check) {
+    const size_t np = ((size_t)d.n + 31) & ~(size_t)31;
+    auto bytes = [&](int S) { return (size_t)S * np * sizeof(DS) + 2 * np * 2; };
+    auto resident = [&](int S) {   // groups an SM holds at a time
+        const int groups = (d.n + S - 1) / S;
+        return std::max(1, std::min({4, (int)((227 * 1024) / (bytes(S) + 1088)), (groups + d.nsm - 1) / d.nsm}));
+    };
+    // Sources per group: an SM's groups cost about their arcs once per source, the masks of
+    // the arcs' tails twice that once per group, and a round's latency, times the rounds,
+    // for every set of groups that run side by side.
+    int S = 1;
+    double best = 0;
+    for (int k = 1; k <= kSsspMaxSources && bytes(k) <= kSsspSmemMax; ++k) {
+        const int groups = (d.n + k - 1) / k, per_sm = (groups + d.nsm - 1) / d.nsm;
+        const double cost = per_sm * arcs_about * (k + 2.0) + (per_sm + resident(k) - 1) / resident(k) * 20000.0;
+        if (k == 1 || cost < best) {
+            best = cost;
+            S = k;
+        }
+    }
+    const size_t smem = bytes(S);
+    SsspArgs<DT> a{d.n, d.ld, arc, w64, arcs, (DT*)d.D, d.err, S, check ? 1 : 0};
+    auto go = [&](auto t) {
+        constexpr int T = decltype(t)::value;
+        auto kern = k_sssp<DT, DS, T>;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
+        const int grid = std::min(d.nsm * std::max(per_sm, 1), (d.n + S - 1) / S);
+        kern<<<grid, T, smem, d.st>>>(a);
+    };
+    // about 1024 threads per SM
+    if (resident(S) >= 3) go(std::integral_constant<int, 256>{});
+    else if (resident(S) == 2) go(std::integral_constant<int, 512>{});
+    else go(std::integral_constant<int, 1024>{});
+}
+
+// Arcs per vertex from which the light search pays: its own kLight arcs per vertex, twice
+// (bc_init_static's device time, complete n = 1024:
+// 4.9 ms so, 25 ms over every arc; complete n = 600, int32: 2.4 ms so, 2.9 ms before).
+constexpr int kDenseDegree = 4 * kLight;
+
+template <typename DT, typename DS>
+static void sssp(const Dev& d, int64_t w_max, bool all_arcs, bool check) {
+    if (!all_arcs && d.g_off && d.g_arcs >= (int64_t)kDenseDegree * d.n) {
+        // the lists live in the memory of the path counts and the dependency rows, which the
+        // accumulation writes only afterwards: each holds n * ld >= arcs entries of 8 bytes
+        Arc* f_arc = reinterpret_cast<Arc*>(d.S);
+        int64_t* f_w64 = reinterpret_cast<int64_t*>(d.Dl);
+        const size_t light = (size_t)2 * kLight * d.n;   // <= arcs / 2
+        Arc* l_arc = reinterpret_cast<Arc*>(d.Dl);
+        int64_t* l_w64 = reinterpret_cast<int64_t*>(l_arc + light);
+        unsigned long long* counts = reinterpret_cast<unsigned long long*>(d.g_count);
+        k_light_arcs<<<std::min((d.n + 7) / 8, d.nsm * 8), 256, 0, d.st>>>(d.n, d.g_off, d.g_arc, d.g_w64, w_max, l_arc,
+                                                                         l_w64, counts + 1);
+        sssp_search<DT, DS>(d, l_arc, l_w64, counts + 1, (double)light, false);
+        k_filter_arcs<DT><<<(int)std::min<int64_t>((d.g_arcs + 255) / 256, d.nsm * 8), 256, 0, d.st>>>(
+            d.ld, d.g_arcs, d.g_arc, d.g_w64, (const DT*)d.D, f_arc, f_w64, counts + 2);
+        sssp_search<DT, DS>(d, f_arc, f_w64, counts + 2, (double)light, check);
+        return;
+    }
+    sssp_search<DT, DS>(d, d.g_arc, d.g_w64, d.g_count, (double)d.g_arcs, check);
+}
+
+// w_max: the largest weight (0: not known).
+void launch_sssp(const Dev& d, int64_t w_max, bool all_arcs) {
+    const int64_t inf = d.dbytes == 4 ? (int64_t)INT32_MAX : INT64_MAX;
+    auto below = [&](int64_t bound) { return w_max > 0 && w_max <= (bound - 1) / std::max(d.n - 1, 1); };
+    if (d.dbytes == 4) sssp<int32_t, uint32_t>(d, w_max, all_arcs, !below(inf));
+    else if (below(INT32_MAX)) sssp<int64_t, uint32_t>(d, w_max, all_arcs, false);
+    else sssp<int64_t, int64_t>(d, w_max, all_arcs, !below(inf));
 }
 
 void launch_estar_flags(const Dev& d, uint8_t* flags) {
     if (d.g_arcs <= 0) return;
     const int blocks = (int)((d.g_arcs + 255) / 256);
     if (d.dbytes == 4)
-        k_estar_flags<int32_t><<<blocks, 256, 0, d.st>>>(d.ld, d.g_arcs, d.g_src, d.g_dst,
-                                                         (const int32_t*)d.g_w, (const int32_t*)d.D, flags);
+        k_estar_flags<int32_t><<<blocks, 256, 0, d.st>>>(d.ld, d.g_arcs, d.g_arc, d.g_w64, (const int32_t*)d.D, flags);
     else
-        k_estar_flags<int64_t><<<blocks, 256, 0, d.st>>>(d.ld, d.g_arcs, d.g_src, d.g_dst,
-                                                         (const int64_t*)d.g_w, (const int64_t*)d.D, flags);
+        k_estar_flags<int64_t><<<blocks, 256, 0, d.st>>>(d.ld, d.g_arcs, d.g_arc, d.g_w64, (const int64_t*)d.D, flags);
 }
 
 }  // namespace bcg

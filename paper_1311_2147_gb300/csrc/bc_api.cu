@@ -5,10 +5,10 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
-#include <unordered_map>
 #include <unordered_set>
 #include <vector>
 
+#include "arc_map.hpp"
 #include "bcgpu.h"
 #include "bc_batch.cuh"
 #include "bc_internal.cuh"
@@ -44,8 +44,8 @@ struct bc_graph {
     bool real_weights = false;
     int32_t w_exp = 0;
     int32_t top_bits = 0;
-    // weights of every arc of G (G_D for undirected graphs)
-    std::unordered_map<uint64_t, int64_t> wmap;
+    // weights of every arc of G (G_D for undirected graphs), and the superset's slots
+    ArcMap amap;
     // host mirror of the E* superset CSR
     // (slots [0, pool_top) hold the laid-out segments and moved ones; a vertex whose
     // segment fills up is moved to pool_top with room to grow, and E* is laid out
@@ -56,7 +56,6 @@ struct bc_graph {
     int64_t estar_rebuilds = 0;
     int64_t estar_moves = 0;
     std::vector<int64_t> e_w;
-    std::unordered_map<uint64_t, int32_t> eslot;
     int64_t estar_arcs = 0;
     // staged batch
     std::vector<bc_update> staged;
@@ -66,8 +65,6 @@ struct bc_graph {
     VEdge* d_entries = nullptr;
     int64_t d_entries_cap = 0;
     // bookkeeping
-    int32_t* h_err = nullptr;             // pinned
-    int64_t* h_stats = nullptr;           // pinned
     uint8_t* d_keep = nullptr;
     int64_t d_keep_cap = 0;
     int64_t ws_cap = 0;
@@ -207,17 +204,21 @@ void collect_profile(bc_graph* g) {
     g->pending.clear();
 }
 
-// Wait for the stream and turn a device-side error into a status (poisoning the handle).
+// Turn the device's error word into a status (poisoning the handle).
+int check_err(bc_graph* g, int32_t err) {
+    if (!err) return BC_OK;
+    g->poisoned = true;
+    g->poison_status = status_of_err(err);
+    return fail(g, g->poison_status, status_text(g->poison_status));
+}
+
+// Wait for the stream and check for a device-side error.
 int sync_check(bc_graph* g) {
+    int32_t err = 0;
+    CK(g, cudaMemcpyAsync(&err, g->d.err, sizeof(int32_t), cudaMemcpyDeviceToHost, g->d.st));
     CK(g, cudaStreamSynchronize(g->d.st));
     collect_profile(g);
-    CK(g, cudaMemcpy(g->h_err, g->d.err, sizeof(int32_t), cudaMemcpyDeviceToHost));
-    if (*g->h_err) {
-        g->poisoned = true;
-        g->poison_status = status_of_err(*g->h_err);
-        return fail(g, g->poison_status, status_text(g->poison_status));
-    }
-    return BC_OK;
+    return check_err(g, err);
 }
 
 // First slot at or after at where a segment of c slots crosses no group boundary (one
@@ -261,15 +262,14 @@ int estar_layout(bc_graph* g, const std::vector<HArc>& arcs, const std::vector<i
     g->e_src.assign(d.e_cap, 0);
     g->e_dst.assign(d.e_cap, -1);
     g->e_w.assign(d.e_cap, 0);
-    g->eslot.clear();
-    g->eslot.reserve(arcs.size() * 2 + 16);
+    g->amap.each([](int32_t, int32_t, ArcMap::Entry& e) { e.slot = -1; });
     for (int32_t a = 0; a < n; ++a)
         for (int32_t s = g->e_off[a]; s < g->e_off[a] + g->e_capv[a]; ++s) g->e_src[s] = a;
     for (const HArc& x : arcs) {
         const int32_t slot = g->e_off[x.a] + g->e_len[x.a]++;
         g->e_dst[slot] = x.b;
         g->e_w[slot] = x.w;
-        g->eslot[arc_key(x.a, x.b)] = slot;
+        g->amap.find(x.a, x.b)->slot = slot;
     }
     g->estar_arcs = (int64_t)arcs.size();
     std::vector<Arc> A(d.e_cap);
@@ -326,17 +326,18 @@ int estar_rebuild(bc_graph* g, const std::vector<HArc>& pending) {
 
 // Validate one update against the host weights and produce its edge entries (at vertex
 // v).  Does not modify anything.
+// over: weights that earlier updates of a batch give, not in the mirror yet.
 int validate_update(bc_graph* g, const bc_update& u, const bc_vedge* edges, int64_t n_edges,
-                    int32_t* v_out, std::vector<VEdge>& ent) {
+                    int32_t* v_out, std::vector<VEdge>& ent, ArcMap* over = nullptr) {
     ent.clear();
     const int32_t n = g->n;
     auto check_arc = [&](int32_t a, int32_t b, int64_t w) -> int {
         if (a < 0 || a >= n || b < 0 || b >= n || a == b)
             return fail(g, BC_ERR_ARG, "edge endpoint out of range or self-loop");
         if (w < 1 || w >= g->inf) return fail(g, BC_ERR_ARG, "weight outside [1, INF-1]");
-        auto it = g->wmap.find(arc_key(a, b));
-        if (it != g->wmap.end() && w >= it->second)
-            return fail(g, BC_ERR_NOT_INCREMENTAL, "new weight is not below the current weight");
+        const ArcMap::Entry* e = over ? over->find(a, b) : nullptr;
+        if (!e) e = g->amap.find(a, b);
+        if (e && w >= e->w) return fail(g, BC_ERR_NOT_INCREMENTAL, "new weight is not below the current weight");
         return BC_OK;
     };
     if (u.kind == BC_UPD_EDGE) {
@@ -377,7 +378,7 @@ bool estar_move(bc_graph* g, int32_t a, int32_t want, std::vector<EMove>& moves)
     for (int32_t i = 0; i < len; ++i) {
         g->e_dst[to + i] = g->e_dst[from + i];
         g->e_w[to + i] = g->e_w[from + i];
-        g->eslot[arc_key(a, g->e_dst[to + i])] = to + i;
+        g->amap.find(a, g->e_dst[to + i])->slot = to + i;
         g->e_dst[from + i] = -1;
     }
     for (int64_t i = 0; i < c; ++i) g->e_src[to + i] = a;
@@ -410,7 +411,8 @@ void mirror_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::v
     // room first: segments that cannot take their new arcs move before any slot is written
     std::vector<std::pair<int32_t, int32_t>> need;   // (vertex, new arcs)
     for (const HArc& x : arcs) {
-        if (g->eslot.count(arc_key(x.a, x.b))) continue;
+        const ArcMap::Entry* e = g->amap.find(x.a, x.b);
+        if (e && e->slot >= 0) continue;
         auto it = std::find_if(need.begin(), need.end(), [&](const std::pair<int32_t, int32_t>& p) {
             return p.first == x.a;
         });
@@ -426,12 +428,12 @@ void mirror_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::v
         }
     }
     for (const HArc& x : arcs) {
-        g->wmap[arc_key(x.a, x.b)] = x.w;
+        ArcMap::Entry& at = g->amap.at(x.a, x.b);
+        at.w = x.w;
         if (*rebuild) continue;
-        auto it = g->eslot.find(arc_key(x.a, x.b));
-        if (it != g->eslot.end()) {
-            g->e_w[it->second] = x.w;
-            ops.push_back({it->second, x.a, x.b, g->e_len[x.a], x.w});
+        if (at.slot >= 0) {
+            g->e_w[at.slot] = x.w;
+            ops.push_back({at.slot, x.a, x.b, g->e_len[x.a], x.w});
             continue;
         }
         const int32_t a = x.a;
@@ -439,7 +441,7 @@ void mirror_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::v
         g->e_src[slot] = a;
         g->e_dst[slot] = x.b;
         g->e_w[slot] = x.w;
-        g->eslot[arc_key(a, x.b)] = slot;
+        at.slot = slot;
         g->estar_arcs++;
         ops.push_back({slot, a, x.b, g->e_len[a], x.w});
     }
@@ -483,8 +485,8 @@ int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const 
         upd.k = (int32_t)ent.size();
         for (int j = 0; j < upd.k; ++j) {
             upd.x[j] = ent[j].x;
-            auto it = g->wmap.find(arc_key(ent[j].x, v));
-            upd.wold[j] = it == g->wmap.end() ? -1 : it->second;
+            const ArcMap::Entry* e = g->amap.find(ent[j].x, v);
+            upd.wold[j] = e ? e->w : -1;
         }
     }
     mirror_update(g, v, ent, ops, moves, arcs, &rebuild);
@@ -609,8 +611,6 @@ void destroy_all(bc_graph* g) {
     g->allocs_async.clear();
     for (void* p : g->allocs) cudaFree(p);
     g->allocs.clear();
-    if (g->h_err) cudaFreeHost(g->h_err);
-    if (g->h_stats) cudaFreeHost(g->h_stats);
     if (g->ev_done) cudaEventDestroy(g->ev_done);
     for (auto& r : g->pending) {
         cudaEventDestroy(r.a);
@@ -669,14 +669,17 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     const int64_t arcs = dir ? m : 2 * m;
     std::vector<HArc> all;
     all.reserve(arcs);
-    g->wmap.reserve(arcs * 2 + 16);
+    g->amap.reserve(arcs);
     for (int64_t i = 0; i < m; ++i) {
         const int32_t a = src[i], b = dst[i];
         if (a < 0 || a >= n || b < 0 || b >= n || a == b || w[i] < 1 || w[i] >= g->inf) {
             destroy_all(g);
             return fail(nullptr, BC_ERR_ARG, "edge out of range, self-loop or weight outside [1, INF-1]");
         }
-        if (!g->wmap.emplace(arc_key(a, b), w[i]).second || (!dir && !g->wmap.emplace(arc_key(b, a), w[i]).second)) {
+        bool added = false, both = true;
+        g->amap.at(a, b, &added).w = w[i];
+        if (!dir) g->amap.at(b, a, &both).w = w[i];
+        if (!added || !both) {
             destroy_all(g);
             return fail(nullptr, BC_ERR_ARG, "repeated edge");
         }
@@ -702,55 +705,67 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     int rc = BC_OK;
     d.nrb_max = (n + kRowsPerBlock - 1) / kRowsPerBlock;
     d.g_arcs = arcs;
-    if (g->dbytes == 4) {
-        int32_t *pD, *pfD, *pcD, *pcD2;
-        if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, d.ld)) ||
-            (rc = dalloc(g, &pcD2, d.ld))) {
-            destroy_all(g);
-            return fail(nullptr, rc, "device allocation failed");
-        }
-        d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2;
-    } else {
-        int64_t *pD, *pfD, *pcD, *pcD2;
-        if ((rc = dalloc(g, &pD, nn)) || (rc = dalloc(g, &pfD, n)) || (rc = dalloc(g, &pcD, d.ld)) ||
-            (rc = dalloc(g, &pcD2, d.ld))) {
-            destroy_all(g);
-            return fail(nullptr, rc, "device allocation failed");
-        }
-        d.D = pD; d.fD = pfD; d.cD = pcD; d.cD2 = pcD2;
-    }
-    if ((rc = dalloc(g, &d.S, nn)) || (rc = dalloc(g, &d.Dl, nn)) || (rc = dalloc(g, &d.bc_hi, n)) ||
-        (rc = dalloc(g, &d.bc_lo, n)) || (rc = dalloc(g, &d.g_arc, arcs)) || (rc = dalloc(g, &d.g_off, n + 1)) || (rc = dalloc(g, &d.g_count, 3)) ||
-        (!i32 && (rc = dalloc(g, &d.g_w64, arcs))) || (rc = dalloc(g, &d.e_off, n + 1)) || (rc = dalloc(g, &d.e_len, n)) ||
-        (rc = dalloc(g, &d.err, 1)) || (rc = dalloc(g, &d.stats, kStats)) || (rc = dalloc(g, &d.mark, n)) ||
-        (rc = dalloc(g, &d.changed, n)) || (rc = dalloc(g, &d.rows, n)) || (rc = dalloc(g, &d.acc_rows, n)) ||
-        (rc = dalloc(g, &d.counts, 8)) || (rc = dalloc(g, &d.fS, n)) || (rc = dalloc(g, &d.fM, n)) ||
-        (rc = dalloc(g, &d.cS, d.ld)) || (rc = dalloc(g, &d.cM, d.ld)) || (rc = dalloc(g, &d.cS2, d.ld)) ||
-        (rc = dalloc(g, &d.partial, (size_t)d.nrb_max * d.ld))) {
-        destroy_all(g);
-        return fail(nullptr, rc, "device allocation failed");
-    }
-    // pair corrections (undirected graphs): change map, old values of changed pairs,
-    // target lists and plans
+    // one allocation for all arrays of the handle's lifetime
+    std::vector<std::pair<void**, size_t>> want;
+    size_t total = 0;
+    auto need = [&](auto** p, size_t count, size_t item) {
+        want.push_back({reinterpret_cast<void**>(p), total});
+        total += (std::max<size_t>(count, 1) * item + 255) & ~(size_t)255;
+    };
+    const size_t db = (size_t)g->dbytes, ld = (size_t)d.ld;
+    need(&d.D, nn, db);
+    need(&d.S, nn, 8);
+    need(&d.Dl, nn, sizeof(ff));
+    need(&d.bc_hi, 2 * (size_t)n + 1, 8);   // bc_hi, bc_lo and the error word are read back together
+    need(&d.fD, n, db);
+    need(&d.cD, ld, db);
+    need(&d.cD2, ld, db);
+    need(&d.fS, n, 8);
+    need(&d.fM, n, 8);
+    need(&d.cS, ld, 8);
+    need(&d.cM, ld, 8);
+    need(&d.cS2, ld, 8);
+    need(&d.g_arc, arcs, sizeof(Arc));
+    if (!i32) need(&d.g_w64, arcs, 8);
+    need(&d.g_off, (size_t)n + 1, 4);
+    need(&d.g_count, 3, 8);
+    need(&d.e_off, (size_t)n + 1, 4);
+    need(&d.e_len, n, 4);
+    need(&d.rows, n, 4);
+    need(&d.acc_rows, n, 4);
+    need(&d.partial, (size_t)d.nrb_max * ld, sizeof(ff));
+    // pair corrections (undirected graphs): old values of changed pairs, target lists, plans
     d.tcap = kPairCap;
     d.chg_words = (n + 31) / 32;
     if (!dir) {
-        uint8_t* poD = nullptr;
-        if ((rc = dalloc(g, &poD, nn * (size_t)g->dbytes)) || (rc = dalloc(g, &d.oldS, nn)) ||
-            (rc = dalloc(g, &d.chg, (size_t)n * d.chg_words)) || (rc = dalloc(g, &d.tcnt, n)) ||
-            (rc = dalloc(g, &d.tlist, (size_t)n * kPairCap)) || (rc = dalloc(g, &d.full_rows, n)) ||
-            (rc = dalloc(g, &d.pair_rows, n)) ||
-            (rc = dalloc(g, reinterpret_cast<uint8_t**>(&d.plan), (size_t)n * kPairCap * 40)) ||
-            (rc = dalloc(g, &d.pair_w, (size_t)n + 1)) || (rc = dalloc(g, &d.bcfix, 2 * (size_t)n))) {
-            destroy_all(g);
-            return fail(nullptr, rc, "device allocation failed");
-        }
-        d.oldD = poD;
+        need(&d.oldD, nn, db);
+        need(&d.oldS, nn, 8);
+        need(&d.tlist, (size_t)n * kPairCap, 4);
+        need(&d.full_rows, n, 4);
+        need(&d.pair_rows, n, 4);
+        need(&d.plan, (size_t)n * kPairCap, 40);
+        need(&d.pair_w, (size_t)n + 1, 8);
         d.pair_on = 1;
     }
-    if (cudaMallocHost(&g->h_err, sizeof(int32_t)) != cudaSuccess ||
-        cudaMallocHost(&g->h_stats, kStats * sizeof(int64_t)) != cudaSuccess ||
-        cudaEventCreateWithFlags(&g->ev_done, cudaEventDisableTiming) != cudaSuccess ||
+    const size_t zero_from = total;   // from here on the arrays start at zero
+    need(&d.stats, kStats, 8);
+    need(&d.mark, n, 1);
+    need(&d.changed, n, 1);
+    need(&d.counts, 8, 4);
+    if (!dir) {
+        need(&d.chg, (size_t)n * d.chg_words, 4);   // the change map
+        need(&d.tcnt, n, 4);
+        need(&d.bcfix, 2 * (size_t)n, 8);
+    }
+    unsigned char* slab = nullptr;
+    if ((rc = dalloc(g, &slab, total))) {
+        destroy_all(g);
+        return fail(nullptr, rc, "device allocation failed");
+    }
+    for (const auto& p : want) *p.first = slab + p.second;
+    d.bc_lo = d.bc_hi + n;
+    d.err = reinterpret_cast<int32_t*>(d.bc_lo + n);
+    if (cudaEventCreateWithFlags(&g->ev_done, cudaEventDisableTiming) != cudaSuccess ||
         (!dir && (cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking) != cudaSuccess ||
                   cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                   cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming) != cudaSuccess ||
@@ -758,7 +773,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
                   cudaEventCreateWithFlags(&g->d.ev3_fork, cudaEventDisableTiming) != cudaSuccess ||
                   cudaEventCreateWithFlags(&g->d.ev3_join, cudaEventDisableTiming) != cudaSuccess))) {
         destroy_all(g);
-        return fail(nullptr, BC_ERR_OOM, "pinned host allocation, stream or event creation failed");
+        return fail(nullptr, BC_ERR_OOM, "stream or event creation failed");
     }
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -783,10 +798,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
         d.pair_walk = 1;
     }
     CKI(cudaMemsetAsync(d.err, 0, sizeof(int32_t), d.st));
-    CKI(cudaMemsetAsync(d.stats, 0, kStats * sizeof(int64_t), d.st));
-    CKI(cudaMemsetAsync(d.mark, 0, n, d.st));
-    CKI(cudaMemsetAsync(d.changed, 0, n, d.st));
-    CKI(cudaMemsetAsync(d.counts, 0, 8 * sizeof(int32_t), d.st));
+    CKI(cudaMemsetAsync(slab + zero_from, 0, total - zero_from, d.st));
     if (d.ld > n) {
         // the column vectors' entries past n: no path (the passes write only the first n)
         std::vector<unsigned char> inf((size_t)(d.ld - n) * g->dbytes);
@@ -798,11 +810,6 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
             CKI(cudaMemcpyAsync(static_cast<unsigned char*>(c) + (size_t)n * g->dbytes, inf.data(), inf.size(),
                                 cudaMemcpyHostToDevice, d.st));
         for (uint64_t* c : {d.cS, d.cM, d.cS2}) CKI(cudaMemsetAsync(c + n, 0, sizeof(uint64_t) * (d.ld - n), d.st));
-    }
-    if (!dir) {
-        CKI(cudaMemsetAsync(d.chg, 0, sizeof(uint32_t) * n * d.chg_words, d.st));
-        CKI(cudaMemsetAsync(d.tcnt, 0, sizeof(int32_t) * n, d.st));
-        CKI(cudaMemsetAsync(d.bcfix, 0, sizeof(int64_t) * 2 * n, d.st));
     }
     CKI(cudaStreamSynchronize(d.st));
     CKI(cudaEventRecord(e0, d.st));
@@ -1077,12 +1084,16 @@ int bc_get_scores(bc_graph* g, double* out) {
     int rc;
     if (!check_alive(g, &rc)) return rc;
     if (!out) return fail(g, BC_ERR_ARG, "out is NULL");
-    if ((rc = sync_check(g))) return rc;
-    std::vector<double> hi(g->n), lo(g->n);
-    CK(g, cudaMemcpy(hi.data(), g->d.bc_hi, sizeof(double) * g->n, cudaMemcpyDeviceToHost));
-    CK(g, cudaMemcpy(lo.data(), g->d.bc_lo, sizeof(double) * g->n, cudaMemcpyDeviceToHost));
+    const size_t n = (size_t)g->n;
+    std::vector<double> hl(2 * n + 1);   // bc_hi, bc_lo, the error word
+    CK(g, cudaMemcpyAsync(hl.data(), g->d.bc_hi, sizeof(double) * 2 * n + sizeof(int32_t), cudaMemcpyDeviceToHost, g->d.st));
+    CK(g, cudaStreamSynchronize(g->d.st));
+    collect_profile(g);
+    int32_t err = 0;
+    std::memcpy(&err, &hl[2 * n], sizeof(err));
+    if ((rc = check_err(g, err))) return rc;
     const double f = g->directed ? 1.0 : 0.5;
-    for (int32_t t = 0; t < g->n; ++t) out[t] = (hi[t] + lo[t]) * f;
+    for (size_t t = 0; t < n; ++t) out[t] = (hl[t] + hl[n + t]) * f;
     return BC_OK;
 }
 
@@ -1118,12 +1129,10 @@ int bc_get_rows(bc_graph* g, int32_t s0, int32_t count, int64_t* d_out, uint64_t
 int bc_get_edges(bc_graph* g, int64_t* m, int32_t* src, int32_t* dst, int64_t* w) {
     if (!g || !m) return BC_ERR_ARG;
     std::vector<std::pair<uint64_t, int64_t>> e;
-    e.reserve(g->wmap.size());
-    for (const auto& kv : g->wmap) {
-        const int32_t a = (int32_t)(kv.first >> 32), b = (int32_t)(kv.first & 0xffffffffu);
-        if (!g->directed && a > b) continue;
-        e.push_back(kv);
-    }
+    e.reserve(g->amap.size());
+    g->amap.each([&](int32_t a, int32_t b, const ArcMap::Entry& x) {
+        if (g->directed || a < b) e.push_back({x.key, x.w});
+    });
     std::sort(e.begin(), e.end());
     if (!src && !dst && !w) {
         *m = (int64_t)e.size();
@@ -1141,27 +1150,28 @@ int bc_get_edges(bc_graph* g, int64_t* m, int32_t* src, int32_t* dst, int64_t* w
 
 int bc_get_info(bc_graph* g, bc_info* out) {
     if (!g || !out) return BC_ERR_ARG;
+    int64_t st[kStats];
+    CK(g, cudaMemcpyAsync(st, g->d.stats, sizeof(st), cudaMemcpyDeviceToHost, g->d.st));
     CK(g, cudaStreamSynchronize(g->d.st));
-    CK(g, cudaMemcpy(g->h_stats, g->d.stats, kStats * sizeof(int64_t), cudaMemcpyDeviceToHost));
     std::memset(out, 0, sizeof(*out));
     out->n = g->n;
     out->directed = g->directed ? 1 : 0;
     out->dist_bytes = g->dbytes;
-    out->m = (int64_t)g->wmap.size();
+    out->m = g->amap.size();
     out->estar_arcs = g->estar_arcs;
-    out->rows_reaccumulated = g->h_stats[0];
-    out->noop_updates = g->h_stats[1];
-    out->max_rows = g->h_stats[2];
-    out->updates_applied = g->h_stats[3];
-    out->pairs_lowered = g->h_stats[4];
-    out->pairs_tied = g->h_stats[5];
-    out->rows_scanned = g->h_stats[6];
-    out->rows_full = g->h_stats[7];
-    out->pair_rows = g->h_stats[8];
-    out->pair_targets = g->h_stats[9];
-    out->walk_pairs = g->h_stats[10];
-    out->walk_vertices = g->h_stats[11];
-    out->walk_arcs = g->h_stats[12];
+    out->rows_reaccumulated = st[0];
+    out->noop_updates = st[1];
+    out->max_rows = st[2];
+    out->updates_applied = st[3];
+    out->pairs_lowered = st[4];
+    out->pairs_tied = st[5];
+    out->rows_scanned = st[6];
+    out->rows_full = st[7];
+    out->pair_rows = st[8];
+    out->pair_targets = st[9];
+    out->walk_pairs = st[10];
+    out->walk_vertices = st[11];
+    out->walk_arcs = st[12];
     out->estar_rebuilds = g->estar_rebuilds;
     out->estar_moves = g->estar_moves;
     out->kernel_launches = g->launches;
@@ -1263,6 +1273,7 @@ struct bc_batch {
     int64_t* d_plans = nullptr;
     int32_t* d_pctr = nullptr;
     int32_t* d_ws = nullptr;
+    int32_t* d_errs = nullptr;       // the graphs' error words after the rounds
     int64_t R_cap = 0, E_cap = 0, O_cap = 0, ws_cap = 0;
     cudaGraphExec_t exec = nullptr;
     int32_t exec_rounds = -1;
@@ -1313,7 +1324,8 @@ void drop_exec(bc_batch* b) {
 void new_arcs_of(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::vector<int32_t>& need) {
     for (const VEdge& e : ent) {
         auto add = [&](int32_t a, int32_t bb) {
-            if (!g->eslot.count(arc_key(a, bb))) need[a]++;
+            const ArcMap::Entry* at = g->amap.find(a, bb);
+            if (!at || at->slot < 0) need[a]++;
         };
         if (!g->directed) {
             add(e.x, v);
@@ -1364,7 +1376,8 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     b->L.acc_threads = 256;
     int rc;
     if ((rc = balloc(b, &b->d_devs, count)) || (rc = balloc(b, &b->d_coff, count + 1)) ||
-        (rc = balloc(b, &b->d_plans, 5 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1))) {
+        (rc = balloc(b, &b->d_plans, 5 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1)) ||
+        (rc = balloc(b, &b->d_errs, count))) {
         bc_batch_destroy(b);
         return rc;
     }
@@ -1427,36 +1440,29 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     int64_t base = 0;
     for (int32_t g = 0; g < G; ++g) {
         bc_graph* gr = b->graphs[g];
-        // validation reads the host weights as they evolve: validate on a copy of the
-        // weights first, then mirror for real once the slack is known to suffice
-        std::unordered_map<uint64_t, int64_t> saved = gr->wmap;
+        // validation reads the host weights as they evolve: the earlier updates' go in a
+        // map of their own first, and into the mirror once the slack is known to suffice
+        ArcMap over;
         std::vector<int32_t> need(gr->n, 0);
         std::vector<VEdge> ent;
         for (int32_t k = 0; k < n_updates[g]; ++k) {
             const bc_update& u = ups[base + k];
             int32_t v = -1;
-            int rc = validate_update(gr, u, edges, n_edges, &v, ent);
+            int rc = validate_update(gr, u, edges, n_edges, &v, ent, &over);
             if (rc) {
                 if (status == BC_OK) status = rc;
                 b->last_error = gr->last_error;
                 break;
             }
             new_arcs_of(gr, v, ent, need);
-            for (const VEdge& e : ent) {   // tentative weights so later updates validate against them
-                if (!gr->directed) {
-                    gr->wmap[arc_key(e.x, v)] = e.w;
-                    gr->wmap[arc_key(v, e.x)] = e.w;
-                } else if (e.dir == 0) {
-                    gr->wmap[arc_key(e.x, v)] = e.w;
-                } else {
-                    gr->wmap[arc_key(v, e.x)] = e.w;
-                }
+            for (const VEdge& e : ent) {
+                if (!gr->directed || e.dir == 0) over.at(e.x, v).w = e.w;
+                if (!gr->directed || e.dir == 1) over.at(v, e.x).w = e.w;
             }
             vtx[g].push_back(v);
             ents[g].push_back(ent);
             ok[g]++;
         }
-        gr->wmap.swap(saved);
         base += n_updates[g];
         bool short_slack = false;
         for (int32_t a = 0; a < gr->n && !short_slack; ++a)
@@ -1590,6 +1596,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     a.plan_pr = b->d_plans + 3 * (G + 1);
     a.plan_pw = b->d_plans + 4 * (G + 1);
     a.pctr = b->d_pctr;
+    a.errs = b->d_errs;
     a.ws = b->d_ws;
     a.ws_stride = b->L.ws_stride;
     b->L.max_eops = std::max<int64_t>(b->L.max_eops, 256);
@@ -1607,13 +1614,16 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     CKB(b, cudaEventRecord(b->e0, b->st));
     if (R > 0) CKB(b, cudaGraphLaunch(b->exec, b->st));
     CKB(b, cudaEventRecord(b->e1, b->st));
+    std::vector<int32_t> errs(G, 0);
+    if (R > 0) CKB(b, cudaMemcpyAsync(errs.data(), b->d_errs, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, b->st));
     CKB(b, cudaStreamSynchronize(b->st));
     float ms = 0.f;
     cudaEventElapsedTime(&ms, b->e0, b->e1);
     b->last_ms = ms;
     for (int32_t g = 0; g < G; ++g) {
         bc_graph* gr = b->graphs[g];
-        int rg = sync_check(gr);
+        collect_profile(gr);
+        int rg = check_err(gr, errs[g]);
         if (rg != BC_OK && status == BC_OK) {
             status = rg;
             b->last_error = gr->last_error;

@@ -39,6 +39,7 @@ struct BatchArgs {
     int64_t* plan_pr;         // [G + 1]: rows listed for pair corrections (graphs with them)
     int64_t* plan_pw;         // [G + 1]: column-test work
     int32_t* pctr;            // column-test pieces handed out past the first wave
+    int32_t* errs;            // [G] error words after the rounds, read back in one copy
     int32_t* ws;              // accumulation work space, acc_grid * ws_stride ints
     int64_t ws_stride;
     AccLayout lay;            // arrays of an accumulation CTA, sized for the largest graph

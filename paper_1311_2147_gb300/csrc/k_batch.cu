@@ -404,11 +404,16 @@ void batch_config(BatchLaunch& L, int dbytes, int n_max, int64_t cap_max) {
     L.ws_stride = (L.lay.ws + 3) / 4;
 }
 
+__global__ void kb_errors(BatchArgs b) {
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < b.G; g += gridDim.x * blockDim.x) b.errs[g] = *b.devs[g].err;
+}
+
 void batch_launch_rounds(const BatchArgs& b, const BatchLaunch& L, int rounds, int dbytes, cudaStream_t st) {
     for (int r = 0; r < rounds; ++r) {
         if (dbytes == 4) round_launches<int32_t>(b, L, r, st);
         else round_launches<int64_t>(b, L, r, st);
     }
+    kb_errors<<<nb(b.G, 256), 256, 0, st>>>(b);
 }
 
 }  // namespace bcg

@@ -498,15 +498,16 @@ int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const 
         for (int j = 0; j < pack.count; ++j) pack.mv[j] = moves[i + j];
         timed(g, 4, 1, [&] { launch_estar_move(d, pack); });
     }
+    // the last pack of slot writes goes along with the update's first kernel
+    EOps last{};
     if (rebuild) {
         int rc = estar_rebuild(g, arcs);
         if (rc) return rc;
     } else {
         for (size_t i = 0; i < ops.size(); i += kMaxEOps) {
-            EOps pack{};
-            pack.count = (int32_t)std::min<size_t>(kMaxEOps, ops.size() - i);
-            for (int j = 0; j < pack.count; ++j) pack.op[j] = ops[i + j];
-            timed(g, 4, 1, [&] { launch_estar_write(d, pack); });
+            if (last.count) timed(g, 4, 1, [&] { launch_estar_write(d, last); });
+            last.count = (int32_t)std::min<size_t>(kMaxEOps, ops.size() - i);
+            for (int j = 0; j < last.count; ++j) last.op[j] = ops[i + j];
         }
     }
     int32_t kin = 0, kout = 0;
@@ -523,70 +524,50 @@ int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const 
     const bool fused = !g->directed && k == 1 && !g->full_scan && g->fused_edges && g->n % (16 / g->dbytes) == 0;
     if (fused) {
         kin = kout = 0;
-        timed(g, 3, 1, [&] { launch_edge_prep(d, ent[0].x, v, ent[0].w); });
+        timed(g, 3, 1, [&] { launch_edge_prep(d, ent[0].x, v, ent[0].w, last); });
         timed(g, 0, 1, [&] { launch_edge_scan(d); });
     }
     if (kin) {
-        timed(g, 3, 1, [&] { launch_alg4_in(d, v, d_ent, k); });
-        timed(g, 4, 1, [&] { launch_compact(d, d.mark, 0, d.rows, d.counts, full, 0); });
+        timed(g, 3, 1, [&] { launch_alg4_in(d, v, d_ent, k, full, last); });
         timed(g, 0, 1, [&] { launch_scan_in(d, v); });
     }
     if (kout) {
-        timed(g, 3, 2, [&] {
-            launch_alg4_out(d, v, d_ent, k);
-            launch_rows_out(d, v, d_ent, k);
-        });
-        timed(g, 4, 1, [&] { launch_compact(d, d.mark, 0, d.rows, d.counts, full, 0); });
+        if (!kin && last.count) timed(g, 4, 1, [&] { launch_estar_write(d, last); });
+        timed(g, 3, 1, [&] { launch_out_prep(d, v, d_ent, k, full); });
         timed(g, 0, 1, [&] { launch_scan_out(d, v); });
         timed(g, 3, 1, [&] { launch_write_row(d, v); });
     }
     if (pair) {
         // rows with more changed targets than kPairCap (and row v): Algorithm 1 in full;
-        // the others: pair corrections of their dependency rows
-        timed(g, 4, 1, [&] { launch_pair_lists(d); });
-        // kernels of launch_pairdep: plan and weights, then the walks (units, two hash-table
-        // row classes, whole-CTA rows) and the gated column test, or the column test alone
-        const int pair_launches = walk ? 7 : 3;
-        // BC: the full rows are subtracted before and added after their re-accumulation;
-        // the corrected rows add their changes to BC's fixed-point change as they are
-        // made, which k_bc_fix folds into BC at the end
+        // the others: pair corrections of their dependency rows.  Both add their changes to
+        // BC's fixed-point change, which k_update_end folds into BC.
+        timed(g, 5, 1, [&] { launch_pair_plan(d); });
+        // kernels of launch_pairdep: weights, then the walks (units, two hash-table row
+        // classes, whole-CTA rows) and the gated column test, or the column test alone
+        const int pair_launches = walk ? 6 : 2;
         if (!g->profile) {
             // the two write disjoint dependency rows and only read the rest of the state:
-            // the (latency-bound, partial-wave) accumulation of the full rows and their
-            // new BC sums run on the second stream beside the pair corrections, which do
-            // not touch BC itself until k_bc_fix, after the join.  The old rows' BC sums
-            // are taken first on this stream, so that the accumulation is the first
-            // kernel of the second stream: launched before the pair corrections, it gets
-            // its SMs before their CTAs (which stay resident until all their work is
-            // taken) fill the GPU.
+            // the (latency-bound, partial-wave) accumulation of the full rows runs on the
+            // second stream beside the pair corrections, its first kernel: launched before
+            // the pair corrections, it gets its SMs before their CTAs (which stay resident
+            // until all their work is taken) fill the GPU.
             Dev ds = d;
             ds.st = g->side;
-            launch_bc_rows_list(d, -1, d.full_rows, d.counts + 3);
             CK(g, cudaEventRecord(g->ev_fork, d.st));
             CK(g, cudaStreamWaitEvent(g->side, g->ev_fork, 0));
             launch_accum_rows(ds, d.full_rows, d.counts + 3);
-            launch_bc_rows_list(ds, +1, d.full_rows, d.counts + 3);
             CK(g, cudaEventRecord(g->ev_join, g->side));
             launch_pairdep(d, walk ? &upd : nullptr);
             CK(g, cudaStreamWaitEvent(d.st, g->ev_join, 0));
-            launch_bc_fix(d);
-            g->launches += 6 + pair_launches;
+            g->launches += 1 + pair_launches;
         } else {
-            timed(g, 2, 2, [&] { launch_bc_rows_list(d, -1, d.full_rows, d.counts + 3); });
             timed(g, 5, pair_launches, [&] { launch_pairdep(d, walk ? &upd : nullptr); });
             timed(g, 1, 1, [&] { launch_accum_rows(d, d.full_rows, d.counts + 3); });
-            timed(g, 2, 3, [&] {
-                launch_bc_rows_list(d, +1, d.full_rows, d.counts + 3);
-                launch_bc_fix(d);
-            });
         }
-        timed(g, 4, 1, [&] { launch_pair_clear(d); });
     } else {
-        timed(g, 4, 1, [&] { launch_compact(d, d.changed, 1, d.acc_rows, d.counts + 1, 0, 1); });
-        timed(g, 2, 2, [&] { launch_bc_rows(d, -1, 0); });
         timed(g, 1, 1, [&] { launch_accum(d, 0); });
-        timed(g, 2, 2, [&] { launch_bc_rows(d, +1, 0); });
     }
+    timed(g, 2, 1, [&] { launch_update_end(d); });
     CK(g, cudaGetLastError());
     return BC_OK;
 }
@@ -732,6 +713,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     need(&d.e_off, (size_t)n + 1, 4);
     need(&d.e_len, n, 4);
     need(&d.rows, n, 4);
+    need(&d.rows2, n, 4);
     need(&d.acc_rows, n, 4);
     need(&d.partial, (size_t)d.nrb_max * ld, sizeof(ff));
     // pair corrections (undirected graphs): old values of changed pairs, target lists, plans
@@ -749,13 +731,12 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     }
     const size_t zero_from = total;   // from here on the arrays start at zero
     need(&d.stats, kStats, 8);
-    need(&d.mark, n, 1);
-    need(&d.changed, n, 1);
+    need(&d.changed, n, 4);
     need(&d.counts, 8, 4);
+    need(&d.bcfix, 2 * (size_t)n, 8);
     if (!dir) {
         need(&d.chg, (size_t)n * d.chg_words, 4);   // the change map
         need(&d.tcnt, n, 4);
-        need(&d.bcfix, 2 * (size_t)n, 8);
     }
     unsigned char* slab = nullptr;
     if ((rc = dalloc(g, &slab, total))) {
@@ -842,7 +823,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     }
     // path counts, DAGs and dependencies of every source; BC as column sums
     launch_accum(d, 1);
-    launch_bc_rows(d, +1, 1);
+    launch_bc_static(d);
     CKI(cudaGetLastError());
     CKI(cudaEventRecord(e1, d.st));
     CKI(cudaEventSynchronize(e1));
@@ -1376,7 +1357,7 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     b->L.acc_threads = 256;
     int rc;
     if ((rc = balloc(b, &b->d_devs, count)) || (rc = balloc(b, &b->d_coff, count + 1)) ||
-        (rc = balloc(b, &b->d_plans, 5 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1)) ||
+        (rc = balloc(b, &b->d_plans, 4 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1)) ||
         (rc = balloc(b, &b->d_errs, count))) {
         bc_batch_destroy(b);
         return rc;
@@ -1591,10 +1572,9 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     a.voff = b->d_voff;
     a.coff = b->d_coff;
     a.plan_scan = b->d_plans;
-    a.plan_bc = b->d_plans + (G + 1);
-    a.plan_acc = b->d_plans + 2 * (G + 1);
-    a.plan_pr = b->d_plans + 3 * (G + 1);
-    a.plan_pw = b->d_plans + 4 * (G + 1);
+    a.plan_acc = b->d_plans + (G + 1);
+    a.plan_pr = b->d_plans + 2 * (G + 1);
+    a.plan_pw = b->d_plans + 3 * (G + 1);
     a.pctr = b->d_pctr;
     a.errs = b->d_errs;
     a.ws = b->d_ws;

@@ -34,9 +34,8 @@ struct BatchArgs {
     const int64_t* voff;      // [rounds * 4 * (G + 1)]: per-vertex pass offsets
     const int64_t* coff;      // [G + 1]: column offsets (prefix of n_g)
     int64_t* plan_scan;       // [G + 1]
-    int64_t* plan_bc;         // [G + 1]
     int64_t* plan_acc;        // [G + 1]
-    int64_t* plan_pr;         // [G + 1]: rows listed for pair corrections (graphs with them)
+    int64_t* plan_pr;         // [G + 1]: changed rows
     int64_t* plan_pw;         // [G + 1]: column-test work
     int32_t* pctr;            // column-test pieces handed out past the first wave
     int32_t* errs;            // [G] error words after the rounds, read back in one copy
@@ -88,7 +87,8 @@ void batch_launch_rounds(const BatchArgs& b, const BatchLaunch& L, int rounds, i
 // corrections of round r (k_pair.cu).
 void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* out, int scan_unroll,
                 cudaStream_t st);
-void batch_pair_lists(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st);
+void batch_pair_plan(const BatchArgs& b, const BatchLaunch& L, int dbytes, cudaStream_t st);
+void batch_round_end(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st);
 void batch_pair_launches(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st);
 
 }  // namespace bcg

@@ -15,11 +15,11 @@ namespace bcg {
 // SYM: the graph is undirected and the state is the one before the update, whose d and
 // sigma are symmetric, so d(s,x) is read as d(x,s) (consecutive threads then read
 // consecutive entries of row x instead of one entry of each row).
+// Returns whether row s can change.
 template <typename DT, bool SYM = false>
-__device__ __forceinline__ void dev_alg4_in(int s, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__device__ __forceinline__ bool dev_alg4_in(int s, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                           int v, const VEdge* __restrict__ e, int k, int directed,
-                          DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
-                          int32_t* err) {
+                          DT* fD, uint64_t* fS, uint64_t* fM, int32_t* err) {
     const int64_t INF = Inf<DT>::v;
     const size_t rs = (size_t)s * ld;
     auto at = [&](int x) { return SYM ? (size_t)x * ld + s : rs + x; };
@@ -54,17 +54,16 @@ __device__ __forceinline__ void dev_alg4_in(int s, int ld, const DT* __restrict_
     fD[s] = (DT)cur;
     fS[s] = sig;
     fM[s] = dec ? sig : hat;
-    mark[s] = aff ? 1 : 0;
-    if (aff) changed[s] = 1;
+    return aff;
 }
 
 // OUT phase, row test: row s (s != v) can change only through a new shortest path
 // s ~> v -> x_j, i.e. d'(s,v) + w'(v,x_j) <= d'(s,x_j) for some out-edge of the update.
+// Returns that.
 template <typename DT>
-__device__ __forceinline__ void dev_rows_out(int s, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__device__ __forceinline__ bool dev_rows_out(int s, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
-                           DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
-                           int32_t* err) {
+                           DT* fD, uint64_t* fS, uint64_t* fM, int32_t* err) {
     const int64_t INF = Inf<DT>::v;
     const size_t rs = (size_t)s * ld;
     const int64_t dsv = D[rs + v];
@@ -88,17 +87,17 @@ __device__ __forceinline__ void dev_rows_out(int s, int ld, const DT* __restrict
     fD[s] = (DT)dsv;
     fS[s] = ssv;
     fM[s] = ssv;
-    mark[s] = aff ? 1 : 0;
-    if (aff) changed[s] = 1;
+    return aff;
 }
 
 // Algorithm 4 on the reversed graph G'_R, for "source" t of G'_R = target t of G: the
 // out-edges (v, x_j) of the update are in-edges of v in G'_R, and d_R(t, x_j) is
-// d'(x_j, t), read from row x_j.  Produces row v of the result.
+// d'(x_j, t), read from row x_j.  Produces row v of the result;
+// returns whether its entry t changes.
 template <typename DT>
-__device__ __forceinline__ void dev_alg4_out(int t, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__device__ __forceinline__ bool dev_alg4_out(int t, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
-                           DT* cD, uint64_t* cS, uint64_t* cM, uint8_t* changed, int32_t* err) {
+                           DT* cD, uint64_t* cS, uint64_t* cM, int32_t* err) {
     const int64_t INF = Inf<DT>::v;
     const size_t rv = (size_t)v * ld;
     const int64_t old = D[rv + t];
@@ -131,85 +130,62 @@ __device__ __forceinline__ void dev_alg4_out(int t, int ld, const DT* __restrict
     cD[t] = (DT)cur;
     cS[t] = sig;
     cM[t] = dec ? sig : hat;
-    if (dec || hat != 0) changed[v] = 1;
+    return dec || hat != 0;
 }
 
-// Stable compaction of {s : mark[s]} (or of all s when full) into rows[], one CTA.
-// Optionally clears mark[] and accumulates the per-update counters.  A thread takes 16
-// consecutive flags per tile (one 16-byte load where aligned), so n = 16384 is one tile:
-// one block scan instead of one per 1024 flags.
-constexpr int kCompactThreads = 1024;
-constexpr int kCompactPerThread = 16;
-// Every thread of the block calls it; blockDim.x is a multiple of 32 (at most 1024).
-__device__ __forceinline__ void dev_compact(int n, uint8_t* mark, int clear, int32_t* rows, int32_t* count,
-                                            int full, int64_t* stats, const int32_t* err) {
-    constexpr int E = kCompactPerThread;
-    __shared__ int32_t wsum[32];
-    __shared__ int32_t s_total;
-    const int nwarps = blockDim.x >> 5;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const bool bad = *err != 0;
-    int base = 0;
-    for (int tile = 0; tile < n; tile += (int)blockDim.x * E) {
-        const int s0 = tile + tid * E;
-        uint32_t fl = 0;   // bit e: flag of s0 + e
-        if (s0 < n) {
-            const bool vec = s0 + E <= n && ((reinterpret_cast<uintptr_t>(mark + s0) & 15) == 0);
-            if (vec) {
-                const uint4 v = *reinterpret_cast<const uint4*>(mark + s0);
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int e = 0; e < E; ++e)
-                    if ((w[e >> 2] >> (8 * (e & 3))) & 0xFFu) fl |= 1u << e;
-                if (clear) *reinterpret_cast<uint4*>(mark + s0) = make_uint4(0u, 0u, 0u, 0u);
-            } else {
-                for (int e = 0; e < E && s0 + e < n; ++e) {
-                    if (mark[s0 + e]) fl |= 1u << e;
-                    if (clear) mark[s0 + e] = 0;
-                }
-            }
-            if (full) fl = (s0 + E <= n) ? 0xFFFFu : ((1u << (n - s0)) - 1u);
-            if (bad) fl = 0;
-        }
-        const int c = __popc(fl);
-        int incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) wsum[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            const int x = lane < nwarps ? wsum[lane] : 0;
-            int winc = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, winc, o);
-                if (lane >= o) winc += y;
-            }
-            if (lane < nwarps) wsum[lane] = winc - x;
-            if (lane == 31) s_total = winc;
-        }
-        __syncthreads();
-        int pos = base + wsum[wid] + incl - c;
-        while (fl) {
-            const int e = __ffs(fl) - 1;
-            fl &= fl - 1;
-            rows[pos++] = s0 + e;
-        }
-        base += s_total;
-        __syncthreads();
+// Appends s to a list where the lane wants to: one atomic per warp (every lane of the
+// warp calls it).
+__device__ __forceinline__ void append_row(bool want, int s, int32_t* rows, int32_t* count) {
+    const unsigned b = __ballot_sync(0xffffffffu, want);
+    if (!b) return;
+    const int lane = threadIdx.x & 31;
+    int p = 0;
+    if (lane == 0) p = atomicAdd(count, __popc(b));
+    p = __shfl_sync(0xffffffffu, p, 0) + __popc(b & ((1u << lane) - 1u));
+    if (want) rows[p] = s;
+}
+
+// One write into the E* superset.
+__device__ __forceinline__ void dev_estar_write(const EOp& o, Arc* e_arc, int64_t* e_w64, int32_t* e_len) {
+    if (o.slot >= 0) {
+        e_arc[o.slot] = make_arc(o.a, o.b, o.w);
+        if (e_w64) e_w64[o.slot] = o.w;
     }
-    if (tid == 0) {
-        *count = base;
-        if (stats) {
-            stats[0] += base;
-            if (base == 0) stats[1] += 1;
-            if (base > stats[2]) stats[2] = base;
-            stats[3] += 1;
-        }
-    }
+    atomicMax(e_len + o.a, o.len_a);   // lengths only grow between rebuilds
+}
+
+// BC's change in an update is summed per column as a fixed-point pair (A in units of
+// 2^-24, B in units of 2^-56) by integer atomics, so the total does not depend on the
+// order in which rows and CTAs add (the result is deterministic) and is exact up to the
+// 2^-56 rounding of each dependency.
+//
+// A dependency v = hi + lo, 0 <= v < 2^15, as such a pair, in single precision only (fp64
+// runs at a small fraction of the fp32 rate here): with h = hi * 2^24 and a = rint(h), h
+// and h - a are exact, and (h - a) * 2^32 and lo * 2^56 (|lo| <= 2^-10) are exact
+// scalings, each rounded to an integer once.  |A| <= 2^39, |B| < 2^47.
+__device__ __forceinline__ void fix_words(ff v, long long* A, long long* B) {
+    const float h = v.hi * 0x1p24f;
+    const float a = rintf(h);
+    *A = __float2ll_rn(a);
+    *B = __float2ll_rn((h - a) * 0x1p32f) + __float2ll_rn(v.lo * 0x1p56f);
+}
+// Adds A, B to column x's pair, B's high bits carried into A: |B| <= 2^31 per addend, and
+// a column has at most 2^15 addends of each kind, so |A| < 2^55 and |B| < 2^47.
+__device__ __forceinline__ void fix_add(int64_t* fix, int x, long long A, long long B) {
+    const long long c = (B + (1ll << 31)) >> 32;
+    A += c;
+    B -= c << 32;
+    unsigned long long* p = reinterpret_cast<unsigned long long*>(fix + 2 * (size_t)x);
+    if (A) atomicAdd(p, (unsigned long long)A);
+    if (B) atomicAdd(p + 1, (unsigned long long)B);
+}
+// BC(x) changes by delta_s(x)'s change from old to now.
+__device__ __forceinline__ void bc_fix_change(int64_t* fix, int x, ff old, ff now) {
+    if (old.hi == now.hi && old.lo == now.lo) return;
+    long long A0, B0, A1, B1;
+    fix_words(old, &A0, &B0);
+    fix_words(now, &A1, &B1);
+    fix_add(fix, x, A1 - A0, B1 - B0);
 }
 
 // Vector access of VEC consecutive distances (16 bytes).
@@ -563,6 +539,7 @@ struct AccArgs {
     int32_t* ws;
     int64_t ws_stride;
     int32_t* err;
+    int64_t* bcfix;      // BC's change (updates)
     AccLayout lay;
 };
 
@@ -905,7 +882,7 @@ __device__ __forceinline__ int dag_levels(const AccArgs<DT>& a, const AccMem& m,
 }
 
 // Eq. 4 back over the levels (level 0 is s: delta_s.(s) is not kept).
-template <typename DT, int T, bool POOLED>
+template <typename DT, bool STATIC, int T, bool POOLED>
 __device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, const DT* Ds, int L, ff* out) {
     const int tid = threadIdx.x, lane = tid & 31;
     for (int l = L - 1; l >= 1; --l) {
@@ -914,6 +891,8 @@ __device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, 
             const int i = i0 + lane;
             const bool have = i < hi;
             const int x = have ? m.order[i] : 0;
+            ff old{0.0f, 0.0f};
+            if (!STATIC && have) old = out[x];   // used last: on its way meanwhile
             const ff sx = ff_from_u64(m.cell[x]), rx = ff_rcp(sx);
             ff acc{0.0f, 0.0f};
             if constexpr (POOLED) {
@@ -958,7 +937,9 @@ __device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, 
             // delta(x) = sigma_sx * acc, rho(x) = (1 + delta(x)) / sigma_sx = acc + 1 / sigma_sx
             if (have) {
                 m.cell[x] = cell_rho(ff_add(acc, rx));
-                out[x] = ff_mul(sx, acc);
+                const ff now = ff_mul(sx, acc);
+                out[x] = now;
+                if (!STATIC) bc_fix_change(a.bcfix, x, old, now);
             }
         }
         __syncthreads();
@@ -981,12 +962,29 @@ __device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m
         __syncthreads();
     }
     const int L = dag_levels<DT, STATIC, T, POOLED>(a, m, sh, s, Ds);
-    for (int x = tid; x < n; x += T) {
-        const uint64_t sg = m.cell[x];
-        if (STATIC) Ss[x] = sg;
-        if (x == s || bit_of(m.sink, x)) {
-            out[x] = ff{0.0f, 0.0f};
-            if (sg != 0) m.cell[x] = cell_rho(ff_rcp(ff_from_u64(sg)));
+    constexpr int VU = 8;
+    for (int x0 = tid; x0 < n; x0 += VU * T) {
+        ff old[VU];
+        bool done[VU];
+#pragma unroll
+        for (int v = 0; v < VU; ++v) {
+            const int x = x0 + v * T;
+            done[v] = x < n && (x == s || bit_of(m.sink, x));
+            old[v] = ff{0.0f, 0.0f};
+            if (!STATIC && done[v]) old[v] = out[x];
+        }
+#pragma unroll
+        for (int v = 0; v < VU; ++v) {
+            const int x = x0 + v * T;
+            if (x >= n) break;
+            const uint64_t sg = m.cell[x];
+            if (STATIC) Ss[x] = sg;
+            if (done[v]) {
+                const ff none{0.0f, 0.0f};
+                if (!STATIC) bc_fix_change(a.bcfix, x, old[v], none);
+                if (STATIC || old[v].hi != 0.0f) out[x] = none;
+                if (sg != 0) m.cell[x] = cell_rho(ff_rcp(ff_from_u64(sg)));
+            }
         }
     }
     if (STATIC && tid < a.ld - n) {   // the entries past n: no path
@@ -994,7 +992,7 @@ __device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m
         out[n + tid] = ff{0.0f, 0.0f};
     }
     __syncthreads();
-    dag_pull<DT, T, POOLED>(a, m, Ds, L, out);
+    dag_pull<DT, STATIC, T, POOLED>(a, m, Ds, L, out);
 }
 template <typename DT, bool STATIC, int T>
 __device__ __noinline__ void dag_source_unpooled(AccArgs<DT> a, AccMem m, AccShared* sh, int s) {
@@ -1048,7 +1046,9 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
     if (STATIC) {
         for (int t = tid; t < n; t += T) m.cell[t] = t == s ? 1ull : 0ull;
     } else {
-        // the cells start as the source's path counts, on their way while the DAG is read off
+        // the old dependencies are on their way to L2 and the path counts, which the cells
+        // start as, here while the DAG is read off
+        for (int t = tid * 16; t < n; t += T * 16) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(out + t));
         for (int t = tid * 2; t < n; t += T * 2) {
             if (SM) async_copy16(m.cell + t, Ss + t);
             else *reinterpret_cast<ulonglong2*>(m.cell + t) = *reinterpret_cast<const ulonglong2*>(Ss + t);
@@ -1103,46 +1103,6 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
     __syncthreads();
     if (sh.arcs <= a.lay.pcap) dag_source<DT, STATIC, T, true>(a, m, sh, s, Ds, Ss, out);
     else dag_source_unpooled<DT, STATIC, T>(a, m, &sh, s);
-}
-
-// partial[rb][t] = sum over rows r of row block rb of Dl[s_r][t] (t != s_r), rows in
-// increasing order, in float-float (all terms are non-negative); rows = nullptr means
-// all n rows.
-__device__ __forceinline__ void dev_bc_partial(int t, int rb, int ld, const int32_t* rows, int total,
-                                               const ff* Dl, ff* partial) {
-    const int r0 = rb * kRowsPerBlock;
-    if (r0 >= total || t >= ld) return;
-    const int r1 = min(total, r0 + kRowsPerBlock);
-    ff acc{0.0f, 0.0f};
-    for (int r = r0; r < r1; ++r) {
-        const int s = rows ? rows[r] : r;
-        if (s != t) acc = ff_add(acc, Dl[(size_t)s * ld + t]);
-    }
-    partial[(size_t)rb * ld + t] = acc;
-}
-
-// bc (hi, lo) += sign * (sum of the row-block partials in block order): the partials are
-// summed in float-float, the total is taken to fp64 and added with TwoSum; overwrite
-// starts from zero (the static computation).
-__device__ __forceinline__ void dev_bc_finish(int t, int ld, int total, const ff* partial, double sign,
-                                              int overwrite, double* hi, double* lo) {
-    const int nrb = (total + kRowsPerBlock - 1) / kRowsPerBlock;
-    if (nrb == 0 && !overwrite) return;
-    ff acc{0.0f, 0.0f};
-    for (int rb = 0; rb < nrb; ++rb) acc = ff_add(acc, partial[(size_t)rb * ld + t]);
-    const double sum = sign * ff_to_double(acc);
-    if (overwrite) {
-        hi[t] = sum;
-        lo[t] = 0.0;
-        return;
-    }
-    // TwoSum (Knuth): h + x = s + e exactly
-    const double h = hi[t];
-    const double s = h + sum;
-    const double bp = s - h;
-    const double e = (h - (s - bp)) + (sum - bp);
-    hi[t] = s;
-    lo[t] += e;
 }
 
 }  // namespace bcg

@@ -207,12 +207,14 @@ struct Dev {
     int64_t* stats;      // [0] rows re-accumulated [1] no-op updates [2] max rows [3] updates
                          // [4] pairs lowered [5] pairs with new ties [6] rows scanned
     // scratch
-    uint8_t* mark;       // [n] rows that change in the current phase
-    uint8_t* changed;    // [n] rows that changed in any phase of the current update
-    int32_t* rows;       // [n] compacted rows of the current phase
-    int32_t* acc_rows;   // [n] compacted rows to re-accumulate
-    int32_t* counts;     // [0] phase rows [1] accumulation rows [3] full rows [4] pair pieces handed
-                         // out [5] rows corrected pair by pair
+    uint32_t* changed;   // [n] 1: the row changed in the current update
+    int32_t* rows;       // [n] rows of the IN phase, or of a fused edge pass's first direction
+    int32_t* rows2;      // [n] rows of the OUT phase, or of the second direction
+    int32_t* acc_rows;   // [n] rows that changed (each list in the order of its atomics: no result
+                         // depends on it)
+    int32_t* counts;     // [0] rows [1] acc_rows [2] rows2 [3] full rows [4] pair pieces handed out
+                         // [5] rows corrected pair by pair [6] CTAs of k_update_end done; all zero
+                         // between updates
     void* fD;            // [n] per-row distance to v after the phase (DT)
     uint64_t* fS;        // [n] per-row path count to v after the phase
     uint64_t* fM;        // [n] per-row multiplier of a tie
@@ -255,7 +257,7 @@ struct Dev {
     int32_t* walk_tl;        // [walk CTAs * n] per-CTA touched columns of a row
     int32_t* walk_ctl;       // [8] units and rows handed out, buffer used (64-bit), overflow
     int32_t* walk_rowE;      // [n] per listed row: vertices found by its walks
-    int64_t* bcfix;      // [2n] BC change of the corrected rows in this update, per column a
+    int64_t* bcfix;      // [2n] BC change of the changed rows in this update, per column a
                          // fixed-point pair (units of 2^-24, units of 2^-56); zero between updates
     cudaStream_t st;
     // a third stream for the heaviest rows of the DAG walks' phase 2 (undirected graphs):
@@ -359,19 +361,16 @@ inline cudaError_t launch_k(void (*kern)(KArgs...), dim3 grid, dim3 block, size_
 cudaError_t scan_setup();
 void launch_estar_write(const Dev& d, const EOps& ops);
 void launch_estar_move(const Dev& d, const EMoves& moves);
-void launch_alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k);
-void launch_rows_out(const Dev& d, int32_t v, const VEdge* e, int32_t k);
-void launch_alg4_out(const Dev& d, int32_t v, const VEdge* e, int32_t k);
-void launch_compact(const Dev& d, const uint8_t* mark, int clear, int32_t* rows,
-                    int32_t* count, int full, int stats);
+void launch_alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k, int full, const EOps& ops);
+void launch_out_prep(const Dev& d, int32_t v, const VEdge* e, int32_t k, int full);
 void launch_scan_in(const Dev& d, int32_t v);
 void launch_scan_out(const Dev& d, int32_t v);
 void launch_write_row(const Dev& d, int32_t v);
-void launch_edge_prep(const Dev& d, int32_t u, int32_t v, int64_t w);
+void launch_edge_prep(const Dev& d, int32_t u, int32_t v, int64_t w, const EOps& ops);
 void launch_edge_scan(const Dev& d);
 void launch_estar_keep(const Dev& d, uint8_t* keep);
 PairRec pair_rec(const Dev& d);
-void launch_pair_lists(const Dev& d);
+void launch_pair_plan(const Dev& d);
 void launch_pairdep(const Dev& d, const WalkUpd* upd);   // upd: DAG walks (k_pairwalk), else column tests
 size_t walk_smem(int n);
 int64_t walk_warps(int nsm);
@@ -379,14 +378,12 @@ int64_t walk_ctas(int nsm);
 // Kernel attributes of the pair corrections (the walks' and the weights pass's dynamic
 // shared memory limits); bc_init_static sets them before it builds a handle.
 cudaError_t walk_setup();
-void launch_pair_clear(const Dev& d);
-void launch_bc_fix(const Dev& d);
+void launch_update_end(const Dev& d);
 
 // ---- launches (k_accum.cu) ----
 void launch_accum(const Dev& d, int is_static);
 void launch_accum_rows(const Dev& d, const int32_t* rows, const int32_t* count);
-void launch_bc_rows(const Dev& d, int sign, int is_static);
-void launch_bc_rows_list(const Dev& d, int sign, const int32_t* rows, const int32_t* count);
+void launch_bc_static(const Dev& d);
 
 // ---- launches (k_static.cu) ----
 void launch_sssp(const Dev& d, int64_t w_max, bool all_arcs);

@@ -21,11 +21,14 @@
 // the heads of the DAG arcs, the levels and a cell per vertex (sigma, then rho); see
 // dev_accum_source.
 //
-// BC is maintained as BC += sum over changed rows of (delta'_s - delta_s): the old rows
-// are subtracted before the rows are rewritten and the new rows added after
-// (Algorithm 3 step 1 recomputes BC from zero; rows that did not change contribute
-// the same amount before and after, so only changed rows are touched).  Column sums
-// run over row blocks in a fixed order into a compensated (hi, lo) pair.
+// BC is maintained as BC += sum over changed rows of (delta'_s - delta_s) (Algorithm 3
+// step 1 recomputes BC from zero; rows that did not change contribute the same amount
+// before and after, so only changed rows are touched): as an entry of delta_s is written,
+// its change goes to BC's fixed-point change of the update (bc_fix_change), which
+// k_update_end folds into the compensated (hi, lo) pair.  Summing the old and the new rows
+// by columns instead took four launches and read every changed row twice (ER n = 4096,
+// 8 updates: 0.33 of 3.6 ms; ER n = 256, 16 updates: 0.31 of 0.98 ms).  The static
+// computation sums the columns in row blocks, in a fixed order.
 #include <algorithm>
 #include <type_traits>
 
@@ -47,17 +50,16 @@ __global__ void __launch_bounds__(T, 1024 / T) k_accum(AccArgs<DT> a) {
     }
 }
 
-// Column partial sums (dev_bc_partial) for two adjacent columns per thread: 16-byte loads
-// of both columns' float-float values, eight rows' loads issued before they are added;
-// each column still adds its rows one by one in list order, as dev_bc_partial does, so
-// the sums are bit-identical.
+// partial[rb][t] = sum over the rows of row block rb of Dl[s][t] (t != s), in increasing
+// order, in float-float (all terms are non-negative), two adjacent columns per thread:
+// 16-byte loads, eight rows' loads issued before they are added.
 constexpr int kBcUnroll = 8;
-__global__ void __launch_bounds__(256) k_bc_partial2(int n, int ld, const int32_t* rows, const int32_t* count,
-                                                     const ff* Dl, ff* partial, const int32_t* err) {
+__global__ void __launch_bounds__(256) k_bc_partial(int n, int ld, const ff* Dl, ff* partial,
+                                                    const int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int t = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-    const int total = rows ? *count : n;
+    const int total = n;
     if (t >= ld) return;
     for (int rb = blockIdx.y; rb * kRowsPerBlock < total; rb += gridDim.y) {
         const int r0 = rb * kRowsPerBlock;
@@ -67,7 +69,7 @@ __global__ void __launch_bounds__(256) k_bc_partial2(int n, int ld, const int32_
             int sr[kBcUnroll];
             float4 v[kBcUnroll];
 #pragma unroll
-            for (int k = 0; k < kBcUnroll; ++k) sr[k] = r + k < r1 ? (rows ? rows[r + k] : r + k) : -1;
+            for (int k = 0; k < kBcUnroll; ++k) sr[k] = r + k < r1 ? r + k : -1;
 #pragma unroll
             for (int k = 0; k < kBcUnroll; ++k)
                 if (sr[k] >= 0) v[k] = __ldcs(reinterpret_cast<const float4*>(Dl + (size_t)sr[k] * ld + t));
@@ -83,12 +85,17 @@ __global__ void __launch_bounds__(256) k_bc_partial2(int n, int ld, const int32_
     }
 }
 
-__global__ void k_bc_finish(int n, int ld, const int32_t* rows, const int32_t* count, const ff* partial,
-                            double sign, int overwrite, double* hi, double* lo, const int32_t* err) {
+// bc (hi, lo) = the sum of the row-block partials in block order.
+__global__ void k_bc_finish(int n, int ld, const ff* partial, double* hi, double* lo, const int32_t* err) {
     pdl_enter();
     if (*err) return;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) dev_bc_finish(t, ld, rows ? *count : n, partial, sign, overwrite, hi, lo);
+    if (t >= n) return;
+    const int nrb = (n + kRowsPerBlock - 1) / kRowsPerBlock;
+    ff acc{0.0f, 0.0f};
+    for (int rb = 0; rb < nrb; ++rb) acc = ff_add(acc, partial[(size_t)rb * ld + t]);
+    hi[t] = ff_to_double(acc);
+    lo[t] = 0.0;
 }
 
 // ------------------------------------------------------------------ launches
@@ -111,6 +118,7 @@ static AccArgs<DT> acc_args(const Dev& d, int is_static, const int32_t* rows, co
     a.ws = d.ws;
     a.ws_stride = d.ws_stride;
     a.err = d.err;
+    a.bcfix = d.bcfix;
     a.lay = d.acc_lay[is_static];
     return a;
 }
@@ -236,29 +244,13 @@ void launch_accum(const Dev& d, int is_static) { accum(d, is_static, d.acc_rows,
 
 void launch_accum_rows(const Dev& d, const int32_t* rows, const int32_t* count) { accum(d, 0, rows, count); }
 
-// sign = -1 / +1: subtract / add the rows listed in acc_rows; is_static: all rows,
-// overwriting BC.
-// The row blocks go to gridDim.y CTAs per column block in turn, about eight CTAs per SM
-// in all (the count of listed rows is known only on the device).
-static int bc_row_ctas(const Dev& d, int col_blocks) {
-    return std::max(1, std::min(d.nrb_max, d.nsm * 8 / col_blocks));
-}
-
-static void bc_rows(const Dev& d, int sign, int is_static, const int32_t* rows, const int32_t* count) {
+// BC of the static computation: the column sums of all rows.  The row blocks go to
+// gridDim.y CTAs per column block in turn, about eight CTAs per SM in all.
+void launch_bc_static(const Dev& d) {
     const int tb = (d.n + 255) / 256, tb2 = (d.ld / 2 + 255) / 256;
-    launch_k(k_bc_partial2, dim3(tb2, bc_row_ctas(d, tb2)), 256, 0, d.st, d.n, d.ld, rows, count, d.Dl, d.partial,
-             d.err);
-    launch_k(k_bc_finish, tb, 256, 0, d.st, d.n, d.ld, rows, count, d.partial, (double)sign, is_static, d.bc_hi, d.bc_lo,
-                                      d.err);
-}
-
-void launch_bc_rows(const Dev& d, int sign, int is_static) {
-    bc_rows(d, sign, is_static, is_static ? nullptr : d.acc_rows, d.counts + 1);
-}
-
-// The same for the rows listed in rows[0..*count).
-void launch_bc_rows_list(const Dev& d, int sign, const int32_t* rows, const int32_t* count) {
-    bc_rows(d, sign, 0, rows, count);
+    launch_k(k_bc_partial, dim3(tb2, std::max(1, std::min(d.nrb_max, d.nsm * 8 / tb2))), 256, 0, d.st, d.n, d.ld, d.Dl,
+             d.partial, d.err);
+    launch_k(k_bc_finish, tb, 256, 0, d.st, d.n, d.ld, d.partial, d.bc_hi, d.bc_lo, d.err);
 }
 
 }  // namespace bcg

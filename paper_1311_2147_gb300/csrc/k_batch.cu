@@ -26,11 +26,7 @@ __global__ void kb_estar(BatchArgs b, int r) {
          j += (int64_t)gridDim.x * blockDim.x) {
         const BatchEOp op = b.eops[j];
         const Dev& d = b.devs[op.g];
-        if (op.op.slot >= 0) {
-            d.e_arc[op.op.slot] = make_arc(op.op.a, op.op.b, op.op.w);
-            if (d.e_w64) d.e_w64[op.op.slot] = op.op.w;
-        }
-        atomicMax(d.e_len + op.op.a, op.op.len_a);
+        dev_estar_write(op.op, d.e_arc, d.e_w64, d.e_len);
     }
 }
 
@@ -54,15 +50,22 @@ __global__ void kb_vertex_pass(BatchArgs b, int r, int kind) {
         const DT* D = (const DT*)d.D;
         switch (kind) {
             case 0:
-                dev_alg4_in<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.mark, d.changed,
-                                d.err);
+                if (dev_alg4_in<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.err)) {
+                    d.changed[x] = 1u;
+                    d.rows[atomicAdd(d.counts, 1)] = x;
+                    d.acc_rows[atomicAdd(d.counts + 1, 1)] = x;
+                }
                 break;
             case 1:
-                dev_rows_out<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.mark, d.changed,
-                                 d.err);
+                if (dev_rows_out<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.fD, d.fS, d.fM, d.err)) {
+                    d.rows2[atomicAdd(d.counts + 2, 1)] = x;
+                    if (atomicExch(d.changed + x, 1u) == 0u) d.acc_rows[atomicAdd(d.counts + 1, 1)] = x;
+                }
                 break;
             case 2:
-                dev_alg4_out<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.cD, d.cS, d.cM, d.changed, d.err);
+                if (dev_alg4_out<DT>(x, d.ld, D, d.S, u.v, e, u.k, d.directed, (DT*)d.cD, d.cS, d.cM, d.err) &&
+                    atomicExch(d.changed + u.v, 1u) == 0u)
+                    d.acc_rows[atomicAdd(d.counts + 1, 1)] = u.v;
                 break;
             default:
                 if (d.pair_on) {
@@ -78,30 +81,12 @@ __global__ void kb_vertex_pass(BatchArgs b, int r, int kind) {
     }
 }
 
-// ---------------------------------------------------------------- compaction
-
-// which 0: IN-phase rows, 1: OUT-phase rows, 2: rows to re-accumulate (clears changed;
-// graphs with pair corrections list theirs in kb_pair_lists).
-__global__ void __launch_bounds__(kCompactThreads) kb_compact(BatchArgs b, int r, int which) {
-    for (int g = blockIdx.x; g < b.G; g += gridDim.x) {
-        const BatchUpd u = b.upd[(int64_t)r * b.G + g];
-        const Dev& d = b.devs[g];
-        if (which == 0 && u.kin == 0) continue;
-        if (which == 1 && u.kout == 0) continue;
-        if (which == 2 && (u.present == 0 || d.pair_on)) continue;
-        if (which < 2) dev_compact(d.n, d.mark, 0, d.rows, d.counts, 0, nullptr, d.err);
-        else dev_compact(d.n, d.changed, 1, d.acc_rows, d.counts + 1, 0, d.stats, d.err);
-        __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------------- plans
 
 // Per-graph work known only on the device, as exclusive prefix offsets over graphs:
-// kind 0: scan items of the phase rows (rows x column chunks); 1: BC partial tasks
-// (column blocks x row blocks of the rows to re-accumulate); 2: sources to
-// re-accumulate; 3: rows listed for pair corrections; 4: column-test weight (and its
-// piece counter back to zero).  One CTA.
+// kind 0: scan items of the phase rows (rows x column chunks); 2: sources to
+// re-accumulate; 3: changed rows; 4: column-test weight (and its piece counter back to
+// zero).  One CTA.
 __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, int phase_active, int64_t* out,
                                                 int scan_unroll) {
     __shared__ int64_t wsum[32];
@@ -119,14 +104,13 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
             if (on && *d.err == 0) {
                 if (kind == 0) {
                     const int cw = kScanThreads * (d.dbytes == 4 ? 4 : 2) * scan_unroll;
-                    v = (int64_t)d.counts[0] * ((d.ld + cw - 1) / cw);
-                    atomicAdd(reinterpret_cast<unsigned long long*>(d.stats + 6), (unsigned long long)d.counts[0]);
-                } else if (kind == 1) {
-                    v = (int64_t)((d.n + 255) / 256) * ((acc_list_count(d) + kRowsPerBlock - 1) / kRowsPerBlock);
+                    const int rows = d.counts[phase_active == 0 ? 0 : 2];
+                    v = (int64_t)rows * ((d.ld + cw - 1) / cw);
+                    atomicAdd(reinterpret_cast<unsigned long long*>(d.stats + 6), (unsigned long long)rows);
                 } else if (kind == 2) {
                     v = acc_list_count(d);
                 } else if (kind == 3) {
-                    v = d.pair_on ? d.counts[1] : 0;
+                    v = d.counts[1];
                 } else if (d.pair_on) {
                     v = d.pair_w[d.counts[5]];
                 }
@@ -195,6 +179,8 @@ __device__ __forceinline__ ScanArgs<DT> batch_scan_args(const Dev& d, const Batc
         a.cD = (const DT*)d.cD;
         a.cS = d.cS;
         a.cM = d.cM;
+        a.rows = d.rows2;
+        a.count = d.counts + 2;
         a.skip_row = u.v;
     }
     return a;
@@ -250,37 +236,6 @@ __global__ void __launch_bounds__(kScanThreads, 4) kb_scan(BatchArgs b, int r, i
     else scan_stats(b.devs[0].stats, 0, 0);
 }
 
-// ---------------------------------------------------------------- BC row sums
-
-__global__ void kb_bc_partial(BatchArgs b, int r, const int64_t* off) {
-    const int G = b.G;
-    const int64_t total = off[G];
-    for (int64_t j = blockIdx.x; j < total; j += gridDim.x) {
-        const int g = graph_of(off, G, j);
-        const Dev& d = b.devs[g];
-        if (*d.err) continue;
-        const int64_t task = j - off[g];
-        const int tb = (d.n + 255) / 256;
-        const int rb = (int)(task / tb);
-        const int t = (int)(task - (int64_t)rb * tb) * 256 + threadIdx.x;
-        dev_bc_partial(t, rb, d.ld, acc_list(d), acc_list_count(d), d.Dl, d.partial);
-    }
-}
-
-__global__ void kb_bc_finish(BatchArgs b, int r, double sign) {
-    const int G = b.G;
-    const int64_t* off = b.coff;
-    const int64_t total = off[G];
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < total;
-         j += (int64_t)gridDim.x * blockDim.x) {
-        const int g = graph_of(off, G, j);
-        const Dev& d = b.devs[g];
-        if (*d.err || b.upd[(int64_t)r * G + g].present == 0) continue;
-        const int t = (int)(j - off[g]);
-        dev_bc_finish(t, d.ld, acc_list_count(d), d.partial, sign, 0, d.bc_hi, d.bc_lo);
-    }
-}
-
 // ---------------------------------------------------------------- accumulation
 
 // One source per CTA of T threads (128, 256 or 512: a tile the autotuner picks), held to
@@ -312,6 +267,7 @@ __global__ void __launch_bounds__(T, 1024 / T) kb_accum(BatchArgs b, int r, cons
         a.ws = b.ws;
         a.ws_stride = b.ws_stride;
         a.err = d.err;
+        a.bcfix = d.bcfix;
         a.lay = b.lay;
         dev_accum_source<DT, false, T, SM>(a, a.rows[j - off[g]], m, sh);
     }
@@ -356,31 +312,24 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     kb_estar<<<nb(L.max_eops, 256), 256, 0, st>>>(b, r);
     // IN phase
     kb_vertex_pass<DT><<<nsm * L.vpass_ctas, 256, 0, st>>>(b, r, 0);
-    kb_compact<<<std::min(b.G, nsm * 2), kCompactThreads, 0, st>>>(b, r, 0);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 0, 0, b.plan_scan, L.scan_unroll);
     batch_scan<DT>(b, L, r, 0, st);
     // OUT phase (graphs without out-edges in this round have no work)
     kb_vertex_pass<DT><<<nsm * L.vpass_ctas, 256, 0, st>>>(b, r, 2);
     kb_vertex_pass<DT><<<nsm * L.vpass_ctas, 256, 0, st>>>(b, r, 1);
-    kb_compact<<<std::min(b.G, nsm * 2), kCompactThreads, 0, st>>>(b, r, 1);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 0, 1, b.plan_scan, L.scan_unroll);
     batch_scan<DT>(b, L, r, 1, st);
     kb_vertex_pass<DT><<<nsm * L.vpass_ctas, 256, 0, st>>>(b, r, 3);
-    // rows to re-accumulate, BC minus the old rows, accumulation, BC plus the new rows;
-    // in graphs with pair corrections only the rows over the target cap, and the others
-    // are corrected pair by pair after (the order of the single-graph path)
-    kb_compact<<<std::min(b.G, nsm * 2), kCompactThreads, 0, st>>>(b, r, 2);
-    if (L.pairs) batch_pair_lists(b, L, r, st);
-    kb_plan<<<1, 1024, 0, st>>>(b, r, 1, 2, b.plan_bc, L.scan_unroll);
+    // the changed rows re-accumulated; in graphs with pair corrections only those over the
+    // target cap, and the others corrected pair by pair after
+    kb_plan<<<1, 1024, 0, st>>>(b, r, 3, 2, b.plan_pr, L.scan_unroll);
+    if (L.pairs) batch_pair_plan(b, L, sizeof(DT), st);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 2, 2, b.plan_acc, L.scan_unroll);
-    kb_bc_partial<<<nsm * L.bc_ctas, 256, 0, st>>>(b, r, b.plan_bc);
-    kb_bc_finish<<<nsm * 2, 256, 0, st>>>(b, r, -1.0);
     if (L.acc_threads == 128) batch_accum<DT, 128>(b, L, r, st);
     else if (L.acc_threads == 256) batch_accum<DT, 256>(b, L, r, st);
     else batch_accum<DT, 512>(b, L, r, st);
-    kb_bc_partial<<<nsm * L.bc_ctas, 256, 0, st>>>(b, r, b.plan_bc);
-    kb_bc_finish<<<nsm * 2, 256, 0, st>>>(b, r, +1.0);
     if (L.pairs) batch_pair_launches(b, L, r, sizeof(DT), st);
+    batch_round_end(b, L, r, st);
 }
 
 void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* out, int scan_unroll,

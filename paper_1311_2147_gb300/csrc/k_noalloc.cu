@@ -166,7 +166,7 @@ extern "C" int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* 
         k_pack_graph<int64_t><<<blocks, 256, 0, d.st>>>(n, arcs, d.g_count, d_off, d_dst, d_w, d.e_arc, d.e_w64, d.e_len, d.err);
     launch_sssp(d, 0, true);
     launch_accum(d, 1);
-    launch_bc_rows(d, +1, 1);
+    launch_bc_static(d);
     k_scores_out<<<(n + 255) / 256, 256, 0, d.st>>>(n, d.bc_hi, d.bc_lo, dir ? 1.0 : 0.5, d_scores, d.err);
     if (cudaGetLastError() != cudaSuccess) return BC_ERR_CUDA;
     int32_t h_err = 0;

@@ -33,103 +33,10 @@ constexpr int kPairCtasPerSm = 4;
 template <int VN> struct PairGroup { static constexpr int value = VN >= 8 ? 1 : 2; };
 constexpr int kPairPieces = 8;  // pieces of equal weight per CTA of the grid
 
-// The row lists of an update's corrections in one pass over the changed-row flags (one
-// CTA, kCompactPerThread flags per thread and tile, as k_compact): acc_rows = the
-// changed rows, full_rows = those with more recorded targets than the cap (Algorithm 1
-// in full), both in increasing order.  The flags are cleared and the per-update counters
-// added as k_compact does for acc_rows.  A thread's two counts travel in one scan word
-// (each tile holds at most 1024 x 16 < 2^16 rows).
-// (CTA-wide; wsum and s_total in shared memory.)
-__device__ __forceinline__ void dev_pair_lists(int n, uint8_t* changed, const int32_t* tcnt, int tcap,
-                                               int32_t* acc_rows, int32_t* acc_count, int32_t* full_rows,
-                                               int32_t* full_count, int64_t* stats, bool bad, int32_t* wsum,
-                                               int32_t& s_total) {
-    constexpr int E = kCompactPerThread;
-    static_assert(kCompactThreads * E < (1 << 16), "a tile's counts fit 16 bits");
-    const int nwarps = blockDim.x >> 5;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    int base_a = 0, base_f = 0;
-    for (int tile = 0; tile < n; tile += (int)blockDim.x * E) {
-        const int s0 = tile + tid * E;
-        uint32_t fl = 0, ffl = 0;   // bit e: row s0 + e changed / goes to the full path
-        if (s0 < n) {
-            if (s0 + E <= n && ((reinterpret_cast<uintptr_t>(changed + s0) & 15) == 0)) {
-                const uint4 v = *reinterpret_cast<const uint4*>(changed + s0);
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int e = 0; e < E; ++e)
-                    if ((w[e >> 2] >> (8 * (e & 3))) & 0xFFu) fl |= 1u << e;
-                *reinterpret_cast<uint4*>(changed + s0) = make_uint4(0u, 0u, 0u, 0u);
-            } else {
-                for (int e = 0; e < E && s0 + e < n; ++e) {
-                    if (changed[s0 + e]) fl |= 1u << e;
-                    changed[s0 + e] = 0;
-                }
-            }
-            if (bad) fl = 0;
-            for (uint32_t b = fl; b; b &= b - 1) {
-                const int e = __ffs(b) - 1;
-                if (tcnt[s0 + e] > tcap) ffl |= 1u << e;
-            }
-        }
-        const int c = __popc(fl) | (__popc(ffl) << 16);
-        int incl = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        if (lane == 31) wsum[wid] = incl;
-        __syncthreads();
-        if (wid == 0) {
-            const int x = lane < nwarps ? wsum[lane] : 0;
-            int winc = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, winc, o);
-                if (lane >= o) winc += y;
-            }
-            if (lane < nwarps) wsum[lane] = winc - x;
-            if (lane == 31) s_total = winc;
-        }
-        __syncthreads();
-        const int excl = wsum[wid] + incl - c;
-        int pa = base_a + (excl & 0xFFFF), pf = base_f + (excl >> 16);
-        while (fl) {
-            const int e = __ffs(fl) - 1;
-            fl &= fl - 1;
-            acc_rows[pa++] = s0 + e;
-            if ((ffl >> e) & 1u) full_rows[pf++] = s0 + e;
-        }
-        base_a += s_total & 0xFFFF;
-        base_f += s_total >> 16;
-        __syncthreads();
-    }
-    if (tid == 0) {
-        *acc_count = base_a;
-        *full_count = base_f;
-        stats[0] += base_a;
-        if (base_a == 0) stats[1] += 1;
-        if (base_a > stats[2]) stats[2] = base_a;
-        stats[3] += 1;
-    }
-}
-
-__global__ void __launch_bounds__(kCompactThreads) k_pair_lists(int n, uint8_t* changed, const int32_t* tcnt,
-                                                                int tcap, int32_t* acc_rows, int32_t* acc_count,
-                                                                int32_t* full_rows, int32_t* full_count,
-                                                                int64_t* stats, const int32_t* err) {
-    pdl_enter();
-    __shared__ int32_t wsum[32];
-    __shared__ int32_t s_total;
-    dev_pair_lists(n, changed, tcnt, tcap, acc_rows, acc_count, full_rows, full_count, stats, *err != 0, wsum,
-                   s_total);
-}
-
 // Per-update records of the rows listed in rows[0..count) back to zero (a pair (s,t)
 // changes only in a changed row s), a warp per row: a row with at most tcap changed
 // targets has its bits only in the words of its listed targets, a longer one is
-// cleared whole.  The rows sent to the full path are added to stats[7].
+// cleared whole.
 __device__ __forceinline__ void dev_pair_clear_row(int s, int32_t* tcnt, const int32_t* tlist, int tcap,
                                                    uint32_t* chg, int words) {
     const int lane = threadIdx.x & 31;
@@ -142,16 +49,6 @@ __device__ __forceinline__ void dev_pair_clear_row(int s, int32_t* tcnt, const i
     }
     __syncwarp();
     if (lane == 0) tcnt[s] = 0;
-}
-
-__global__ void k_pair_clear(const int32_t* rows, const int32_t* count, int32_t* tcnt, const int32_t* tlist,
-                             int tcap, uint32_t* chg, int words, const int32_t* full_count, int64_t* stats) {
-    pdl_enter();
-    const int cnt = *count;
-    if (blockIdx.x == 0 && threadIdx.x == 0) stats[7] += *full_count;
-    const int wpb = blockDim.x >> 5;
-    for (int i = blockIdx.x * wpb + (threadIdx.x >> 5); i < cnt; i += gridDim.x * wpb)
-        dev_pair_clear_row(rows[i], tcnt, tlist, tcap, chg, words);
 }
 
 // One changed target t of a row s, as prepared by k_pair_plan: the pair's distance and
@@ -187,35 +84,24 @@ struct PairArgs {
     int tcap;
     const int32_t* rows;
     const int32_t* count;
+    int32_t* full_rows;     // rows with more targets than tcap
+    int32_t* full_count;
     ff* Dl;
-    int64_t* bcfix;         // [2n] BC change of this update (fixed point, see bc_fix_add)
+    int64_t* bcfix;         // [2n] BC change of this update (fixed point, see fix_add)
     int32_t* err;
 };
 
-// BC(x) += v for one corrected entry delta_s(x): v is added to the column's fixed-point
-// pair (A in units of 2^-24, B in units of 2^-56) by two integer atomics, so the total
-// does not depend on the order in which rows and CTAs add (the result is deterministic)
-// and is exact up to the 2^-56 rounding of each entry.  Bounds: each pair term
-// delta_st(x) lies in [0, 1] and a row has at most kPairCap targets, so |v| <= 128 and
-// |A| <= 2^31, |B| <= 2^31 per entry (the DAG walks add a row's column sum with
-// 0 <= B < 2^32); a column receives at most one entry per row, so for n < 2^20 both
-// sums stay below 2^52 and k_bc_fix converts them exactly.
+// BC(x) += v for one corrected entry delta_s(x) (fix_add): each pair term delta_st(x)
+// lies in [0, 1] and a row has at most kPairCap targets, so |v| <= 128, and a column
+// receives at most one entry per row.
 __device__ __forceinline__ void bc_fix_add(int64_t* fix, int x, ff v) {
-    // in single precision, as fix_split: h = hi * 2^24 is exact (|h| <= 2^31) and so is
-    // h - rint(h); (h - a) * 2^32 and lo * 2^56 (|lo| <= 2^-17) are exact scalings, each
-    // rounded to an integer once, and a carry keeps |B| <= 2^31
-    const float h = v.hi * 0x1p24f;
-    const float a = rintf(h);
-    long long b = __float2ll_rn((h - a) * 0x1p32f) + __float2ll_rn(v.lo * 0x1p56f);
-    const long long c = (b + (1ll << 31)) >> 32;
-    const long long A = __float2ll_rn(a) + c;
-    b -= c << 32;
-    unsigned long long* p = reinterpret_cast<unsigned long long*>(fix + 2 * (size_t)x);
-    atomicAdd(p, (unsigned long long)A);
-    if (b) atomicAdd(p + 1, (unsigned long long)b);
+    long long A, B;
+    fix_words(v, &A, &B);
+    fix_add(fix, x, A, B);
 }
 
-// One warp per listed row with 1..tcap changed targets (most rows have a few): rank
+// One warp per listed row: a row with more changed targets than the cap goes to the list of
+// those re-accumulated in full; one with 1..tcap (most rows have a few): rank
 // them (the sums then run in a fixed order) and write the per-target scalars of the
 // plan.  Every target of row s has its bit set, so its old values are the saved ones.
 constexpr int kPlanThreads = 256;
@@ -226,6 +112,7 @@ __device__ __forceinline__ void dev_pair_plan_row(const PairArgs<DT>& a, int s, 
     const int64_t INF = Inf<DT>::v;
     const int lane = threadIdx.x & 31;
     const int T = a.tcnt[s];
+    if (T > a.tcap && lane == 0) a.full_rows[atomicAdd(a.full_count, 1)] = s;
     if (T == 0 || T > a.tcap) return;   // warp-uniform
     for (int j = lane; j < T; j += 32) sv[j] = a.tlist[(size_t)s * a.tcap + j];
     __syncwarp();
@@ -366,8 +253,7 @@ struct PairWeightsSmem {
 // the last pass overwrites with the prefix.
 __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int32_t* count, const int32_t* tcnt,
                                                  int tcap, int nchunks, int32_t* prows, int32_t* pcount,
-                                                 int64_t* wpre, int64_t* stats, int32_t* next_piece,
-                                                 int32_t* walk_ctl, int32_t* walk_rowE, PairWeightsSmem& sm,
+                                                 int64_t* wpre, int64_t* stats, int32_t* walk_ctl, int32_t* walk_rowE, PairWeightsSmem& sm,
                                                  int32_t* s_r, int32_t* s_T, int scap) {
     int64_t* wsum = sm.wsum;
     int64_t& s_total = sm.s_total;
@@ -485,7 +371,6 @@ __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int3
             t += s_tgts[k];
         }
         wpre[cnt] = base;
-        *next_piece = 0;
         if (walk_ctl)
             for (int k = 0; k < 8; ++k) walk_ctl[k] = 0;
         stats[8] += r;
@@ -496,14 +381,13 @@ __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int3
 __global__ void __launch_bounds__(1024) k_pair_weights(const int32_t* rows, const int32_t* count,
                                                        const int32_t* tcnt, int tcap, int nchunks,
                                                        int32_t* prows, int32_t* pcount,
-                                                       int64_t* wpre, int64_t* stats, int32_t* next_piece,
-                                                       int32_t* walk_ctl, int32_t* walk_rowE, const int32_t* err,
+                                                       int64_t* wpre, int64_t* stats, int32_t* walk_ctl, int32_t* walk_rowE, const int32_t* err,
                                                        int scap) {
     pdl_enter();
     __shared__ PairWeightsSmem sm;
     extern __shared__ int32_t s_stage[];   // 2 * scap ints
     if (*err) return;
-    dev_pair_weights(rows, count, tcnt, tcap, nchunks, prows, pcount, wpre, stats, next_piece, walk_ctl, walk_rowE,
+    dev_pair_weights(rows, count, tcnt, tcap, nchunks, prows, pcount, wpre, stats, walk_ctl, walk_rowE,
                      sm, s_stage, s_stage + scap, scap);
 }
 
@@ -764,25 +648,60 @@ __device__ __forceinline__ void dev_bc_fix(int t, int64_t* fix, double* hi, doub
     lo[t] += e + x2;
 }
 
-__global__ void k_bc_fix(int n, int64_t* fix, double* hi, double* lo, const int32_t* err) {
+// Counters of a finished update, from its lists: [0] rows changed [1] updates without any
+// [2] most rows [3] updates [7] rows re-accumulated in full among those with corrections.
+__device__ __forceinline__ void dev_update_stats(int64_t* stats, int changed, int full) {
+    stats[0] += changed;
+    if (changed == 0) stats[1] += 1;
+    if (changed > stats[2]) stats[2] = changed;
+    stats[3] += 1;
+    stats[7] += full;
+}
+
+// The last kernel of an update: BC takes its change, the changed rows' flags and records go
+// back to zero, and the CTA that finishes last adds the counters and zeroes the lists'
+// counts for the next update.
+struct EndArgs {
+    int n;
+    int64_t* fix;
+    double* hi;
+    double* lo;
+    const int32_t* rows;
+    int32_t* counts;
+    uint32_t* changed;
+    int32_t* tcnt;       // NULL: no records
+    const int32_t* tlist;
+    int tcap;
+    uint32_t* chg;
+    int words;
+    int64_t* stats;
+    const int32_t* err;
+};
+__global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
     pdl_enter();
-    if (*err) return;
+    if (*a.err) return;   // the handle is poisoned: no further update
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) dev_bc_fix(t, fix, hi, lo);
+    for (int x = t; x < a.n; x += gridDim.x * blockDim.x) dev_bc_fix(x, a.fix, a.hi, a.lo);
+    const int cnt = a.counts[1];
+    for (int i = t; i < cnt; i += gridDim.x * blockDim.x) a.changed[a.rows[i]] = 0u;
+    if (a.tcnt)
+        for (int i = t >> 5; i < cnt; i += (gridDim.x * blockDim.x) >> 5)
+            dev_pair_clear_row(a.rows[i], a.tcnt, a.tlist, a.tcap, a.chg, a.words);
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(a.counts + 6, 1) == (int)gridDim.x - 1) {
+        dev_update_stats(a.stats, cnt, a.counts[3]);
+        for (int k = 0; k < 8; ++k) a.counts[k] = 0;
+    }
 }
 
 // ------------------------------------------------------------------ launches
 
 PairRec pair_rec(const Dev& d) { return make_pair_rec(d); }
 
-void launch_pair_lists(const Dev& d) {
-    launch_k(k_pair_lists, 1, kCompactThreads, 0, d.st, d.n, d.changed, d.tcnt, d.tcap, d.acc_rows, d.counts + 1,
-                                                  d.full_rows, d.counts + 3, d.stats, d.err);
-}
-
-void launch_pair_clear(const Dev& d) {
-    launch_k(k_pair_clear, d.nsm * 4, 256, 0, d.st, d.acc_rows, d.counts + 1, d.tcnt, d.tlist, d.tcap, d.chg,
-                                              d.chg_words, d.counts + 3, d.stats);
+void launch_update_end(const Dev& d) {
+    EndArgs a{d.n, d.bcfix, d.bc_hi, d.bc_lo, d.acc_rows, d.counts, d.changed, d.pair_on ? d.tcnt : nullptr, d.tlist,
+              d.tcap, d.chg, d.chg_words, d.stats, d.err};
+    launch_k(k_update_end, std::min(d.nsm * 4, std::max(1, (d.n + 31) / 32)), 256, 0, d.st, a);
 }
 
 template <typename DT>
@@ -807,6 +726,8 @@ __host__ __device__ inline PairArgs<DT> pair_args(const Dev& d) {
     a.tcap = d.tcap;
     a.rows = d.acc_rows;
     a.count = d.counts + 1;
+    a.full_rows = d.full_rows;
+    a.full_count = d.counts + 3;
     a.Dl = d.Dl;
     a.bcfix = d.bcfix;
     a.err = d.err;
@@ -827,19 +748,6 @@ __device__ __forceinline__ bool batch_pair_graph(const BatchArgs& b, int r, int 
     return d.pair_on && b.upd[(int64_t)r * b.G + g].present && *d.err == 0;
 }
 
-// One CTA per graph in turn: the row lists of its corrections (k_pair_lists).
-__global__ void __launch_bounds__(kCompactThreads) kb_pair_lists(BatchArgs b, int r) {
-    __shared__ int32_t wsum[32];
-    __shared__ int32_t s_total;
-    for (int g = blockIdx.x; g < b.G; g += gridDim.x) {
-        const Dev& d = b.devs[g];
-        if (!d.pair_on || b.upd[(int64_t)r * b.G + g].present == 0) continue;   // block-uniform
-        dev_pair_lists(d.n, d.changed, d.tcnt, d.tcap, d.acc_rows, d.counts + 1, d.full_rows, d.counts + 3, d.stats,
-                       *d.err != 0, wsum, s_total);
-        __syncthreads();
-    }
-}
-
 // A warp per listed row of every graph (k_pair_plan); plan_pr offsets the rows.
 template <typename DT>
 __global__ void __launch_bounds__(kPlanThreads) kb_pair_plan(BatchArgs b) {
@@ -851,6 +759,7 @@ __global__ void __launch_bounds__(kPlanThreads) kb_pair_plan(BatchArgs b) {
     for (int64_t j = (int64_t)blockIdx.x * (kPlanThreads / 32) + wib; j < total; j += nw) {
         const int g = graph_of(b.plan_pr, G, j);
         const Dev& d = b.devs[g];
+        if (!d.pair_on) continue;
         const PairArgs<DT> a = pair_args<DT>(d);
         dev_pair_plan_row<DT>(a, d.acc_rows[j - b.plan_pr[g]], s_val[wib]);
     }
@@ -867,7 +776,7 @@ __global__ void __launch_bounds__(1024) kb_pair_weights(BatchArgs b, int r, int 
         const int cw = kPairThreads * pair_vn(d.dbytes);
         const int nchunks = (d.n + cw - 1) / cw;
         dev_pair_weights(d.acc_rows, d.counts + 1, d.tcnt, d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w,
-                         d.stats, d.counts + 4, nullptr, nullptr, sm, s_stage, s_stage + scap, scap);
+                         d.stats, nullptr, nullptr, sm, s_stage, s_stage + scap, scap);
         __syncthreads();
     }
 }
@@ -971,49 +880,56 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) kb_pairdep(Batch
     }
 }
 
-// BC += the fixed-point change of each column of every graph with corrections (k_bc_fix).
-__global__ void kb_bc_fix(BatchArgs b, int r) {
+// The end of a round (k_update_end): BC takes its change in every graph with an update, the
+// changed rows' flags and records go back to zero (a warp per listed row); then, a thread
+// per graph, the counters and the lists' counts.
+__global__ void kb_update_end(BatchArgs b, int r) {
     const int G = b.G;
     const int64_t total = b.coff[G];
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < total;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int g = graph_of(b.coff, G, j);
-        if (!batch_pair_graph(b, r, g)) continue;
         const Dev& d = b.devs[g];
+        if (*d.err || b.upd[(int64_t)r * G + g].present == 0) continue;
         dev_bc_fix((int)(j - b.coff[g]), d.bcfix, d.bc_hi, d.bc_lo);
     }
-}
-
-// The per-update records back to zero, a warp per listed row (k_pair_clear).
-__global__ void kb_pair_clear(BatchArgs b, int r) {
-    const int G = b.G;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
-        if (batch_pair_graph(b, r, g)) b.devs[g].stats[7] += b.devs[g].counts[3];
-    const int64_t total = b.plan_pr[G];
+    const int64_t rows = b.plan_pr[G];
     const int wpb = blockDim.x >> 5;
-    for (int64_t j = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); j < total; j += (int64_t)gridDim.x * wpb) {
+    for (int64_t j = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); j < rows; j += (int64_t)gridDim.x * wpb) {
         const int g = graph_of(b.plan_pr, G, j);
         const Dev& d = b.devs[g];
-        dev_pair_clear_row(d.acc_rows[j - b.plan_pr[g]], d.tcnt, d.tlist, d.tcap, d.chg, d.chg_words);
+        const int s = d.acc_rows[j - b.plan_pr[g]];
+        if ((threadIdx.x & 31) == 0) d.changed[s] = 0u;
+        if (d.pair_on) dev_pair_clear_row(s, d.tcnt, d.tlist, d.tcap, d.chg, d.chg_words);
+    }
+}
+__global__ void kb_update_stats(BatchArgs b, int r) {
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < b.G; g += gridDim.x * blockDim.x) {
+        const Dev& d = b.devs[g];
+        if (*d.err || b.upd[(int64_t)r * b.G + g].present == 0) continue;
+        dev_update_stats(d.stats, d.counts[1], d.counts[3]);
+        for (int k = 0; k < 8; ++k) d.counts[k] = 0;
     }
 }
 
-void batch_pair_lists(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st) {
-    kb_pair_lists<<<std::min(b.G, L.nsm * 2), kCompactThreads, 0, st>>>(b, r);
+void batch_pair_plan(const BatchArgs& b, const BatchLaunch& L, int dbytes, cudaStream_t st) {
+    if (dbytes == 4) kb_pair_plan<int32_t><<<L.nsm * 8, kPlanThreads, 0, st>>>(b);
+    else kb_pair_plan<int64_t><<<L.nsm * 8, kPlanThreads, 0, st>>>(b);
+}
+
+void batch_round_end(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st) {
+    kb_update_end<<<L.nsm * 4, 256, 0, st>>>(b, r);
+    kb_update_stats<<<std::max(1, (b.G + 255) / 256), 256, 0, st>>>(b, r);
 }
 
 template <typename DT>
 static void batch_pairs(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st) {
     const int G = b.G, nsm = L.nsm;
-    batch_plan(b, r, 3, 2, b.plan_pr, L.scan_unroll, st);
-    kb_pair_plan<DT><<<nsm * 8, kPlanThreads, 0, st>>>(b);
     const int scap = weights_stage(b.n_max);
     kb_pair_weights<<<std::min(G, nsm * 2), 1024, 2 * sizeof(int32_t) * (size_t)scap, st>>>(b, r, scap);
     const int pgrid = nsm * kPairCtasPerSm;
     batch_plan(b, r, 4, 2, b.plan_pw, L.scan_unroll, st);
     kb_pairdep<DT, pair_vn(sizeof(DT))><<<pgrid, kPairThreads, 0, st>>>(b);
-    kb_bc_fix<<<nsm * 4, 256, 0, st>>>(b, r);
-    kb_pair_clear<<<nsm * 4, 256, 0, st>>>(b, r);
 }
 
 void batch_pair_launches(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st) {
@@ -1495,16 +1411,19 @@ static void launch_walks(const Dev& d, const WalkUpd& upd, int nchunks) {
     launch_k(k_pairdep<DT, pair_vn(sizeof(DT))>, pgrid, kPairThreads, 0, d.st, a);
 }
 
-void launch_pairdep(const Dev& d, const WalkUpd* upd) {
+void launch_pair_plan(const Dev& d) {
     const int pgrid = d.nsm * 8;
     if (d.dbytes == 4) launch_k(k_pair_plan<int32_t>, pgrid, kPlanThreads, 0, d.st, pair_args<int32_t>(d));
     else launch_k(k_pair_plan<int64_t>, pgrid, kPlanThreads, 0, d.st, pair_args<int64_t>(d));
+}
+
+void launch_pairdep(const Dev& d, const WalkUpd* upd) {
     const int vn = pair_vn(d.dbytes);
     const int cw = kPairThreads * vn;
     const int nchunks = (d.n + cw - 1) / cw;
     const int scap = weights_stage(d.n);
     launch_k(k_pair_weights, 1, 1024, 2 * sizeof(int32_t) * (size_t)scap, d.st, d.acc_rows, d.counts + 1, d.tcnt,
-             d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w, d.stats, d.counts + 4,
+             d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w, d.stats,
              upd ? d.walk_ctl : nullptr, upd ? d.walk_rowE : nullptr, d.err, scap);
     if (upd) {
         if (d.dbytes == 4) launch_walks<int32_t>(d, *upd, nchunks);
@@ -1514,10 +1433,6 @@ void launch_pairdep(const Dev& d, const WalkUpd* upd) {
     const int grid = d.nsm * kPairCtasPerSm;   // one resident wave; later pieces go to the first free CTA
     if (d.dbytes == 4) launch_k(k_pairdep<int32_t, 8>, grid, kPairThreads, 0, d.st, pair_args<int32_t>(d));
     else launch_k(k_pairdep<int64_t, 2>, grid, kPairThreads, 0, d.st, pair_args<int64_t>(d));
-}
-
-void launch_bc_fix(const Dev& d) {
-    launch_k(k_bc_fix, (d.n + 255) / 256, 256, 0, d.st, d.n, d.bcfix, d.bc_hi, d.bc_lo, d.err);
 }
 
 }  // namespace bcg

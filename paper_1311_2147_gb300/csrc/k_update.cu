@@ -7,14 +7,13 @@
 // (Section 3, "Undirected graphs").  Per phase:
 //
 //   IN  (E_i):  k_alg4_in   Algorithm 4 for every source s -> d'(s,v), sigma'_sv,
-//                           sigma-hat'_sv, and whether row s can change;
-//               k_compact   rows that change, in increasing order;
-//               k_scan_cs    Lemma 4 over those rows: D(s,t) = d'(s,v) + d(v,t).
-//   OUT (E_o):  k_alg4_out  Algorithm 4 on the reversed graph G'_R for every target t
+//                           sigma-hat'_sv, and the list of rows that can change;
+//               k_scan_cs   Lemma 4 over those rows: D(s,t) = d'(s,v) + d(v,t).
+//   OUT (E_o):  k_out_prep  Algorithm 4 on the reversed graph G'_R for every target t
 //                           -> d''(v,t), sigma''_vt, sigma-hat''_vt (row v of the
-//                           result; reads rows x_j of D', which are contiguous);
-//               k_rows_out  rows s with d'(s,v) + w'(v,x_j) <= d'(s,x_j) for some j;
-//               k_compact, k_scan_cs  Lemma 4 read on G'_R: D(s,t) = d'(s,v) + d''(v,t);
+//                           result; reads rows x_j of D', which are contiguous), and the
+//                           rows s with d'(s,v) + w'(v,x_j) <= d'(s,x_j) for some j;
+//               k_scan_cs   Lemma 4 read on G'_R: D(s,t) = d'(s,v) + d''(v,t);
 //               k_write_row row v <- (d''(v,.), sigma''_v.).
 //
 // Lemma 1 (and its vertex analogue) makes the in-place scan race free: during the IN
@@ -23,16 +22,10 @@
 
 namespace bcg {
 
-__global__ void k_estar_write(Arc* e_arc, int64_t* e_w64, int32_t* e_len, EOps ops) {
+__global__ void k_estar_write(Arc* e_arc, int64_t* e_w64, int32_t* e_len, const __grid_constant__ EOps ops) {
     pdl_enter();
-    int i = threadIdx.x;
-    if (i >= ops.count) return;
-    const EOp o = ops.op[i];
-    if (o.slot >= 0) {
-        e_arc[o.slot] = make_arc(o.a, o.b, o.w);
-        if (e_w64) e_w64[o.slot] = o.w;
-    }
-    atomicMax(e_len + o.a, o.len_a);   // lengths only grow between rebuilds
+    const int i = threadIdx.x;
+    if (i < ops.count) dev_estar_write(ops.op[i], e_arc, e_w64, e_len);
 }
 
 // One CTA per move: copy the segment, empty its old slots, point e_off[a] at the copy.
@@ -49,45 +42,56 @@ __global__ void k_estar_move(int32_t* e_off, Arc* e_arc, int64_t* e_w64, EMoves 
     if (threadIdx.x == 0) e_off[m.a] = m.to;
 }
 
+// The first kernel of an update also writes its arcs into the E* superset (ops; nothing
+// reads that before the accumulation), a launch of its own otherwise.  full: every row is
+// listed for the rank-1 pass.
 template <typename DT>
 __global__ void k_alg4_in(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                           int v, const VEdge* __restrict__ e, int k, int directed,
-                          DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
-                          int32_t* err) {
+                          DT* fD, uint64_t* fS, uint64_t* fM, int32_t* rows, int32_t* acc_rows, int32_t* counts,
+                          uint32_t* changed, int full, int32_t* err, Arc* e_arc, int64_t* e_w64, int32_t* e_len,
+                          const __grid_constant__ EOps ops) {
     pdl_enter();
-    if (*err) return;
+    if (*reinterpret_cast<const volatile int32_t*>(err)) return;
+    if (blockIdx.x == 0 && (int)threadIdx.x < ops.count) dev_estar_write(ops.op[threadIdx.x], e_arc, e_w64, e_len);
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    if (directed) dev_alg4_in<DT, false>(s, ld, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
-    else dev_alg4_in<DT, true>(s, ld, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
+    bool aff = false;
+    if (s < n) {
+        if (directed) aff = dev_alg4_in<DT, false>(s, ld, D, S, v, e, k, directed, fD, fS, fM, err);
+        else aff = dev_alg4_in<DT, true>(s, ld, D, S, v, e, k, directed, fD, fS, fM, err);
+        if (aff) changed[s] = 1u;
+    }
+    append_row(s < n && (aff || full), s, rows, counts);
+    append_row(aff, s, acc_rows, counts + 1);
 }
 
+// The OUT phase's two per-vertex passes, which only read the state: CTAs 0 .. nb-1
+// Algorithm 4 on the reversed graph, CTAs nb .. 2nb-1 the row test.
 template <typename DT>
-__global__ void k_rows_out(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
+__global__ void k_out_prep(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
                            int v, const VEdge* __restrict__ e, int k, int directed,
-                           DT* fD, uint64_t* fS, uint64_t* fM, uint8_t* mark, uint8_t* changed,
+                           DT* cD, uint64_t* cS, uint64_t* cM, DT* fD, uint64_t* fS, uint64_t* fM,
+                           int32_t* rows, int32_t* acc_rows, int32_t* counts, uint32_t* changed, int full,
                            int32_t* err) {
     pdl_enter();
-    if (*err) return;
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) dev_rows_out<DT>(s, ld, D, S, v, e, k, directed, fD, fS, fM, mark, changed, err);
-}
-
-template <typename DT>
-__global__ void k_alg4_out(int n, int ld, const DT* __restrict__ D, const uint64_t* __restrict__ S,
-                           int v, const VEdge* __restrict__ e, int k, int directed,
-                           DT* cD, uint64_t* cS, uint64_t* cM, uint8_t* changed, int32_t* err) {
-    pdl_enter();
-    if (*err) return;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n) dev_alg4_out<DT>(t, ld, D, S, v, e, k, directed, cD, cS, cM, changed, err);
-}
-
-__global__ void __launch_bounds__(kCompactThreads)
-k_compact(int n, uint8_t* mark, int clear, int32_t* rows, int32_t* count, int full,
-          int64_t* stats, const int32_t* err) {
-    pdl_enter();
-    dev_compact(n, mark, clear, rows, count, full, stats, err);
+    if (*reinterpret_cast<const volatile int32_t*>(err)) return;
+    const int nb = gridDim.x / 2;
+    if ((int)blockIdx.x < nb) {
+        const int t = blockIdx.x * blockDim.x + threadIdx.x;
+        if (t < n && dev_alg4_out<DT>(t, ld, D, S, v, e, k, directed, cD, cS, cM, err) &&
+            atomicExch(changed + v, 1u) == 0u)
+            acc_rows[atomicAdd(counts + 1, 1)] = v;
+    } else {
+        const int s = (blockIdx.x - nb) * blockDim.x + threadIdx.x;
+        bool aff = false, fresh = false;
+        if (s < n) {
+            aff = dev_rows_out<DT>(s, ld, D, S, v, e, k, directed, fD, fS, fM, err);
+            fresh = aff && changed[s] == 0u;   // s != v where aff: no other thread touches its flag
+            if (fresh) changed[s] = 1u;
+        }
+        append_row(s < n && (aff || full), s, rows, counts + 2);
+        append_row(fresh, s, acc_rows, counts + 1);
+    }
 }
 
 // K2: in-place rank-1 min-plus / path-count pass over rows[0..count) x all columns, by
@@ -373,17 +377,17 @@ __global__ void k_estar_keep(int ld, const DT* D, const Arc* e_arc, const int64_
 // paths are added).  A shortest simple path uses the edge in at most one direction, and
 // a candidate whose prefix already used the edge the other way is longer than d(s,t),
 // so one pass with both candidates taken from the old state gives the two directed
-// passes' d and sigma.  Rows are appended with one atomic per warp and list (the counts
-// start at zero); the order of a list does not affect any result.
+// passes' d and sigma.
 template <typename DT>
 __global__ void k_edge_prep(int n, int ld, const DT* D, const uint64_t* S, int u, int v, int64_t w, DT* cDv,
                             uint64_t* cSv, DT* cDu, uint64_t* cSu, DT* fD, uint64_t* fS, uint64_t* fM,
-                            int32_t* rows1, int32_t* count1, int32_t* rows2, int32_t* count2,
-                            uint8_t* changed, int32_t* err) {
+                            int32_t* rows1, int32_t* rows2, int32_t* acc_rows, int32_t* counts, uint32_t* changed,
+                            int32_t* err, Arc* e_arc, int64_t* e_w64, int32_t* e_len,
+                            const __grid_constant__ EOps ops) {
     pdl_enter();
     if (*reinterpret_cast<const volatile int32_t*>(err)) return;   // grid-uniform for this launch
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    const int lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && (int)threadIdx.x < ops.count) dev_estar_write(ops.op[threadIdx.x], e_arc, e_w64, e_len);
     const int64_t INF = Inf<DT>::v;
     bool in1 = false, in2 = false;
     if (s < n) {
@@ -419,20 +423,12 @@ __global__ void k_edge_prep(int n, int ld, const DT* D, const uint64_t* S, int u
             fD[s] = (DT)rd;
             fS[s] = rs;
             fM[s] = rm;
-            changed[s] = 1;
+            changed[s] = 1u;
         }
     }
-    const unsigned b1 = __ballot_sync(0xffffffffu, in1), b2 = __ballot_sync(0xffffffffu, in2);
-    int p1 = 0, p2 = 0;
-    if (lane == 0) {
-        if (b1) p1 = atomicAdd(count1, __popc(b1));
-        if (b2) p2 = atomicAdd(count2, __popc(b2));
-    }
-    p1 = __shfl_sync(0xffffffffu, p1, 0);
-    p2 = __shfl_sync(0xffffffffu, p2, 0);
-    const unsigned lt = (1u << lane) - 1u;
-    if (in1) rows1[p1 + __popc(b1 & lt)] = s;
-    if (in2) rows2[p2 + __popc(b2 & lt)] = s;
+    append_row(in1, s, rows1, counts);
+    append_row(in2, s, rows2, counts + 2);
+    append_row(in1 || in2, s, acc_rows, counts + 1);
 }
 
 // ------------------------------------------------------------------ launches
@@ -449,37 +445,24 @@ void launch_estar_move(const Dev& d, const EMoves& moves) {
     launch_k(k_estar_move, moves.count, 128, 0, d.st, d.e_off, d.e_arc, d.e_w64, moves);
 }
 
-void launch_alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
-    if (d.dbytes == 4)
-        launch_k(k_alg4_in<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.fD, d.fS, d.fM,
-            d.mark, d.changed, d.err);
-    else
-        launch_k(k_alg4_in<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.fD, d.fS, d.fM,
-            d.mark, d.changed, d.err);
+template <typename DT>
+static void alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k, int full, const EOps& ops) {
+    launch_k(k_alg4_in<DT>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const DT*)d.D, d.S, v, e, k, d.directed, (DT*)d.fD,
+             d.fS, d.fM, d.rows, d.acc_rows, d.counts, d.changed, full, d.err, d.e_arc, d.e_w64, d.e_len, ops);
+}
+void launch_alg4_in(const Dev& d, int32_t v, const VEdge* e, int32_t k, int full, const EOps& ops) {
+    if (d.dbytes == 4) alg4_in<int32_t>(d, v, e, k, full, ops);
+    else alg4_in<int64_t>(d, v, e, k, full, ops);
 }
 
-void launch_rows_out(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
-    if (d.dbytes == 4)
-        launch_k(k_rows_out<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.fD, d.fS, d.fM,
-            d.mark, d.changed, d.err);
-    else
-        launch_k(k_rows_out<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.fD, d.fS, d.fM,
-            d.mark, d.changed, d.err);
+template <typename DT>
+static void out_prep(const Dev& d, int32_t v, const VEdge* e, int32_t k, int full) {
+    launch_k(k_out_prep<DT>, 2 * nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const DT*)d.D, d.S, v, e, k, d.directed,
+             (DT*)d.cD, d.cS, d.cM, (DT*)d.fD, d.fS, d.fM, d.rows2, d.acc_rows, d.counts, d.changed, full, d.err);
 }
-
-void launch_alg4_out(const Dev& d, int32_t v, const VEdge* e, int32_t k) {
-    if (d.dbytes == 4)
-        launch_k(k_alg4_out<int32_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, v, e, k, d.directed, (int32_t*)d.cD, d.cS, d.cM,
-            d.changed, d.err);
-    else
-        launch_k(k_alg4_out<int64_t>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, v, e, k, d.directed, (int64_t*)d.cD, d.cS, d.cM,
-            d.changed, d.err);
-}
-
-void launch_compact(const Dev& d, const uint8_t* mark, int clear, int32_t* rows, int32_t* count,
-                    int full, int stats) {
-    launch_k(k_compact, 1, kCompactThreads, 0, d.st, d.n, const_cast<uint8_t*>(mark), clear, rows, count,
-                                               full, stats ? d.stats : nullptr, d.err);
+void launch_out_prep(const Dev& d, int32_t v, const VEdge* e, int32_t k, int full) {
+    if (d.dbytes == 4) out_prep<int32_t>(d, v, e, k, full);
+    else out_prep<int64_t>(d, v, e, k, full);
 }
 
 // Dynamic shared memory of k_scan_cs: its ring of kCsStages row chunks, then a queue
@@ -561,11 +544,13 @@ void launch_scan_in(const Dev& d, int32_t v) {
     }
 }
 
-// OUT phase: columns come from the new row v computed by k_alg4_out; row v itself is
+// OUT phase: columns come from the new row v computed by k_out_prep; row v itself is
 // written afterwards by k_write_row.
 void launch_scan_out(const Dev& d, int32_t v) {
     if (d.dbytes == 4) {
         ScanArgs<int32_t> a = scan_args<int32_t>(d);
+        a.rows = d.rows2;
+        a.count = d.counts + 2;
         a.cD = (const int32_t*)d.cD;
         a.cS = d.cS;
         a.cM = d.cM;
@@ -574,6 +559,8 @@ void launch_scan_out(const Dev& d, int32_t v) {
         scan_dispatch<int32_t>(d, a);
     } else {
         ScanArgs<int64_t> a = scan_args<int64_t>(d);
+        a.rows = d.rows2;
+        a.count = d.counts + 2;
         a.cD = (const int64_t*)d.cD;
         a.cS = d.cS;
         a.cM = d.cM;
@@ -598,18 +585,17 @@ void launch_write_row(const Dev& d, int32_t v) {
 
 // The fused pass of an undirected edge update {u, v} with weight w: the row lists and
 // column snapshots (k_edge_prep), then one rank-1 pass over both lists, each against its
-// own column vector, every change a first change of the update.  List 1 goes to rows /
-// counts[0] against row v; list 2 to acc_rows / counts[2] (free until the pair lists are
-// built after the pass) against row u.
-void launch_edge_prep(const Dev& d, int32_t u, int32_t v, int64_t w) {
-    cudaMemsetAsync(d.counts, 0, 3 * sizeof(int32_t), d.st);   // counts[0..2]; [1] is rewritten later
-    const int grid = (d.n + 255) / 256;
-    if (d.dbytes == 4)
-        launch_k(k_edge_prep<int32_t>, grid, 256, 0, d.st, d.n, d.ld, (const int32_t*)d.D, d.S, u, v, w, (int32_t*)d.cD, d.cS, (int32_t*)d.cD2, d.cS2, (int32_t*)d.fD,
-            d.fS, d.fM, d.rows, d.counts, d.acc_rows, d.counts + 2, d.changed, d.err);
-    else
-        launch_k(k_edge_prep<int64_t>, grid, 256, 0, d.st, d.n, d.ld, (const int64_t*)d.D, d.S, u, v, w, (int64_t*)d.cD, d.cS, (int64_t*)d.cD2, d.cS2, (int64_t*)d.fD,
-            d.fS, d.fM, d.rows, d.counts, d.acc_rows, d.counts + 2, d.changed, d.err);
+// own column vector, every change a first change of the update.  List 1 (rows) goes
+// against row v, list 2 (rows2) against row u.
+template <typename DT>
+static void edge_prep(const Dev& d, int32_t u, int32_t v, int64_t w, const EOps& ops) {
+    launch_k(k_edge_prep<DT>, nblk(d.n, 256), 256, 0, d.st, d.n, d.ld, (const DT*)d.D, d.S, u, v, w, (DT*)d.cD, d.cS,
+             (DT*)d.cD2, d.cS2, (DT*)d.fD, d.fS, d.fM, d.rows, d.rows2, d.acc_rows, d.counts, d.changed, d.err, d.e_arc,
+             d.e_w64, d.e_len, ops);
+}
+void launch_edge_prep(const Dev& d, int32_t u, int32_t v, int64_t w, const EOps& ops) {
+    if (d.dbytes == 4) edge_prep<int32_t>(d, u, v, w, ops);
+    else edge_prep<int64_t>(d, u, v, w, ops);
 }
 
 template <typename DT>
@@ -620,7 +606,7 @@ static void edge_scan(const Dev& d) {
     a.cD = (const DT*)d.cD;
     a.cS = d.cS;
     a.cM = d.cS;
-    a.rows2 = d.acc_rows;
+    a.rows2 = d.rows2;
     a.count2 = d.counts + 2;
     a.cD2 = (const DT*)d.cD2;
     a.cS2 = d.cS2;

@@ -120,9 +120,8 @@ typedef struct bc_info {
     int64_t estar_moves;         /* vertex segments of E* moved to the free region instead */
     int64_t pair_rows;           /* rows whose dependencies were corrected pair by pair */
     int64_t pair_targets;        /* (row, changed target) pairs of those corrections */
-    int64_t walk_pairs;          /* of pair_targets: pairs whose columns were found by DAG walks
-                                    ("pair_walk") */
-    int64_t walk_vertices;       /* vertices on their shortest paths (both states) found by the walks */
+    int64_t walk_pairs;          /* of pair_targets: pairs corrected by DAG walks ("pair_walk") */
+    int64_t walk_vertices;       /* vertices on their shortest paths found by the walks, per row */
     int64_t walk_arcs;           /* E* superset arcs the walks examined */
 } bc_info;
 
@@ -264,14 +263,16 @@ int bc_get_profile(bc_graph* g, double* ms, int64_t* launches, int32_t reset);
  *                     (one source's passes spread over more threads); 0: the
  *                     CTAs chosen by n for thousands of sources, which share SMs better
  *                     with other handles' work (the server sets 0 for its graphs).  Same results bit for bit.
- *   "pair_walk" 0|1 (undirected graphs only; BC_ERR_ARG on a directed graph): find the
- *                     columns of each changed pair (s,t) -- the vertices on a shortest
- *                     s-t path of the old and of the new state -- by walking DAG(s) of
- *                     Eq. 1 backwards from t over the E* superset, instead of testing
- *                     every column.  Same results bit for bit.  Turning it on allocates
- *                     its scratch (16 bytes per vertex per warp of the walk grid) once;
- *                     BC_ERR_OOM if that fails, BC_ERR_ARG if n is too large for the
- *                     walk's per-warp bit sets (n above ~100k).
+ *   "pair_walk" 0|1 (undirected graphs only; BC_ERR_ARG on a directed graph): correct a
+ *                     row by walking DAG(s) of Eq. 1 backwards from its changed targets
+ *                     over the E* superset, instead of testing every column of every
+ *                     pair.  Same D and sigma bit for bit, dependencies within rounding.
+ *                     On by default from 3072 vertices (where its scratch fits).  Turning
+ *                     it on allocates that scratch (about 80 bytes per vertex and SM) once;
+ *                     BC_ERR_OOM if that fails.
+ *   "walk_cap"        (with "pair_walk" on): most entries of a row's table in shared
+ *                     memory to use; a row that needs more takes one in device memory.
+ *                     Same results bit for bit.
  */
 int bc_set_option(bc_graph* g, const char* name, int64_t value);
 

@@ -74,7 +74,6 @@ struct bc_graph {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int64_t bytes = 0;
     double last_init_ms = 0.0;
-    int64_t walk_cap_alloc = 0;   // entries allocated for the DAG walks' buffer
     std::vector<void*> allocs;
     std::vector<void*> allocs_async;   // stream-ordered (replaced while the handle lives)
     // launch accounting and optional per-class event timing
@@ -447,27 +446,28 @@ void mirror_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::v
     }
 }
 
-// Scratch of the DAG walks (per warp of the walk grid: a vertex list, a touched-column
-// list and a row of column sums), allocated once per handle.
+// Range of the option "walk_cap" (far above any table's size).
+int64_t walk_cap_max(const Dev& d) { return (8ll << 20) + 64ll * d.n + 131072ll * d.nsm; }
+
+// Scratch of the DAG walks, allocated once per handle (in one piece: nothing is left behind
+// where it does not fit).
 int walk_alloc(bc_graph* g) {
     Dev& d = g->d;
-    if (d.walk_list) return BC_OK;
-    if (walk_smem(d.n) > kWalkSmemMax) return fail(g, BC_ERR_ARG, "pair_walk: n too large for the walk's bit sets");
-    const size_t n = (size_t)d.n;
-    // expected use is ~25 entries per changed pair; every warp may leave part of a block unused
-    d.walk_cap = (int64_t)(8u << 20) + 64 * (int64_t)n + walk_warps(d.nsm) * kWalkBlock;
-    g->walk_cap_alloc = d.walk_cap;
-    int rc;
-    if ((rc = dalloc(g, &d.walk_list, (size_t)walk_warps(d.nsm) * n)) ||
-        (rc = dalloc(g, &d.walk_buf, (size_t)d.walk_cap)) || (rc = dalloc(g, &d.walk_useg, n * kPairCap * 4)) ||
-        (rc = dalloc(g, &d.walk_acc2, (size_t)walk_ctas(d.nsm) * 2 * n)) ||
-        (rc = dalloc(g, &d.walk_tl, (size_t)walk_ctas(d.nsm) * n)) || (rc = dalloc(g, &d.walk_ctl, 8)) ||
-        (rc = dalloc(g, &d.walk_rowE, n)))
-        return rc;
-    cudaError_t e = cudaMemsetAsync(d.walk_acc2, 0, sizeof(int64_t) * (size_t)walk_ctas(d.nsm) * 2 * n, d.st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.walk_ctl, 0, sizeof(int32_t) * 8, d.st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d.walk_rowE, 0, sizeof(int32_t) * n, d.st);
-    if (e != cudaSuccess) return cuda_fail(g, e, "cudaMemsetAsync");
+    if (d.walk_rows) return BC_OK;
+    const size_t lists = (2 * (size_t)d.n + 8 + 63) / 64 * 64 * sizeof(int32_t);
+    unsigned char* p = nullptr;
+    int rc = dalloc(g, &p, lists + walk_dense_bytes(d.n, d.dbytes) * (size_t)d.nsm);
+    if (rc) return rc;
+    d.walk_rows = reinterpret_cast<int32_t*>(p);
+    d.walk_ctl = d.walk_rows + 2 * (size_t)d.n;
+    d.walk_dense = p + lists;
+    d.walk_cap = walk_cap_max(d);
+    cudaError_t e = cudaMemsetAsync(d.walk_ctl, 0, sizeof(int32_t) * 8, d.st);
+    if (e == cudaSuccess) e = walk_setup(d);
+    if (e != cudaSuccess) {
+        d.walk_rows = nullptr;
+        return cuda_fail(g, e, "walk_alloc");
+    }
     return BC_OK;
 }
 
@@ -541,27 +541,36 @@ int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const 
         // rows with more changed targets than kPairCap (and row v): Algorithm 1 in full;
         // the others: pair corrections of their dependency rows.  Both add their changes to
         // BC's fixed-point change, which k_update_end folds into BC.
-        timed(g, 5, 1, [&] { launch_pair_plan(d); });
-        // kernels of launch_pairdep: weights, then the walks (units, two hash-table row
-        // classes, whole-CTA rows) and the gated column test, or the column test alone
-        const int pair_launches = walk ? 6 : 2;
+        timed(g, 5, 1, [&] {
+            if (walk) launch_walk_class(d);
+            else launch_pair_plan(d);
+        });
+        // the walks of the rows of a CTA each, of the light ones, of those that outgrew
+        // their tables; or the weights and the column test
+        const int pair_launches = walk ? 3 : 2;
+        auto corrections = [&](const Dev& dd, cudaEvent_t ready) {
+            if (walk) launch_walks(dd, upd, ready);
+            else launch_pairdep(dd);
+        };
         if (!g->profile) {
             // the two write disjoint dependency rows and only read the rest of the state:
-            // the (latency-bound, partial-wave) accumulation of the full rows runs on the
-            // second stream beside the pair corrections, its first kernel: launched before
-            // the pair corrections, it gets its SMs before their CTAs (which stay resident
-            // until all their work is taken) fill the GPU.
+            // the (latency-bound, partial-wave) accumulation of the full rows runs beside the
+            // pair corrections, its first kernel: launched before the pair corrections, it gets
+            // its SMs before their CTAs (which stay resident until all their work is taken)
+            // fill the GPU.  Hence the walks, which start at once, go to the other streams,
+            // while the column test waits for its weights.
             Dev ds = d;
             ds.st = g->side;
             CK(g, cudaEventRecord(g->ev_fork, d.st));
             CK(g, cudaStreamWaitEvent(g->side, g->ev_fork, 0));
-            launch_accum_rows(ds, d.full_rows, d.counts + 3);
+            launch_accum_rows(walk ? d : ds, d.full_rows, d.counts + 3);
+            if (walk) corrections(ds, g->ev_fork);
             CK(g, cudaEventRecord(g->ev_join, g->side));
-            launch_pairdep(d, walk ? &upd : nullptr);
+            if (!walk) corrections(d, nullptr);
             CK(g, cudaStreamWaitEvent(d.st, g->ev_join, 0));
             g->launches += 1 + pair_launches;
         } else {
-            timed(g, 5, pair_launches, [&] { launch_pairdep(d, walk ? &upd : nullptr); });
+            timed(g, 5, pair_launches, [&] { corrections(d, nullptr); });
             timed(g, 1, 1, [&] { launch_accum_rows(d, d.full_rows, d.counts + 3); });
         }
     } else {
@@ -585,7 +594,6 @@ void destroy_all(bc_graph* g) {
         cudaStreamSynchronize(g->d.st3);
         cudaStreamDestroy(g->d.st3);
     }
-    if (g->d.ev3_fork) cudaEventDestroy(g->d.ev3_fork);
     if (g->d.ev3_join) cudaEventDestroy(g->d.ev3_join);
     for (void* p : g->allocs_async) cudaFreeAsync(p, g->d.st);
     if (!g->allocs_async.empty()) cudaStreamSynchronize(g->d.st);
@@ -751,7 +759,6 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
                   cudaEventCreateWithFlags(&g->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                   cudaEventCreateWithFlags(&g->ev_join, cudaEventDisableTiming) != cudaSuccess ||
                   cudaStreamCreateWithFlags(&g->d.st3, cudaStreamNonBlocking) != cudaSuccess ||
-                  cudaEventCreateWithFlags(&g->d.ev3_fork, cudaEventDisableTiming) != cudaSuccess ||
                   cudaEventCreateWithFlags(&g->d.ev3_join, cudaEventDisableTiming) != cudaSuccess))) {
         destroy_all(g);
         return fail(nullptr, BC_ERR_OOM, "stream or event creation failed");
@@ -773,10 +780,13 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
                         std::string(#call) + ": " + cudaGetErrorString(e_));               \
     } while (0)
     CKI(scan_setup());
-    CKI(walk_setup());
+    CKI(pair_setup());
     if (!dir && n >= kWalkDefaultMinN) {
-        if ((rc = walk_alloc(g))) return bail(rc, g->last_error);
-        d.pair_walk = 1;
+        // (no room for its scratch: the column test, which needs none)
+        rc = walk_alloc(g);
+        if (rc != BC_OK && rc != BC_ERR_OOM) return bail(rc, g->last_error);
+        d.pair_walk = rc == BC_OK ? 1 : 0;
+        cudaGetLastError();
     }
     CKI(cudaMemsetAsync(d.err, 0, sizeof(int32_t), d.st));
     CKI(cudaMemsetAsync(slab + zero_from, 0, total - zero_from, d.st));
@@ -1193,10 +1203,10 @@ int bc_set_option(bc_graph* g, const char* name, int64_t value) {
         return BC_OK;
     }
     if (std::strcmp(name, "walk_cap") == 0) {
-        // entries of the walks' buffer to use (at most the allocated size; a test knob:
-        // an update whose walks do not fit is done by the column test)
-        if (!g->d.walk_list) return fail(g, BC_ERR_ARG, "walk_cap needs pair_walk on");
-        if (value < 0 || value > g->walk_cap_alloc) return fail(g, BC_ERR_ARG, "walk_cap out of range");
+        // entries of a row's table in shared memory to use at most (a test knob: a row that
+        // needs more takes a table in device memory; same results bit for bit)
+        if (!g->d.walk_rows) return fail(g, BC_ERR_ARG, "walk_cap needs pair_walk on");
+        if (value < 0 || value > walk_cap_max(g->d)) return fail(g, BC_ERR_ARG, "walk_cap out of range");
         g->d.walk_cap = value;
         return BC_OK;
     }

@@ -118,12 +118,11 @@ struct WalkUpd {
     int32_t x[kWalkMaxEdges];
     int64_t wold[kWalkMaxEdges];
 };
-constexpr int kWalkThreads = 256;
-constexpr int kWalkCtasPerSm = 8;      // walks: latency-bound, 32 registers, a few KB of shared memory
-constexpr int kWalkRowCtasPerSm = 8;
-constexpr size_t kWalkSmemMax = 200 * 1024;
-constexpr int kWalkBlock = 2048;     // walk buffer entries a warp reserves at a time
-constexpr int kWalkDefaultMinN = 12288;   // undirected graphs with at least this many vertices walk by default
+// Undirected graphs with at least this many vertices walk by default.  The walks are the
+// faster from n = 512 on (per update, column test / walks, int32: n = 512 153 / 76 us, 2048
+// 159 / 98, 4096 245 / 156, 8192 547 / 267; int64, n = 1500: 116 / 96), but a batch uses the
+// column test, and small graphs get the same bits alone and in a batch.
+constexpr int kWalkDefaultMinN = 3072;
 
 // One edge of a vertex update, as staged on the device (matches bc_vedge).
 struct VEdge {
@@ -248,22 +247,20 @@ struct Dev {
     int64_t* pair_w;     // [n + 1] prefix of the pair corrections' work item weights
     int32_t* full_rows;  // [n] rows re-accumulated in full (counts[3])
     int32_t* pair_rows;  // [n] rows corrected pair by pair, most targets first (counts[5])
-    int32_t pair_walk;   // 1: pair corrections by DAG walks (k_walk_units, k_walk_rows), scratch below
-    int32_t* walk_list;      // [walk warps * n] per-warp vertex lists of a walk
-    int32_t* walk_buf;       // [walk_cap] vertices found by the walks of an update
-    int64_t walk_cap;
-    int32_t* walk_useg;      // [n * tcap * 4] per (row, target): segments of the old and new walk
-    int64_t* walk_acc2;      // [walk CTAs * 2n] per-CTA fixed-point column sums of a row (zero between rows)
-    int32_t* walk_tl;        // [walk CTAs * n] per-CTA touched columns of a row
-    int32_t* walk_ctl;       // [8] units and rows handed out, buffer used (64-bit), overflow
-    int32_t* walk_rowE;      // [n] per listed row: vertices found by its walks
+    int32_t pair_walk;   // 1: pair corrections by DAG walks (k_walk.cu), scratch below
+    int64_t walk_cap;    // most entries of a walk's table in shared memory
+    int32_t walk_grid[2];    // CTAs of the walks of light rows, of rows with more targets
+    int32_t* walk_rows;      // [2n] rows with more targets, rows that outgrew their table
+    int32_t* walk_ctl;       // [8] rows in the lists of light rows and these two, and taken from
+                             // each; zero between updates
+    unsigned char* walk_dense;   // [nsm * walk_dense_bytes] tables of rows that outgrow shared memory
     int64_t* bcfix;      // [2n] BC change of the changed rows in this update, per column a
                          // fixed-point pair (units of 2^-24, units of 2^-56); zero between updates
     cudaStream_t st;
-    // a third stream for the heaviest rows of the DAG walks' phase 2 (undirected graphs):
-    // forked from st after the walks, joined back before the BC fix-up
+    // a third stream for the rows walked by a CTA each (undirected graphs): forked from st
+    // before the light rows, joined back after them
     cudaStream_t st3;
-    cudaEvent_t ev3_fork, ev3_join;
+    cudaEvent_t ev3_join;
 };
 
 constexpr int kRowsPerBlock = 64;   // rows per partial sum of the BC reduction
@@ -371,13 +368,13 @@ void launch_edge_scan(const Dev& d);
 void launch_estar_keep(const Dev& d, uint8_t* keep);
 PairRec pair_rec(const Dev& d);
 void launch_pair_plan(const Dev& d);
-void launch_pairdep(const Dev& d, const WalkUpd* upd);   // upd: DAG walks (k_pairwalk), else column tests
-size_t walk_smem(int n);
-int64_t walk_warps(int nsm);
-int64_t walk_ctas(int nsm);
-// Kernel attributes of the pair corrections (the walks' and the weights pass's dynamic
-// shared memory limits); bc_init_static sets them before it builds a handle.
-cudaError_t walk_setup();
+void launch_pairdep(const Dev& d);
+cudaError_t pair_setup();   // kernel attributes (the weights pass's dynamic shared memory)
+// The pair corrections by walks: rows to their classes (k_pair_plan's place), then the walks.
+void launch_walk_class(const Dev& d);
+void launch_walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready);   // ready: when the classes are (NULL: one stream)
+size_t walk_dense_bytes(int n, int dbytes);   // of one table (a table per SM)
+cudaError_t walk_setup(Dev& d);               // launch shapes, kernel attributes, empty tables
 void launch_update_end(const Dev& d);
 
 // ---- launches (k_accum.cu) ----

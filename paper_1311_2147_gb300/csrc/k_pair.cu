@@ -80,7 +80,6 @@ struct PairArgs {
     int32_t* next_piece;    // pieces of the work handed out so far past the first wave
     const int32_t* prows;   // the rows corrected pair by pair, most targets first
     const int32_t* pcount;
-    const int32_t* gate;    // when set: the column test runs only if *gate != 0 (walk overflow)
     int tcap;
     const int32_t* rows;
     const int32_t* count;
@@ -253,7 +252,7 @@ struct PairWeightsSmem {
 // the last pass overwrites with the prefix.
 __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int32_t* count, const int32_t* tcnt,
                                                  int tcap, int nchunks, int32_t* prows, int32_t* pcount,
-                                                 int64_t* wpre, int64_t* stats, int32_t* walk_ctl, int32_t* walk_rowE, PairWeightsSmem& sm,
+                                                 int64_t* wpre, int64_t* stats, PairWeightsSmem& sm,
                                                  int32_t* s_r, int32_t* s_T, int scap) {
     int64_t* wsum = sm.wsum;
     int64_t& s_total = sm.s_total;
@@ -295,8 +294,6 @@ __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int3
     }
     __syncthreads();
     const int cnt = s_hist[0];
-    if (walk_rowE)
-        for (int i = tid; i < cnt_all; i += blockDim.x) walk_rowE[i] = 0;
     for (int i0 = 0; i0 < cnt_all; i0 += blockDim.x) {
         const int i = i0 + tid;
         const int r = i < cnt_all ? (staged ? s_r[i] : rows[i]) : 0;
@@ -371,8 +368,6 @@ __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int3
             t += s_tgts[k];
         }
         wpre[cnt] = base;
-        if (walk_ctl)
-            for (int k = 0; k < 8; ++k) walk_ctl[k] = 0;
         stats[8] += r;
         stats[9] += t;
     }
@@ -381,13 +376,13 @@ __device__ __forceinline__ void dev_pair_weights(const int32_t* rows, const int3
 __global__ void __launch_bounds__(1024) k_pair_weights(const int32_t* rows, const int32_t* count,
                                                        const int32_t* tcnt, int tcap, int nchunks,
                                                        int32_t* prows, int32_t* pcount,
-                                                       int64_t* wpre, int64_t* stats, int32_t* walk_ctl, int32_t* walk_rowE, const int32_t* err,
+                                                       int64_t* wpre, int64_t* stats, const int32_t* err,
                                                        int scap) {
     pdl_enter();
     __shared__ PairWeightsSmem sm;
     extern __shared__ int32_t s_stage[];   // 2 * scap ints
     if (*err) return;
-    dev_pair_weights(rows, count, tcnt, tcap, nchunks, prows, pcount, wpre, stats, walk_ctl, walk_rowE,
+    dev_pair_weights(rows, count, tcnt, tcap, nchunks, prows, pcount, wpre, stats,
                      sm, s_stage, s_stage + scap, scap);
 }
 
@@ -563,7 +558,6 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) k_pairdep(PairAr
     __shared__ PairQueue s_wq[kPairThreads / 32];
     __shared__ int s_i, s_c, s_p;
     if (*a.err) return;
-    if (a.gate && *a.gate == 0) return;
     constexpr int CW = kPairThreads * VN;
     const int n = a.n;
     const int nchunks = (n + CW - 1) / CW;
@@ -675,6 +669,7 @@ struct EndArgs {
     uint32_t* chg;
     int words;
     int64_t* stats;
+    int32_t* walk_ctl;   // NULL: no walks
     const int32_t* err;
 };
 __global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
@@ -691,6 +686,8 @@ __global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
     if (threadIdx.x == 0 && atomicAdd(a.counts + 6, 1) == (int)gridDim.x - 1) {
         dev_update_stats(a.stats, cnt, a.counts[3]);
         for (int k = 0; k < 8; ++k) a.counts[k] = 0;
+        if (a.walk_ctl)
+            for (int k = 0; k < 8; ++k) a.walk_ctl[k] = 0;
     }
 }
 
@@ -700,7 +697,7 @@ PairRec pair_rec(const Dev& d) { return make_pair_rec(d); }
 
 void launch_update_end(const Dev& d) {
     EndArgs a{d.n, d.bcfix, d.bc_hi, d.bc_lo, d.acc_rows, d.counts, d.changed, d.pair_on ? d.tcnt : nullptr, d.tlist,
-              d.tcap, d.chg, d.chg_words, d.stats, d.err};
+              d.tcap, d.chg, d.chg_words, d.stats, d.walk_ctl, d.err};
     launch_k(k_update_end, std::min(d.nsm * 4, std::max(1, (d.n + 31) / 32)), 256, 0, d.st, a);
 }
 
@@ -722,7 +719,6 @@ __host__ __device__ inline PairArgs<DT> pair_args(const Dev& d) {
     a.next_piece = d.counts + 4;
     a.prows = d.pair_rows;
     a.pcount = d.counts + 5;
-    a.gate = nullptr;
     a.tcap = d.tcap;
     a.rows = d.acc_rows;
     a.count = d.counts + 1;
@@ -776,7 +772,7 @@ __global__ void __launch_bounds__(1024) kb_pair_weights(BatchArgs b, int r, int 
         const int cw = kPairThreads * pair_vn(d.dbytes);
         const int nchunks = (d.n + cw - 1) / cw;
         dev_pair_weights(d.acc_rows, d.counts + 1, d.tcnt, d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w,
-                         d.stats, nullptr, nullptr, sm, s_stage, s_stage + scap, scap);
+                         d.stats, sm, s_stage, s_stage + scap, scap);
         __syncthreads();
     }
 }
@@ -937,478 +933,11 @@ void batch_pair_launches(const BatchArgs& b, const BatchLaunch& L, int r, int db
     else batch_pairs<int64_t>(b, L, r, st);
 }
 
-// ------------------------------------------------------------------ DAG walks
-//
-// The same corrections with the columns found by walking the shortest-path DAG instead
-// of testing every column.  The columns on a shortest s-t path of a state are the
-// vertices from which t is reachable in DAG(s) of that state (Eq. 1: the arcs (x, y)
-// with d(s,x) + w(x,y) = d(s,y)), so a walk backwards from t over those arcs visits
-// exactly them -- about 20 per changed pair against n column tests.  In G_D of an
-// undirected graph the arcs into y are y's own arcs reversed (same weight), read from
-// the E* superset; before the update E*+ held every arc of the old E* (arcs are only
-// added between re-layouts, and a re-layout keeps the arcs of the state it reads), and
-// the arcs of the update itself carry their old weight from `upd` (or did not exist).
-//
-// Phase 1 (k_walk_units): a unit is one changed pair (row s, target); any free warp
-// takes the next units, walks both states level by level (the arcs of a level's
-// vertices spread over the lanes) and appends the vertices found -- t excluded -- to a
-// global buffer, recording each walk's segment.  Phase 2 (k_walk_rows): one CTA per row;
-// its warps share out the row's segments, evaluate the terms and add them to a per-CTA
-// row of fixed-point column sums (integer atomics, so the sums do not depend on which
-// warp adds first), which is then added to delta_s and to BC's fixed-point change.  If
-// the buffer overflows, phase 2 does nothing and the column test runs instead.
-
-template <typename DT>
-struct WalkArgs {
-    const int32_t* e_off;
-    const int32_t* e_len;
-    const Arc* e_arc;
-    const int64_t* e_w64;
-    int32_t* list;      // [walk warps * n] vertices of a walk, level by level (phase 1)
-    int32_t* buf;       // [cap] vertices found by the walks of the update's units
-    int64_t cap;
-    int32_t* useg;      // [n * tcap * 4] per unit: start and length of the old, then the new walk
-    int64_t* acc2;      // [CTAs * 2n] per CTA: fixed-point column sums of a row (zero between rows)
-    int32_t* tl;        // [CTAs * n] per CTA: columns of the row with a sum
-    int32_t* ctl;       // [0] units handed out [1] rows handed out [2..3] buffer used (64-bit) [4] overflow
-                        // [5] light rows handed out [6] mid-size rows handed out
-    int32_t* rowE;      // [n] per listed row: vertices its walks found (zeroed by k_pair_weights)
-    int64_t* stats;     // [10] pairs walked [11] vertices found [12] arcs examined
-    int nchunks;        // items per row in the weight prefix wpre
-    WalkUpd upd;
-};
-
-constexpr int kWalkWarps = kWalkThreads / 32;
-constexpr int kWalkGrab = 1;         // units a warp takes at a time (unit costs vary too much for more)
-constexpr int kWalkLightRowMax = 128;   // rows whose walks found at most this many vertices: light CTAs
-constexpr int kWalkMidRowMax = 512;     // up to this many: mid-size CTAs; more: k_walk_rows
-
-// d(s,x) and sigma_sx of a state: the saved values where the pair changed in this update
-// (old state).  The change-map word and the current value are loaded together (one
-// round trip); the saved value is read only where the bit is set, rarely.
-template <typename DT>
-__device__ __forceinline__ int64_t walk_d(const PairArgs<DT>& a, size_t rs, int s, int x, bool is_new) {
-    const size_t i = rs + x;
-    const int64_t cur = (int64_t)a.D[i];
-    if (is_new) return cur;
-    const uint32_t word = a.chg[(size_t)s * a.words + (x >> 5)];
-    return ((word >> (x & 31)) & 1u) ? (int64_t)a.oD[i] : cur;
-}
-template <typename DT>
-__device__ __forceinline__ uint64_t walk_sigma(const PairArgs<DT>& a, size_t rs, int s, int x, bool is_new) {
-    const size_t i = rs + x;
-    const uint64_t cur = a.S[i];
-    if (is_new) return cur;
-    const uint32_t word = a.chg[(size_t)s * a.words + (x >> 5)];
-    return ((word >> (x & 31)) & 1u) ? a.oS[i] : cur;
-}
-
-// First unit of row index r: the targets of the rows before it (wpre counts T + 1 per
-// row and item chunk).
-template <typename DT>
-__device__ __forceinline__ int64_t unit_start(const PairArgs<DT>& a, int nchunks, int r) {
-    return a.wpre[r] / nchunks - r;
-}
-
-template <typename DT>
-__global__ void __launch_bounds__(kWalkThreads, kWalkCtasPerSm) k_walk_units(PairArgs<DT> a, WalkArgs<DT> w) {
-    pdl_enter();
-    extern __shared__ uint32_t wbits[];   // per warp: visited bits
-    if (*a.err) return;
-    const int n = a.n, words = a.words;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
-    const int64_t INF = Inf<DT>::v;
-    uint32_t* vis = wbits + (size_t)wib * words;
-    int32_t* list = w.list + ((size_t)blockIdx.x * kWalkWarps + wib) * n;
-    for (int i = lane; i < words; i += 32) vis[i] = 0u;
-    __syncwarp();
-    const int cnt = *a.pcount;
-    const int64_t nunits = unit_start<DT>(a, w.nchunks, cnt);
-    const int v = w.upd.v;
-    // this warp's block of the buffer: [bnext, bend)
-    long long bnext = 0, bend = 0;
-    __shared__ unsigned long long s_cnt[kWalkWarps][2];   // per warp: vertices found, arcs examined
-    if (lane == 0) s_cnt[wib][0] = s_cnt[wib][1] = 0ull;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd(reinterpret_cast<unsigned long long*>(w.stats + 10), (unsigned long long)nunits);
-    for (;;) {
-        int g0 = 0;
-        if (lane == 0) g0 = atomicAdd(w.ctl, kWalkGrab);
-        g0 = __shfl_sync(0xffffffffu, g0, 0);
-        if (g0 >= nunits) break;
-        for (int64_t id = g0; id < min((int64_t)g0 + kWalkGrab, nunits); ++id) {
-            // the unit's row: the last r with unit_start(r) <= id, i.e. wpre[r] <= (id + r) *
-            // nchunks (wpre[r] is a multiple of nchunks)
-            int L = 0, R = cnt;
-            while (R - L > 1) {
-                const int m = (L + R) >> 1;
-                if (a.wpre[m] <= (id + m) * w.nchunks) L = m; else R = m;
-            }
-            const int s = a.prows[L];
-            const int u = (int)(id - unit_start<DT>(a, w.nchunks, L));
-            const PairTgt& pt = a.plan[(size_t)s * a.tcap + u];
-            const int t = pt.t;
-            const size_t rs = (size_t)s * a.ld;
-            for (int stt = 0; stt < 2; ++stt) {
-                const bool is_new = stt == 1;
-                int found = 0;   // warp-uniform
-                if ((is_new ? pt.dnew : pt.dold) >= 0) {
-                    if (lane == 0) {
-                        list[0] = t;
-                        vis[t >> 5] |= 1u << (t & 31);
-                    }
-                    __syncwarp();
-                    int head = 0, tail = 1;   // list[head, tail) is the current level
-                    while (head < tail) {
-                        const int l0 = head, l1 = tail;
-                        head = l1;
-                        for (int b0 = l0; b0 < l1; b0 += 32) {
-                            const int nb = min(32, l1 - b0);
-                            int y = 0, off = 0, len = 0;
-                            int64_t dy = 0;
-                            if (lane < nb) {
-                                y = list[b0 + lane];
-                                off = w.e_off[y];
-                                len = w.e_len[y];
-                                dy = walk_d<DT>(a, rs, s, y, is_new);
-                            }
-                            int incl = len;
-#pragma unroll
-                            for (int o = 1; o < 32; o <<= 1) {
-                                const int z = __shfl_up_sync(0xffffffffu, incl, o);
-                                if (lane >= o) incl += z;
-                            }
-                            const int tot = __shfl_sync(0xffffffffu, incl, 31);
-                            const int excl = incl - len;
-                            // first step of the owner search: the largest power of two below nb
-                            const int top = nb > 1 ? 1 << (31 - __clz(nb - 1)) : 0;
-                            if (lane == 0) s_cnt[wib][1] += (unsigned)tot;
-                            for (int k0 = 0; k0 < tot; k0 += 32) {   // the batch's arcs, one per lane
-                                const int k = k0 + lane;
-                                int j = 0;   // owner: the last lane j < nb whose arcs start at or before k
-                                for (int step = top; step >= 1; step >>= 1) {
-                                    const int c = j + step;
-                                    const int ex = __shfl_sync(0xffffffffu, excl, c & 31);
-                                    if (c < nb && ex <= k) j = c;
-                                }
-                                const int yj = __shfl_sync(0xffffffffu, y, j);
-                                const int offj = __shfl_sync(0xffffffffu, off, j);
-                                const int exj = __shfl_sync(0xffffffffu, excl, j);
-                                const int64_t dyj = __shfl_sync(0xffffffffu, dy, j);
-                                bool fresh = false;
-                                int x = -1;
-                                if (k < tot) {
-                                    const int e = offj + (k - exj);
-                                    const Arc arc = w.e_arc[e];
-                                    x = arc.dst();
-                                    int64_t wv = sizeof(DT) == 4 ? (int64_t)arc.w : w.e_w64[e];
-                                    if (!is_new && (yj == v || x == v)) {
-                                        const int o = yj == v ? x : yj;
-                                        for (int u = 0; u < w.upd.k; ++u)
-                                            if (w.upd.x[u] == o) wv = w.upd.wold[u];
-                                    }
-                                    if (x >= 0 && x != s && wv >= 0 && wv <= dyj) {   // else no predecessor
-                                        const int64_t dx = walk_d<DT>(a, rs, s, x, is_new);
-                                        if (dx != INF && dx + wv == dyj) {
-                                            const uint32_t bit = 1u << (x & 31);
-                                            fresh = !(atomicOr(&vis[x >> 5], bit) & bit);
-                                        }
-                                    }
-                                }
-                                const unsigned bal = __ballot_sync(0xffffffffu, fresh);
-                                if (fresh) list[tail + __popc(bal & lt)] = x;
-                                tail += __popc(bal);
-                            }
-                        }
-                        __syncwarp();
-                    }
-                    found = tail - 1;
-                    if (lane == 0) s_cnt[wib][0] += (unsigned)found;
-                    // the walk's vertices (t excluded) into the buffer
-                    // room in the warp's block, else a new block (a walk longer than a block
-                    // gets a block of its own size); one atomic per block, not per walk
-                    if (bnext + found > bend) {
-                        const long long want = found > kWalkBlock ? found : kWalkBlock;
-                        long long b = 0;
-                        if (lane == 0)
-                            b = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(w.ctl + 2),
-                                                     (unsigned long long)want);
-                        bnext = __shfl_sync(0xffffffffu, b, 0);
-                        bend = bnext + want;
-                    }
-                    const long long base = bnext;
-                    bnext += found;
-                    if (base + found <= w.cap) {
-                        for (int i = lane; i < found; i += 32) w.buf[base + i] = list[1 + i];
-                    } else {
-                        if (lane == 0) w.ctl[4] = 1;
-                        found = 0;
-                    }
-                    if (lane == 0) w.useg[id * 4 + 2 * stt] = (int32_t)base;
-                    for (int i = lane; i < tail; i += 32) vis[list[i] >> 5] = 0u;
-                    __syncwarp();
-                }
-                if (lane == 0) {
-                    w.useg[id * 4 + 2 * stt + 1] = found;
-                    if (found) atomicAdd(w.rowE + L, found);
-                }
-            }
-        }
-    }
-    if (lane == 0 && (s_cnt[wib][0] | s_cnt[wib][1])) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(w.stats + 11), s_cnt[wib][0]);
-        atomicAdd(reinterpret_cast<unsigned long long*>(w.stats + 12), s_cnt[wib][1]);
-    }
-}
-
-// A term v = hi + lo (|v| <= 1 + 2^-40, a pair dependency) as a fixed-point pair (units
-// of 2^-24 and 2^-56, as in bc_fix_add) in single precision only (fp64 runs at a small
-// fraction of the fp32 rate here): with h = hi * 2^24 and a = rint(h), h - a is exact
-// (|h| <= 2^24 + 1), and (h - a) * 2^32 and lo * 2^56 are exact scalings, each rounded to
-// an integer once, so B is within one unit of v * 2^56 - A * 2^32; a carry keeps
-// |B| <= 2^31.
-__device__ __forceinline__ void fix_split(ff v, long long* A, long long* B) {
-    const float h = v.hi * 0x1p24f;
-    const float a = rintf(h);
-    long long b = __float2ll_rn((h - a) * 0x1p32f) + __float2ll_rn(v.lo * 0x1p56f);
-    const long long c = (b + (1ll << 31)) >> 32;
-    *A = (long long)__float2int_rn(a) + c;
-    *B = b - (c << 32);
-}
-
-// A column's fixed-point sum (A in units of 2^-24 plus B in units of 2^-56, 0 <= B <
-// 2^32, |A| < 2^47) as a float-float: four exactly representable parts, added with
-// error-free sums.
-__device__ __forceinline__ ff fix_to_ff(long long A, long long B) {
-    const float p0 = (float)(int)(A >> 24);
-    const float p1 = (float)(int)(A & 0xFFFFFF) * 0x1p-24f;
-    const float p2 = (float)(int)(B >> 24) * 0x1p-32f;
-    const float p3 = (float)(int)(B & 0xFFFFFF) * 0x1p-56f;
-    return ff_add(two_sum(p0, p1), two_sum(p2, p3));
-}
-
-template <typename DT>
-__global__ void __launch_bounds__(kWalkThreads, kWalkRowCtasPerSm) k_walk_rows(PairArgs<DT> a, WalkArgs<DT> w) {
-    pdl_enter();
-    extern __shared__ uint32_t tbits[];   // touched columns of the row
-    __shared__ int s_r, s_nt;
-    if (*a.err) return;
-    if (*(volatile int32_t*)(w.ctl + 4)) return;   // overflow: the column test does the update
-    const int n = a.n, words = a.words;
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    long long* acc = reinterpret_cast<long long*>(w.acc2) + (size_t)blockIdx.x * 2 * n;
-    int32_t* tl = w.tl + (size_t)blockIdx.x * n;
-    for (int i = threadIdx.x; i < words; i += blockDim.x) tbits[i] = 0u;
-    const int cnt = *a.pcount;
-    for (;;) {
-        if (threadIdx.x == 0) {
-            s_r = atomicAdd(w.ctl + 1, 1);
-            s_nt = 0;
-        }
-        __syncthreads();
-        const int r = s_r;
-        if (r >= cnt) break;
-        if (w.rowE[r] <= kWalkMidRowMax) {   // none found, or taken by k_walk_rows_hash
-            __syncthreads();
-            continue;
-        }
-        const int s = a.prows[r];
-        const int T = a.tcnt[s];
-        const int64_t id0 = unit_start<DT>(a, w.nchunks, r);
-        const size_t rs = (size_t)s * a.ld;
-        // the row's walks (2 per target) go to the warps in turn
-        for (int q = wib; q < 2 * T; q += kWalkWarps) {
-            const int u = q >> 1;
-            const bool is_new = q & 1;
-            const PairTgt& pt = a.plan[(size_t)s * a.tcap + u];
-            const int64_t base = w.useg[(id0 + u) * 4 + 2 * (q & 1)];
-            const int len = w.useg[(id0 + u) * 4 + 2 * (q & 1) + 1];
-            const ff rcp = is_new ? pt.rnew : pt.rold;
-            const size_t rt = (size_t)pt.t * a.ld;
-            for (int i = lane; i < len; i += 32) {
-                const int x = w.buf[base + i];
-                ff term = pair_term(walk_sigma<DT>(a, rs, s, x, is_new), walk_sigma<DT>(a, rt, pt.t, x, is_new), rcp);
-                if (!is_new) term = ff{-term.hi, -term.lo};
-                long long A, B;
-                fix_split(term, &A, &B);
-                atomicAdd(reinterpret_cast<unsigned long long*>(acc + 2 * x), (unsigned long long)A);
-                if (B) atomicAdd(reinterpret_cast<unsigned long long*>(acc + 2 * x + 1), (unsigned long long)B);
-                const uint32_t bit = 1u << (x & 31);
-                if (!(atomicOr(&tbits[x >> 5], bit) & bit)) tl[atomicAdd(&s_nt, 1)] = x;
-            }
-        }
-        __syncthreads();
-        // the row's sums: delta_s and BC's change once per column, then the scratch back to zero
-        const int nt = s_nt;
-        for (int i = threadIdx.x; i < nt; i += blockDim.x) {
-            const int x = tl[i];
-            const long long A0 = acc[2 * x], B0 = acc[2 * x + 1];
-            acc[2 * x] = 0;
-            acc[2 * x + 1] = 0;
-            const long long A = A0 + (B0 >> 32), B = B0 & 0xFFFFFFFFll;   // 0 <= B < 2^32
-            const ff v = fix_to_ff(A, B);
-            ff* p = a.Dl + rs + x;
-            *p = ff_add(*p, v);
-            unsigned long long* bp = reinterpret_cast<unsigned long long*>(a.bcfix + 2 * (size_t)x);
-            atomicAdd(bp, (unsigned long long)A);
-            if (B) atomicAdd(bp + 1, (unsigned long long)B);
-            tbits[x >> 5] = 0u;
-        }
-        __syncthreads();
-    }
-}
-
-// The rows whose walks found at most kMaxE vertices (and more than kMinE) in CTAs of
-// kThreads threads, many per SM so that many rows are in flight: the warps share out the
-// row's walks and add the terms to a hash table of fixed-point column sums in shared
-// memory (kHash slots, at least twice the vertices, so it never fills and every probe
-// ends), which is then added to delta_s and to BC's change and emptied.  Two classes:
-// light rows (at most 128 vertices; most rows, one to three changed targets) in 64-thread
-// CTAs, 32 per SM, and mid-size rows (129 to 512 vertices) in 256-thread CTAs with a
-// 1024-slot table, 8 per SM.  Rows with more vertices go to k_walk_rows.
-template <int kThreads, int kCtas, int kHash, int kMinE, int kMaxE, int kCtl>
-struct WalkHash {
-    static constexpr int threads = kThreads, ctas = kCtas, hash = kHash, min_e = kMinE, max_e = kMaxE, ctl = kCtl;
-    static_assert(kHash >= 2 * kMaxE, "the hash table stays at most half full");
-    static_assert((kHash & (kHash - 1)) == 0, "a power of two");
-    static constexpr int bits = kHash == 256 ? 8 : kHash == 512 ? 9 : kHash == 1024 ? 10 : kHash == 2048 ? 11 : 12;
-    static_assert((1 << bits) == kHash, "table size");
-    static constexpr size_t smem = (size_t)kHash * (2 * sizeof(unsigned long long) + sizeof(int32_t)) +
-                                   (size_t)kMaxE * sizeof(int32_t);
-};
-using WalkLight = WalkHash<64, 32, 256, 0, kWalkLightRowMax, 5>;
-using WalkMid = WalkHash<256, 8, 1024, kWalkLightRowMax, kWalkMidRowMax, 6>;
-static_assert(WalkMid::smem * WalkMid::ctas <= 200 * 1024, "mid-size tables fit the SM");
-static_assert(WalkMid::smem <= 48 * 1024 && WalkLight::smem <= 48 * 1024, "no opt-in shared memory needed");
-
-template <typename DT, typename H>
-__global__ void __launch_bounds__(H::threads, H::ctas) k_walk_rows_hash(PairArgs<DT> a, WalkArgs<DT> w) {
-    pdl_enter();
-    extern __shared__ unsigned long long hsm[];
-    unsigned long long* hval = hsm;                                        // [2 * hash]
-    int32_t* hkey = reinterpret_cast<int32_t*>(hsm + 2 * H::hash);         // [hash]
-    int32_t* hused = hkey + H::hash;                                       // [max_e]
-    __shared__ int s_r, s_nu;
-    if (*a.err) return;
-    if (*(volatile int32_t*)(w.ctl + 4)) return;   // overflow: the column test does the update
-    const int n = a.n;
-    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-    constexpr int kW = H::threads / 32;
-    for (int i = tid; i < H::hash; i += H::threads) {
-        hkey[i] = -1;
-        hval[2 * i] = 0ull;
-        hval[2 * i + 1] = 0ull;
-    }
-    const int cnt = *a.pcount;
-    for (;;) {
-        if (tid == 0) {
-            s_r = atomicAdd(w.ctl + H::ctl, 1);
-            s_nu = 0;
-        }
-        __syncthreads();
-        const int r = s_r;
-        if (r >= cnt) break;
-        const int e = w.rowE[r];
-        if (e <= H::min_e || e > H::max_e || e == 0) {   // nothing found / another class
-            __syncthreads();
-            continue;
-        }
-        const int s = a.prows[r];
-        const int T = a.tcnt[s];
-        const int64_t id0 = unit_start<DT>(a, w.nchunks, r);
-        const size_t rs = (size_t)s * a.ld;
-        for (int q = wib; q < 2 * T; q += kW) {
-            const int u = q >> 1;
-            const bool is_new = q & 1;
-            const PairTgt& pt = a.plan[(size_t)s * a.tcap + u];
-            const int64_t base = w.useg[(id0 + u) * 4 + 2 * (q & 1)];
-            const int len = w.useg[(id0 + u) * 4 + 2 * (q & 1) + 1];
-            const ff rcp = is_new ? pt.rnew : pt.rold;
-            const size_t rt = (size_t)pt.t * a.ld;
-            for (int i = lane; i < len; i += 32) {
-                const int x = w.buf[base + i];
-                ff term = pair_term(walk_sigma<DT>(a, rs, s, x, is_new), walk_sigma<DT>(a, rt, pt.t, x, is_new), rcp);
-                if (!is_new) term = ff{-term.hi, -term.lo};
-                long long A, B;
-                fix_split(term, &A, &B);
-                int slot = (int)(((uint32_t)x * 2654435761u) >> (32 - H::bits));
-                for (;;) {
-                    const int old = atomicCAS(&hkey[slot], -1, x);
-                    if (old == -1) {
-                        hused[atomicAdd(&s_nu, 1)] = slot;
-                        break;
-                    }
-                    if (old == x) break;
-                    slot = (slot + 1) & (H::hash - 1);
-                }
-                atomicAdd(&hval[2 * slot], (unsigned long long)A);
-                if (B) atomicAdd(&hval[2 * slot + 1], (unsigned long long)B);
-            }
-        }
-        __syncthreads();
-        const int nu = s_nu;
-        for (int i = tid; i < nu; i += H::threads) {
-            const int slot = hused[i];
-            const int x = hkey[slot];
-            const long long A0 = (long long)hval[2 * slot], B0 = (long long)hval[2 * slot + 1];
-            hkey[slot] = -1;
-            hval[2 * slot] = 0ull;
-            hval[2 * slot + 1] = 0ull;
-            const long long A = A0 + (B0 >> 32), B = B0 & 0xFFFFFFFFll;   // 0 <= B < 2^32
-            const ff v = fix_to_ff(A, B);
-            ff* p = a.Dl + rs + x;
-            *p = ff_add(*p, v);
-            unsigned long long* bp = reinterpret_cast<unsigned long long*>(a.bcfix + 2 * (size_t)x);
-            atomicAdd(bp, (unsigned long long)A);
-            if (B) atomicAdd(bp + 1, (unsigned long long)B);
-        }
-        __syncthreads();
-    }
-}
-
-size_t walk_smem(int n) { return (size_t)kWalkWarps * (size_t)((n + 31) / 32) * sizeof(uint32_t); }
-int64_t walk_warps(int nsm) { return (int64_t)nsm * kWalkCtasPerSm * kWalkWarps; }
-int64_t walk_ctas(int nsm) { return (int64_t)nsm * kWalkRowCtasPerSm; }
-
-cudaError_t walk_setup() {
+cudaError_t pair_setup() {
     const int wmax = 2 * (int)sizeof(int32_t) * kWeightsStageMax;
-    cudaError_t e0 = cudaFuncSetAttribute(k_pair_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax);
-    if (e0 == cudaSuccess) e0 = cudaFuncSetAttribute(kb_pair_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax);
-    if (e0 != cudaSuccess) return e0;
-    cudaError_t e = cudaFuncSetAttribute(k_walk_units<int32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kWalkSmemMax);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_walk_units<int64_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kWalkSmemMax);
+    cudaError_t e = cudaFuncSetAttribute(k_pair_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_pair_weights, cudaFuncAttributeMaxDynamicSharedMemorySize, wmax);
     return e;
-}
-
-template <typename DT>
-static void launch_walks(const Dev& d, const WalkUpd& upd, int nchunks) {
-    const int grid = d.nsm * kWalkCtasPerSm, rgrid = d.nsm * kWalkRowCtasPerSm;
-    WalkArgs<DT> w{d.e_off, d.e_len, d.e_arc, d.e_w64, d.walk_list, d.walk_buf, d.walk_cap, d.walk_useg,
-                   d.walk_acc2, d.walk_tl, d.walk_ctl, d.walk_rowE, d.stats, nchunks, upd};
-    launch_k(k_walk_units<DT>, grid, kWalkThreads, walk_smem(d.n), d.st, pair_args<DT>(d), w);
-    // phase 2: the heaviest rows (a few CTAs with a long tail) on the third stream beside
-    // the two hash-table classes (disjoint rows, their own counters and scratch)
-    const bool third = d.st3 != nullptr;
-    cudaStream_t sr = d.st;
-    if (third) {
-        cudaEventRecord(d.ev3_fork, d.st);
-        cudaStreamWaitEvent(d.st3, d.ev3_fork, 0);
-        sr = d.st3;
-    }
-    launch_k(k_walk_rows<DT>, rgrid, kWalkThreads, (size_t)((d.n + 31) / 32) * sizeof(uint32_t), sr, pair_args<DT>(d), w);
-    if (third) cudaEventRecord(d.ev3_join, d.st3);
-    launch_k(k_walk_rows_hash<DT, WalkLight>, d.nsm * WalkLight::ctas, WalkLight::threads, WalkLight::smem, d.st, pair_args<DT>(d), w);
-    launch_k(k_walk_rows_hash<DT, WalkMid>, d.nsm * WalkMid::ctas, WalkMid::threads, WalkMid::smem, d.st, pair_args<DT>(d), w);
-    if (third) cudaStreamWaitEvent(d.st, d.ev3_join, 0);
-    // the column test, which does nothing unless the walks' buffer overflowed
-    PairArgs<DT> a = pair_args<DT>(d);
-    a.gate = d.walk_ctl + 4;
-    const int pgrid = d.nsm * kPairCtasPerSm;
-    launch_k(k_pairdep<DT, pair_vn(sizeof(DT))>, pgrid, kPairThreads, 0, d.st, a);
 }
 
 void launch_pair_plan(const Dev& d) {
@@ -1417,19 +946,13 @@ void launch_pair_plan(const Dev& d) {
     else launch_k(k_pair_plan<int64_t>, pgrid, kPlanThreads, 0, d.st, pair_args<int64_t>(d));
 }
 
-void launch_pairdep(const Dev& d, const WalkUpd* upd) {
+void launch_pairdep(const Dev& d) {
     const int vn = pair_vn(d.dbytes);
     const int cw = kPairThreads * vn;
     const int nchunks = (d.n + cw - 1) / cw;
     const int scap = weights_stage(d.n);
     launch_k(k_pair_weights, 1, 1024, 2 * sizeof(int32_t) * (size_t)scap, d.st, d.acc_rows, d.counts + 1, d.tcnt,
-             d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w, d.stats,
-             upd ? d.walk_ctl : nullptr, upd ? d.walk_rowE : nullptr, d.err, scap);
-    if (upd) {
-        if (d.dbytes == 4) launch_walks<int32_t>(d, *upd, nchunks);
-        else launch_walks<int64_t>(d, *upd, nchunks);
-        return;
-    }
+             d.tcap, nchunks, d.pair_rows, d.counts + 5, d.pair_w, d.stats, d.err, scap);
     const int grid = d.nsm * kPairCtasPerSm;   // one resident wave; later pieces go to the first free CTA
     if (d.dbytes == 4) launch_k(k_pairdep<int32_t, 8>, grid, kPairThreads, 0, d.st, pair_args<int32_t>(d));
     else launch_k(k_pairdep<int64_t, 2>, grid, kPairThreads, 0, d.st, pair_args<int64_t>(d));

@@ -1,0 +1,723 @@
+// k_walk.cu -- pair corrections of a row at a time, by walks of the shortest-path DAG.
+//
+// The rows of an update with at most kPairCap changed targets are corrected by
+//     delta'_s(x) = delta_s(x) + sum over changed pairs (s,t) of [delta'_st(x) - delta_st(x)]
+// (k_pair.cu).  For one state and the set T of the row's changed targets,
+//     delta_T(x) = sum over t in T of sigma_sx * sigma_xt / sigma_st
+// is the dependency of s on x restricted to the targets in T, and it obeys Eq. 4 with
+// the 1 replaced by "y is in T":
+//     delta_T(x) = sum over arcs (x,y) of DAG(s) of sigma_sx / sigma_sy * ([y in T] + delta_T(y)).
+// It is zero outside the ancestors of T, so a walk backwards from T over the arcs with
+// d(s,x) + w(x,y) = d(s,y) (Eq. 1) finds every vertex with a correction, and the
+// recurrence over the arcs found gives all the sums, without a term per target and
+// without reading row t.  In G_D of an undirected graph the arcs into y are y's own arcs
+// reversed (same weight), read from the E* superset; before the update E*+ held every
+// arc of the old E* (arcs are only added between re-layouts, and a re-layout keeps the
+// arcs of the state it reads), and the arcs of the update itself carry their old weight
+// from `upd` (or did not exist).  The old row is the new one except at T, where the
+// saved values hold.
+//
+// A pair (s,y) with y not in T keeps its whole set of shortest paths, so every ancestor of
+// y is outside T and has the same DAG arcs in both states: past T the two recurrences
+// differ only in the values that they carry, and, being linear, run as one on the
+// difference.  So a target has two entries in the row's table (old, carrying minus its
+// sum, and new), any other vertex one, and each is expanded once.
+//
+// A warp takes a light row with a table of 128 entries, a CTA a row with more targets and
+// a larger table, both hash tables in shared memory; rows that outgrow theirs are taken
+// by a last launch, whose CTAs fall back to dense arrays in device memory.  Sums are
+// fixed-point integers in units of 2^-55 added by atomics, so a row's result depends
+// neither on the order of its arcs nor on the class it ran in.
+//
+// Bound by latency and by the instructions of short, uneven loops (ncu, light rows at
+// n = 8192: 42 % of the issue slots, 17 % of the memory rate): per level of a walk the
+// segment, an arc, its tail's distance; hence many rows in flight (a warp and 5.4 KB each)
+// and several arcs of a lane in flight.  It replaced a walk per pair and state that listed
+// the vertices found, and a second pass that evaluated sigma_sx * sigma_xt / sigma_st for
+// each from rows s and t (Barabasi-Albert, 8 edges a vertex, weights 1..100): at n = 8192,
+// 31,500 pairs an update, 267 us an update against 391, with 64-bit distances 348 against
+// 443; 16 updates at n = 16384 8.6 ms against 11.4.  Of that: one walk for both states
+// 560 -> 446 us an update at n = 16384 (a quarter fewer arcs, half the entries); two warps
+// a CTA with 64 registers instead of 48 and more warps, 478 -> 436.
+#include <algorithm>
+
+#include "bc_device.cuh"
+
+namespace bcg {
+
+namespace {
+
+constexpr int kNone = -1;                 // the end of a list of DAG arcs
+constexpr int kManyArcs = 48;               // vertices with as many are walked one by one
+constexpr int kLightTargets = 16;         // rows with more changed targets: a CTA each
+
+template <typename DT>
+struct WalkArgs {
+    int n, ld, tcap;
+    const DT* D;
+    const uint64_t* S;
+    const DT* oD;          // values before the update, valid at the changed pairs
+    const uint64_t* oS;
+    const int32_t* tcnt;
+    const int32_t* tlist;
+    const int32_t* e_off;
+    const int32_t* e_len;
+    const Arc* e_arc;
+    const int64_t* e_w64;
+    ff* Dl;
+    int64_t* bcfix;
+    const int32_t* rows;   // rows that changed
+    const int32_t* count;
+    int32_t* full_rows;    // rows with more targets than tcap
+    int32_t* full_count;
+    int32_t* list[3];      // light rows, CTA rows, rows that outgrew their table
+    int32_t* ctl;          // [0..2] rows in the lists [3..5] rows taken past each warp's or CTA's first
+    int64_t* stats;        // [8] rows and [9] pairs corrected [10] pairs walked [11] vertices found [12] arcs examined
+    const int32_t* err;
+    int cap;               // most entries of a shared-memory table to use
+    unsigned char* dense;  // per CTA of the last launch
+    int64_t dense_stride;
+    WalkUpd upd;
+};
+
+// Each listed row to its class; the rows over the cap to those re-accumulated in full.
+template <typename DT>
+__global__ void __launch_bounds__(256) k_walk_class(const __grid_constant__ WalkArgs<DT> a) {
+    pdl_enter();
+    if (*a.err) return;
+    const int cnt = *a.count;
+    int rows = 0, tgts = 0;
+    for (int i0 = blockIdx.x * blockDim.x; i0 < cnt; i0 += gridDim.x * blockDim.x) {   // warp-uniform
+        const int i = i0 + threadIdx.x;
+        const int s = i < cnt ? a.rows[i] : 0;
+        const int T = i < cnt ? a.tcnt[s] : 0;
+        append_row(T > a.tcap, s, a.full_rows, a.full_count);
+        append_row(T > 0 && T <= min(kLightTargets, a.tcap), s, a.list[0], a.ctl + 0);
+        append_row(T > kLightTargets && T <= a.tcap, s, a.list[1], a.ctl + 1);
+        if (T <= a.tcap) {
+            rows += T > 0;
+            tgts += T;
+        }
+    }
+    rows = __reduce_add_sync(FULL, rows);
+    tgts = __reduce_add_sync(FULL, tgts);
+    if ((threadIdx.x & 31) == 0 && rows) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 8), (unsigned long long)rows);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 9), (unsigned long long)tgts);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 10), (unsigned long long)tgts);
+    }
+}
+
+// Counters of the group (warp or CTA) that has a row.
+struct WalkShared {
+    int seen;    // entries made, less the targets' without a path
+    int bare;    // those
+    int nodes;   // DAG arcs found
+    int ready;   // entries whose children are done
+    int over;    // the table is too small for the row
+    int row;
+};
+
+// A row's table.  An entry's key is 2 * vertex + 1, a target's old entry's 2 * vertex; -1
+// where free.  IX numbers entries and DAG arcs ("nodes").
+template <typename DT, typename IX>
+struct WalkTable {
+    uint64_t* sig;              // sigma_sx
+    unsigned long long* acc;    // the difference's share of x so far, at a target with a path plus 1
+                                // (old: all of it negative), in units of 2^-55
+    DT* d;                      // d(s,x)
+    int32_t* key;
+    int32_t* head;              // DAG arcs into x: first node
+    int32_t* cnt;               // DAG children of x not done yet
+    IX* seen;                   // entries made, in order (the targets first; without a path: not in it)
+    IX* ready;                  // entries whose children are done, in order
+    IX* node_x;                 // a DAG arc's tail
+    IX* node_next;              // the next arc with the same head
+
+    __host__ __device__ static constexpr size_t entry_bytes() {
+        return sizeof(uint64_t) * 2 + sizeof(DT) + 3 * sizeof(int32_t) + 2 * sizeof(IX);
+    }
+    __host__ __device__ static constexpr size_t bytes(size_t entries, size_t nodes) {
+        return (entries * entry_bytes() + nodes * 2 * sizeof(IX) + 15) & ~(size_t)15;
+    }
+    __device__ __forceinline__ WalkTable(unsigned char* p, size_t entries, size_t nodes) {
+        auto take = [&](size_t b) {
+            unsigned char* q = p;
+            p += b;
+            return q;
+        };
+        sig = reinterpret_cast<uint64_t*>(take(8 * entries));
+        acc = reinterpret_cast<unsigned long long*>(take(8 * entries));
+        d = reinterpret_cast<DT*>(take(sizeof(DT) * entries));
+        key = reinterpret_cast<int32_t*>(take(4 * entries));
+        head = reinterpret_cast<int32_t*>(take(4 * entries));
+        cnt = reinterpret_cast<int32_t*>(take(4 * entries));
+        seen = reinterpret_cast<IX*>(take(sizeof(IX) * entries));
+        ready = reinterpret_cast<IX*>(take(sizeof(IX) * entries));
+        node_x = reinterpret_cast<IX*>(take(sizeof(IX) * nodes));
+        node_next = reinterpret_cast<IX*>(take(sizeof(IX) * nodes));
+    }
+    __device__ __forceinline__ void free_entry(int e) const {
+        key[e] = -1;
+        head[e] = kNone;
+        cnt[e] = 0;
+        acc[e] = 0ull;
+    }
+    // All m entries (a multiple of four; the arrays start on 16-byte boundaries).
+    __device__ __forceinline__ void free_all(int m, int rank, int threads) const {
+        for (int i = rank; i < m / 4; i += threads) {
+            reinterpret_cast<int4*>(key)[i] = make_int4(-1, -1, -1, -1);
+            reinterpret_cast<int4*>(head)[i] = make_int4(kNone, kNone, kNone, kNone);
+            reinterpret_cast<int4*>(cnt)[i] = make_int4(0, 0, 0, 0);
+            reinterpret_cast<ulonglong2*>(acc)[2 * i] = make_ulonglong2(0ull, 0ull);
+            reinterpret_cast<ulonglong2*>(acc)[2 * i + 1] = make_ulonglong2(0ull, 0ull);
+        }
+    }
+};
+
+// v in (-2^8, 2^8) to units of 2^-55 and back: h - a is exact, each part is rounded once;
+// the four parts of the way back are exact.
+__device__ __forceinline__ long long to_units(ff v) {
+    const float h = v.hi * 0x1p24f;
+    const float a = rintf(h);
+    return __float2ll_rn(a) * (1ll << 31) + __float2ll_rn((h - a) * 0x1p31f) + __float2ll_rn(v.lo * 0x1p55f);
+}
+__device__ __forceinline__ ff from_units(long long v) {
+    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
+    const uint32_t A = (uint32_t)(m >> 31), B = (uint32_t)m & 0x7FFFFFFFu;
+    const ff r = ff_add(two_sum((float)(A >> 24), (float)(A & 0xFFFFFFu) * 0x1p-24f),
+                        two_sum((float)(B >> 24) * 0x1p-31f, (float)(B & 0xFFFFFFu) * 0x1p-55f));
+    return v < 0 ? ff{-r.hi, -r.lo} : r;
+}
+constexpr long long kOne = 1ll << 55;
+
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// GS threads work on a row: a warp, or the CTA.  H: entries of the hash table (0: dense,
+// entry = key); NODES: room for DAG arcs (dense: none are kept, the arcs are read again).
+template <typename DT, typename IX, int GS, int H, int NODES>
+struct RowWalk {
+    const WalkArgs<DT>& a;
+    const WalkTable<DT, IX>& t;
+    WalkShared& sh;
+    int limit;   // entries from which the hash table counts as too small
+    int s, T;    // the row and its changed targets
+    unsigned long long* totals;   // vertices found, arcs examined (of this lane 0)
+
+    __device__ __forceinline__ static void sync() {
+        if (GS == 32) __syncwarp();
+        else __syncthreads();
+    }
+    __device__ __forceinline__ static int rank() { return GS == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x; }
+    __device__ __forceinline__ static int home(int k) {
+        constexpr int bits = H == 0 ? 1 : 31 - __builtin_clz(H | 1);
+        return (int)(((uint32_t)k * 2654435761u) >> (32 - bits));
+    }
+    // The entry of key k, or -1.  A hash table always has a free entry, so the probe ends:
+    // past the limit every thread makes at most one more (see over()).
+    __device__ __forceinline__ int find(int k) const {
+        if constexpr (H == 0) {
+            return *(volatile int32_t*)(t.key + k) == k ? k : -1;
+        } else {
+            for (int e = home(k);; e = (e + 1) & (H - 1)) {
+                const int c = *(volatile int32_t*)(t.key + e);
+                if (c == k) return e;
+                if (c == -1) return -1;
+            }
+        }
+    }
+    // The entry of key k, made if there is none.
+    __device__ __forceinline__ int insert(int k, DT d, bool count, bool* made) const {
+        for (int e = H == 0 ? k : home(k);; e = (e + 1) & (H - 1)) {
+            const int c = atomicCAS(t.key + e, -1, k);
+            if (c != -1 && c != k) continue;
+            *made = c == -1;
+            if (c == -1) {
+                t.d[e] = d;
+                if (count) {
+                    const int u = atomicAdd(&sh.seen, 1);
+                    t.seen[u] = (IX)e;
+                    if (H != 0 && u + *(volatile int*)&sh.bare >= limit) *(volatile int*)&sh.over = 1;
+                } else {
+                    atomicAdd(&sh.bare, 1);
+                }
+            }
+            return e;
+        }
+    }
+    // Warp-uniform; asked before each step that makes at most one entry per thread.
+    __device__ __forceinline__ bool over() const { return H != 0 && __any_sync(FULL, *(volatile int*)&sh.over); }
+
+    // The old weight of an arc between x and y that weighs w now (negative: it did not exist).
+    __device__ __forceinline__ DT old_weight(DT w, int x, int y) const {
+        if (y == a.upd.v || x == a.upd.v) {
+            const int o = y == a.upd.v ? x : y;
+            for (int u = 0; u < a.upd.k; ++u)
+                if (a.upd.x[u] == o) w = (DT)min(a.upd.wold[u], Inf<DT>::v);
+        }
+        return w;
+    }
+
+    // The changed targets, each with an entry per state (2 * kPairCap of them fit any table).
+    __device__ __forceinline__ void seed() const {
+        const size_t rs = (size_t)s * a.ld;
+        for (int j0 = 0; j0 < 2 * T; j0 += GS) {
+            const int j = j0 + rank();
+            if (j < 2 * T) {
+                const int x = a.tlist[(size_t)s * a.tcap + (j >> 1)], st = j & 1;
+                const uint64_t sg = st ? a.S[rs + x] : a.oS[rs + x];
+                DT d = st ? a.D[rs + x] : a.oD[rs + x];
+                if (sg == 0) d = (DT)Inf<DT>::v;
+                bool made;
+                const bool path = (int64_t)d != Inf<DT>::v;
+                const int e = insert(2 * x + st, d, path, &made);
+                t.sig[e] = sg;
+                if (path) {
+                    t.acc[e] = (unsigned long long)(st ? kOne : -kOne);
+                    prefetch_l2(a.Dl + rs + x);
+                }
+            }
+        }
+    }
+
+    // The arcs [0, tot) of a warp's vertices (lane's: entry and state in ey, distance dy, slots
+    // from off + excl on), 32 * U at a time so that the loads of U arcs per
+    // lane overlap.  ONE: all are vertex `one`'s; else an arc's owner is the last vertex j < nb
+    // whose arcs start at or before it.
+    template <bool ONE>
+    __device__ __forceinline__ void expand(int ey, DT dy, int off, int excl, int tot, int nb, int one) const {
+        const int lane = threadIdx.x & 31;
+        const size_t rs = (size_t)s * a.ld;
+        const int top = nb > 1 ? 1 << (31 - __clz(nb - 1)) : 0;
+        if (ONE) {
+            ey = __shfl_sync(FULL, ey, one);
+            dy = __shfl_sync(FULL, dy, one);
+            off = __shfl_sync(FULL, off, one);
+        }
+        constexpr int U = ONE ? 4 : 2;
+        for (int k0 = 0; k0 < tot; k0 += 32 * U) {
+            int ej[U], x[U];
+            DT dyj[U], dx[U], w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                x[u] = -1;
+                ej[u] = ey;
+                dyj[u] = dy;
+                if (k0 + 32 * u >= tot) continue;   // uniform
+                const int k = k0 + 32 * u + lane;
+                int at = off + k;
+                if (!ONE) {
+                    int j = 0;
+                    for (int step = top; step >= 1; step >>= 1) {
+                        const int c = j + step;
+                        const int ex = __shfl_sync(FULL, excl, c & 31);
+                        if (c < nb && ex <= k) j = c;
+                    }
+                    ej[u] = __shfl_sync(FULL, ey, j);
+                    dyj[u] = __shfl_sync(FULL, dy, j);
+                    at = __shfl_sync(FULL, off, j) + k;
+                }
+                if (k < tot) {
+                    const Arc arc = a.e_arc[at];
+                    x[u] = arc.dst();
+                    w[u] = sizeof(DT) == 4 ? (DT)arc.w : (DT)a.e_w64[at];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (x[u] < 0) continue;
+                if (!(ej[u] & 1)) w[u] = old_weight(w[u], x[u], t.key[ej[u] >> 1] >> 1);
+                if (x[u] == s || w[u] < 0 || w[u] > dyj[u]) x[u] = -1;   // no predecessor
+                else dx[u] = a.D[rs + x[u]];
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (k0 + 32 * u >= tot) continue;   // uniform
+                bool is = false;
+                int f = -1;
+                int k = (x[u] << 1) | 1;
+                const DT want = dyj[u] - w[u];   // below INF: dyj is
+                if (x[u] >= 0) {
+                    is = dx[u] == want;
+                    if (!(ej[u] & 1)) {   // old: a target's distance is that of its old entry
+                        f = find(k ^ 1);
+                        if (f >= 0) {
+                            k ^= 1;
+                            is = t.d[f] == want;
+                        }
+                    }
+                }
+                if (!__any_sync(FULL, is)) continue;
+                if (over()) return;
+                if (is) {
+                    if (f < 0) {
+                        bool made;
+                        f = insert(k, want, true, &made);
+                        if (made) {
+                            prefetch_l2(a.S + rs + x[u]);
+                            prefetch_l2(a.Dl + rs + x[u]);
+                        }
+                    }
+                    atomicAdd(t.cnt + f, 1);
+                    if (H != 0) {
+                        const int q = atomicAdd(&sh.nodes, 1);
+                        if (q < NODES) {
+                            t.node_x[q] = (IX)f;
+                            t.node_next[q] = (IX)atomicExch(t.head + (ej[u] >> 1), q);
+                        } else {
+                            *(volatile int*)&sh.over = 1;
+                        }
+                    }
+                }
+                __syncwarp();
+            }
+        }
+    }
+
+    // Backwards from the entries seen, level by level, a level's vertices shared out to the
+    // warps.  Every DAG arc (x,y) counts in cnt[x], and is linked into y's list.
+    __device__ __forceinline__ void walk() const {
+        const int lane = threadIdx.x & 31;
+        constexpr int W = GS / 32;
+        const int wid = rank() >> 5;
+        for (int lo = 0;;) {
+            sync();
+            const int hi = *(volatile int*)&sh.seen;
+            const int ov = *(volatile int*)&sh.over;
+            sync();
+            if (lo >= hi || ov) break;
+            const int per = W == 1 ? 32 : min(32, (hi - lo + W - 1) / W);
+            for (int b0 = lo + wid * per; b0 < hi; b0 += W * per) {
+                const int nb = min(per, hi - b0);
+                int ey = 0;
+                int off = 0, len = 0;
+                DT dy = 0;
+                if (lane < nb) {
+                    const int e = t.seen[b0 + lane], k = t.key[e];
+                    ey = 2 * e + (k & 1);
+                    off = a.e_off[k >> 1];
+                    len = a.e_len[k >> 1];
+                    dy = t.d[e];
+                }
+                const int arcs = __reduce_add_sync(FULL, len);
+                if (lane == 0) totals[1] += (unsigned)arcs;
+                // vertices with many arcs one by one, the others together
+                for (unsigned m = __ballot_sync(FULL, len >= kManyArcs); m; m &= m - 1) {
+                    const int one = __ffs(m) - 1;
+                    expand<true>(ey, dy, off, 0, __shfl_sync(FULL, len, one), nb, one);
+                }
+                if (len >= kManyArcs) len = 0;
+                int incl = len;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int z = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += z;
+                }
+                const int tot = __shfl_sync(FULL, incl, 31);
+                expand<false>(ey, dy, off - (incl - len), incl - len, tot, nb, 0);
+            }
+            lo = hi;
+        }
+    }
+
+    // What a vertex y whose children are done has for its DAG parents: its sum c, and the
+    // sum over its path count, r, for parents with another count.
+    struct Share {
+        long long c;
+        uint64_t sig;
+        ff r;
+    };
+    __device__ __forceinline__ void share(int e, Share& h) const {
+        h.c = (long long)*(volatile unsigned long long*)(t.acc + e);
+        h.sig = t.sig[e];
+        h.r.hi = -1.f;
+        h.r.lo = 2.f;   // not computed (no float-float has |lo| > |hi|)
+    }
+    // One DAG arc (x,y): sigma_sx / sigma_sy of y's sum, which is the whole of it where x is
+    // y's only parent, mostly.
+    __device__ __forceinline__ void push(int f, Share& h) const {
+        const uint64_t sx = t.sig[f];
+        long long c = h.c;
+        if (sx != h.sig) {
+            if (h.r.lo == 2.f) h.r = ff_mul(from_units(h.c), ff_rcp(ff_from_u64(h.sig)));
+            c = to_units(ff_mul(h.r, ff_from_u64(sx)));
+        }
+        atomicAdd(t.acc + f, (unsigned long long)c);
+        if (atomicSub(t.cnt + f, 1) == 1) t.ready[atomicAdd(&sh.ready, 1)] = (IX)f;
+    }
+
+    // The recurrence: an entry pushes to its DAG parents once its own children are done.
+    __device__ __forceinline__ void pull(int nseed) const {
+        const size_t rs = (size_t)s * a.ld;
+        const int seen = *(volatile int*)&sh.seen;
+        for (int i = rank(); i < seen; i += GS) {
+            const int e = t.seen[i];
+            if (i >= nseed) t.sig[e] = a.S[rs + (t.key[e] >> 1)];
+            if (t.cnt[e] == 0) t.ready[atomicAdd(&sh.ready, 1)] = (IX)e;
+        }
+        for (int lo = 0;;) {
+            sync();
+            const int hi = *(volatile int*)&sh.ready;
+            sync();
+            if (lo >= hi) break;
+            if (H != 0) {
+                for (int i = lo + rank(); i < hi; i += GS) {
+                    const int e = t.ready[i];
+                    int q = t.head[e];
+                    if (q < 0) continue;
+                    Share r;
+                    share(e, r);
+                    while (q >= 0) {   // the list of y: at most NODES arcs
+                        push(t.node_x[q], r);
+                        q = t.node_next[q];
+                        if (q == (int)(IX)kNone) q = kNone;
+                    }
+                }
+            } else {   // a warp per entry; the arcs are read again
+                for (int i = lo + (rank() >> 5); i < hi; i += GS / 32) {
+                    const int e = t.ready[i], y = e >> 1, st = e & 1;
+                    const int off = a.e_off[y], len = a.e_len[y];
+                    const DT dy = t.d[e];
+                    Share r;
+                    share(e, r);
+                    for (int k = threadIdx.x & 31; k < len; k += 32) {
+                        const Arc arc = a.e_arc[off + k];
+                        const int x = arc.dst();
+                        DT w = sizeof(DT) == 4 ? (DT)arc.w : (DT)a.e_w64[off + k];
+                        if (!st) w = old_weight(w, x, y);
+                        if (x == s || w < 0 || w > dy) continue;
+                        int f = st ? -1 : find(2 * x);
+                        if (f < 0) f = find(2 * x + 1);
+                        if (f >= 0 && t.d[f] == dy - w) push(f, r);
+                    }
+                }
+            }
+            lo = hi;
+        }
+    }
+
+    // delta_s(x) and BC(x) change by the difference; a target's in its two entries.
+    __device__ __forceinline__ void finish(int e) const {
+        const int k = t.key[e];
+        if (k < 0 || !(k & 1)) return;
+        const int o = find(k ^ 1);
+        long long v = (long long)t.acc[e];
+        if (o >= 0) v += (long long)t.acc[o];
+        if (v == 0) return;
+        const int x = k >> 1;
+        ff* p = a.Dl + (size_t)s * a.ld + x;
+        *p = ff_add(*p, from_units(v));
+        fix_add(a.bcfix, x, v >> 31, (v & 0x7FFFFFFFll) << 1);   // units of 2^-24 and 2^-56
+    }
+
+    // The whole row; false: it outgrew the table and nothing was written but the table.
+    // The table is free before and after.
+    __device__ __forceinline__ bool run() const {
+        if (rank() == 0) sh.seen = sh.bare = sh.nodes = sh.ready = sh.over = 0;
+        sync();
+        seed();
+        sync();
+        const int nseed = *(volatile int*)&sh.seen;
+        walk();
+        const bool ok = *(volatile int*)&sh.over == 0;   // (walk ends with a sync)
+        if (ok) {
+            pull(nseed);
+            for (int i = rank(); i < nseed; i += GS) {
+                const int e = t.seen[i];
+                t.acc[e] -= (unsigned long long)(t.key[e] & 1 ? kOne : -kOne);
+            }
+            sync();
+            const int seen = *(volatile int*)&sh.seen;
+            for (int i = rank(); i < seen; i += GS) finish(t.seen[i]);
+            if (rank() == 0) totals[0] += (unsigned)(seen - nseed);
+        }
+        sync();
+        if constexpr (H != 0) {
+            t.free_all(H, rank(), GS);
+        } else {
+            const int m = *(volatile int*)&sh.seen;
+            for (int i = rank(); i < m; i += GS) t.free_entry(t.seen[i]);
+            for (int j = rank(); j < 2 * T; j += GS) t.free_entry(2 * a.tlist[(size_t)s * a.tcap + (j >> 1)] + (j & 1));
+        }
+        sync();
+        return ok;
+    }
+};
+
+__device__ __forceinline__ void walk_totals(int64_t* stats, const unsigned long long* totals) {
+    if (totals[0]) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 11), totals[0]);
+    if (totals[1]) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 12), totals[1]);
+}
+
+// Light rows: a warp each.
+constexpr int kLightWarps = 2, kLightH = 128, kLightLimit = kLightH - 33, kLightNodes = 192;
+template <typename DT> using LightTable = WalkTable<DT, uint16_t>;
+template <typename DT>
+__host__ __device__ constexpr size_t light_bytes() { return LightTable<DT>::bytes(kLightH, kLightNodes); }
+
+template <typename DT>
+__global__ void __launch_bounds__(kLightWarps * 32, 16) k_walk_light(const __grid_constant__ WalkArgs<DT> a) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char wsm[];
+    __shared__ WalkShared s_sh[kLightWarps];
+    if (*a.err) return;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const LightTable<DT> t(wsm + wib * light_bytes<DT>(), kLightH, kLightNodes);
+    t.free_all(kLightH, lane, 32);
+    __syncwarp();
+    const int limit = min(a.cap, kLightLimit);
+    const int cnt = a.ctl[0], nw = gridDim.x * kLightWarps;
+    unsigned long long totals[2] = {0ull, 0ull};
+    for (int i = blockIdx.x * kLightWarps + wib; i < cnt;) {
+        int nx = 0;   // the next row's number arrives while this one is worked on
+        if (lane == 0) nx = nw + atomicAdd(a.ctl + 3, 1);
+        const int s = a.list[0][i];
+        const RowWalk<DT, uint16_t, 32, kLightH, kLightNodes> w{a, t, s_sh[wib], limit, s, a.tcnt[s], totals};
+        if (!w.run() && lane == 0) a.list[2][atomicAdd(a.ctl + 2, 1)] = s;
+        i = __shfl_sync(FULL, nx, 0);
+    }
+    if (lane == 0) walk_totals(a.stats, totals);
+}
+
+// Rows with more targets (RETRY: rows that outgrew their table, in the dense arrays if
+// they outgrow this one too): a CTA each.  A light row has at most 16 targets (22 entries
+// in the mean, and up to 95 fit); one of more has some hundred entries, so 512 are enough
+// for most and leave eight CTAs an SM.
+template <bool RETRY>
+struct Cta {
+    static_assert(4 * kPairCap <= 512 && 2 * kLightTargets < kLightH, "room for the targets");
+    static constexpr int threads = RETRY ? 512 : 128, h = RETRY ? 2048 : 512, limit = h - threads - 1,
+                         nodes = RETRY ? 3072 : 768, per_sm = RETRY ? 1 : 8;
+    template <typename DT>
+    __host__ __device__ static constexpr size_t bytes() { return WalkTable<DT, uint16_t>::bytes(h, nodes); }
+};
+
+template <typename DT, bool RETRY>
+__global__ void __launch_bounds__(Cta<RETRY>::threads, Cta<RETRY>::per_sm) k_walk_cta(const __grid_constant__ WalkArgs<DT> a) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char wsm[];
+    __shared__ WalkShared sh;
+    if (*a.err) return;
+    using C = Cta<RETRY>;
+    constexpr int L = RETRY ? 2 : 1;
+    const int cnt = a.ctl[L];
+    if ((int)blockIdx.x >= cnt) return;
+    const WalkTable<DT, uint16_t> t(wsm, C::h, C::nodes);
+    t.free_all(C::h, threadIdx.x, C::threads);
+    const int limit = min(a.cap, C::limit);
+    unsigned long long totals[2] = {0ull, 0ull};
+    for (int i = blockIdx.x; i < cnt;) {
+        int nx = 0;
+        if (threadIdx.x == 0) nx = (int)gridDim.x + atomicAdd(a.ctl + 3 + L, 1);
+        const int s = a.list[L][i];
+        const RowWalk<DT, uint16_t, C::threads, C::h, C::nodes> w{a, t, sh, limit, s, a.tcnt[s], totals};
+        if (!w.run()) {
+            if (RETRY) {
+                const WalkTable<DT, int32_t> dt(a.dense + (size_t)blockIdx.x * a.dense_stride, 2 * (size_t)a.n, 0);
+                const RowWalk<DT, int32_t, C::threads, 0, 0> dw{a, dt, sh, 0, s, a.tcnt[s], totals};
+                dw.run();
+            } else if (threadIdx.x == 0) {
+                a.list[2][atomicAdd(a.ctl + 2, 1)] = s;
+            }
+        }
+        if (threadIdx.x == 0) sh.row = nx;
+        __syncthreads();
+        i = sh.row;
+        __syncthreads();
+    }
+    if ((threadIdx.x & 31) == 0) walk_totals(a.stats, totals);
+}
+
+// The dense arrays start free.
+template <typename DT>
+__global__ void k_walk_dense_init(unsigned char* dense, int64_t stride, int n) {
+    const WalkTable<DT, int32_t> t(dense + (size_t)blockIdx.x * stride, 2 * (size_t)n, 0);
+    for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) t.free_entry(e);
+}
+
+template <typename DT>
+WalkArgs<DT> walk_args(const Dev& d) {
+    WalkArgs<DT> a{};
+    a.n = d.n;
+    a.ld = d.ld;
+    a.tcap = d.tcap;
+    a.D = (const DT*)d.D;
+    a.S = d.S;
+    a.oD = (const DT*)d.oldD;
+    a.oS = d.oldS;
+    a.tcnt = d.tcnt;
+    a.tlist = d.tlist;
+    a.e_off = d.e_off;
+    a.e_len = d.e_len;
+    a.e_arc = d.e_arc;
+    a.e_w64 = d.e_w64;
+    a.Dl = d.Dl;
+    a.bcfix = d.bcfix;
+    a.rows = d.acc_rows;
+    a.count = d.counts + 1;
+    a.full_rows = d.full_rows;
+    a.full_count = d.counts + 3;
+    a.list[0] = d.pair_rows;
+    a.list[1] = d.walk_rows;
+    a.list[2] = d.walk_rows + d.n;
+    a.ctl = d.walk_ctl;
+    a.stats = d.stats;
+    a.err = d.err;
+    a.cap = (int)std::min<int64_t>(d.walk_cap, 1 << 20);
+    a.dense = d.walk_dense;
+    a.dense_stride = (int64_t)walk_dense_bytes(d.n, d.dbytes);
+    return a;
+}
+
+int resident(const void* f, int threads, size_t smem, int nsm) {
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, threads, smem) != cudaSuccess || b < 1) b = 1;
+    return b * nsm;
+}
+
+template <typename DT>
+void walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready) {
+    WalkArgs<DT> a = walk_args<DT>(d);
+    a.upd = upd;
+    // rows of CTAs on the third stream beside the light ones, then those that outgrew
+    // their table
+    const cudaStream_t sr = ready ? d.st3 : d.st;
+    if (ready) cudaStreamWaitEvent(sr, ready, 0);
+    launch_k(k_walk_cta<DT, false>, d.walk_grid[1], Cta<false>::threads, Cta<false>::bytes<DT>(), sr, a);
+    if (ready) cudaEventRecord(d.ev3_join, sr);
+    launch_k(k_walk_light<DT>, d.walk_grid[0], kLightWarps * 32, kLightWarps * light_bytes<DT>(), d.st, a);
+    if (ready) cudaStreamWaitEvent(d.st, d.ev3_join, 0);
+    launch_k(k_walk_cta<DT, true>, d.nsm, Cta<true>::threads, Cta<true>::bytes<DT>(), d.st, a);
+}
+
+template <typename DT>
+cudaError_t setup(Dev& d) {
+    cudaError_t e = cudaFuncSetAttribute(k_walk_cta<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Cta<true>::bytes<DT>());
+    if (e != cudaSuccess) return e;
+    d.walk_grid[0] = resident((const void*)k_walk_light<DT>, kLightWarps * 32, kLightWarps * light_bytes<DT>(), d.nsm);
+    d.walk_grid[1] = resident((const void*)k_walk_cta<DT, false>, Cta<false>::threads, Cta<false>::bytes<DT>(), d.nsm);
+    k_walk_dense_init<DT><<<d.nsm, 256, 0, d.st>>>(d.walk_dense, (int64_t)walk_dense_bytes(d.n, d.dbytes), d.n);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t walk_dense_bytes(int n, int dbytes) {
+    return dbytes == 4 ? WalkTable<int32_t, int32_t>::bytes(2 * (size_t)n, 0)
+                       : WalkTable<int64_t, int32_t>::bytes(2 * (size_t)n, 0);
+}
+cudaError_t walk_setup(Dev& d) { return d.dbytes == 4 ? setup<int32_t>(d) : setup<int64_t>(d); }
+
+void launch_walk_class(const Dev& d) {
+    const int grid = std::max(1, std::min((d.n + 255) / 256, d.nsm * 4));
+    if (d.dbytes == 4) launch_k(k_walk_class<int32_t>, grid, 256, 0, d.st, walk_args<int32_t>(d));
+    else launch_k(k_walk_class<int64_t>, grid, 256, 0, d.st, walk_args<int64_t>(d));
+}
+
+void launch_walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready) {
+    if (d.dbytes == 4) walks<int32_t>(d, upd, ready);
+    else walks<int64_t>(d, upd, ready);
+}
+
+}  // namespace bcg

@@ -267,9 +267,7 @@ int bc_get_profile(bc_graph* g, double* ms, int64_t* launches, int32_t reset);
  *                     row by walking DAG(s) of Eq. 1 backwards from its changed targets
  *                     over the E* superset, instead of testing every column of every
  *                     pair.  Same D and sigma bit for bit, dependencies within rounding.
- *                     On by default from 3072 vertices (where its scratch fits).  Turning
- *                     it on allocates that scratch (about 80 bytes per vertex and SM) once;
- *                     BC_ERR_OOM if that fails.
+ *                     On by default.  Updates of more than 32 edges use the column test.
  *   "walk_cap"        (with "pair_walk" on): most entries of a row's table in shared
  *                     memory to use; a row that needs more takes one in device memory.
  *                     Same results bit for bit.
@@ -344,11 +342,9 @@ int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* d_off, cons
  * of all graphs at once, and the rounds are captured once into a CUDA graph that is
  * replayed by one graph launch per call.  Undirected graphs with pair corrections on
  * (option "pair_updates", the default) re-accumulate only their rows over the target
- * cap and correct the others pair by pair with the column test; the DAG walks are not
- * used in batches.  A graph's result is bit-identical to applying the same updates to it
- * alone with the same options (for an undirected graph alone: the column test, i.e. n
- * below the walks' default or "pair_walk" 0; with the walks the dependencies agree
- * within rounding).  The graphs must share the distance type; they stay owned by the
+ * cap and correct the others, by the walks or the column test (option "pair_walk").  A
+ * graph's result is bit-identical to applying the same updates to it alone with the same
+ * options.  The graphs must share the distance type; they stay owned by the
  * caller and must not be used by other calls while a batch call runs.
  */
 typedef struct bc_batch bc_batch;

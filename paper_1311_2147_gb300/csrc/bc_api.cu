@@ -449,28 +449,6 @@ void mirror_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::v
 // Range of the option "walk_cap" (far above any table's size).
 int64_t walk_cap_max(const Dev& d) { return (8ll << 20) + 64ll * d.n + 131072ll * d.nsm; }
 
-// Scratch of the DAG walks, allocated once per handle (in one piece: nothing is left behind
-// where it does not fit).
-int walk_alloc(bc_graph* g) {
-    Dev& d = g->d;
-    if (d.walk_rows) return BC_OK;
-    const size_t lists = (2 * (size_t)d.n + 8 + 63) / 64 * 64 * sizeof(int32_t);
-    unsigned char* p = nullptr;
-    int rc = dalloc(g, &p, lists + walk_dense_bytes(d.n, d.dbytes) * (size_t)d.nsm);
-    if (rc) return rc;
-    d.walk_rows = reinterpret_cast<int32_t*>(p);
-    d.walk_ctl = d.walk_rows + 2 * (size_t)d.n;
-    d.walk_dense = p + lists;
-    d.walk_cap = walk_cap_max(d);
-    cudaError_t e = cudaMemsetAsync(d.walk_ctl, 0, sizeof(int32_t) * 8, d.st);
-    if (e == cudaSuccess) e = walk_setup(d);
-    if (e != cudaSuccess) {
-        d.walk_rows = nullptr;
-        return cuda_fail(g, e, "walk_alloc");
-    }
-    return BC_OK;
-}
-
 int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const VEdge* d_ent) {
     Dev& d = g->d;
     std::vector<EOp> ops;
@@ -479,7 +457,7 @@ int enqueue_update(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, const 
     bool rebuild = false;
     // the DAG walks of the pair corrections need the update's edges with their old weights
     WalkUpd upd{};
-    const bool walk = d.pair_on && d.pair_walk && !g->directed && (int)ent.size() <= kWalkMaxEdges;
+    const bool walk = update_walks(d, (int)ent.size());
     if (walk) {
         upd.v = v;
         upd.k = (int32_t)ent.size();
@@ -733,14 +711,17 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
         need(&d.tlist, (size_t)n * kPairCap, 4);
         need(&d.full_rows, n, 4);
         need(&d.pair_rows, n, 4);
-        need(&d.plan, (size_t)n * kPairCap, 40);
+        need(&d.plan, (size_t)n * kPairCap, kPairPlanBytes);
+        need(&d.walk_rows, 2 * (size_t)n, 4);
         need(&d.pair_w, (size_t)n + 1, 8);
         d.pair_on = 1;
+        d.pair_walk = 1;
+        d.walk_cap = walk_cap_max(d);
     }
     const size_t zero_from = total;   // from here on the arrays start at zero
     need(&d.stats, kStats, 8);
     need(&d.changed, n, 4);
-    need(&d.counts, 8, 4);
+    need(&d.counts, 16, 4);
     need(&d.bcfix, 2 * (size_t)n, 8);
     if (!dir) {
         need(&d.chg, (size_t)n * d.chg_words, 4);   // the change map
@@ -781,13 +762,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     } while (0)
     CKI(scan_setup());
     CKI(pair_setup());
-    if (!dir && n >= kWalkDefaultMinN) {
-        // (no room for its scratch: the column test, which needs none)
-        rc = walk_alloc(g);
-        if (rc != BC_OK && rc != BC_ERR_OOM) return bail(rc, g->last_error);
-        d.pair_walk = rc == BC_OK ? 1 : 0;
-        cudaGetLastError();
-    }
+    CKI(walk_setup());
     CKI(cudaMemsetAsync(d.err, 0, sizeof(int32_t), d.st));
     CKI(cudaMemsetAsync(slab + zero_from, 0, total - zero_from, d.st));
     if (d.ld > n) {
@@ -1195,17 +1170,13 @@ int bc_set_option(bc_graph* g, const char* name, int64_t value) {
     }
     if (std::strcmp(name, "pair_walk") == 0) {
         if (value != 0 && g->directed) return fail(g, BC_ERR_ARG, "pair_walk needs an undirected graph");
-        if (value != 0) {
-            const int rc = walk_alloc(g);
-            if (rc) return rc;
-        }
         g->d.pair_walk = value != 0 ? 1 : 0;
         return BC_OK;
     }
     if (std::strcmp(name, "walk_cap") == 0) {
         // entries of a row's table in shared memory to use at most (a test knob: a row that
         // needs more takes a table in device memory; same results bit for bit)
-        if (!g->d.walk_rows) return fail(g, BC_ERR_ARG, "walk_cap needs pair_walk on");
+        if (g->directed) return fail(g, BC_ERR_ARG, "walk_cap needs pair_walk on");
         if (value < 0 || value > walk_cap_max(g->d)) return fail(g, BC_ERR_ARG, "walk_cap out of range");
         g->d.walk_cap = value;
         return BC_OK;
@@ -1258,6 +1229,10 @@ struct bc_batch {
     BatchUpd* d_upd = nullptr;
     VEdge* d_entries = nullptr;
     BatchEOp* d_eops = nullptr;
+    int64_t* d_wold = nullptr;       // the entries' weights before their update
+    int32_t* d_wctl = nullptr;       // the walks' counters and lists
+    int2* d_wlist = nullptr;
+    int64_t wrows = 0;
     int64_t* d_eop_off = nullptr;
     int64_t* d_voff = nullptr;
     int64_t* d_coff = nullptr;
@@ -1355,6 +1330,7 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
             return BC_ERR_ARG;
         }
         b->n_max = std::max(b->n_max, g->n);
+        b->wrows += g->n;
     }
     b->dbytes = graphs[0]->dbytes;
     b->L.nsm = graphs[0]->d.nsm;
@@ -1368,7 +1344,8 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     int rc;
     if ((rc = balloc(b, &b->d_devs, count)) || (rc = balloc(b, &b->d_coff, count + 1)) ||
         (rc = balloc(b, &b->d_plans, 4 * ((size_t)count + 1))) || (rc = balloc(b, &b->d_pctr, 1)) ||
-        (rc = balloc(b, &b->d_errs, count))) {
+        (rc = balloc(b, &b->d_errs, count)) || (rc = balloc(b, &b->d_wctl, 8)) ||
+        (rc = balloc(b, &b->d_wlist, 3 * (size_t)b->wrows))) {
         bc_batch_destroy(b);
         return rc;
     }
@@ -1469,7 +1446,9 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     // ---- host records of every round
     std::vector<BatchUpd> upd((size_t)R * G);
     std::vector<VEdge> entries;
+    std::vector<int64_t> wold;
     std::vector<BatchEOp> eops;
+    int32_t pairs = 0;   // the kinds of corrections (BatchLaunch::pairs)
     std::vector<int64_t> eop_off(R + 1, 0);
     std::vector<int64_t> voff((size_t)R * 4 * (G + 1), 0);
     std::vector<std::vector<EOp>> gops(G);
@@ -1484,6 +1463,11 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
             std::vector<EMove> moves;
             std::vector<HArc> arcs;
             bool rebuild = false;
+            for (const VEdge& e : ent) {
+                const ArcMap::Entry* at = gr->amap.find(e.x, vtx[g][r]);
+                wold.push_back(at ? at->w : -1);
+            }
+            if (gr->d.pair_on) pairs |= update_walks(gr->d, (int)ent.size()) ? 2 : 1;
             mirror_update(gr, vtx[g][r], ent, ops, moves, arcs, &rebuild);
             if (rebuild || !moves.empty()) return bfail(b, BC_ERR_CUDA, "internal: E* slack sized too small");
             u.v = vtx[g][r];
@@ -1509,11 +1493,9 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
         }
     }
     // ---- device buffers and launch shape
-    // graphs with pair corrections (undirected, option on): a round launches their kernels
-    int32_t pairs = 0;
-    for (bc_graph* g : b->graphs) pairs |= g->d.pair_on ? 1 : 0;
-    if (pairs != b->L.pairs) {
-        b->L.pairs = pairs;
+    // corrections that no round launches kernels of yet (those of earlier calls stay)
+    if (pairs & ~b->L.pairs) {
+        b->L.pairs |= pairs;
         drop_exec(b);
     }
     int64_t cap_max = 0;
@@ -1544,8 +1526,9 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     }
     if ((int64_t)entries.size() > b->E_cap) {
         bfree(b, b->d_entries);
+        bfree(b, b->d_wold);
         const int64_t c = std::max<int64_t>((int64_t)entries.size() * 2, 1024);
-        if ((rc = balloc(b, &b->d_entries, c))) return rc;
+        if ((rc = balloc(b, &b->d_entries, c)) || (rc = balloc(b, &b->d_wold, c))) return rc;
         b->E_cap = c;
         drop_exec(b);
     }
@@ -1565,9 +1548,11 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
                                b->st));
         CKB(b, cudaMemcpyAsync(b->d_voff, voff.data(), sizeof(int64_t) * voff.size(), cudaMemcpyHostToDevice, b->st));
     }
-    if (!entries.empty())
+    if (!entries.empty()) {
         CKB(b, cudaMemcpyAsync(b->d_entries, entries.data(), sizeof(VEdge) * entries.size(), cudaMemcpyHostToDevice,
                                b->st));
+        CKB(b, cudaMemcpyAsync(b->d_wold, wold.data(), sizeof(int64_t) * wold.size(), cudaMemcpyHostToDevice, b->st));
+    }
     if (!eops.empty())
         CKB(b, cudaMemcpyAsync(b->d_eops, eops.data(), sizeof(BatchEOp) * eops.size(), cudaMemcpyHostToDevice, b->st));
     BatchArgs& a = b->args;
@@ -1586,6 +1571,10 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     a.plan_pr = b->d_plans + 2 * (G + 1);
     a.plan_pw = b->d_plans + 3 * (G + 1);
     a.pctr = b->d_pctr;
+    a.wctl = b->d_wctl;
+    a.wlist = b->d_wlist;
+    a.wrows = b->wrows;
+    a.wold = b->d_wold;
     a.errs = b->d_errs;
     a.ws = b->d_ws;
     a.ws_stride = b->L.ws_stride;

@@ -37,6 +37,10 @@ struct BatchArgs {
     int64_t* plan_acc;        // [G + 1]
     int64_t* plan_pr;         // [G + 1]: changed rows
     int64_t* plan_pw;         // [G + 1]: column-test work
+    int32_t* wctl;            // [8] the walks' counters: rows in the three lists, rows taken from them
+    int2* wlist;              // [3 * wrows] (graph, row): light rows, CTA rows, rows that outgrew their table
+    int64_t wrows;            // rows of all graphs
+    const int64_t* wold;      // weights of `entries` before their update (-1: a new edge)
     int32_t* pctr;            // column-test pieces handed out past the first wave
     int32_t* errs;            // [G] error words after the rounds, read back in one copy
     int32_t* ws;              // accumulation work space, acc_grid * ws_stride ints
@@ -57,8 +61,8 @@ struct BatchLaunch {
                           // turn (item = CTA + k * grid)                (tunable)
     int32_t acc_threads;  // threads of an accumulation CTA: 512, 256 or 128 (more sources
                           // in flight per SM)                           (tunable)
-    int32_t pairs;        // 1: some graph of the batch has pair corrections (0: the round skips
-                          // the pair kernels)
+    int32_t pairs;        // some update of the batch is corrected by [bit 0] the column test [bit 1]
+                          // the walks (a round launches only these kernels)
     int32_t acc_grid;
     AccLayout lay;
     int64_t ws_stride;
@@ -76,6 +80,15 @@ __device__ __forceinline__ int graph_of(const int64_t* off, int G, int64_t j) {
     return lo;
 }
 
+// Whether the update of round r in graph g walks (else its rows are corrected by the column
+// test, if the graph has pair corrections at all).
+__host__ __device__ inline bool update_walks(const Dev& d, int k) {
+    return d.pair_on && d.pair_walk && !d.directed && k <= kWalkMaxEdges;
+}
+__device__ __forceinline__ bool batch_walks_graph(const BatchArgs& b, int r, int g) {
+    return update_walks(b.devs[g], b.upd[(int64_t)r * b.G + g].k);
+}
+
 // The rows a round re-accumulates by Algorithm 1 in graph d: with pair corrections the
 // rows over the target cap, else every changed row.
 __device__ __forceinline__ const int32_t* acc_list(const Dev& d) { return d.pair_on ? d.full_rows : d.acc_rows; }
@@ -87,7 +100,9 @@ void batch_launch_rounds(const BatchArgs& b, const BatchLaunch& L, int rounds, i
 // corrections of round r (k_pair.cu).
 void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* out, int scan_unroll,
                 cudaStream_t st);
-void batch_pair_plan(const BatchArgs& b, const BatchLaunch& L, int dbytes, cudaStream_t st);
+void batch_pair_plan(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st);
+void batch_walk_class(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st);
+void batch_walk_launches(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st);
 void batch_round_end(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st);
 void batch_pair_launches(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st);
 

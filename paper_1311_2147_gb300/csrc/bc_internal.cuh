@@ -118,11 +118,7 @@ struct WalkUpd {
     int32_t x[kWalkMaxEdges];
     int64_t wold[kWalkMaxEdges];
 };
-// Undirected graphs with at least this many vertices walk by default.  The walks are the
-// faster from n = 512 on (per update, column test / walks, int32: n = 512 153 / 76 us, 2048
-// 159 / 98, 4096 245 / 156, 8192 547 / 267; int64, n = 1500: 116 / 96), but a batch uses the
-// column test, and small graphs get the same bits alone and in a batch.
-constexpr int kWalkDefaultMinN = 3072;
+constexpr int kPairPlanBytes = 40;   // of the column test's plan per target (the walks' dense tables lie there too)
 
 // One edge of a vertex update, as staged on the device (matches bc_vedge).
 struct VEdge {
@@ -212,8 +208,9 @@ struct Dev {
     int32_t* acc_rows;   // [n] rows that changed (each list in the order of its atomics: no result
                          // depends on it)
     int32_t* counts;     // [0] rows [1] acc_rows [2] rows2 [3] full rows [4] pair pieces handed out
-                         // [5] rows corrected pair by pair [6] CTAs of k_update_end done; all zero
-                         // between updates
+                         // [5] rows corrected pair by pair [6] CTAs of k_update_end done [8..10] rows
+                         // in the walks' lists (light rows and the two below) [11..13] rows taken
+                         // from them; all zero between updates
     void* fD;            // [n] per-row distance to v after the phase (DT)
     uint64_t* fS;        // [n] per-row path count to v after the phase
     uint64_t* fM;        // [n] per-row multiplier of a tie
@@ -249,11 +246,7 @@ struct Dev {
     int32_t* pair_rows;  // [n] rows corrected pair by pair, most targets first (counts[5])
     int32_t pair_walk;   // 1: pair corrections by DAG walks (k_walk.cu), scratch below
     int64_t walk_cap;    // most entries of a walk's table in shared memory
-    int32_t walk_grid[2];    // CTAs of the walks of light rows, of rows with more targets
-    int32_t* walk_rows;      // [2n] rows with more targets, rows that outgrew their table
-    int32_t* walk_ctl;       // [8] rows in the lists of light rows and these two, and taken from
-                             // each; zero between updates
-    unsigned char* walk_dense;   // [nsm * walk_dense_bytes] tables of rows that outgrow shared memory
+    int32_t* walk_rows;  // [2n] rows with more targets, rows that outgrew their table
     int64_t* bcfix;      // [2n] BC change of the changed rows in this update, per column a
                          // fixed-point pair (units of 2^-24, units of 2^-56); zero between updates
     cudaStream_t st;
@@ -373,8 +366,7 @@ cudaError_t pair_setup();   // kernel attributes (the weights pass's dynamic sha
 // The pair corrections by walks: rows to their classes (k_pair_plan's place), then the walks.
 void launch_walk_class(const Dev& d);
 void launch_walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready);   // ready: when the classes are (NULL: one stream)
-size_t walk_dense_bytes(int n, int dbytes);   // of one table (a table per SM)
-cudaError_t walk_setup(Dev& d);               // launch shapes, kernel attributes, empty tables
+cudaError_t walk_setup();   // kernel attributes
 void launch_update_end(const Dev& d);
 
 // ---- launches (k_accum.cu) ----

@@ -85,7 +85,7 @@ __global__ void kb_vertex_pass(BatchArgs b, int r, int kind) {
 
 // Per-graph work known only on the device, as exclusive prefix offsets over graphs:
 // kind 0: scan items of the phase rows (rows x column chunks); 2: sources to
-// re-accumulate; 3: changed rows; 4: column-test weight (and its piece counter back to
+// re-accumulate; 3: changed rows (and the walks' counters back to zero); 4: column-test weight (and its piece counter back to
 // zero).  One CTA.
 __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, int phase_active, int64_t* out,
                                                 int scan_unroll) {
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
                     v = acc_list_count(d);
                 } else if (kind == 3) {
                     v = d.counts[1];
-                } else if (d.pair_on) {
+                } else if (d.pair_on && !update_walks(d, u.k)) {
                     v = d.pair_w[d.counts[5]];
                 }
             }
@@ -144,6 +144,8 @@ __global__ void __launch_bounds__(1024) kb_plan(BatchArgs b, int r, int kind, in
     if (threadIdx.x == 0) {
         out[G] = s_base;
         if (kind == 4) *b.pctr = 0;
+        if (kind == 3)
+            for (int k = 0; k < 8; ++k) b.wctl[k] = 0;
     }
 }
 
@@ -323,12 +325,14 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     // the changed rows re-accumulated; in graphs with pair corrections only those over the
     // target cap, and the others corrected pair by pair after
     kb_plan<<<1, 1024, 0, st>>>(b, r, 3, 2, b.plan_pr, L.scan_unroll);
-    if (L.pairs) batch_pair_plan(b, L, sizeof(DT), st);
+    if (L.pairs & 1) batch_pair_plan(b, L, r, sizeof(DT), st);
+    if (L.pairs & 2) batch_walk_class(b, L, r, st);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 2, 2, b.plan_acc, L.scan_unroll);
     if (L.acc_threads == 128) batch_accum<DT, 128>(b, L, r, st);
     else if (L.acc_threads == 256) batch_accum<DT, 256>(b, L, r, st);
     else batch_accum<DT, 512>(b, L, r, st);
-    if (L.pairs) batch_pair_launches(b, L, r, sizeof(DT), st);
+    if (L.pairs & 1) batch_pair_launches(b, L, r, sizeof(DT), st);
+    if (L.pairs & 2) batch_walk_launches(b, L, r, sizeof(DT), st);
     batch_round_end(b, L, r, st);
 }
 

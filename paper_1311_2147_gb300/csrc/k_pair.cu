@@ -61,7 +61,7 @@ struct PairTgt {
     ff rold;
     ff rnew;
 };
-static_assert(sizeof(PairTgt) == 40, "the plan is allocated with 40 bytes per target");
+static_assert(sizeof(PairTgt) == kPairPlanBytes, "the plan is allocated with these bytes per target");
 
 template <typename DT>
 struct PairArgs {
@@ -669,7 +669,6 @@ struct EndArgs {
     uint32_t* chg;
     int words;
     int64_t* stats;
-    int32_t* walk_ctl;   // NULL: no walks
     const int32_t* err;
 };
 __global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
@@ -685,9 +684,7 @@ __global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(a.counts + 6, 1) == (int)gridDim.x - 1) {
         dev_update_stats(a.stats, cnt, a.counts[3]);
-        for (int k = 0; k < 8; ++k) a.counts[k] = 0;
-        if (a.walk_ctl)
-            for (int k = 0; k < 8; ++k) a.walk_ctl[k] = 0;
+        for (int k = 0; k < 16; ++k) a.counts[k] = 0;
     }
 }
 
@@ -697,7 +694,7 @@ PairRec pair_rec(const Dev& d) { return make_pair_rec(d); }
 
 void launch_update_end(const Dev& d) {
     EndArgs a{d.n, d.bcfix, d.bc_hi, d.bc_lo, d.acc_rows, d.counts, d.changed, d.pair_on ? d.tcnt : nullptr, d.tlist,
-              d.tcap, d.chg, d.chg_words, d.stats, d.walk_ctl, d.err};
+              d.tcap, d.chg, d.chg_words, d.stats, d.err};
     launch_k(k_update_end, std::min(d.nsm * 4, std::max(1, (d.n + 31) / 32)), 256, 0, d.st, a);
 }
 
@@ -736,17 +733,16 @@ __host__ __device__ inline PairArgs<DT> pair_args(const Dev& d) {
 // the round is in k_batch.cu).  Each kernel runs the single-graph kernel's device
 // function on the concatenated work of all graphs, a task mapped to its graph by binary
 // search over prefix offsets, so a graph's result in a batch is bit-identical to its
-// result alone.  The column test always serves a batch (the DAG walks are for graphs far
-// larger than a batch's).
+// result alone.  Graphs whose update walks are k_walk.cu's.
 
 __device__ __forceinline__ bool batch_pair_graph(const BatchArgs& b, int r, int g) {
     const Dev& d = b.devs[g];
-    return d.pair_on && b.upd[(int64_t)r * b.G + g].present && *d.err == 0;
+    return d.pair_on && b.upd[(int64_t)r * b.G + g].present && *d.err == 0 && !batch_walks_graph(b, r, g);
 }
 
 // A warp per listed row of every graph (k_pair_plan); plan_pr offsets the rows.
 template <typename DT>
-__global__ void __launch_bounds__(kPlanThreads) kb_pair_plan(BatchArgs b) {
+__global__ void __launch_bounds__(kPlanThreads) kb_pair_plan(BatchArgs b, int r) {
     __shared__ int32_t s_val[kPlanThreads / 32][kPairCap];
     const int G = b.G;
     const int64_t total = b.plan_pr[G];
@@ -755,7 +751,7 @@ __global__ void __launch_bounds__(kPlanThreads) kb_pair_plan(BatchArgs b) {
     for (int64_t j = (int64_t)blockIdx.x * (kPlanThreads / 32) + wib; j < total; j += nw) {
         const int g = graph_of(b.plan_pr, G, j);
         const Dev& d = b.devs[g];
-        if (!d.pair_on) continue;
+        if (!d.pair_on || batch_walks_graph(b, r, g)) continue;
         const PairArgs<DT> a = pair_args<DT>(d);
         dev_pair_plan_row<DT>(a, d.acc_rows[j - b.plan_pr[g]], s_val[wib]);
     }
@@ -908,9 +904,9 @@ __global__ void kb_update_stats(BatchArgs b, int r) {
     }
 }
 
-void batch_pair_plan(const BatchArgs& b, const BatchLaunch& L, int dbytes, cudaStream_t st) {
-    if (dbytes == 4) kb_pair_plan<int32_t><<<L.nsm * 8, kPlanThreads, 0, st>>>(b);
-    else kb_pair_plan<int64_t><<<L.nsm * 8, kPlanThreads, 0, st>>>(b);
+void batch_pair_plan(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st) {
+    if (dbytes == 4) kb_pair_plan<int32_t><<<L.nsm * 8, kPlanThreads, 0, st>>>(b, r);
+    else kb_pair_plan<int64_t><<<L.nsm * 8, kPlanThreads, 0, st>>>(b, r);
 }
 
 void batch_round_end(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st) {

@@ -39,8 +39,14 @@
 // 443; 16 updates at n = 16384 8.6 ms against 11.4.  Of that: one walk for both states
 // 560 -> 446 us an update at n = 16384 (a quarter fewer arcs, half the entries); two warps
 // a CTA with 64 registers instead of 48 and more warps, 478 -> 436.
+//
+// Every undirected graph walks by default, alone and in a batch.  Per update alone, column
+// test / walks: n = 512 153 / 79 us, 1024 168 / 89, 2048 159 / 104, 4096 246 / 157, 8192
+// 547 / 271; 64-bit distances, n = 1500: 116 / 97.  A batch of 96 graphs of 32..512 vertices,
+// 8 rounds: the column test's kernels 3.4 ms, the walks' 1.0.
 #include <algorithm>
 
+#include "bc_batch.cuh"
 #include "bc_device.cuh"
 
 namespace bcg {
@@ -51,9 +57,11 @@ constexpr int kNone = -1;                 // the end of a list of DAG arcs
 constexpr int kManyArcs = 48;               // vertices with as many are walked one by one
 constexpr int kLightTargets = 16;         // rows with more changed targets: a CTA each
 
+// The state of a graph as the walks read and write it.
 template <typename DT>
-struct WalkArgs {
+struct WalkGraph {
     int n, ld, tcap;
+    int cap;               // most entries of a shared-memory table to use
     const DT* D;
     const uint64_t* S;
     const DT* oD;          // values before the update, valid at the changed pairs
@@ -66,17 +74,58 @@ struct WalkArgs {
     const int64_t* e_w64;
     ff* Dl;
     int64_t* bcfix;
+    int64_t* stats;        // [8] rows and [9] pairs corrected [10] pairs walked [11] vertices found [12] arcs examined
+    unsigned char* dense;  // dense_tables(n) tables
+};
+template <typename DT>
+__host__ __device__ __forceinline__ WalkGraph<DT> walk_graph(const Dev& d) {
+    WalkGraph<DT> a;
+    a.n = d.n;
+    a.ld = d.ld;
+    a.tcap = d.tcap;
+    a.cap = d.walk_cap < (1 << 20) ? (int)d.walk_cap : 1 << 20;
+    a.D = (const DT*)d.D;
+    a.S = d.S;
+    a.oD = (const DT*)d.oldD;
+    a.oS = d.oldS;
+    a.tcnt = d.tcnt;
+    a.tlist = d.tlist;
+    a.e_off = d.e_off;
+    a.e_len = d.e_len;
+    a.e_arc = d.e_arc;
+    a.e_w64 = d.e_w64;
+    a.Dl = d.Dl;
+    a.bcfix = d.bcfix;
+    a.stats = d.stats;
+    a.dense = reinterpret_cast<unsigned char*>(d.plan);
+    return a;
+}
+
+// An update's edges in a batch (alone: WalkUpd).
+struct BatchWalkUpd {
+    int32_t v, k;
+    const VEdge* ent;
+    const int64_t* old_w;
+    __device__ __forceinline__ int32_t x(int u) const { return ent[u].x; }
+    __device__ __forceinline__ int64_t wold(int u) const { return old_w[u]; }
+};
+struct OneWalkUpd {
+    int32_t v, k;
+    const WalkUpd& upd;
+    __device__ __forceinline__ int32_t x(int u) const { return upd.x[u]; }
+    __device__ __forceinline__ int64_t wold(int u) const { return upd.wold[u]; }
+};
+
+template <typename DT>
+struct WalkArgs {
+    WalkGraph<DT> g;
     const int32_t* rows;   // rows that changed
     const int32_t* count;
     int32_t* full_rows;    // rows with more targets than tcap
     int32_t* full_count;
     int32_t* list[3];      // light rows, CTA rows, rows that outgrew their table
     int32_t* ctl;          // [0..2] rows in the lists [3..5] rows taken past each warp's or CTA's first
-    int64_t* stats;        // [8] rows and [9] pairs corrected [10] pairs walked [11] vertices found [12] arcs examined
     const int32_t* err;
-    int cap;               // most entries of a shared-memory table to use
-    unsigned char* dense;  // per CTA of the last launch
-    int64_t dense_stride;
     WalkUpd upd;
 };
 
@@ -90,11 +139,11 @@ __global__ void __launch_bounds__(256) k_walk_class(const __grid_constant__ Walk
     for (int i0 = blockIdx.x * blockDim.x; i0 < cnt; i0 += gridDim.x * blockDim.x) {   // warp-uniform
         const int i = i0 + threadIdx.x;
         const int s = i < cnt ? a.rows[i] : 0;
-        const int T = i < cnt ? a.tcnt[s] : 0;
-        append_row(T > a.tcap, s, a.full_rows, a.full_count);
-        append_row(T > 0 && T <= min(kLightTargets, a.tcap), s, a.list[0], a.ctl + 0);
-        append_row(T > kLightTargets && T <= a.tcap, s, a.list[1], a.ctl + 1);
-        if (T <= a.tcap) {
+        const int T = i < cnt ? a.g.tcnt[s] : 0;
+        append_row(T > a.g.tcap, s, a.full_rows, a.full_count);
+        append_row(T > 0 && T <= min(kLightTargets, a.g.tcap), s, a.list[0], a.ctl + 0);
+        append_row(T > kLightTargets && T <= a.g.tcap, s, a.list[1], a.ctl + 1);
+        if (T <= a.g.tcap) {
             rows += T > 0;
             tgts += T;
         }
@@ -102,9 +151,54 @@ __global__ void __launch_bounds__(256) k_walk_class(const __grid_constant__ Walk
     rows = __reduce_add_sync(FULL, rows);
     tgts = __reduce_add_sync(FULL, tgts);
     if ((threadIdx.x & 31) == 0 && rows) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 8), (unsigned long long)rows);
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 9), (unsigned long long)tgts);
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.stats + 10), (unsigned long long)tgts);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.g.stats + 8), (unsigned long long)rows);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.g.stats + 9), (unsigned long long)tgts);
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.g.stats + 10), (unsigned long long)tgts);
+    }
+}
+
+// The same over a batch: the graphs whose update of round r walks.
+__device__ __forceinline__ BatchWalkUpd batch_upd(const BatchArgs& b, int r, int g) {
+    const BatchUpd& u = b.upd[(int64_t)r * b.G + g];
+    return BatchWalkUpd{u.v, u.k, b.entries + u.first, b.wold + u.first};
+}
+__device__ __forceinline__ void append_pair(bool want, int2 gs, int2* list, int32_t* count) {
+    const unsigned m = __ballot_sync(FULL, want);
+    if (!m) return;
+    const int lane = threadIdx.x & 31;
+    int p = 0;
+    if (lane == 0) p = atomicAdd(count, __popc(m));
+    p = __shfl_sync(FULL, p, 0) + __popc(m & ((1u << lane) - 1u));
+    if (want) list[p] = gs;
+}
+__global__ void __launch_bounds__(256) kb_walk_class(BatchArgs b, int r) {
+    const int64_t total = b.plan_pr[b.G];
+    for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x; j0 < total; j0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = j0 + threadIdx.x;
+        int g = -1, s = 0, T = 0, cap = 0;
+        if (j < total) {
+            g = graph_of(b.plan_pr, b.G, j);
+            const Dev& d = b.devs[g];
+            if (batch_walks_graph(b, r, g)) {
+                s = d.acc_rows[j - b.plan_pr[g]];
+                T = d.tcnt[s];
+                cap = d.tcap;
+                if (T > cap) d.full_rows[atomicAdd(d.counts + 3, 1)] = s;
+            }
+        }
+        const int2 gs = make_int2(g, s);
+        append_pair(T > 0 && T <= min(kLightTargets, cap), gs, b.wlist, b.wctl + 0);
+        append_pair(T > kLightTargets && T <= cap, gs, b.wlist + b.wrows, b.wctl + 1);
+        // the counters of a graph, once per warp
+        const unsigned peers = __match_any_sync(FULL, g);
+        const int rows = __popc(__ballot_sync(FULL, T > 0 && T <= cap) & peers);
+        const int tgts = __reduce_add_sync(peers, T <= cap ? T : 0);
+        if (rows && (int)(threadIdx.x & 31) == __ffs(peers) - 1) {
+            unsigned long long* st = reinterpret_cast<unsigned long long*>(b.devs[g].stats);
+            atomicAdd(st + 8, (unsigned long long)rows);
+            atomicAdd(st + 9, (unsigned long long)tgts);
+            atomicAdd(st + 10, (unsigned long long)tgts);
+        }
     }
 }
 
@@ -115,7 +209,7 @@ struct WalkShared {
     int nodes;   // DAG arcs found
     int ready;   // entries whose children are done
     int over;    // the table is too small for the row
-    int row;
+    int row;     // the next row
 };
 
 // A row's table.  An entry's key is 2 * vertex + 1, a target's old entry's 2 * vertex; -1
@@ -194,10 +288,12 @@ constexpr long long kOne = 1ll << 55;
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // GS threads work on a row: a warp, or the CTA.  H: entries of the hash table (0: dense,
-// entry = key); NODES: room for DAG arcs (dense: none are kept, the arcs are read again).
-template <typename DT, typename IX, int GS, int H, int NODES>
+// entry = vertex, or n + j for the j-th target's old one, which the vertex's head names);
+// NODES: room for DAG arcs (dense: none are kept, the arcs are read again).
+template <typename DT, typename UPD, typename IX, int GS, int H, int NODES>
 struct RowWalk {
-    const WalkArgs<DT>& a;
+    const WalkGraph<DT>& a;
+    const UPD& upd;
     const WalkTable<DT, IX>& t;
     WalkShared& sh;
     int limit;   // entries from which the hash table counts as too small
@@ -217,7 +313,8 @@ struct RowWalk {
     // past the limit every thread makes at most one more (see over()).
     __device__ __forceinline__ int find(int k) const {
         if constexpr (H == 0) {
-            return *(volatile int32_t*)(t.key + k) == k ? k : -1;
+            if (!(k & 1)) return *(volatile int32_t*)(t.head + (k >> 1));
+            return *(volatile int32_t*)(t.key + (k >> 1)) == k ? k >> 1 : -1;
         } else {
             for (int e = home(k);; e = (e + 1) & (H - 1)) {
                 const int c = *(volatile int32_t*)(t.key + e);
@@ -226,14 +323,15 @@ struct RowWalk {
             }
         }
     }
-    // The entry of key k, made if there is none.
-    __device__ __forceinline__ int insert(int k, DT d, bool count, bool* made) const {
-        for (int e = H == 0 ? k : home(k);; e = (e + 1) & (H - 1)) {
+    // The entry of key k (the j-th target's old one), made if there is none.
+    __device__ __forceinline__ int insert(int k, int j, DT d, bool count, bool* made) const {
+        for (int e = H != 0 ? home(k) : (k & 1) ? k >> 1 : a.n + j;; e = (e + 1) & (H - 1)) {
             const int c = atomicCAS(t.key + e, -1, k);
             if (c != -1 && c != k) continue;
             *made = c == -1;
             if (c == -1) {
                 t.d[e] = d;
+                if (H == 0 && !(k & 1)) t.head[k >> 1] = e;
                 if (count) {
                     const int u = atomicAdd(&sh.seen, 1);
                     t.seen[u] = (IX)e;
@@ -250,10 +348,10 @@ struct RowWalk {
 
     // The old weight of an arc between x and y that weighs w now (negative: it did not exist).
     __device__ __forceinline__ DT old_weight(DT w, int x, int y) const {
-        if (y == a.upd.v || x == a.upd.v) {
-            const int o = y == a.upd.v ? x : y;
-            for (int u = 0; u < a.upd.k; ++u)
-                if (a.upd.x[u] == o) w = (DT)min(a.upd.wold[u], Inf<DT>::v);
+        if (y == upd.v || x == upd.v) {
+            const int o = y == upd.v ? x : y;
+            for (int u = 0; u < upd.k; ++u)
+                if (upd.x(u) == o) w = (DT)min(upd.wold(u), Inf<DT>::v);
         }
         return w;
     }
@@ -270,7 +368,7 @@ struct RowWalk {
                 if (sg == 0) d = (DT)Inf<DT>::v;
                 bool made;
                 const bool path = (int64_t)d != Inf<DT>::v;
-                const int e = insert(2 * x + st, d, path, &made);
+                const int e = insert(2 * x + st, j >> 1, d, path, &made);
                 t.sig[e] = sg;
                 if (path) {
                     t.acc[e] = (unsigned long long)(st ? kOne : -kOne);
@@ -352,7 +450,7 @@ struct RowWalk {
                 if (is) {
                     if (f < 0) {
                         bool made;
-                        f = insert(k, want, true, &made);
+                        f = insert(k, 0, want, true, &made);
                         if (made) {
                             prefetch_l2(a.S + rs + x[u]);
                             prefetch_l2(a.Dl + rs + x[u]);
@@ -475,7 +573,7 @@ struct RowWalk {
                 }
             } else {   // a warp per entry; the arcs are read again
                 for (int i = lo + (rank() >> 5); i < hi; i += GS / 32) {
-                    const int e = t.ready[i], y = e >> 1, st = e & 1;
+                    const int e = t.ready[i], y = t.key[e] >> 1, st = t.key[e] & 1;
                     const int off = a.e_off[y], len = a.e_len[y];
                     const DT dy = t.d[e];
                     Share r;
@@ -537,26 +635,36 @@ struct RowWalk {
         } else {
             const int m = *(volatile int*)&sh.seen;
             for (int i = rank(); i < m; i += GS) t.free_entry(t.seen[i]);
-            for (int j = rank(); j < 2 * T; j += GS) t.free_entry(2 * a.tlist[(size_t)s * a.tcap + (j >> 1)] + (j & 1));
+            for (int j = rank(); j < T; j += GS) {
+                t.free_entry(a.tlist[(size_t)s * a.tcap + j]);
+                t.free_entry(a.n + j);
+            }
         }
         sync();
         return ok;
     }
 };
 
-__device__ __forceinline__ void walk_totals(int64_t* stats, const unsigned long long* totals) {
-    if (totals[0]) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 11), totals[0]);
-    if (totals[1]) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 12), totals[1]);
-}
-
 // Light rows: a warp each.
-constexpr int kLightWarps = 2, kLightH = 128, kLightLimit = kLightH - 33, kLightNodes = 192;
+constexpr int kLightPerSm = 16, kLightWarps = 2, kLightH = 128, kLightLimit = kLightH - 33, kLightNodes = 192;
 template <typename DT> using LightTable = WalkTable<DT, uint16_t>;
 template <typename DT>
 __host__ __device__ constexpr size_t light_bytes() { return LightTable<DT>::bytes(kLightH, kLightNodes); }
 
+template <typename DT, typename UPD>
+__device__ __forceinline__ bool light_row(const WalkGraph<DT>& g, const UPD& upd, const LightTable<DT>& t,
+                                          WalkShared& sh, int s, unsigned long long* totals) {
+    const RowWalk<DT, UPD, uint16_t, 32, kLightH, kLightNodes> w{g, upd, t, sh, min(g.cap, kLightLimit), s, g.tcnt[s], totals};
+    return w.run();
+}
+__device__ __forceinline__ void walk_totals(int64_t* stats, unsigned long long* totals) {
+    if (totals[0]) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 11), totals[0]);
+    if (totals[1]) atomicAdd(reinterpret_cast<unsigned long long*>(stats + 12), totals[1]);
+    totals[0] = totals[1] = 0ull;
+}
+
 template <typename DT>
-__global__ void __launch_bounds__(kLightWarps * 32, 16) k_walk_light(const __grid_constant__ WalkArgs<DT> a) {
+__global__ void __launch_bounds__(kLightWarps * 32, kLightPerSm) k_walk_light(const __grid_constant__ WalkArgs<DT> a) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char wsm[];
     __shared__ WalkShared s_sh[kLightWarps];
@@ -565,18 +673,50 @@ __global__ void __launch_bounds__(kLightWarps * 32, 16) k_walk_light(const __gri
     const LightTable<DT> t(wsm + wib * light_bytes<DT>(), kLightH, kLightNodes);
     t.free_all(kLightH, lane, 32);
     __syncwarp();
-    const int limit = min(a.cap, kLightLimit);
+    const OneWalkUpd upd{a.upd.v, a.upd.k, a.upd};
     const int cnt = a.ctl[0], nw = gridDim.x * kLightWarps;
     unsigned long long totals[2] = {0ull, 0ull};
     for (int i = blockIdx.x * kLightWarps + wib; i < cnt;) {
         int nx = 0;   // the next row's number arrives while this one is worked on
         if (lane == 0) nx = nw + atomicAdd(a.ctl + 3, 1);
         const int s = a.list[0][i];
-        const RowWalk<DT, uint16_t, 32, kLightH, kLightNodes> w{a, t, s_sh[wib], limit, s, a.tcnt[s], totals};
-        if (!w.run() && lane == 0) a.list[2][atomicAdd(a.ctl + 2, 1)] = s;
+        if (!light_row(a.g, upd, t, s_sh[wib], s, totals) && lane == 0) a.list[2][atomicAdd(a.ctl + 2, 1)] = s;
         i = __shfl_sync(FULL, nx, 0);
     }
-    if (lane == 0) walk_totals(a.stats, totals);
+    if (lane == 0) walk_totals(a.g.stats, totals);
+}
+
+// The same over a batch: rows are (graph, row) pairs, a warp's graph is in shared memory.
+template <typename DT>
+__global__ void __launch_bounds__(kLightWarps * 32, kLightPerSm) kb_walk_light(BatchArgs b, int r) {
+    extern __shared__ __align__(16) unsigned char wsm[];
+    __shared__ WalkShared s_sh[kLightWarps];
+    __shared__ WalkGraph<DT> s_g[kLightWarps];
+    __shared__ BatchWalkUpd s_u[kLightWarps];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const LightTable<DT> t(wsm + wib * light_bytes<DT>(), kLightH, kLightNodes);
+    t.free_all(kLightH, lane, 32);
+    const int cnt = b.wctl[0], nw = gridDim.x * kLightWarps;
+    unsigned long long totals[2] = {0ull, 0ull};
+    int cg = -1;
+    for (int i = blockIdx.x * kLightWarps + wib; i < cnt;) {
+        int nx = 0;
+        if (lane == 0) nx = nw + atomicAdd(b.wctl + 3, 1);
+        const int2 gs = b.wlist[i];
+        if (gs.x != cg) {
+            if (lane == 0) {
+                if (cg >= 0) walk_totals(s_g[wib].stats, totals);
+                s_g[wib] = walk_graph<DT>(b.devs[gs.x]);
+                s_u[wib] = batch_upd(b, r, gs.x);
+            }
+            cg = gs.x;
+        }
+        __syncwarp();
+        if (!light_row(s_g[wib], s_u[wib], t, s_sh[wib], gs.y, totals) && lane == 0)
+            b.wlist[2 * b.wrows + atomicAdd(b.wctl + 2, 1)] = gs;
+        i = __shfl_sync(FULL, nx, 0);
+    }
+    if (lane == 0 && cg >= 0) walk_totals(s_g[wib].stats, totals);
 }
 
 // Rows with more targets (RETRY: rows that outgrew their table, in the dense arrays if
@@ -592,6 +732,30 @@ struct Cta {
     __host__ __device__ static constexpr size_t bytes() { return WalkTable<DT, uint16_t>::bytes(h, nodes); }
 };
 
+// A dense table: the vertices, then the targets' old entries.
+__host__ __device__ constexpr int dense_entries(int n) { return n + (n < kPairCap ? n : kPairCap); }
+
+template <typename DT, bool RETRY, typename UPD>
+__device__ __forceinline__ bool cta_row(const WalkGraph<DT>& g, const UPD& upd, const WalkTable<DT, uint16_t>& t,
+                                        WalkShared& sh, int s, unsigned long long* totals, bool& dense_free) {
+    using C = Cta<RETRY>;
+    const int T = g.tcnt[s];
+    const RowWalk<DT, UPD, uint16_t, C::threads, C::h, C::nodes> w{g, upd, t, sh, min(g.cap, C::limit), s, T, totals};
+    if (w.run()) return true;
+    if constexpr (RETRY) {
+        const int m = dense_entries(g.n);
+        const WalkTable<DT, int32_t> dt(g.dense + blockIdx.x * WalkTable<DT, int32_t>::bytes(m, 0), m, 0);
+        if (!dense_free) {   // (what was there before: another update's plan)
+            for (int e = threadIdx.x; e < m; e += C::threads) dt.free_entry(e);
+            __syncthreads();
+        }
+        dense_free = true;
+        const RowWalk<DT, UPD, int32_t, C::threads, 0, 0> dw{g, upd, dt, sh, 0, s, T, totals};
+        return dw.run();
+    }
+    return false;
+}
+
 template <typename DT, bool RETRY>
 __global__ void __launch_bounds__(Cta<RETRY>::threads, Cta<RETRY>::per_sm) k_walk_cta(const __grid_constant__ WalkArgs<DT> a) {
     pdl_enter();
@@ -604,55 +768,67 @@ __global__ void __launch_bounds__(Cta<RETRY>::threads, Cta<RETRY>::per_sm) k_wal
     if ((int)blockIdx.x >= cnt) return;
     const WalkTable<DT, uint16_t> t(wsm, C::h, C::nodes);
     t.free_all(C::h, threadIdx.x, C::threads);
-    const int limit = min(a.cap, C::limit);
+    const OneWalkUpd upd{a.upd.v, a.upd.k, a.upd};
     unsigned long long totals[2] = {0ull, 0ull};
+    bool dense_free = false;
     for (int i = blockIdx.x; i < cnt;) {
         int nx = 0;
         if (threadIdx.x == 0) nx = (int)gridDim.x + atomicAdd(a.ctl + 3 + L, 1);
         const int s = a.list[L][i];
-        const RowWalk<DT, uint16_t, C::threads, C::h, C::nodes> w{a, t, sh, limit, s, a.tcnt[s], totals};
-        if (!w.run()) {
-            if (RETRY) {
-                const WalkTable<DT, int32_t> dt(a.dense + (size_t)blockIdx.x * a.dense_stride, 2 * (size_t)a.n, 0);
-                const RowWalk<DT, int32_t, C::threads, 0, 0> dw{a, dt, sh, 0, s, a.tcnt[s], totals};
-                dw.run();
-            } else if (threadIdx.x == 0) {
-                a.list[2][atomicAdd(a.ctl + 2, 1)] = s;
-            }
-        }
+        if (!cta_row<DT, RETRY>(a.g, upd, t, sh, s, totals, dense_free) && threadIdx.x == 0)
+            a.list[2][atomicAdd(a.ctl + 2, 1)] = s;
         if (threadIdx.x == 0) sh.row = nx;
         __syncthreads();
         i = sh.row;
         __syncthreads();
     }
-    if ((threadIdx.x & 31) == 0) walk_totals(a.stats, totals);
+    if ((threadIdx.x & 31) == 0) walk_totals(a.g.stats, totals);
 }
 
-// The dense arrays start free.
-template <typename DT>
-__global__ void k_walk_dense_init(unsigned char* dense, int64_t stride, int n) {
-    const WalkTable<DT, int32_t> t(dense + (size_t)blockIdx.x * stride, 2 * (size_t)n, 0);
-    for (int e = threadIdx.x; e < 2 * n; e += blockDim.x) t.free_entry(e);
+template <typename DT, bool RETRY>
+__global__ void __launch_bounds__(Cta<RETRY>::threads, Cta<RETRY>::per_sm) kb_walk_cta(BatchArgs b, int r) {
+    extern __shared__ __align__(16) unsigned char wsm[];
+    __shared__ WalkShared sh;
+    __shared__ WalkGraph<DT> s_g;
+    __shared__ BatchWalkUpd s_u;
+    using C = Cta<RETRY>;
+    constexpr int L = RETRY ? 2 : 1;
+    const int cnt = b.wctl[L];
+    if ((int)blockIdx.x >= cnt) return;
+    const WalkTable<DT, uint16_t> t(wsm, C::h, C::nodes);
+    t.free_all(C::h, threadIdx.x, C::threads);
+    unsigned long long totals[2] = {0ull, 0ull};
+    int cg = -1;
+    bool dense_free = false;
+    for (int i = blockIdx.x; i < cnt;) {
+        int nx = 0;
+        if (threadIdx.x == 0) nx = (int)gridDim.x + atomicAdd(b.wctl + 3 + L, 1);
+        const int2 gs = b.wlist[L * b.wrows + i];
+        if (gs.x != cg) {
+            if (cg >= 0 && (threadIdx.x & 31) == 0) walk_totals(s_g.stats, totals);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                s_g = walk_graph<DT>(b.devs[gs.x]);
+                s_u = batch_upd(b, r, gs.x);
+            }
+            cg = gs.x;
+            dense_free = false;
+        }
+        __syncthreads();
+        if (!cta_row<DT, RETRY>(s_g, s_u, t, sh, gs.y, totals, dense_free) && threadIdx.x == 0)
+            b.wlist[2 * b.wrows + atomicAdd(b.wctl + 2, 1)] = gs;
+        if (threadIdx.x == 0) sh.row = nx;
+        __syncthreads();
+        i = sh.row;
+        __syncthreads();
+    }
+    if (cg >= 0 && (threadIdx.x & 31) == 0) walk_totals(s_g.stats, totals);
 }
 
 template <typename DT>
 WalkArgs<DT> walk_args(const Dev& d) {
     WalkArgs<DT> a{};
-    a.n = d.n;
-    a.ld = d.ld;
-    a.tcap = d.tcap;
-    a.D = (const DT*)d.D;
-    a.S = d.S;
-    a.oD = (const DT*)d.oldD;
-    a.oS = d.oldS;
-    a.tcnt = d.tcnt;
-    a.tlist = d.tlist;
-    a.e_off = d.e_off;
-    a.e_len = d.e_len;
-    a.e_arc = d.e_arc;
-    a.e_w64 = d.e_w64;
-    a.Dl = d.Dl;
-    a.bcfix = d.bcfix;
+    a.g = walk_graph<DT>(d);
     a.rows = d.acc_rows;
     a.count = d.counts + 1;
     a.full_rows = d.full_rows;
@@ -660,20 +836,21 @@ WalkArgs<DT> walk_args(const Dev& d) {
     a.list[0] = d.pair_rows;
     a.list[1] = d.walk_rows;
     a.list[2] = d.walk_rows + d.n;
-    a.ctl = d.walk_ctl;
-    a.stats = d.stats;
+    a.ctl = d.counts + 8;
     a.err = d.err;
-    a.cap = (int)std::min<int64_t>(d.walk_cap, 1 << 20);
-    a.dense = d.walk_dense;
-    a.dense_stride = (int64_t)walk_dense_bytes(d.n, d.dbytes);
     return a;
 }
 
-int resident(const void* f, int threads, size_t smem, int nsm) {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, f, threads, smem) != cudaSuccess || b < 1) b = 1;
-    return b * nsm;
+// The dense tables take the place of the column test's plan, which an update that walks has
+// no use for: as many of them as fit.
+template <typename DT>
+int dense_tables(int n) {
+    return (int)((size_t)n * kPairCap * kPairPlanBytes / WalkTable<DT, int32_t>::bytes(dense_entries(n), 0));
 }
+// The least of dense_tables (n = 1, 64-bit distances; a batch's graphs have any n).
+constexpr int kDenseTablesMin =
+    (int)((size_t)kPairCap * kPairPlanBytes / WalkTable<int64_t, int32_t>::bytes(dense_entries(1), 0));
+static_assert(kDenseTablesMin >= 48, "CTAs for the rows that outgrow shared memory");
 
 template <typename DT>
 void walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready) {
@@ -683,31 +860,42 @@ void walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready) {
     // their table
     const cudaStream_t sr = ready ? d.st3 : d.st;
     if (ready) cudaStreamWaitEvent(sr, ready, 0);
-    launch_k(k_walk_cta<DT, false>, d.walk_grid[1], Cta<false>::threads, Cta<false>::bytes<DT>(), sr, a);
+    launch_k(k_walk_cta<DT, false>, d.nsm * Cta<false>::per_sm, Cta<false>::threads, Cta<false>::bytes<DT>(), sr, a);
     if (ready) cudaEventRecord(d.ev3_join, sr);
-    launch_k(k_walk_light<DT>, d.walk_grid[0], kLightWarps * 32, kLightWarps * light_bytes<DT>(), d.st, a);
+    launch_k(k_walk_light<DT>, d.nsm * kLightPerSm, kLightWarps * 32, kLightWarps * light_bytes<DT>(), d.st, a);
     if (ready) cudaStreamWaitEvent(d.st, d.ev3_join, 0);
-    launch_k(k_walk_cta<DT, true>, d.nsm, Cta<true>::threads, Cta<true>::bytes<DT>(), d.st, a);
+    launch_k(k_walk_cta<DT, true>, std::min(d.nsm, dense_tables<DT>(d.n)), Cta<true>::threads, Cta<true>::bytes<DT>(), d.st, a);
 }
 
 template <typename DT>
-cudaError_t setup(Dev& d) {
-    cudaError_t e = cudaFuncSetAttribute(k_walk_cta<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)Cta<true>::bytes<DT>());
-    if (e != cudaSuccess) return e;
-    d.walk_grid[0] = resident((const void*)k_walk_light<DT>, kLightWarps * 32, kLightWarps * light_bytes<DT>(), d.nsm);
-    d.walk_grid[1] = resident((const void*)k_walk_cta<DT, false>, Cta<false>::threads, Cta<false>::bytes<DT>(), d.nsm);
-    k_walk_dense_init<DT><<<d.nsm, 256, 0, d.st>>>(d.walk_dense, (int64_t)walk_dense_bytes(d.n, d.dbytes), d.n);
-    return cudaGetLastError();
+cudaError_t setup() {
+    const int smem = (int)Cta<true>::bytes<DT>();
+    cudaError_t e = cudaFuncSetAttribute(k_walk_cta<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_walk_cta<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    return e;
+}
+
+template <typename DT>
+void batch_walks(const BatchArgs& b, int nsm, int r, cudaStream_t st) {
+    kb_walk_cta<DT, false><<<nsm * Cta<false>::per_sm, Cta<false>::threads, Cta<false>::bytes<DT>(), st>>>(b, r);
+    kb_walk_light<DT><<<nsm * kLightPerSm, kLightWarps * 32, kLightWarps * light_bytes<DT>(), st>>>(b, r);
+    kb_walk_cta<DT, true><<<std::min(nsm, kDenseTablesMin), Cta<true>::threads, Cta<true>::bytes<DT>(), st>>>(b, r);
 }
 
 }  // namespace
 
-size_t walk_dense_bytes(int n, int dbytes) {
-    return dbytes == 4 ? WalkTable<int32_t, int32_t>::bytes(2 * (size_t)n, 0)
-                       : WalkTable<int64_t, int32_t>::bytes(2 * (size_t)n, 0);
+cudaError_t walk_setup() {
+    const cudaError_t e = setup<int32_t>();
+    return e == cudaSuccess ? setup<int64_t>() : e;
 }
-cudaError_t walk_setup(Dev& d) { return d.dbytes == 4 ? setup<int32_t>(d) : setup<int64_t>(d); }
+
+void batch_walk_class(const BatchArgs& b, const BatchLaunch& L, int r, cudaStream_t st) {
+    kb_walk_class<<<L.nsm * 8, 256, 0, st>>>(b, r);
+}
+void batch_walk_launches(const BatchArgs& b, const BatchLaunch& L, int r, int dbytes, cudaStream_t st) {
+    if (dbytes == 4) batch_walks<int32_t>(b, L.nsm, r, st);
+    else batch_walks<int64_t>(b, L.nsm, r, st);
+}
 
 void launch_walk_class(const Dev& d) {
     const int grid = std::max(1, std::min((d.n + 255) / 256, d.nsm * 4));

@@ -54,7 +54,7 @@ namespace bcg {
 namespace {
 
 constexpr int kNone = -1;                 // the end of a list of DAG arcs
-constexpr int kManyArcs = 48;               // vertices with as many are walked one by one
+constexpr int kManyArcs = 96;               // vertices with as many are walked one by one
 constexpr int kLightTargets = 16;         // rows with more changed targets: a CTA each
 
 // The state of a graph as the walks read and write it.
@@ -392,7 +392,7 @@ struct RowWalk {
             dy = __shfl_sync(FULL, dy, one);
             off = __shfl_sync(FULL, off, one);
         }
-        constexpr int U = ONE ? 4 : 2;
+        constexpr int U = ONE ? 4 : 1;
         for (int k0 = 0; k0 < tot; k0 += 32 * U) {
             int ej[U], x[U];
             DT dyj[U], dx[U], w[U];
@@ -726,8 +726,8 @@ __global__ void __launch_bounds__(kLightWarps * 32, kLightPerSm) kb_walk_light(B
 template <bool RETRY>
 struct Cta {
     static_assert(4 * kPairCap <= 512 && 2 * kLightTargets < kLightH, "room for the targets");
-    static constexpr int threads = RETRY ? 512 : 128, h = RETRY ? 2048 : 512, limit = h - threads - 1,
-                         nodes = RETRY ? 3072 : 768, per_sm = RETRY ? 1 : 8;
+    static constexpr int threads = RETRY ? 512 : 256, h = RETRY ? 2048 : 1024, limit = h - threads - 1,
+                         nodes = RETRY ? 3072 : 1536, per_sm = RETRY ? 1 : 4;
     template <typename DT>
     __host__ __device__ static constexpr size_t bytes() { return WalkTable<DT, uint16_t>::bytes(h, nodes); }
 };

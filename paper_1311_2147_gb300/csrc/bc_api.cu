@@ -1351,6 +1351,12 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     }
     cudaEventCreate(&b->e0);
     cudaEventCreate(&b->e1);
+    if (cudaStreamCreateWithFlags(&b->L.side, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->L.fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&b->L.join, cudaEventDisableTiming) != cudaSuccess) {
+        bc_batch_destroy(b);
+        return BC_ERR_CUDA;
+    }
     std::vector<int64_t> coff(count + 1, 0);
     for (int32_t i = 0; i < count; ++i) coff[i + 1] = coff[i] + graphs[i]->n;
     if (cudaMemcpy(b->d_coff, coff.data(), sizeof(int64_t) * (count + 1), cudaMemcpyHostToDevice) != cudaSuccess) {
@@ -1627,6 +1633,9 @@ void bc_batch_destroy(bc_batch* b) {
     for (void* p : b->allocs) cudaFree(p);
     if (b->e0) cudaEventDestroy(b->e0);
     if (b->e1) cudaEventDestroy(b->e1);
+    if (b->L.side) cudaStreamDestroy(b->L.side);
+    if (b->L.fork) cudaEventDestroy(b->L.fork);
+    if (b->L.join) cudaEventDestroy(b->L.join);
     if (b->own_stream) cudaStreamDestroy(b->st);
     delete b;
 }

@@ -67,6 +67,8 @@ struct BatchLaunch {
     AccLayout lay;
     int64_t ws_stride;
     int64_t max_eops;
+    cudaStream_t side;    // the accumulation's, beside the corrections
+    cudaEvent_t fork, join;
 };
 
 // Graph g of task j: last g with off[g] <= j (off non-decreasing, off[0] = 0).

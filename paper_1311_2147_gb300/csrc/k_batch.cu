@@ -328,11 +328,17 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     if (L.pairs & 1) batch_pair_plan(b, L, r, sizeof(DT), st);
     if (L.pairs & 2) batch_walk_class(b, L, r, st);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 2, 2, b.plan_acc, L.scan_unroll);
-    if (L.acc_threads == 128) batch_accum<DT, 128>(b, L, r, st);
-    else if (L.acc_threads == 256) batch_accum<DT, 256>(b, L, r, st);
-    else batch_accum<DT, 512>(b, L, r, st);
+    // (disjoint dependency rows, the rest of the state only read: a branch each of the
+    // captured graph)
+    cudaEventRecord(L.fork, st);
+    cudaStreamWaitEvent(L.side, L.fork, 0);
+    if (L.acc_threads == 128) batch_accum<DT, 128>(b, L, r, L.side);
+    else if (L.acc_threads == 256) batch_accum<DT, 256>(b, L, r, L.side);
+    else batch_accum<DT, 512>(b, L, r, L.side);
+    cudaEventRecord(L.join, L.side);
     if (L.pairs & 1) batch_pair_launches(b, L, r, sizeof(DT), st);
     if (L.pairs & 2) batch_walk_launches(b, L, r, sizeof(DT), st);
+    cudaStreamWaitEvent(st, L.join, 0);
     batch_round_end(b, L, r, st);
 }
 

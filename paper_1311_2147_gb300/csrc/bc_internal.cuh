@@ -170,6 +170,10 @@ inline __host__ __device__ int64_t group_slots(int64_t slots) {
     return (slots + kGroupSlots - 1) / kGroupSlots * kGroupSlots;
 }
 AccLayout acc_layout(int n, int64_t e_cap, bool is_static);
+// Most shared memory of an accumulation CTA (of the 227 KB a CTA may have), and what its
+// kernels are allowed: the allowance belongs to the kernel, which every handle and every
+// batch launches with a layout of its own, so none of them sets less.
+constexpr int32_t kAccSmemMax = 224 * 1024;
 inline bool acc_all_smem(const AccLayout& l) { return l.all_smem != 0; }
 
 // Device state of one handle (plain pointers; owned by the host-side bc_graph).

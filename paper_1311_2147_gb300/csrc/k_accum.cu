@@ -123,7 +123,6 @@ static AccArgs<DT> acc_args(const Dev& d, int is_static, const int32_t* rows, co
     return a;
 }
 
-constexpr int32_t kAccSmemMax = 224 * 1024;   // of the 227 KB a CTA may have
 // The cells (8 bytes per vertex, the largest array) stay in shared memory while two CTAs
 // fit an SM with them: past that (n above ~5500) they go to the work space, in L2, and
 // more threads per SM pay for it (BA n = 8192, every changed row: 0.48 us per row with

@@ -300,7 +300,7 @@ template <typename DT, int T>
 static int batch_accum_occupancy(const AccLayout& l) {
     int per_sm = 1;
     auto occ = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, l.smem);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAccSmemMax);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, l.smem);
     };
     if (acc_all_smem(l)) occ(kb_accum<DT, T, true>);

@@ -360,7 +360,9 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
  * updates are validated in order; a graph stops at its first invalid update (the updates
  * before it are applied) and the first such status is returned.  n_done (optional, G
  * entries) receives how many updates each graph applied.  Synchronous; device-side
- * errors poison only the graphs they occur in.
+ * errors poison only the graphs they occur in.  A call that fails with BC_ERR_CUDA or
+ * BC_ERR_OOM before its rounds have run poisons the graphs it had valid updates for (their
+ * weights on the host are already the new ones).
  */
 int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, const bc_vedge* edges,
                    int64_t n_edges, int32_t* n_done);

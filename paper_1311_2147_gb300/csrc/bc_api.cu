@@ -97,7 +97,10 @@ int fail(bc_graph* g, int code, const std::string& msg) {
     return code;
 }
 
+// (The runtime keeps the error for the next cudaGetLastError, which another handle's call
+// would take for its own launches'; it is reported here.)
 int cuda_fail(bc_graph* g, cudaError_t e, const char* what) {
+    cudaGetLastError();
     std::string m = std::string(what) + ": " + cudaGetErrorString(e);
     if (e == cudaErrorMemoryAllocation) return fail(g, BC_ERR_OOM, m);
     return fail(g, BC_ERR_CUDA, m);
@@ -756,7 +759,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
 #define CKI(call)                                                                          \
     do {                                                                                   \
         cudaError_t e_ = (call);                                                           \
-        if (e_ != cudaSuccess)                                                             \
+        if (e_ != cudaSuccess && (cudaGetLastError(), true))                               \
             return bail(e_ == cudaErrorMemoryAllocation ? BC_ERR_OOM : BC_ERR_CUDA,        \
                         std::string(#call) + ": " + cudaGetErrorString(e_));               \
     } while (0)
@@ -1259,16 +1262,21 @@ int bfail(bc_batch* b, int code, const std::string& msg) {
 #define CKB(b, call)                                                                           \
     do {                                                                                       \
         cudaError_t e_ = (call);                                                               \
-        if (e_ != cudaSuccess)                                                                 \
+        if (e_ != cudaSuccess) {                                                               \
+            cudaGetLastError();                                                                \
             return bfail((b), e_ == cudaErrorMemoryAllocation ? BC_ERR_OOM : BC_ERR_CUDA,        \
                          std::string(#call) + ": " + cudaGetErrorString(e_));                   \
+        }                                                                                      \
     } while (0)
 
 template <typename T>
 int balloc(bc_batch* b, T** p, size_t count) {
     *p = nullptr;
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(T));
-    if (e != cudaSuccess) return bfail(b, BC_ERR_OOM, "cudaMalloc failed for a batch buffer");
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return bfail(b, BC_ERR_OOM, "cudaMalloc failed for a batch buffer");
+    }
     b->allocs.push_back(*p);
     return BC_OK;
 }
@@ -1285,6 +1293,18 @@ void drop_exec(bc_batch* b) {
     b->exec = nullptr;
     b->exec_rounds = -1;
 }
+
+// The graphs whose weights or superset a batch call has changed on the host: until the
+// rounds have run these are ahead of the device, so a call that ends before poisons them.
+struct Ahead {
+    std::vector<bc_graph*> graphs;
+    ~Ahead() {
+        for (bc_graph* g : graphs) {
+            g->poisoned = true;
+            g->poison_status = BC_ERR_CUDA;
+        }
+    }
+};
 
 // Arcs the update would add to the E* superset (not yet in it).
 void new_arcs_of(bc_graph* g, int32_t v, const std::vector<VEdge>& ent, std::vector<int32_t>& need) {
@@ -1412,6 +1432,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     std::vector<std::vector<std::vector<VEdge>>> ents(G);
     std::vector<int32_t> ok(G, 0);
     int64_t base = 0;
+    Ahead ahead;
     for (int32_t g = 0; g < G; ++g) {
         bc_graph* gr = b->graphs[g];
         // validation reads the host weights as they evolve: the earlier updates' go in a
@@ -1445,8 +1466,10 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
             std::vector<HArc> arcs;
             for (size_t s2 = 0; s2 < gr->e_dst.size(); ++s2)
                 if (gr->e_dst[s2] >= 0) arcs.push_back({gr->e_src[s2], gr->e_dst[s2], gr->e_w[s2]});
+            ahead.graphs.push_back(gr);
             int rc = estar_layout(gr, arcs, &need);
             if (rc) return bfail(b, rc, gr->last_error);
+            ahead.graphs.pop_back();
         }
     }
     // ---- host records of every round
@@ -1464,6 +1487,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
             u = BatchUpd{};
             if (r >= ok[g]) continue;
             bc_graph* gr = b->graphs[g];
+            if (r == 0) ahead.graphs.push_back(gr);
             const std::vector<VEdge>& ent = ents[g][r];
             std::vector<EOp> ops;
             std::vector<EMove> moves;
@@ -1515,6 +1539,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     const int64_t ws_need = (int64_t)b->L.acc_grid * b->L.ws_stride;
     if (ws_need > b->ws_cap) {
         bfree(b, b->d_ws);
+        b->ws_cap = 0;
         if ((rc = balloc(b, &b->d_ws, ws_need))) return rc;
         b->ws_cap = ws_need;
         drop_exec(b);
@@ -1523,6 +1548,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
         bfree(b, b->d_upd);
         bfree(b, b->d_eop_off);
         bfree(b, b->d_voff);
+        b->R_cap = 0;   // until all are there
         const int64_t rc2 = std::max<int64_t>(R, 8);
         if ((rc = balloc(b, &b->d_upd, rc2 * G)) || (rc = balloc(b, &b->d_eop_off, rc2 + 1)) ||
             (rc = balloc(b, &b->d_voff, rc2 * 4 * (G + 1))))
@@ -1533,6 +1559,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     if ((int64_t)entries.size() > b->E_cap) {
         bfree(b, b->d_entries);
         bfree(b, b->d_wold);
+        b->E_cap = 0;
         const int64_t c = std::max<int64_t>((int64_t)entries.size() * 2, 1024);
         if ((rc = balloc(b, &b->d_entries, c)) || (rc = balloc(b, &b->d_wold, c))) return rc;
         b->E_cap = c;
@@ -1540,6 +1567,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     }
     if ((int64_t)eops.size() > b->O_cap) {
         bfree(b, b->d_eops);
+        b->O_cap = 0;
         const int64_t c = std::max<int64_t>((int64_t)eops.size() * 2, 1024);
         if ((rc = balloc(b, &b->d_eops, c))) return rc;
         b->O_cap = c;
@@ -1588,12 +1616,18 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     if (R > 0 && (!b->exec || b->exec_rounds != R)) {
         drop_exec(b);
         cudaGraph_t graph = nullptr;
+        cudaGetLastError();   // what is read below is the launches'
         CKB(b, cudaStreamBeginCapture(b->st, cudaStreamCaptureModeThreadLocal));
         batch_launch_rounds(a, b->L, R, b->dbytes, b->st);
-        CKB(b, cudaStreamEndCapture(b->st, &graph));
-        cudaError_t e = cudaGraphInstantiate(&b->exec, graph, 0);
-        cudaGraphDestroy(graph);
-        if (e != cudaSuccess) return bfail(b, BC_ERR_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
+        const cudaError_t launched = cudaGetLastError(), ended = cudaStreamEndCapture(b->st, &graph);
+        cudaGetLastError();
+        cudaError_t e = launched != cudaSuccess ? launched : ended;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, graph, 0);
+        if (graph) cudaGraphDestroy(graph);
+        if (e != cudaSuccess) {
+            b->exec = nullptr;
+            return bfail(b, BC_ERR_CUDA, std::string("capture of the rounds: ") + cudaGetErrorString(e));
+        }
         b->exec_rounds = R;
     }
     CKB(b, cudaEventRecord(b->e0, b->st));
@@ -1602,6 +1636,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
     std::vector<int32_t> errs(G, 0);
     if (R > 0) CKB(b, cudaMemcpyAsync(errs.data(), b->d_errs, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, b->st));
     CKB(b, cudaStreamSynchronize(b->st));
+    ahead.graphs.clear();
     float ms = 0.f;
     cudaEventElapsedTime(&ms, b->e0, b->e1);
     b->last_ms = ms;

@@ -315,7 +315,8 @@ int bc_get_weight_unit(bc_graph* g, int32_t* exp2);
  * every GPU that loads the library until the process exits).
  *   n            vertices, 1 .. 512; larger graphs are rejected with BC_ERR_ARG.
  *   arcs         arcs in d_dst / d_w, 0 .. 32768 (BC_ERR_ARG beyond).
- *   d_off        DEVICE int32[n+1]: CSR offsets by tail (arcs of a in [d_off[a], d_off[a+1])).
+ *   d_off        DEVICE int32[n+1]: CSR offsets by tail (arcs of a in [d_off[a], d_off[a+1]),
+ *                d_off[0] = 0, d_off[n] = arcs; anything else returns BC_ERR_ARG).
  *   d_dst, d_w   DEVICE int32 / int64 [arcs]: head and weight of each arc, weight in
  *                [1, INF-1] of the distance type.  An undirected graph is passed as
  *                G_D (both arcs of every edge).  The graph must be simple (repeated

@@ -75,13 +75,18 @@ cudaError_t scratch_address(unsigned char** out) {
 }
 
 // Pack the caller's CSR into the slot format of the accumulation (every arc a slot),
-// and check each arc: endpoints in range, no self-loop, weight in [1, INF-1].  The
-// slots past the arcs, up to a whole group, are empty.
+// and check each arc: endpoints in range, no self-loop, weight in [1, INF-1].  The offsets
+// cover every slot (0 first, the number of arcs last, none smaller than the one before):
+// the search goes over all of them, and one left out would hold an earlier call's arc.
+// The slots past the arcs, up to a whole group, are empty.
 template <typename DT>
 __global__ void k_pack_graph(int n, int64_t arcs, unsigned long long* count, const int32_t* off, const int32_t* dst, const int64_t* w,
                              Arc* arc, int64_t* w64, int32_t* len, int32_t* err) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0) *count = (unsigned long long)arcs;
+    if (i == 0) {
+        *count = (unsigned long long)arcs;
+        if (off[0] != 0 || off[n] != arcs) set_err(err, ERRF_ARG_DEVICE);
+    }
     if (i < n) {
         const int32_t a = off[i], b = off[i + 1];
         if (a < 0 || b < a || b > arcs) {

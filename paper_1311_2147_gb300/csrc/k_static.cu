@@ -26,7 +26,6 @@
 // one global distance order over all sources; this finds a little more than E* and keeps
 // the sources independent.
 #include <algorithm>
-#include <type_traits>
 
 #include "bc_internal.cuh"
 
@@ -58,17 +57,43 @@ struct SsspArgs {
     int check;             // a distance might not fit its type
 };
 
-// A group of S sources per CTA: their distance rows (DS) and two change masks per vertex
-// (bit k: d(s_k, x) dropped in the last round / in this one) in shared memory.  A round
+// What a CTA keeps in shared memory.  Groups: S distance rows and 16 mask bits per vertex.
+// Where not even one such row and its masks fit (n above 28672, or 19104 with 64-bit
+// rows), one source at a time: its row and one mask bit per vertex, and where that does not
+// fit either (64-bit rows, n above 27776), the mask bits alone, the distances in the
+// source's row of D.  bc_init_static's device time, G(n, 4n) directed: kOne 158 ms at
+// n = 29100 (32-bit) and 85 ms at n = 20000 (64-bit rows), kOneInD 352 ms at n = 32768; with a
+// search of the changed vertices' arcs, source by source, these took 565, 297 and 560 ms.
+enum class SsspForm { kGroups, kOne, kOneInD };
+
+// Two change masks, one bit per vertex and source of the group: whether its distance
+// dropped in the last round (cur) or in this one (nxt).
+template <bool GROUPS>
+struct SsspMask {
+    static __host__ __device__ constexpr int words(int np) { return GROUPS ? np / 2 : np / 32; }
+    static __device__ __forceinline__ unsigned get(const uint32_t* m, int x) {
+        if (GROUPS) return reinterpret_cast<const volatile uint16_t*>(m)[x];
+        return (*reinterpret_cast<const volatile uint32_t*>(m + (x >> 5)) >> (x & 31)) & 1u;
+    }
+    static __device__ __forceinline__ void set(uint32_t* m, int x, int k) {
+        if (GROUPS) atomicOr(m + (x >> 1), (1u << k) << ((x & 1) << 4));
+        else atomicOr(m + (x >> 5), 1u << (x & 31));
+    }
+};
+
+// A group of S sources per CTA: their distance rows (DS) and the two change masks.  A round
 // goes over all arcs, a lane per arc; a vector of 32 arcs is skipped for the sources in
 // which none of its tails changed.
-template <typename DT, typename DS, int T>
+template <typename DT, typename DS, int T, SsspForm F>
 __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int n = a.n, np = (n + 31) & ~31;
-    DS* dist = reinterpret_cast<DS*>(smem);
-    uint32_t* cur = reinterpret_cast<uint32_t*>(dist + (size_t)a.S * np);
-    uint32_t* nxt = cur + np / 2;
+    constexpr bool kRowInD = F == SsspForm::kOneInD;
+    static_assert(!kRowInD || sizeof(DS) == sizeof(DT), "the search's rows are D's");
+    using Mask = SsspMask<F == SsspForm::kGroups>;
+    const int n = a.n, np = (n + 31) & ~31, words = Mask::words(np);
+    DS* const rows = reinterpret_cast<DS*>(smem);
+    uint32_t* cur = reinterpret_cast<uint32_t*>(smem + (kRowInD ? 0 : (size_t)a.S * np * sizeof(DS)));
+    uint32_t* nxt = cur + words;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = T / 32, U = 4;
     const int64_t arcs = (int64_t)*a.arcs;
@@ -76,12 +101,13 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
     for (int s0 = blockIdx.x * a.S; s0 < n; s0 += gridDim.x * a.S) {
         if (block_err(a.err)) return;
         const int S = min(a.S, n - s0);
-        for (int t = tid; t < S * np; t += T) dist[t] = Far<DS>::v;
-        for (int t = tid; t < np / 2; t += T) cur[t] = nxt[t] = 0u;
+        DS* const dist = kRowInD ? reinterpret_cast<DS*>(a.D + (size_t)s0 * a.ld) : rows;
+        for (int t = tid; t < (kRowInD ? a.ld : S * np); t += T) dist[t] = Far<DS>::v;
+        for (int t = tid; t < words; t += T) cur[t] = nxt[t] = 0u;
         __syncthreads();
         if (tid < S) {
             dist[(size_t)tid * np + s0 + tid] = (DS)0;
-            atomicOr(cur + ((s0 + tid) >> 1), (1u << tid) << (((s0 + tid) & 1) << 4));
+            Mask::set(cur, s0 + tid, tid);
         }
         __syncthreads();
         bool converged = false;
@@ -103,8 +129,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int x = r[u].src(), b = r[u].dst();
-                    const unsigned mine =
-                        r[u].empty() ? 0u : (unsigned)reinterpret_cast<const volatile uint16_t*>(cur)[x];
+                    const unsigned mine = r[u].empty() ? 0u : Mask::get(cur, x);
                     for (unsigned m = __reduce_or_sync(0xffffffffu, mine); m; m &= m - 1u) {
                         const int k = __ffs(m) - 1;
                         if (!((mine >> k) & 1u)) continue;
@@ -113,7 +138,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
                         const DS nd = through(dx, sizeof(DS) == 8 ? (DS)w[u] : (DS)r[u].w);
                         if (nd < *(volatile DS*)(d + b)) {
                             atomic_min_dist(d + b, nd);
-                            atomicOr(nxt + (b >> 1), (1u << k) << ((b & 1) << 4));
+                            Mask::set(nxt, b, k);
                             any = true;
                         }
                     }
@@ -126,7 +151,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
             uint32_t* t = cur;
             cur = nxt;
             nxt = t;
-            for (int q = tid; q < np / 2; q += T) nxt[q] = 0u;
+            for (int q = tid; q < words; q += T) nxt[q] = 0u;
             __syncthreads();
         }
         // positive weights converge within n-1 rounds; anything else is reported
@@ -140,13 +165,14 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
                     if (dist[(size_t)k * np + r.src()] != Far<DS>::v && dist[(size_t)k * np + r.dst()] == Far<DS>::v)
                         set_err(a.err, ERRF_DIST);
             }
-        for (int k = 0; k < S; ++k) {
-            DT* row = a.D + (size_t)(s0 + k) * a.ld;
-            for (int t = tid; t < a.ld; t += T) {   // the entries past n: no path
-                const DS d = t < n ? dist[(size_t)k * np + t] : Far<DS>::v;
-                row[t] = d == Far<DS>::v ? (DT)Inf<DT>::v : (DT)d;
+        if constexpr (!kRowInD)
+            for (int k = 0; k < S; ++k) {
+                DT* row = a.D + (size_t)(s0 + k) * a.ld;
+                for (int t = tid; t < a.ld; t += T) {   // the entries past n: no path
+                    const DS d = t < n ? dist[(size_t)k * np + t] : Far<DS>::v;
+                    row[t] = d == Far<DS>::v ? (DT)Inf<DT>::v : (DT)d;
+                }
             }
-        }
         __syncthreads();
     }
 }
@@ -230,14 +256,35 @@ __global__ void __launch_bounds__(256) k_filter_arcs(int ld, int64_t arcs, const
     }
 }
 
+// Most shared memory of a search CTA, and what its kernels are allowed (the allowance
+// belongs to the kernel, which other host threads may be launching: none sets less).
 constexpr size_t kSsspSmemMax = 224 * 1024;
+
+template <typename DT, typename DS, int T, SsspForm F>
+static void sssp_launch(const Dev& d, const SsspArgs<DT>& a, size_t smem) {
+    auto kern = k_sssp<DT, DS, T, F>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSsspSmemMax);
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
+    const int grid = std::min(d.nsm * std::max(per_sm, 1), (d.n + a.S - 1) / a.S);
+    kern<<<grid, T, smem, d.st>>>(a);
+}
 
 // arcs_about: the number of arcs, for the choice of S (it is known only on the device).
 template <typename DT, typename DS>
 static void sssp_search(const Dev& d, const Arc* arc, const int64_t* w64, const unsigned long long* arcs,
                         double arcs_about, bool check) {
     const size_t np = ((size_t)d.n + 31) & ~(size_t)31;
+    SsspArgs<DT> a{d.n, d.ld, arc, w64, arcs, (DT*)d.D, d.err, 1, check ? 1 : 0};
     auto bytes = [&](int S) { return (size_t)S * np * sizeof(DS) + 2 * np * 2; };
+    if (bytes(1) > kSsspSmemMax) {
+        const size_t masks = 2 * (np / 8), one = np * sizeof(DS) + masks;
+        if constexpr (sizeof(DS) == sizeof(int64_t)) {
+            // (a row of D: as many threads an SM, in small CTAs, which wait for it one by one)
+            if (one > kSsspSmemMax) return sssp_launch<DT, DS, 256, SsspForm::kOneInD>(d, a, masks);
+        }
+        return sssp_launch<DT, DS, 1024, SsspForm::kOne>(d, a, one);   // 32-bit rows fit up to kMaxVertices
+    }
     auto resident = [&](int S) {   // groups an SM holds at a time
         const int groups = (d.n + S - 1) / S;
         return std::max(1, std::min({4, (int)((227 * 1024) / (bytes(S) + 1088)), (groups + d.nsm - 1) / d.nsm}));
@@ -245,32 +292,22 @@ static void sssp_search(const Dev& d, const Arc* arc, const int64_t* w64, const 
     // Sources per group: an SM's groups cost about their arcs once per source, the masks of
     // the arcs' tails twice that once per group, and a round's latency, times the rounds,
     // for every set of groups that run side by side.
-    int S = 1;
     double best = 0;
     for (int k = 1; k <= kSsspMaxSources && bytes(k) <= kSsspSmemMax; ++k) {
         const int groups = (d.n + k - 1) / k, per_sm = (groups + d.nsm - 1) / d.nsm;
         const double cost = per_sm * arcs_about * (k + 2.0) + (per_sm + resident(k) - 1) / resident(k) * 20000.0;
         if (k == 1 || cost < best) {
             best = cost;
-            S = k;
+            a.S = k;
         }
     }
-    const size_t smem = bytes(S);
-    SsspArgs<DT> a{d.n, d.ld, arc, w64, arcs, (DT*)d.D, d.err, S, check ? 1 : 0};
-    auto go = [&](auto t) {
-        constexpr int T = decltype(t)::value;
-        auto kern = k_sssp<DT, DS, T>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
-        const int grid = std::min(d.nsm * std::max(per_sm, 1), (d.n + S - 1) / S);
-        kern<<<grid, T, smem, d.st>>>(a);
-    };
     // about 1024 threads per SM
-    if (resident(S) >= 3) go(std::integral_constant<int, 256>{});
-    else if (resident(S) == 2) go(std::integral_constant<int, 512>{});
-    else go(std::integral_constant<int, 1024>{});
+    const size_t smem = bytes(a.S);
+    if (resident(a.S) >= 3) sssp_launch<DT, DS, 256, SsspForm::kGroups>(d, a, smem);
+    else if (resident(a.S) == 2) sssp_launch<DT, DS, 512, SsspForm::kGroups>(d, a, smem);
+    else sssp_launch<DT, DS, 1024, SsspForm::kGroups>(d, a, smem);
 }
+static_assert((size_t)kMaxVertices * sizeof(uint32_t) + 2 * kMaxVertices / 8 <= kSsspSmemMax, "SsspForm::kOne of 32-bit rows");
 
 // Arcs per vertex from which the light search pays: its own kLight arcs per vertex, twice
 // (bc_init_static's device time, complete n = 1024:

@@ -191,7 +191,7 @@ struct Dev {
     // full graph (G or G_D), used by the static computation
     Arc* g_arc;          // [g_arcs] by tail
     int64_t* g_w64;      // [g_arcs] weights in full (int64 distances; else NULL)
-    int32_t* g_off;      // [n + 1] first arc of each tail (NULL: the search takes every arc)
+    int32_t* g_off;      // [n + 1] first arc of each tail
     int64_t g_arcs;
     unsigned long long* g_count;   // [3] number of arcs in g_arc, and of two lists of the search
     // E*+ CSR with slack

@@ -152,6 +152,7 @@ extern "C" int bc_static_scores_noalloc(int32_t n, int64_t arcs, const int32_t* 
     d.e_cap = d.e_used = arcs;
     d.g_arc = d.e_arc;
     d.g_w64 = d.e_w64;
+    d.g_off = d.e_off;
     d.err = reinterpret_cast<int32_t*>(base + kOffErr);
     d.counts = reinterpret_cast<int32_t*>(base + kOffCnt);
     d.stats = reinterpret_cast<int64_t*>(base + kOffStats);

@@ -10,10 +10,11 @@
 // What bounds it: shared-memory gathers (two per arc, source and round in which the tail
 // changed; the random one takes about three bank cycles) and, for few sources per group,
 // the arcs' L2 reads of every round.  The arcs are read in order, 8 bytes each, once per
-// round for all sources of the group; before, a warp took the changed vertices of one
-// source one after the other, a chain of two L2 reads each.  Static search, before and
-// now: BA n = 4096 4.79 and 1.71 ms, ER n = 3001 (int64) 2.32 and 0.66 ms, BA n = 16384
-// 91 and 33 ms.
+// round for all sources of the group (or, in rounds of few changed vertices, these
+// vertices' arcs); before, a warp took the changed vertices of one source one after the
+// other, a chain of two L2 reads each.  Static search, before and now: BA n = 4096 5.04 and
+// 1.66 ms, ER n = 3001 (int64) 2.31 and 0.64 ms, BA n = 16384 90 and 42 ms, grid 128 x 128
+// 300 and 112 ms.
 //
 // E* (Section 1: arcs on some shortest path) is then {(a,b) : w(a,b) = d(a,b)}: the
 // one-arc path a->b is shortest exactly when the arc lies on a shortest path (a
@@ -26,6 +27,7 @@
 // one global distance order over all sources; this finds a little more than E* and keeps
 // the sources independent.
 #include <algorithm>
+#include <type_traits>
 
 #include "bc_internal.cuh"
 
@@ -51,6 +53,7 @@ struct SsspArgs {
     const Arc* arc;        // arcs, by tail
     const int64_t* w64;    // their weights in full (int64 distances)
     const unsigned long long* arcs;   // their number
+    const int32_t* off;    // [n + 1] first arc of each tail (NULL: they are in no order)
     DT* D;
     int32_t* err;
     int S;                 // sources of a group
@@ -61,8 +64,8 @@ struct SsspArgs {
 // Where not even one such row and its masks fit (n above 28672, or 19104 with 64-bit
 // rows), one source at a time: its row and one mask bit per vertex, and where that does not
 // fit either (64-bit rows, n above 27776), the mask bits alone, the distances in the
-// source's row of D.  bc_init_static's device time, G(n, 4n) directed: kOne 158 ms at
-// n = 29100 (32-bit) and 85 ms at n = 20000 (64-bit rows), kOneInD 352 ms at n = 32768; with a
+// source's row of D.  bc_init_static's device time, G(n, 4n) directed: kOne 129 ms at
+// n = 29100 (32-bit) and 72 ms at n = 20000 (64-bit rows), kOneInD 328 ms at n = 32768; with a
 // search of the changed vertices' arcs, source by source, these took 565, 297 and 560 ms.
 enum class SsspForm { kGroups, kOne, kOneInD };
 
@@ -79,14 +82,39 @@ struct SsspMask {
         if (GROUPS) atomicOr(m + (x >> 1), (1u << k) << ((x & 1) << 4));
         else atomicOr(m + (x >> 5), 1u << (x & 31));
     }
+    // Returns x's bits before.
+    static __device__ __forceinline__ unsigned set_old(uint32_t* m, int x, int k) {
+        if (GROUPS) return (atomicOr(m + (x >> 1), (1u << k) << ((x & 1) << 4)) >> ((x & 1) << 4)) & 0xFFFFu;
+        return (atomicOr(m + (x >> 5), 1u << (x & 31)) >> (x & 31)) & 1u;
+    }
+    // By x's own thread alone.
+    static __device__ __forceinline__ void clear(uint32_t* m, int x) {
+        if (GROUPS) *reinterpret_cast<volatile uint16_t*>(reinterpret_cast<uint16_t*>(m) + x) = 0;
+        else atomicAnd(m + (x >> 5), ~(1u << (x & 31)));
+    }
+};
+
+// Rounds in which few vertices changed go over these vertices' arcs only (LISTS).  A round
+// over all arcs costs the same however few changed, and on a path or a cycle nearly every
+// round has a vertex or two per source.  Search without and with lists: path of n = 1024
+// 1.56 and 0.91 ms, 4096 22.6 and 8.6 ms (64-bit rows 46 and 15.7), 16384 2860 and 590 ms;
+// BA n = 4096, whose last rounds change few, 1.72 and 1.66 ms.  A round goes over a list where
+// that is at most a quarter as long as there are vectors of 32 arcs.
+constexpr int kSsspList = 512;
+constexpr int kListsMinN = 2048;
+struct SsspLists {
+    int n[3];                      // vertices listed for a round, by round modulo 3
+    uint16_t v[2][kSsspList];      // by round modulo 2 (more than fit are only counted)
 };
 
 // A group of S sources per CTA: their distance rows (DS) and the two change masks.  A round
 // goes over all arcs, a lane per arc; a vector of 32 arcs is skipped for the sources in
-// which none of its tails changed.
-template <typename DT, typename DS, int T, SsspForm F>
+// which none of its tails changed.  Or, where few vertices are listed as changed, over the
+// arcs of 32 of these at a time.
+template <typename DT, typename DS, int T, SsspForm F, bool LISTS>
 __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ SsspLists sh;
     constexpr bool kRowInD = F == SsspForm::kOneInD;
     static_assert(!kRowInD || sizeof(DS) == sizeof(DT), "the search's rows are D's");
     using Mask = SsspMask<F == SsspForm::kGroups>;
@@ -98,6 +126,7 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
     constexpr int NW = T / 32, U = 4;
     const int64_t arcs = (int64_t)*a.arcs;
     const int nchunk = (int)((arcs + 31) >> 5);
+    const int few = LISTS && a.off ? min(kSsspList, nchunk / 4) : 0;   // vertices, for a round over a list
     for (int s0 = blockIdx.x * a.S; s0 < n; s0 += gridDim.x * a.S) {
         if (block_err(a.err)) return;
         const int S = min(a.S, n - s0);
@@ -108,51 +137,126 @@ __global__ void __launch_bounds__(T, 1024 / T) k_sssp(SsspArgs<DT> a) {
         if (tid < S) {
             dist[(size_t)tid * np + s0 + tid] = (DS)0;
             Mask::set(cur, s0 + tid, tid);
+            sh.v[0][tid] = (uint16_t)(s0 + tid);
         }
+        if (tid < 3) sh.n[tid] = tid == 0 ? S : 0;
         __syncthreads();
         bool converged = false;
+        bool listed = LISTS && S <= few;   // the vertices in cur are all in this round's list
         for (int round = 0; round <= n; ++round) {
-            bool any = false;
-            for (int c0 = warp * U; c0 < nchunk; c0 += U * NW) {
-                Arc r[U];
-                int64_t w[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int64_t e = ((int64_t)(c0 + u) << 5) + lane;
-                    r[u] = empty_arc();
-                    w[u] = 0;
-                    if (e < arcs) {
-                        r[u] = a.arc[e];
-                        if (sizeof(DS) == 8) w[u] = a.w64[e];
+            const uint16_t* const list = sh.v[round & 1];
+            uint16_t* const list_next = sh.v[(round + 1) & 1];
+            int* const n_next = &sh.n[(round + 1) % 3];
+            int changed;
+            if (LISTS && listed) {
+                const int count = sh.n[round % 3], per = min(32, (count + NW - 1) / NW);
+                if (tid == 0) sh.n[(round + 2) % 3] = 0;
+                for (int b0 = warp * per; b0 < count; b0 += NW * per) {   // warp-uniform
+                    int x = 0, beg = 0, len = 0;
+                    unsigned mine = 0;
+                    if (lane < min(per, count - b0)) {
+                        x = list[b0 + lane];
+                        beg = a.off[x];
+                        len = a.off[x + 1] - beg;
+                        mine = Mask::get(cur, x);
+                        Mask::clear(cur, x);
                     }
-                }
+                    int incl = len;
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int x = r[u].src(), b = r[u].dst();
-                    const unsigned mine = r[u].empty() ? 0u : Mask::get(cur, x);
-                    for (unsigned m = __reduce_or_sync(0xffffffffu, mine); m; m &= m - 1u) {
-                        const int k = __ffs(m) - 1;
-                        if (!((mine >> k) & 1u)) continue;
-                        DS* d = dist + (size_t)k * np;
-                        const DS dx = *(volatile DS*)(d + x);
-                        const DS nd = through(dx, sizeof(DS) == 8 ? (DS)w[u] : (DS)r[u].w);
-                        if (nd < *(volatile DS*)(d + b)) {
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int z = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (lane >= o) incl += z;
+                    }
+                    const int tot = __shfl_sync(0xffffffffu, incl, 31), excl = incl - len;
+                    for (int k0 = 0; k0 < tot; k0 += 32) {
+                        // the arc's tail: the last vertex whose arcs start at or before it
+                        int j = 0;
+#pragma unroll
+                        for (int step = 16; step >= 1; step >>= 1) {
+                            const int ex = __shfl_sync(0xffffffffu, excl, j + step);
+                            if (ex <= k0 + lane) j += step;
+                        }
+                        const int xj = __shfl_sync(0xffffffffu, x, j);
+                        const int64_t e = __shfl_sync(0xffffffffu, beg - excl, j) + k0 + lane;
+                        unsigned m = __shfl_sync(0xffffffffu, mine, j);
+                        if (k0 + lane >= tot) continue;
+                        const Arc r = a.arc[e];
+                        const DS w = sizeof(DS) == 8 ? (DS)a.w64[e] : (DS)r.w;
+                        for (; m; m &= m - 1u) {
+                            const int k = __ffs(m) - 1, b = r.dst();
+                            DS* d = dist + (size_t)k * np;
+                            const DS nd = through(*(volatile DS*)(d + xj), w);
+                            if (nd >= *(volatile DS*)(d + b)) continue;
                             atomic_min_dist(d + b, nd);
-                            Mask::set(nxt, b, k);
-                            any = true;
+                            if (Mask::set_old(nxt, b, k) != 0u) continue;   // listed already
+                            const int p = atomicAdd(n_next, 1);
+                            if (p < kSsspList) list_next[p] = (uint16_t)b;
                         }
                     }
                 }
+                __syncthreads();
+                changed = *n_next;
+                listed = changed <= few;
+            } else {
+                bool any = false;
+                if (tid == 0) sh.n[(round + 2) % 3] = 0;
+                for (int c0 = warp * U; c0 < nchunk; c0 += U * NW) {
+                    Arc r[U];
+                    int64_t w[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int64_t e = ((int64_t)(c0 + u) << 5) + lane;
+                        r[u] = empty_arc();
+                        w[u] = 0;
+                        if (e < arcs) {
+                            r[u] = a.arc[e];
+                            if (sizeof(DS) == 8) w[u] = a.w64[e];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int x = r[u].src(), b = r[u].dst();
+                        const unsigned mine = r[u].empty() ? 0u : Mask::get(cur, x);
+                        for (unsigned m = __reduce_or_sync(0xffffffffu, mine); m; m &= m - 1u) {
+                            const int k = __ffs(m) - 1;
+                            if (!((mine >> k) & 1u)) continue;
+                            DS* d = dist + (size_t)k * np;
+                            const DS dx = *(volatile DS*)(d + x);
+                            const DS nd = through(dx, sizeof(DS) == 8 ? (DS)w[u] : (DS)r[u].w);
+                            if (nd < *(volatile DS*)(d + b)) {
+                                atomic_min_dist(d + b, nd);
+                                Mask::set(nxt, b, k);
+                                any = true;
+                            }
+                        }
+                    }
+                }
+                changed = __syncthreads_count(any);   // threads that found one
+                listed = false;
+                for (int q = tid; q < words; q += T) cur[q] = 0u;
+                if (LISTS && changed <= min(few, T / 4)) {   // block-uniform: perhaps few vertices
+                    for (int q = tid; q < words; q += T) {
+                        constexpr int per_word = F == SsspForm::kGroups ? 2 : 32;
+                        uint32_t w = nxt[q];
+                        for (int i = 0; w; ++i, w = per_word == 2 ? w >> 16 : w >> 1) {
+                            if (!(w & (per_word == 2 ? 0xFFFFu : 1u))) continue;
+                            const int p = atomicAdd(n_next, 1);
+                            if (p < kSsspList) list_next[p] = (uint16_t)(q * per_word + i);
+                        }
+                    }
+                    __syncthreads();
+                    listed = *n_next <= few;
+                } else {
+                    __syncthreads();
+                }
             }
-            if (!__syncthreads_or(any)) {
+            if (changed == 0) {
                 converged = true;
                 break;
             }
             uint32_t* t = cur;
             cur = nxt;
             nxt = t;
-            for (int q = tid; q < words; q += T) nxt[q] = 0u;
-            __syncthreads();
         }
         // positive weights converge within n-1 rounds; anything else is reported
         if (!converged && tid == 0) set_err(a.err, ERRF_TIMEOUT);
@@ -260,9 +364,9 @@ __global__ void __launch_bounds__(256) k_filter_arcs(int ld, int64_t arcs, const
 // belongs to the kernel, which other host threads may be launching: none sets less).
 constexpr size_t kSsspSmemMax = 224 * 1024;
 
-template <typename DT, typename DS, int T, SsspForm F>
+template <typename DT, typename DS, int T, SsspForm F, bool LISTS>
 static void sssp_launch(const Dev& d, const SsspArgs<DT>& a, size_t smem) {
-    auto kern = k_sssp<DT, DS, T, F>;
+    auto kern = k_sssp<DT, DS, T, F, LISTS>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSsspSmemMax);
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
@@ -273,21 +377,21 @@ static void sssp_launch(const Dev& d, const SsspArgs<DT>& a, size_t smem) {
 // arcs_about: the number of arcs, for the choice of S (it is known only on the device).
 template <typename DT, typename DS>
 static void sssp_search(const Dev& d, const Arc* arc, const int64_t* w64, const unsigned long long* arcs,
-                        double arcs_about, bool check) {
+                        const int32_t* off, double arcs_about, bool check) {
     const size_t np = ((size_t)d.n + 31) & ~(size_t)31;
-    SsspArgs<DT> a{d.n, d.ld, arc, w64, arcs, (DT*)d.D, d.err, 1, check ? 1 : 0};
+    SsspArgs<DT> a{d.n, d.ld, arc, w64, arcs, off, (DT*)d.D, d.err, 1, check ? 1 : 0};
     auto bytes = [&](int S) { return (size_t)S * np * sizeof(DS) + 2 * np * 2; };
     if (bytes(1) > kSsspSmemMax) {
         const size_t masks = 2 * (np / 8), one = np * sizeof(DS) + masks;
         if constexpr (sizeof(DS) == sizeof(int64_t)) {
             // (a row of D: as many threads an SM, in small CTAs, which wait for it one by one)
-            if (one > kSsspSmemMax) return sssp_launch<DT, DS, 256, SsspForm::kOneInD>(d, a, masks);
+            if (one > kSsspSmemMax) return sssp_launch<DT, DS, 256, SsspForm::kOneInD, true>(d, a, masks);
         }
-        return sssp_launch<DT, DS, 1024, SsspForm::kOne>(d, a, one);   // 32-bit rows fit up to kMaxVertices
+        return sssp_launch<DT, DS, 1024, SsspForm::kOne, true>(d, a, one);   // 32-bit rows fit up to kMaxVertices
     }
     auto resident = [&](int S) {   // groups an SM holds at a time
         const int groups = (d.n + S - 1) / S;
-        return std::max(1, std::min({4, (int)((227 * 1024) / (bytes(S) + 1088)), (groups + d.nsm - 1) / d.nsm}));
+        return std::max(1, std::min({4, (int)((227 * 1024) / (bytes(S) + sizeof(SsspLists) + 1088)), (groups + d.nsm - 1) / d.nsm}));
     };
     // Sources per group: an SM's groups cost about their arcs once per source, the masks of
     // the arcs' tails twice that once per group, and a round's latency, times the rounds,
@@ -303,9 +407,17 @@ static void sssp_search(const Dev& d, const Arc* arc, const int64_t* w64, const 
     }
     // about 1024 threads per SM
     const size_t smem = bytes(a.S);
-    if (resident(a.S) >= 3) sssp_launch<DT, DS, 256, SsspForm::kGroups>(d, a, smem);
-    else if (resident(a.S) == 2) sssp_launch<DT, DS, 512, SsspForm::kGroups>(d, a, smem);
-    else sssp_launch<DT, DS, 1024, SsspForm::kGroups>(d, a, smem);
+    auto go = [&](auto lists) {
+        constexpr bool L = decltype(lists)::value;
+        if (resident(a.S) >= 3) sssp_launch<DT, DS, 256, SsspForm::kGroups, L>(d, a, smem);
+        else if (resident(a.S) == 2) sssp_launch<DT, DS, 512, SsspForm::kGroups, L>(d, a, smem);
+        else sssp_launch<DT, DS, 1024, SsspForm::kGroups, L>(d, a, smem);
+    };
+    // Lists for large graphs and for those with about one edge per vertex (k_sssp): they cost a
+    // small one some 3 us for their part of the kernel (G(256, 2048) 20.1 us without, 23.4 with;
+    // G(1024, 8192) 85.7 and 87.0).
+    if (off && (d.n >= kListsMinN || 2 * d.g_arcs <= 5 * (int64_t)d.n)) go(std::true_type{});
+    else go(std::false_type{});
 }
 static_assert((size_t)kMaxVertices * sizeof(uint32_t) + 2 * kMaxVertices / 8 <= kSsspSmemMax, "SsspForm::kOne of 32-bit rows");
 
@@ -327,13 +439,13 @@ static void sssp(const Dev& d, int64_t w_max, bool all_arcs, bool check) {
         unsigned long long* counts = reinterpret_cast<unsigned long long*>(d.g_count);
         k_light_arcs<<<std::min((d.n + 7) / 8, d.nsm * 8), 256, 0, d.st>>>(d.n, d.g_off, d.g_arc, d.g_w64, w_max, l_arc,
                                                                          l_w64, counts + 1);
-        sssp_search<DT, DS>(d, l_arc, l_w64, counts + 1, (double)light, false);
+        sssp_search<DT, DS>(d, l_arc, l_w64, counts + 1, nullptr, (double)light, false);
         k_filter_arcs<DT><<<(int)std::min<int64_t>((d.g_arcs + 255) / 256, d.nsm * 8), 256, 0, d.st>>>(
             d.ld, d.g_arcs, d.g_arc, d.g_w64, (const DT*)d.D, f_arc, f_w64, counts + 2);
-        sssp_search<DT, DS>(d, f_arc, f_w64, counts + 2, (double)light, check);
+        sssp_search<DT, DS>(d, f_arc, f_w64, counts + 2, nullptr, (double)light, check);
         return;
     }
-    sssp_search<DT, DS>(d, d.g_arc, d.g_w64, d.g_count, (double)d.g_arcs, check);
+    sssp_search<DT, DS>(d, d.g_arc, d.g_w64, d.g_count, d.g_off, (double)d.g_arcs, check);
 }
 
 // w_max: the largest weight (0: not known).

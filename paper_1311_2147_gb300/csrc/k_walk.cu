@@ -26,12 +26,12 @@
 // A warp takes a light row with a table of 128 entries, a CTA a row with more targets and
 // a larger table, both hash tables in shared memory; rows that outgrow theirs are taken
 // by a last launch, whose CTAs fall back to dense arrays in device memory.  Sums are
-// fixed-point integers in units of 2^-55 added by atomics, so a row's result depends
-// neither on the order of its arcs nor on the class it ran in.
+// fixed-point integers of two words, in units of 2^-119, added by atomics, so a row's result
+// depends neither on the order of its arcs nor on the class it ran in.
 //
 // Bound by latency and by the instructions of short, uneven loops (ncu, light rows at
 // n = 8192: 42 % of the issue slots, 17 % of the memory rate): per level of a walk the
-// segment, an arc, its tail's distance; hence many rows in flight (a warp and 5.4 KB each)
+// segment, an arc, its tail's distance; hence many rows in flight (a warp and 5.5 KB each)
 // and several arcs of a lane in flight.  It replaced a walk per pair and state that listed
 // the vertices found, and a second pass that evaluated sigma_sx * sigma_xt / sigma_st for
 // each from rows s and t (Barabasi-Albert, 8 edges a vertex, weights 1..100): at n = 8192,
@@ -218,23 +218,26 @@ template <typename DT, typename IX>
 struct WalkTable {
     uint64_t* sig;              // sigma_sx
     unsigned long long* acc;    // the difference's share of x so far, at a target with a path plus 1
-                                // (old: all of it negative), in units of 2^-55
+                                // (old: all of it negative), in units of 2^-55,
+    unsigned long long* low;    // and what is below that, in units of 2^-119
     DT* d;                      // d(s,x)
     int32_t* key;
     int32_t* head;              // DAG arcs into x: first node
-    int32_t* cnt;               // DAG children of x not done yet
+    uint32_t* cnt;              // DAG children of x not done yet, in 16-bit halves (a vertex has fewer
+                                // than n, and one more for each target with two entries)
     IX* seen;                   // entries made, in order (the targets first; without a path: not in it)
     IX* ready;                  // entries whose children are done, in order
     IX* node_x;                 // a DAG arc's tail
     IX* node_next;              // the next arc with the same head
 
     __host__ __device__ static constexpr size_t entry_bytes() {
-        return sizeof(uint64_t) * 2 + sizeof(DT) + 3 * sizeof(int32_t) + 2 * sizeof(IX);
+        return sizeof(uint64_t) * 3 + sizeof(DT) + 2 * sizeof(int32_t) + sizeof(uint16_t) + 2 * sizeof(IX);
     }
     __host__ __device__ static constexpr size_t bytes(size_t entries, size_t nodes) {
-        return (entries * entry_bytes() + nodes * 2 * sizeof(IX) + 15) & ~(size_t)15;
+        return ((entries + (entries & 1)) * entry_bytes() + nodes * 2 * sizeof(IX) + 15) & ~(size_t)15;
     }
     __device__ __forceinline__ WalkTable(unsigned char* p, size_t entries, size_t nodes) {
+        entries += entries & 1;
         auto take = [&](size_t b) {
             unsigned char* q = p;
             p += b;
@@ -242,10 +245,11 @@ struct WalkTable {
         };
         sig = reinterpret_cast<uint64_t*>(take(8 * entries));
         acc = reinterpret_cast<unsigned long long*>(take(8 * entries));
+        low = reinterpret_cast<unsigned long long*>(take(8 * entries));
         d = reinterpret_cast<DT*>(take(sizeof(DT) * entries));
         key = reinterpret_cast<int32_t*>(take(4 * entries));
         head = reinterpret_cast<int32_t*>(take(4 * entries));
-        cnt = reinterpret_cast<int32_t*>(take(4 * entries));
+        cnt = reinterpret_cast<uint32_t*>(take(2 * entries));
         seen = reinterpret_cast<IX*>(take(sizeof(IX) * entries));
         ready = reinterpret_cast<IX*>(take(sizeof(IX) * entries));
         node_x = reinterpret_cast<IX*>(take(sizeof(IX) * nodes));
@@ -254,36 +258,73 @@ struct WalkTable {
     __device__ __forceinline__ void free_entry(int e) const {
         key[e] = -1;
         head[e] = kNone;
-        cnt[e] = 0;
-        acc[e] = 0ull;
+        reinterpret_cast<uint16_t*>(cnt)[e] = 0;
+        acc[e] = low[e] = 0ull;
+    }
+    __device__ __forceinline__ bool no_children(int e) const { return reinterpret_cast<const uint16_t*>(cnt)[e] == 0; }
+    __device__ __forceinline__ void count_child(int e) const { atomicAdd(cnt + (e >> 1), 1u << ((e & 1) << 4)); }
+    __device__ __forceinline__ bool last_child(int e) const {
+        const int sh = (e & 1) << 4;
+        return ((atomicSub(cnt + (e >> 1), 1u << sh) >> sh) & 0xFFFFu) == 1u;
+    }
+    __device__ __forceinline__ __int128 sum(int e) const {
+        const long long hi = (long long)*(volatile unsigned long long*)(acc + e);
+        return ((__int128)hi << 64) + *(volatile unsigned long long*)(low + e);
+    }
+    // The low word's carry goes along; most shares have nothing below 2^-55.
+    __device__ __forceinline__ void add(int e, __int128 v) const {
+        unsigned long long hi = (unsigned long long)(v >> 64);
+        const unsigned long long lo = (unsigned long long)v;
+        if (lo) hi += atomicAdd(low + e, lo) + lo < lo;
+        atomicAdd(acc + e, hi);
     }
     // All m entries (a multiple of four; the arrays start on 16-byte boundaries).
     __device__ __forceinline__ void free_all(int m, int rank, int threads) const {
         for (int i = rank; i < m / 4; i += threads) {
             reinterpret_cast<int4*>(key)[i] = make_int4(-1, -1, -1, -1);
             reinterpret_cast<int4*>(head)[i] = make_int4(kNone, kNone, kNone, kNone);
-            reinterpret_cast<int4*>(cnt)[i] = make_int4(0, 0, 0, 0);
-            reinterpret_cast<ulonglong2*>(acc)[2 * i] = make_ulonglong2(0ull, 0ull);
-            reinterpret_cast<ulonglong2*>(acc)[2 * i + 1] = make_ulonglong2(0ull, 0ull);
+            reinterpret_cast<int2*>(cnt)[i] = make_int2(0, 0);
+            const ulonglong2 none = make_ulonglong2(0ull, 0ull);
+            reinterpret_cast<ulonglong2*>(acc)[2 * i] = reinterpret_cast<ulonglong2*>(acc)[2 * i + 1] = none;
+            reinterpret_cast<ulonglong2*>(low)[2 * i] = reinterpret_cast<ulonglong2*>(low)[2 * i + 1] = none;
         }
     }
 };
 
-// v in (-2^8, 2^8) to units of 2^-55 and back: h - a is exact, each part is rounded once;
-// the four parts of the way back are exact.
-__device__ __forceinline__ long long to_units(ff v) {
-    const float h = v.hi * 0x1p24f;
-    const float a = rintf(h);
-    return __float2ll_rn(a) * (1ll << 31) + __float2ll_rn((h - a) * 0x1p31f) + __float2ll_rn(v.lo * 0x1p55f);
+// v in (-2^8, 2^8) to units of 2^-119 and back.  A share is at least 2^-64 (one path of fewer
+// than 2^64), so these keep every bit of a float-float, and sums of them by integer atomics
+// are exact whatever their order.  (With 2^-55 and one word a share of 2^-40 kept 15 bits.)
+// h - a, r - c and the products with powers of two are exact.
+__device__ __forceinline__ __int128 to_units(ff v) {
+    const float h = v.hi * 0x1p24f, a = rintf(h);
+    float r0 = (h - a) * 0x1p31f, r1 = v.lo * 0x1p55f;   // units of 2^-55
+    const float b0 = rintf(r0), b1 = rintf(r1);
+    const long long hi = __float2ll_rn(a) * (1ll << 31) + __float2ll_rn(b0) + __float2ll_rn(b1);
+    r0 -= b0;
+    r1 -= b1;
+    __int128 x = (__int128)hi << 64;
+    if (r0 != 0.f || r1 != 0.f) {
+        r0 *= 0x1p32f;
+        r1 *= 0x1p32f;
+        const float c0 = rintf(r0), c1 = rintf(r1);
+        x += (__int128)(__float2ll_rn(c0) + __float2ll_rn(c1)) << 32;
+        x += __float2ll_rn((r0 - c0) * 0x1p32f) + __float2ll_rn((r1 - c1) * 0x1p32f);
+    }
+    return x;
 }
-__device__ __forceinline__ ff from_units(long long v) {
-    const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
-    const uint32_t A = (uint32_t)(m >> 31), B = (uint32_t)m & 0x7FFFFFFFu;
-    const ff r = ff_add(two_sum((float)(A >> 24), (float)(A & 0xFFFFFFu) * 0x1p-24f),
-                        two_sum((float)(B >> 24) * 0x1p-31f, (float)(B & 0xFFFFFFu) * 0x1p-55f));
+__device__ __forceinline__ float pow2f(int e) { return e < -126 ? 0.f : __int_as_float((e + 127) << 23); }
+__device__ __forceinline__ ff from_units(__int128 v) {
+    const unsigned __int128 m = v < 0 ? -(unsigned __int128)v : (unsigned __int128)v;
+    const uint64_t m1 = (uint64_t)(m >> 64), m0 = (uint64_t)m;
+    // its 64 leading bits, in units of 2^(-55 - z)
+    const int z = m1 ? __clzll((long long)m1) : 64 + __clzll((long long)m0);
+    const uint64_t top = z == 0 ? m1 : z < 64 ? (m1 << z) | (m0 >> (64 - z)) : z < 128 ? m0 << (z - 64) : 0ull;
+    const ff r = ff_add(two_sum((float)(uint32_t)(top >> 40) * pow2f(-15 - z),
+                                (float)((uint32_t)(top >> 16) & 0xFFFFFFu) * pow2f(-39 - z)),
+                        ff{(float)((uint32_t)top & 0xFFFFu) * pow2f(-55 - z), 0.f});
     return v < 0 ? ff{-r.hi, -r.lo} : r;
 }
-constexpr long long kOne = 1ll << 55;
+constexpr long long kOne = 1ll << 55;   // 1 in acc
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
@@ -456,7 +497,7 @@ struct RowWalk {
                             prefetch_l2(a.Dl + rs + x[u]);
                         }
                     }
-                    atomicAdd(t.cnt + f, 1);
+                    t.count_child(f);
                     if (H != 0) {
                         const int q = atomicAdd(&sh.nodes, 1);
                         if (q < NODES) {
@@ -521,12 +562,12 @@ struct RowWalk {
     // What a vertex y whose children are done has for its DAG parents: its sum c, and the
     // sum over its path count, r, for parents with another count.
     struct Share {
-        long long c;
+        __int128 c;
         uint64_t sig;
         ff r;
     };
     __device__ __forceinline__ void share(int e, Share& h) const {
-        h.c = (long long)*(volatile unsigned long long*)(t.acc + e);
+        h.c = t.sum(e);
         h.sig = t.sig[e];
         h.r.hi = -1.f;
         h.r.lo = 2.f;   // not computed (no float-float has |lo| > |hi|)
@@ -535,13 +576,13 @@ struct RowWalk {
     // y's only parent, mostly.
     __device__ __forceinline__ void push(int f, Share& h) const {
         const uint64_t sx = t.sig[f];
-        long long c = h.c;
+        __int128 c = h.c;
         if (sx != h.sig) {
             if (h.r.lo == 2.f) h.r = ff_mul(from_units(h.c), ff_rcp(ff_from_u64(h.sig)));
             c = to_units(ff_mul(h.r, ff_from_u64(sx)));
         }
-        atomicAdd(t.acc + f, (unsigned long long)c);
-        if (atomicSub(t.cnt + f, 1) == 1) t.ready[atomicAdd(&sh.ready, 1)] = (IX)f;
+        t.add(f, c);
+        if (t.last_child(f)) t.ready[atomicAdd(&sh.ready, 1)] = (IX)f;
     }
 
     // The recurrence: an entry pushes to its DAG parents once its own children are done.
@@ -551,7 +592,7 @@ struct RowWalk {
         for (int i = rank(); i < seen; i += GS) {
             const int e = t.seen[i];
             if (i >= nseed) t.sig[e] = a.S[rs + (t.key[e] >> 1)];
-            if (t.cnt[e] == 0) t.ready[atomicAdd(&sh.ready, 1)] = (IX)e;
+            if (t.no_children(e)) t.ready[atomicAdd(&sh.ready, 1)] = (IX)e;
         }
         for (int lo = 0;;) {
             sync();
@@ -599,13 +640,14 @@ struct RowWalk {
         const int k = t.key[e];
         if (k < 0 || !(k & 1)) return;
         const int o = find(k ^ 1);
-        long long v = (long long)t.acc[e];
-        if (o >= 0) v += (long long)t.acc[o];
+        __int128 v = t.sum(e);
+        if (o >= 0) v += t.sum(o);
         if (v == 0) return;
         const int x = k >> 1;
         ff* p = a.Dl + (size_t)s * a.ld + x;
         *p = ff_add(*p, from_units(v));
-        fix_add(a.bcfix, x, v >> 31, (v & 0x7FFFFFFFll) << 1);   // units of 2^-24 and 2^-56
+        v += (__int128)1 << 62;   // to the nearest 2^-56
+        fix_add(a.bcfix, x, (long long)(v >> 95), (long long)(uint32_t)(v >> 63));   // units of 2^-24 and 2^-56
     }
 
     // The whole row; false: it outgrew the table and nothing was written but the table.
@@ -645,16 +687,19 @@ struct RowWalk {
     }
 };
 
-// Light rows: a warp each.
+// Light rows: a warp each.  16 CTAs' tables (with 32-bit distances) leave an SM 60 KB of L1, as
+// do four of the CTA rows' (below): both are kept under 196 KB an SM.  With 6.4 and 51 KB, past
+// it, 16 updates at n = 16384 took 9.5 ms instead of 9.1.
 constexpr int kLightPerSm = 16, kLightWarps = 2, kLightH = 128, kLightLimit = kLightH - 33, kLightNodes = 192;
-template <typename DT> using LightTable = WalkTable<DT, uint16_t>;
+static_assert(kLightH <= 255 && kLightNodes < 255, "numbered in 8 bits");
+template <typename DT> using LightTable = WalkTable<DT, uint8_t>;
 template <typename DT>
 __host__ __device__ constexpr size_t light_bytes() { return LightTable<DT>::bytes(kLightH, kLightNodes); }
 
 template <typename DT, typename UPD>
 __device__ __forceinline__ bool light_row(const WalkGraph<DT>& g, const UPD& upd, const LightTable<DT>& t,
                                           WalkShared& sh, int s, unsigned long long* totals) {
-    const RowWalk<DT, UPD, uint16_t, 32, kLightH, kLightNodes> w{g, upd, t, sh, min(g.cap, kLightLimit), s, g.tcnt[s], totals};
+    const RowWalk<DT, UPD, uint8_t, 32, kLightH, kLightNodes> w{g, upd, t, sh, min(g.cap, kLightLimit), s, g.tcnt[s], totals};
     return w.run();
 }
 __device__ __forceinline__ void walk_totals(int64_t* stats, unsigned long long* totals) {
@@ -727,7 +772,7 @@ template <bool RETRY>
 struct Cta {
     static_assert(4 * kPairCap <= 512 && 2 * kLightTargets < kLightH, "room for the targets");
     static constexpr int threads = RETRY ? 512 : 256, h = RETRY ? 2048 : 1024, limit = h - threads - 1,
-                         nodes = RETRY ? 3072 : 1536, per_sm = RETRY ? 1 : 4;
+                         nodes = RETRY ? 3072 : 1408, per_sm = RETRY ? 1 : 4;
     template <typename DT>
     __host__ __device__ static constexpr size_t bytes() { return WalkTable<DT, uint16_t>::bytes(h, nodes); }
 };
@@ -850,7 +895,7 @@ int dense_tables(int n) {
 // The least of dense_tables (n = 1, 64-bit distances; a batch's graphs have any n).
 constexpr int kDenseTablesMin =
     (int)((size_t)kPairCap * kPairPlanBytes / WalkTable<int64_t, int32_t>::bytes(dense_entries(1), 0));
-static_assert(kDenseTablesMin >= 48, "CTAs for the rows that outgrow shared memory");
+static_assert(kDenseTablesMin >= 40, "CTAs for the rows that outgrow shared memory");
 
 template <typename DT>
 void walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready) {
@@ -869,9 +914,13 @@ void walks(const Dev& d, const WalkUpd& upd, cudaEvent_t ready) {
 
 template <typename DT>
 cudaError_t setup() {
-    const int smem = (int)Cta<true>::bytes<DT>();
-    cudaError_t e = cudaFuncSetAttribute(k_walk_cta<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kb_walk_cta<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto allow = [](auto kern, size_t smem) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+    cudaError_t e = allow(k_walk_cta<DT, false>, Cta<false>::bytes<DT>());
+    if (e == cudaSuccess) e = allow(kb_walk_cta<DT, false>, Cta<false>::bytes<DT>());
+    if (e == cudaSuccess) e = allow(k_walk_cta<DT, true>, Cta<true>::bytes<DT>());
+    if (e == cudaSuccess) e = allow(kb_walk_cta<DT, true>, Cta<true>::bytes<DT>());
     return e;
 }
 

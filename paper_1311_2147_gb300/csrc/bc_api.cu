@@ -726,7 +726,7 @@ int bc_init_static(bc_graph** out, int32_t n, int64_t m, const int32_t* src, con
     need(&d.stats, kStats, 8);
     need(&d.changed, n, 4);
     need(&d.counts, 16, 4);
-    need(&d.bcfix, 2 * (size_t)n, 8);
+    need(&d.bcfix, 3 * (size_t)n + 1, 8);
     if (!dir) {
         need(&d.chg, (size_t)n * d.chg_words, 4);   // the change map
         need(&d.tcnt, n, 4);

@@ -154,38 +154,55 @@ __device__ __forceinline__ void dev_estar_write(const EOp& o, Arc* e_arc, int64_
     atomicMax(e_len + o.a, o.len_a);   // lengths only grow between rebuilds
 }
 
-// BC's change in an update is summed per column as a fixed-point pair (A in units of
-// 2^-24, B in units of 2^-56) by integer atomics, so the total does not depend on the
-// order in which rows and CTAs add (the result is deterministic) and is exact up to the
-// 2^-56 rounding of each dependency.
+// BC's change in an update is summed per column as fixed-point words (A in units of 2^-24,
+// B of 2^-71) by integer atomics, so the total does not depend on the order in which rows
+// and CTAs add (the result is deterministic) and is exact up to the rounding of each
+// dependency to 2^-71, its own last bit or less from 2^-23 on.  Where pairs have very many
+// shortest paths dependencies, and BC with them, are smaller; what those have below 2^-71
+// goes to a third word (C in units of 2^-112), which few updates touch (fix[3n] tells).
 //
-// A dependency v = hi + lo, 0 <= v < 2^15, as such a pair, in single precision only (fp64
+// A dependency v = hi + lo, |v| < 2^15, as these words, in single precision only (fp64
 // runs at a small fraction of the fp32 rate here): with h = hi * 2^24 and a = rint(h), h
-// and h - a are exact, and (h - a) * 2^32 and lo * 2^56 (|lo| <= 2^-10) are exact
-// scalings, each rounded to an integer once.  |A| <= 2^39, |B| < 2^47.
-__device__ __forceinline__ void fix_words(ff v, long long* A, long long* B) {
-    const float h = v.hi * 0x1p24f;
-    const float a = rintf(h);
-    *A = __float2ll_rn(a);
-    *B = __float2ll_rn((h - a) * 0x1p32f) + __float2ll_rn(v.lo * 0x1p56f);
+// and h - a are exact, and (h - a) * 2^47 and lo * 2^71 (|lo| <= 2^-10) are exact
+// scalings, each rounded to an integer once.  |A| <= 2^39, |B| <= 2^61 + 2^46, |C| <= 2^41.
+struct FixWords {
+    long long A, B, C;
+};
+__device__ __forceinline__ FixWords fix_words(ff v) {   // but C
+    const float h = v.hi * 0x1p24f, a = rintf(h);
+    return FixWords{__float2ll_rn(a), __float2ll_rn((h - a) * 0x1p47f) + __float2ll_rn(v.lo * 0x1p71f), 0};
 }
-// Adds A, B to column x's pair, B's high bits carried into A: |B| <= 2^31 per addend, and
-// a column has at most 2^15 addends of each kind, so |A| < 2^55 and |B| < 2^47.
-__device__ __forceinline__ void fix_add(int64_t* fix, int x, long long A, long long B) {
-    const long long c = (B + (1ll << 31)) >> 32;
-    A += c;
-    B -= c << 32;
+// 0 < |v| < 2^-23, and its C: what the two roundings of B leave, exactly.
+__device__ __forceinline__ bool fix_small(ff v) { return (__float_as_uint(v.hi) & 0x7FFFFFFFu) - 1u < 0x33FFFFFFu; }
+__device__ __forceinline__ long long fix_rest(ff v) {
+    const float h = v.hi * 0x1p24f, r = (h - rintf(h)) * 0x1p47f, l = v.lo * 0x1p71f;
+    return __float2ll_rn((r - rintf(r)) * 0x1p41f) + __float2ll_rn((l - rintf(l)) * 0x1p41f);
+}
+// B's high bits carried into A: |B| <= 2^46 is left.
+__device__ __forceinline__ void fix_carry(FixWords& w) {
+    const long long c = (w.B + (1ll << 46)) >> 47;
+    w.A += c;
+    w.B -= c << 47;
+}
+// Adds w to column x's words (A and B side by side, the C of all n columns behind them): a
+// column has at most 2^15 addends of each kind, so |A| < 2^55, |B| <= 2^62 and |C| < 2^58.
+__device__ __forceinline__ void fix_add(int64_t* fix, int n, int x, FixWords w) {
+    fix_carry(w);
     unsigned long long* p = reinterpret_cast<unsigned long long*>(fix + 2 * (size_t)x);
-    if (A) atomicAdd(p, (unsigned long long)A);
-    if (B) atomicAdd(p + 1, (unsigned long long)B);
+    if (w.A) atomicAdd(p, (unsigned long long)w.A);
+    if (w.B) atomicAdd(p + 1, (unsigned long long)w.B);
+    if (w.C) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(fix + 2 * (size_t)n + x), (unsigned long long)w.C);
+        fix[3 * (size_t)n] = 1;
+    }
 }
 // BC(x) changes by delta_s(x)'s change from old to now.
-__device__ __forceinline__ void bc_fix_change(int64_t* fix, int x, ff old, ff now) {
+__device__ __forceinline__ void bc_fix_change(int64_t* fix, int n, int x, ff old, ff now) {
     if (old.hi == now.hi && old.lo == now.lo) return;
-    long long A0, B0, A1, B1;
-    fix_words(old, &A0, &B0);
-    fix_words(now, &A1, &B1);
-    fix_add(fix, x, A1 - A0, B1 - B0);
+    const FixWords w0 = fix_words(old), w1 = fix_words(now);
+    FixWords w{w1.A - w0.A, w1.B - w0.B, 0};
+    if (fix_small(old) || fix_small(now)) w.C = fix_rest(now) - fix_rest(old);
+    fix_add(fix, n, x, w);
 }
 
 // Vector access of VEC consecutive distances (16 bytes).
@@ -939,7 +956,7 @@ __device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, 
                 m.cell[x] = cell_rho(ff_add(acc, rx));
                 const ff now = ff_mul(sx, acc);
                 out[x] = now;
-                if (!STATIC) bc_fix_change(a.bcfix, x, old, now);
+                if (!STATIC) bc_fix_change(a.bcfix, a.n, x, old, now);
             }
         }
         __syncthreads();
@@ -981,7 +998,7 @@ __device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m
             if (STATIC) Ss[x] = sg;
             if (done[v]) {
                 const ff none{0.0f, 0.0f};
-                if (!STATIC) bc_fix_change(a.bcfix, x, old[v], none);
+                if (!STATIC) bc_fix_change(a.bcfix, n, x, old[v], none);
                 if (STATIC || old[v].hi != 0.0f) out[x] = none;
                 if (sg != 0) m.cell[x] = cell_rho(ff_rcp(ff_from_u64(sg)));
             }

@@ -251,8 +251,10 @@ struct Dev {
     int32_t pair_walk;   // 1: pair corrections by DAG walks (k_walk.cu), scratch below
     int64_t walk_cap;    // most entries of a walk's table in shared memory
     int32_t* walk_rows;  // [2n] rows with more targets, rows that outgrew their table
-    int64_t* bcfix;      // [2n] BC change of the changed rows in this update, per column a
-                         // fixed-point pair (units of 2^-24, units of 2^-56); zero between updates
+    int64_t* bcfix;      // [3n + 1] BC change of the changed rows in this update, per column
+                         // fixed-point words (units of 2^-24, 2^-71 and, behind those of all
+                         // columns, 2^-112), then whether any of the last is used; zero between
+                         // updates
     cudaStream_t st;
     // a third stream for the rows walked by a CTA each (undirected graphs): forked from st
     // before the light rows, joined back after them

@@ -86,17 +86,17 @@ struct PairArgs {
     int32_t* full_rows;     // rows with more targets than tcap
     int32_t* full_count;
     ff* Dl;
-    int64_t* bcfix;         // [2n] BC change of this update (fixed point, see fix_add)
+    int64_t* bcfix;         // [3n + 1] BC change of this update (fixed point, see fix_add)
     int32_t* err;
 };
 
 // BC(x) += v for one corrected entry delta_s(x) (fix_add): each pair term delta_st(x)
 // lies in [0, 1] and a row has at most kPairCap targets, so |v| <= 128, and a column
 // receives at most one entry per row.
-__device__ __forceinline__ void bc_fix_add(int64_t* fix, int x, ff v) {
-    long long A, B;
-    fix_words(v, &A, &B);
-    fix_add(fix, x, A, B);
+__device__ __forceinline__ void bc_fix_add(int64_t* fix, int n, int x, ff v) {
+    FixWords w = fix_words(v);
+    if (fix_small(v)) w.C = fix_rest(v);
+    fix_add(fix, n, x, w);
 }
 
 // One warp per listed row: a row with more changed targets than the cap goes to the list of
@@ -537,7 +537,7 @@ __device__ __forceinline__ void pair_item(const PairArgs<DT>& a, int s, int U_, 
             const ff acc = s_acc[q][threadIdx.x];
             ff* p = a.Dl + rs + x0 + q;
             *p = ff_add(*p, acc);
-            bc_fix_add(a.bcfix, x0 + q, acc);
+            bc_fix_add(a.bcfix, a.n, x0 + q, acc);
         }
 }
 
@@ -622,18 +622,19 @@ __global__ void __launch_bounds__(kPairThreads, kPairCtasPerSm) k_pairdep(PairAr
     }
 }
 
-// BC (hi, lo) += the fixed-point change of each column, then the pair is zeroed for the
-// next update: B's high bits are carried into A (A' = A + (B >> 32), B' = B mod 2^32),
-// so A' * 2^-24 and B' * 2^-56 are exact doubles, added with TwoSum as in
-// dev_bc_finish.
-__device__ __forceinline__ void dev_bc_fix(int t, int64_t* fix, double* hi, double* lo) {
+// BC (hi, lo) += the fixed-point change of each column, then its words are zeroed for the
+// next update: B's high bits are carried into A, so that A * 2^-24 and B * 2^-71 are exact
+// doubles, the first added with TwoSum.  third: some column has a C.
+__device__ __forceinline__ void dev_bc_fix(int t, int n, int64_t* fix, bool third, double* hi, double* lo) {
     const longlong2 f = *reinterpret_cast<const longlong2*>(fix + 2 * (size_t)t);
-    if (f.x == 0 && f.y == 0) return;
+    FixWords w{f.x, f.y, 0};
+    if (third) w.C = fix[2 * (size_t)n + t];
+    if ((w.A | w.B | w.C) == 0) return;
     *reinterpret_cast<longlong2*>(fix + 2 * (size_t)t) = make_longlong2(0, 0);
-    const long long A = f.x + (f.y >> 32);
-    const long long B = f.y & 0xFFFFFFFFll;
-    const double x1 = (double)A * 0x1p-24;
-    const double x2 = (double)B * 0x1p-56;
+    if (third) fix[2 * (size_t)n + t] = 0;
+    fix_carry(w);
+    const double x1 = (double)w.A * 0x1p-24;
+    const double x2 = (double)w.B * 0x1p-71 + (double)w.C * 0x1p-112;
     const double h = hi[t];
     const double s = h + x1;
     const double bp = s - h;
@@ -675,7 +676,8 @@ __global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
     pdl_enter();
     if (*a.err) return;   // the handle is poisoned: no further update
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    for (int x = t; x < a.n; x += gridDim.x * blockDim.x) dev_bc_fix(x, a.fix, a.hi, a.lo);
+    const bool third = a.fix[3 * (size_t)a.n] != 0;
+    for (int x = t; x < a.n; x += gridDim.x * blockDim.x) dev_bc_fix(x, a.n, a.fix, third, a.hi, a.lo);
     const int cnt = a.counts[1];
     for (int i = t; i < cnt; i += gridDim.x * blockDim.x) a.changed[a.rows[i]] = 0u;
     if (a.tcnt)
@@ -685,6 +687,7 @@ __global__ void __launch_bounds__(256) k_update_end(EndArgs a) {
     if (threadIdx.x == 0 && atomicAdd(a.counts + 6, 1) == (int)gridDim.x - 1) {
         dev_update_stats(a.stats, cnt, a.counts[3]);
         for (int k = 0; k < 16; ++k) a.counts[k] = 0;
+        if (third) a.fix[3 * (size_t)a.n] = 0;
     }
 }
 
@@ -883,7 +886,7 @@ __global__ void kb_update_end(BatchArgs b, int r) {
         const int g = graph_of(b.coff, G, j);
         const Dev& d = b.devs[g];
         if (*d.err || b.upd[(int64_t)r * G + g].present == 0) continue;
-        dev_bc_fix((int)(j - b.coff[g]), d.bcfix, d.bc_hi, d.bc_lo);
+        dev_bc_fix((int)(j - b.coff[g]), d.n, d.bcfix, d.bcfix[3 * (size_t)d.n] != 0, d.bc_hi, d.bc_lo);
     }
     const int64_t rows = b.plan_pr[G];
     const int wpb = blockDim.x >> 5;
@@ -901,6 +904,7 @@ __global__ void kb_update_stats(BatchArgs b, int r) {
         if (*d.err || b.upd[(int64_t)r * b.G + g].present == 0) continue;
         dev_update_stats(d.stats, d.counts[1], d.counts[3]);
         for (int k = 0; k < 8; ++k) d.counts[k] = 0;
+        d.bcfix[3 * (size_t)d.n] = 0;
     }
 }
 

@@ -646,8 +646,12 @@ struct RowWalk {
         const int x = k >> 1;
         ff* p = a.Dl + (size_t)s * a.ld + x;
         *p = ff_add(*p, from_units(v));
-        v += (__int128)1 << 62;   // to the nearest 2^-56
-        fix_add(a.bcfix, x, (long long)(v >> 95), (long long)(uint32_t)(v >> 63));   // units of 2^-24 and 2^-56
+        // units of 2^-24, 2^-71 and, of a small one, 2^-112
+        FixWords w{(long long)(v >> 95), (long long)(v >> 48) & ((1ll << 47) - 1), 0};
+        const long long rest = (long long)v & ((1ll << 48) - 1);
+        if (w.A == 0 || w.A == -1) w.C = (rest + 64) >> 7;
+        else w.B += rest >> 47;
+        fix_add(a.bcfix, a.n, x, w);
     }
 
     // The whole row; false: it outgrew the table and nothing was written but the table.

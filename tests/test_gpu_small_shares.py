@@ -1,10 +1,11 @@
 """Dependencies far below one: where pairs have 3^k shortest paths, a vertex on one of them
 has a dependency of about 3^-k.  Updates bring such a vertex onto the shortest paths; the
-corrected and the re-accumulated rows keep its relative accuracy.
+corrected and the re-accumulated rows, and BC, keep its relative accuracy.
 
 Tolerance: a result goes through at most a few hundred float-float operations, each with a
 relative error of a few units of 2^-46 (ff.cuh), all on terms of one sign for the vertices
-compared (new on the paths, so nothing cancels): 512 * 4 * 2^-46 = 2.9e-11."""
+compared (new on the paths, so nothing cancels): 512 * 4 * 2^-46 = 2.9e-11.  BC's change keeps
+each of these to 2^-112, far below that of the entries here."""
 import numpy as np
 import pytest
 
@@ -51,6 +52,8 @@ def check(h, g, x, a0, label):
     got, exp = dl[:, x], st.DEL[:, x]
     assert exp[a0] > 0
     assert bool(np.all(np.abs(got - exp) <= RTOL * exp)), f"{label}: dependency {got[a0]} expected {exp[a0]}"
+    bc = h.bc_get_scores()[x]
+    assert abs(bc - st.BC[x]) <= RTOL * st.BC[x], f"{label}: BC {bc} expected {st.BC[x]}"
 
 
 @pytest.mark.parametrize("dist", ["i32", "i64"])

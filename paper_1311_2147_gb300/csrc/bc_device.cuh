@@ -600,7 +600,8 @@ struct AccMem {
     uint32_t* cnt;     // [np / 2] (over row) in-degrees
     uint32_t* mask;    // [words] bit per slot of the superset: its arc is in DAG'(s)
     uint16_t* base;    // [words] first pool entry of a mask word's arcs
-    uint16_t* order;   // [np] (over mask and base) vertices with DAG out-arcs, level by level
+    uint16_t* order;   // [np] (over mask and base; without the pool over first) vertices with DAG
+                       // out-arcs, level by level
     uint16_t* pool;    // [pcap + 4] heads of the DAG arcs
     uint64_t* cell;    // [np] sigma_sx, then rho(x) once x is finished
     uint32_t* sink;    // [np / 32] bit per vertex: no DAG out-arc
@@ -769,40 +770,135 @@ __device__ __forceinline__ int count_dag(const AccMem& m, int beg, int len, int*
     return k + __popc(m.mask[w1] & (0xffffffffu >> (31 - ((end - 1) & 31))));
 }
 
-// First pool entry of the heads of a vertex with k > 0 DAG out-arcs; p as count_dag gives
-// it.  Marks the last head.  Heads that lie in several groups, and those of a big vertex
-// behind their number, are copied to the end of the pool (past its end they are only
-// counted).
+// Mask word w of the segment of slots [beg, end].
+__device__ __forceinline__ uint32_t segment_word(const AccMem& m, int w, int beg, int end) {
+    uint32_t b = m.mask[w];
+    if (w == beg >> 5) b &= 0xffffffffu << (beg & 31);
+    if (w == end >> 5) b &= 0xffffffffu >> (31 - (end & 31));
+    return b;
+}
+// First pool entry of the heads of a vertex with 0 < k < kBigDag DAG out-arcs; p as count_dag
+// gives it.  Marks the last head.  Heads that lie in several groups are copied to the end of
+// the pool (past its end they are only counted).
 __device__ __forceinline__ uint16_t place_heads(const AccMem& m, int pcap, int* s_arcs, int beg, int len, int k, int p) {
-    const int h = k >= kBigDag ? 1 : 0;
-    if (h || beg / kGroupSlots != (beg + len - 1) / kGroupSlots) {
-        p = atomicAdd(s_arcs, k + h);
-        if (p + k + h > pcap) return 0;
+    const int end = beg + len - 1;
+    if (beg / kGroupSlots != end / kGroupSlots) {
+        p = atomicAdd(s_arcs, k);
+        if (p + k > pcap) return 0;
         int at = p;
-        if (h) m.pool[at++] = (uint16_t)k;
-        const int w0 = beg >> 5, w1 = (beg + len - 1) >> 5;
-        for (int w = w0; w <= w1; ++w) {
-            const uint32_t word = m.mask[w], low = w == w0 ? (1u << (beg & 31)) - 1u : 0u;
-            uint32_t b = word & ~low;
-            if (w == w1) b &= 0xffffffffu >> (31 - ((beg + len - 1) & 31));
-            const int p0 = (int)m.base[w] + __popc(word & low), c = __popc(b);
+        for (int w = beg >> 5; w <= end >> 5; ++w) {
+            const uint32_t b = segment_word(m, w, beg, end);
+            const int p0 = (int)m.base[w] + (w == beg >> 5 ? __popc(m.mask[w] & ((1u << (beg & 31)) - 1u)) : 0);
+            const int c = __popc(b);
             for (int q = 0; q < c; ++q) m.pool[at++] = m.pool[p0 + q] & kHeadMask;
         }
     }
-    if (p + k + h <= pcap) m.pool[p + k + h - 1] |= kLastHead;
+    if (p + k <= pcap) m.pool[p + k - 1] |= kLastHead;
+    return (uint16_t)p;
+}
+// A vertex with more is placed by the whole warp: its heads are copied behind their number.
+__device__ __forceinline__ uint16_t place_big(const AccMem& m, int pcap, int* s_arcs, int beg, int len) {
+    const int lane = threadIdx.x & 31, end = beg + len - 1;
+    int k = 0;
+    for (int w = (beg >> 5) + lane; w <= end >> 5; w += 32) k += __popc(segment_word(m, w, beg, end));
+    k = __reduce_add_sync(FULL, k);
+    int p = 0;
+    if (lane == 0) p = atomicAdd(s_arcs, k + 1);
+    p = __shfl_sync(FULL, p, 0);
+    if (p + k + 1 > pcap) return 0;
+    if (lane == 0) m.pool[p] = (uint16_t)k;
+    int at = p + 1;
+    for (int w0 = beg >> 5; w0 <= end >> 5; w0 += 32) {   // 32 words at a time
+        const int w = w0 + lane;
+        int c = 0, p0 = 0;
+        if (w <= end >> 5) {
+            c = __popc(segment_word(m, w, beg, end));
+            p0 = (int)m.base[w] + (w == beg >> 5 ? __popc(m.mask[w] & ((1u << (beg & 31)) - 1u)) : 0);
+        }
+        int incl = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int z = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += z;
+        }
+        const int words = min(32, (end >> 5) - w0 + 1);
+        for (int j = 0; j < words; ++j) {
+            const int cj = __shfl_sync(FULL, c, j), from = __shfl_sync(FULL, p0, j), to = __shfl_sync(FULL, at + incl - c, j);
+            if (lane < cj) m.pool[to + lane] = m.pool[from + lane] & kHeadMask;
+        }
+        at += __shfl_sync(FULL, incl, 31);
+    }
     return (uint16_t)p;
 }
 
-// The DAG heads of vertex x from the superset and the distance row in memory, for a DAG
-// with more arcs than the pool holds (ties everywhere).
-template <typename DT, typename F>
-__device__ __forceinline__ void dag_heads(const AccArgs<DT>& a, const DT* Ds, int x, F&& f) {
-    const int64_t dx = Ds[x];
-    const int beg = a.e_off[x], end = beg + a.e_len[x];
-    for (int e = beg; e < end; ++e) {
-        const Arc arc = a.e_arc[e];
-        const int64_t w = sizeof(DT) == 4 ? (int64_t)arc.w : a.e_w64[e];
-        if (dx + w == (int64_t)Ds[arc.dst()]) f(arc.dst());
+// ---- the heads of a DAG with more arcs than the pool holds (ties everywhere, a hub whose
+// heads would be copied), from the masks and the superset: the masks stay and `order` takes
+// the place of `first`.  One L2 read a head in place of a shared-memory one, as many at a time
+// as in the pool's form.  Testing every slot of a vertex again, a thread a vertex, took 13.0 ms
+// where this takes 3.7 (k_accum of the static computation, BA n = 4096 with unit weights; BA
+// n = 12000 174 and 45 ms), and 27 and 1.1 ms for a star of 4096 vertices.
+
+// As four_heads, for the vertex whose segment is [beg, beg + len).
+template <typename F>
+__device__ __forceinline__ void four_heads_masked(const Arc* e_arc, const AccMem& m, int beg, int len, bool go, F&& f) {
+    const int end = beg + len - 1;
+    int w = beg >> 5;
+    uint32_t b = go ? segment_word(m, w, beg, end) : 0u;
+    while (__any_sync(FULL, go)) {
+        int at[4];
+        unsigned valid = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            at[u] = 0;
+            while (go && b == 0u && w < end >> 5) b = segment_word(m, ++w, beg, end);
+            if (b == 0u) continue;
+            at[u] = 32 * w + __ffs(b) - 1;
+            valid |= 1u << u;
+            b &= b - 1u;
+        }
+        go = go && (b != 0u || w < end >> 5);
+        uint32_t h[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h[u] = (valid >> u) & 1u ? (uint32_t)e_arc[at[u]].dst() : 0u;
+        f(h, valid);
+    }
+}
+// Position of bit number i (from 0) of b, which has more than i.
+__device__ __forceinline__ int nth_bit(uint32_t b, int i) {
+    int p = 0;
+#pragma unroll
+    for (int s = 16; s >= 1; s >>= 1) {
+        const int c = __popc(b & ((1u << s) - 1u));
+        if (i >= c) {
+            i -= c;
+            b >>= s;
+            p += s;
+        }
+    }
+    return p;
+}
+// The heads of one vertex by a whole warp, head number r by lane r mod 32 in increasing order,
+// as from the pool (so a lane's sum has the same terms in the same order): f(have, head).
+template <typename F>
+__device__ __forceinline__ void big_heads_masked(const Arc* e_arc, const AccMem& m, int beg, int len, F&& f) {
+    constexpr int U = 4;
+    const int lane = threadIdx.x & 31, end = beg + len - 1;
+    int rank = 0;   // warp-uniform
+    for (int w0 = beg >> 5; w0 <= end >> 5; w0 += U) {
+        uint32_t b[U];
+        bool have[U];
+        int h[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            b[u] = w0 + u <= end >> 5 ? segment_word(m, w0 + u, beg, end) : 0u;
+            const int i = (lane - rank) & 31, c = __popc(b[u]);
+            have[u] = i < c;
+            h[u] = have[u] ? e_arc[32 * (w0 + u) + nth_bit(b[u], i)].dst() : 0;
+            rank += c;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (b[u]) f(have[u], h[u]);
     }
 }
 
@@ -811,14 +907,14 @@ __device__ __forceinline__ void dag_heads(const AccArgs<DT>& a, const DT* Ds, in
 // counts go along: sigma_sb is the sum of sigma_sa over the DAG in-arcs (a, b).  Returns
 // the number of levels; level l is order[level_at(l) .. level_at(l + 1)).
 template <typename DT, bool STATIC, int T, bool POOLED>
-__device__ __forceinline__ int dag_levels(const AccArgs<DT>& a, const AccMem& m, AccShared& sh, int s, const DT* Ds) {
+__device__ __forceinline__ int dag_levels(const AccArgs<DT>& a, const AccMem& m, AccShared& sh, int s) {
     const int tid = threadIdx.x, lane = tid & 31;
     int lo = 0, hi = bit_of(m.sink, s) ? 0 : 1, L = 0;
     if (tid == 0) {
         m.order[0] = (uint16_t)s;
         m.level_at(0) = 0;
     }
-    __syncthreads();   // the masks under order are dead from here on
+    __syncthreads();   // what lies under order (POOLED: the masks) is dead from here on
     while (lo < hi) {
         int* q = &sh.q[L % 3];
         if (tid == 0) sh.q[(L + 1) % 3] = 0;
@@ -882,10 +978,24 @@ __device__ __forceinline__ int dag_levels(const AccArgs<DT>& a, const AccMem& m,
                         append4(m, q, hi, ready, b);
                     }
                 }
-            } else if (have) {
-                dag_heads(a, Ds, x, [&](int b) {
-                    if (take(b, sx) && !bit_of(m.sink, b)) m.order[hi + atomicAdd(q, 1)] = (uint16_t)b;
+            } else {
+                const bool big = have && bit_of(m.big, x);
+                const int beg = have ? a.e_off[x] : 0, len = have ? a.e_len[x] : 0;
+                four_heads_masked(a.e_arc, m, beg, len, have && !big, [&](const uint32_t* b, unsigned valid) {
+                    unsigned ready = 0;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if ((valid >> u) & 1u) ready |= take((int)b[u], sx) && !bit_of(m.sink, (int)b[u]) ? 1u << u : 0u;
+                    append4(m, q, hi, ready, b);
                 });
+                for (unsigned bb = __ballot_sync(FULL, big); bb; bb &= bb - 1u) {
+                    const int src = __ffs(bb) - 1;
+                    const uint64_t sb = STATIC ? m.cell[__shfl_sync(FULL, x, src)] : 0ull;
+                    big_heads_masked(a.e_arc, m, __shfl_sync(FULL, beg, src), __shfl_sync(FULL, len, src), [&](bool got, int h) {
+                        const uint32_t b[4] = {(uint32_t)h, 0u, 0u, 0u};
+                        append4(m, q, hi, got && take(h, sb) && !bit_of(m.sink, h) ? 1u : 0u, b);
+                    });
+                }
             }
         }
         __syncthreads();
@@ -900,7 +1010,7 @@ __device__ __forceinline__ int dag_levels(const AccArgs<DT>& a, const AccMem& m,
 
 // Eq. 4 back over the levels (level 0 is s: delta_s.(s) is not kept).
 template <typename DT, bool STATIC, int T, bool POOLED>
-__device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, const DT* Ds, int L, ff* out) {
+__device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, int L, ff* out) {
     const int tid = threadIdx.x, lane = tid & 31;
     for (int l = L - 1; l >= 1; --l) {
         const int lo = m.level_at(l), hi = m.level_at(l + 1);
@@ -931,24 +1041,22 @@ __device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, 
                     part = warp_sum(part);
                     if (lane == src) acc = part;
                 }
-            } else if (have) {
-                // kBigDag heads or more are summed as a warp would: 32 sums by rank, then a butterfly
-                int k = 0;
-                dag_heads(a, Ds, x, [&](int b) {
-                    ++k;
-                    acc = ff_add(acc, cell_ff(m.cell[b]));
+            } else {
+                const bool big = have && bit_of(m.big, x);
+                const int beg = have ? a.e_off[x] : 0, len = have ? a.e_len[x] : 0;
+                four_heads_masked(a.e_arc, m, beg, len, have && !big, [&](const uint32_t* b, unsigned valid) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if ((valid >> u) & 1u) acc = ff_add(acc, cell_ff(m.cell[b[u]]));
                 });
-                if (k >= kBigDag) {
-                    ff part[32];
-                    for (int c = 0; c < 32; ++c) part[c] = ff{0.0f, 0.0f};
-                    k = 0;
-                    dag_heads(a, Ds, x, [&](int b) {
-                        part[k & 31] = ff_add(part[k & 31], cell_ff(m.cell[b]));
-                        ++k;
+                for (unsigned bb = __ballot_sync(FULL, big); bb; bb &= bb - 1u) {
+                    const int src = __ffs(bb) - 1;
+                    ff part{0.0f, 0.0f};
+                    big_heads_masked(a.e_arc, m, __shfl_sync(FULL, beg, src), __shfl_sync(FULL, len, src), [&](bool got, int h) {
+                        if (got) part = ff_add(part, cell_ff(m.cell[h]));
                     });
-                    for (int o = 16; o > 0; o >>= 1)
-                        for (int c = 0; c < o; ++c) part[c] = ff_add(part[c], part[c + o]);
-                    acc = part[0];
+                    part = warp_sum(part);
+                    if (lane == src) acc = part;
                 }
             }
             // delta(x) = sigma_sx * acc, rho(x) = (1 + delta(x)) / sigma_sx = acc + 1 / sigma_sx
@@ -966,19 +1074,23 @@ __device__ __forceinline__ void dag_pull(const AccArgs<DT>& a, const AccMem& m, 
 // Once the DAG's levels are known: the vertices without DAG out-arcs are finished, then
 // the others back over the levels.
 template <typename DT, bool STATIC, int T, bool POOLED>
-__device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m, AccShared& sh, int s, const DT* Ds,
-                                           uint64_t* Ss, ff* out) {
+__device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m, AccShared& sh, int s, uint64_t* Ss,
+                                           ff* out) {
     const int n = a.n, tid = threadIdx.x;
-    if (!POOLED) {   // the pool's heads were counted as they came; now from the superset
+    if (!POOLED) {   // the pool's heads were counted as they came; now those of the masks
         for (int t = tid; t < (n + 1) / 2; t += T) m.cnt[t] = 0u;
         __syncthreads();
-        for (int x = tid; x < n; x += T)
-            if (!bit_of(m.sink, x)) dag_heads(a, Ds, x, [&](int b) { cnt_inc(m.cnt, b); });
+        constexpr int U = kGroupSlots / 32;
+        for (int g = tid >> 5; g < (int)(a.e_used / kGroupSlots); g += T / 32)
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if ((m.mask[g * U + u] >> (tid & 31)) & 1u)
+                    cnt_inc(m.cnt, a.e_arc[(int64_t)g * kGroupSlots + 32 * u + (tid & 31)].dst());
         __syncthreads();
         for (int x = tid; x < n; x += T) cnt_mark(m.cnt, x, !STATIC && bit_of(m.sink, x));
         __syncthreads();
     }
-    const int L = dag_levels<DT, STATIC, T, POOLED>(a, m, sh, s, Ds);
+    const int L = dag_levels<DT, STATIC, T, POOLED>(a, m, sh, s);
     constexpr int VU = 8;
     for (int x0 = tid; x0 < n; x0 += VU * T) {
         ff old[VU];
@@ -1009,12 +1121,13 @@ __device__ __forceinline__ void dag_source(const AccArgs<DT>& a, const AccMem& m
         out[n + tid] = ff{0.0f, 0.0f};
     }
     __syncthreads();
-    dag_pull<DT, STATIC, T, POOLED>(a, m, Ds, L, out);
+    dag_pull<DT, STATIC, T, POOLED>(a, m, L, out);
 }
 template <typename DT, bool STATIC, int T>
 __device__ __noinline__ void dag_source_unpooled(AccArgs<DT> a, AccMem m, AccShared* sh, int s) {
+    m.order = m.first;   // the masks are still read
     const size_t row = (size_t)s * a.ld;
-    dag_source<DT, STATIC, T, false>(a, m, *sh, s, a.D + row, a.S + row, a.Dl + row);
+    dag_source<DT, STATIC, T, false>(a, m, *sh, s, a.S + row, a.Dl + row);
 }
 
 // Re-accumulate source s (whole block; every thread calls it): stage its distance row,
@@ -1088,6 +1201,7 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
         for (int q = tid; q < arcs; q += T) cnt_inc(m.cnt, m.pool[q]);
     __syncthreads();   // the lists below mark and copy pool entries
     constexpr int VU = 8;
+    unsigned any_big = 0;
     for (int i0 = 0; i0 * T < n; i0 += VU) {
         int beg[VU], len[VU];
 #pragma unroll
@@ -1106,19 +1220,28 @@ __device__ __forceinline__ void dev_accum_source(const AccArgs<DT>& a, int s, co
             int p = 0;
             const int k = count_dag(m, beg[v], len[v], &p);
             if (x < n) {
-                m.first[x] = k > 0 ? place_heads(m, a.lay.pcap, &sh.arcs, beg[v], len[v], k, p) : (uint16_t)0;
+                if (k < kBigDag)
+                    m.first[x] = k > 0 ? place_heads(m, a.lay.pcap, &sh.arcs, beg[v], len[v], k, p) : (uint16_t)0;
                 cnt_mark(m.cnt, x, !STATIC && k == 0);
             }
             const unsigned sinks = __ballot_sync(FULL, k == 0), bigs = __ballot_sync(FULL, k >= kBigDag);
+            any_big |= bigs;
             if (lane == 0 && x < n) {
                 m.sink[x >> 5] = sinks;
                 m.big[x >> 5] = bigs;
             }
         }
     }
+    __syncwarp();
+    for (int q = tid >> 5; any_big && q * 32 < n; q += T / 32)   // the words of big that this warp wrote
+        for (uint32_t bb = m.big[q]; bb; bb &= bb - 1u) {
+            const int x = 32 * q + __ffs(bb) - 1;
+            const uint16_t first = place_big(m, a.lay.pcap, &sh.arcs, a.e_off[x], a.e_len[x]);
+            if (lane == 0) m.first[x] = first;
+        }
     if (SM && !STATIC) async_wait_all();
     __syncthreads();
-    if (sh.arcs <= a.lay.pcap) dag_source<DT, STATIC, T, true>(a, m, sh, s, Ds, Ss, out);
+    if (sh.arcs <= a.lay.pcap) dag_source<DT, STATIC, T, true>(a, m, sh, s, Ss, out);
     else dag_source_unpooled<DT, STATIC, T>(a, m, &sh, s);
 }
 

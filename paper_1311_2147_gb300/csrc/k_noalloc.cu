@@ -78,7 +78,9 @@ cudaError_t scratch_address(unsigned char** out) {
 // and check each arc: endpoints in range, no self-loop, weight in [1, INF-1].  The offsets
 // cover every slot (0 first, the number of arcs last, none smaller than the one before):
 // the search goes over all of them, and one left out would hold an earlier call's arc.
-// The slots past the arcs, up to a whole group, are empty.
+// The slots past the arcs, up to a whole group, are empty.  A thread per slot, its tail found
+// in the offsets by bisection: a thread per vertex took 34 us for BA n = 512 (8150 arcs) and
+// 76 us for the complete graph of 181 (32580), this takes 2.8 and 2.6.
 template <typename DT>
 __global__ void k_pack_graph(int n, int64_t arcs, unsigned long long* count, const int32_t* off, const int32_t* dst, const int64_t* w,
                              Arc* arc, int64_t* w64, int32_t* len, int32_t* err) {
@@ -89,22 +91,22 @@ __global__ void k_pack_graph(int n, int64_t arcs, unsigned long long* count, con
     }
     if (i < n) {
         const int32_t a = off[i], b = off[i + 1];
-        if (a < 0 || b < a || b > arcs) {
-            len[i] = 0;
-            set_err(err, ERRF_ARG_DEVICE);
-        } else {
-            len[i] = b - a;
-            for (int32_t e = a; e < b; ++e) {
-                if (dst[e] == (int32_t)i) set_err(err, ERRF_ARG_DEVICE);   // self-loop
-                arc[e] = make_arc((int32_t)i, dst[e], w[e]);
-                if (sizeof(DT) == 8) w64[e] = w[e];
-            }
-        }
+        const bool ok = a >= 0 && b >= a && b <= arcs;
+        len[i] = ok ? b - a : 0;
+        if (!ok) set_err(err, ERRF_ARG_DEVICE);
     }
     if (i < arcs) {
         const int32_t b = dst[i];
         const int64_t x = w[i];
-        if (b < 0 || b >= n || x < 1 || x >= Inf<DT>::v) set_err(err, ERRF_ARG_DEVICE);
+        int lo = 0, hi = n;   // the last vertex below hi whose arcs start at or before i, or 0
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (off[mid] <= i) lo = mid;
+            else hi = mid;
+        }
+        if (b < 0 || b >= n || b == lo || x < 1 || x >= Inf<DT>::v) set_err(err, ERRF_ARG_DEVICE);
+        arc[i] = make_arc(lo, b, x);
+        if (sizeof(DT) == 8) w64[i] = x;
     } else if (i < group_slots(arcs)) {
         arc[i] = empty_arc();
     }

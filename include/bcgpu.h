@@ -111,7 +111,8 @@ typedef struct bc_info {
     int64_t rows_scanned;        /* rows passed through the rank-1 pass (all phases) */
     int64_t pairs_lowered;       /* pairs whose distance dropped (Lemma 2/4 last case) */
     int64_t pairs_tied;          /* pairs that gained tied shortest paths */
-    int64_t kernel_launches;     /* kernels enqueued by this handle since init */
+    int64_t kernel_launches;     /* kernels enqueued by this handle since init; in a batch, those of the
+                                    rounds it had an update in */
     int64_t state_bytes;         /* device bytes owned by the handle */
     double last_init_ms;         /* device time of the static computation in bc_init_static */
     int64_t rows_full;           /* of rows_reaccumulated: rows rebuilt by Algorithm 1 rather than
@@ -370,7 +371,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
 
 /* bc_batch_set_tiles -- launch shape of the batch kernels (what the autotuner varies):
  * tiles[0] CTAs per SM of the per-vertex passes (1..64), tiles[1] of the rank-1 pass,
- * tiles[2] of the BC row sums, tiles[3] cap on accumulation CTAs per SM (0 = as many as
+ * tiles[2] (1..64) is not used, tiles[3] cap on accumulation CTAs per SM (0 = as many as
  * fit); with count >= 6 also the rank-1 pass's tile and schedule: tiles[4] 16-byte
  * vectors per thread per work item (1, 2, 4 or 8: the item's column chunk is 256
  * threads x tiles[4] x 16 bytes), tiles[5] 0 = a contiguous block of items per CTA,

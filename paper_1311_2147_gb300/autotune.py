@@ -1,7 +1,7 @@
 """Autotuner for the launch shape of batches of graphs (bc_batch_set_tiles).
 
-The tunable shape is (CTAs per SM of the per-vertex passes, of the rank-1 pass, of the
-BC row sums, cap on accumulation CTAs per SM, the rank-1 pass's tile -- 16-byte vectors
+The tunable shape is (CTAs per SM of the per-vertex passes, of the rank-1 pass, a place
+that is not used, cap on accumulation CTAs per SM, the rank-1 pass's tile -- 16-byte vectors
 per thread per work item, so its column chunk -- its schedule -- contiguous item
 blocks per CTA or items dealt out in turn -- and the threads of an accumulation CTA,
 512, 256 or 128).  The tuner runs coordinate descent from a
@@ -19,7 +19,7 @@ import os
 from . import build as _build
 
 DEFAULT = [4, 8, 8, 0, 4, 0, 256]
-CANDIDATES = [[2, 4, 8], [4, 8, 16], [4, 8, 16], [0, 1], [1, 2, 4, 8], [0, 1], [512, 256, 128]]
+CANDIDATES = [[2, 4, 8], [4, 8, 16], [8], [0, 1], [1, 2, 4, 8], [0, 1], [512, 256, 128]]
 CACHE = os.path.join(_build.BUILD, "autotune.json")
 TIMED_STEPS = 2   # timed batch steps per candidate (after one untimed step that captures the graph)
 

@@ -1383,7 +1383,6 @@ int bc_batch_create(bc_batch** out, int32_t count, bc_graph* const* graphs, void
     b->L.nsm = graphs[0]->d.nsm;
     b->L.vpass_ctas = 4;
     b->L.scan_ctas = 8;
-    b->L.bc_ctas = 8;
     b->L.acc_per_sm = 0;
     b->L.scan_unroll = 4;
     b->L.scan_sched = 0;
@@ -1426,7 +1425,6 @@ int bc_batch_set_tiles(bc_batch* b, const int32_t* tiles, int32_t count) {
         return bfail(b, BC_ERR_ARG, "accumulation CTA threads must be 128, 256 or 512");
     b->L.vpass_ctas = tiles[0];
     b->L.scan_ctas = tiles[1];
-    b->L.bc_ctas = tiles[2];
     b->L.acc_per_sm = tiles[3];
     if (count >= 6) {
         b->L.scan_unroll = tiles[4];
@@ -1537,7 +1535,6 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
                 entries.push_back(e);
             }
             for (const EOp& op : ops) eops.push_back(BatchEOp{g, 0, op});
-            gr->launches += 20;
         }
         eop_off[r + 1] = (int64_t)eops.size();
         for (int kind = 0; kind < 4; ++kind) {
@@ -1676,6 +1673,7 @@ int bc_batch_apply(bc_batch* b, const int32_t* n_updates, const bc_update* ups, 
             b->last_error = gr->last_error;
         }
         if (n_done) n_done[g] = ok[g];
+        if (ok[g]) gr->launches += (int64_t)ok[g] * batch_round_kernels(b->L) + 1;   // the errors' once a call
     }
     return status;
 }

@@ -53,7 +53,6 @@ struct BatchLaunch {
     int32_t nsm;
     int32_t vpass_ctas;   // CTAs per SM of the per-vertex passes      (tunable)
     int32_t scan_ctas;    // CTAs per SM of the rank-1 pass             (tunable)
-    int32_t bc_ctas;      // CTAs per SM of the BC row sums             (tunable)
     int32_t acc_per_sm;   // cap on accumulation CTAs per SM, 0 = max   (tunable)
     int32_t scan_unroll;  // 16-byte vectors per thread per rank-1 item: the item's column
                           // chunk is 256 threads x this x the vector width (1, 2, 4, 8; tunable)
@@ -98,6 +97,7 @@ __device__ __forceinline__ int32_t acc_list_count(const Dev& d) { return d.pair_
 
 void batch_config(BatchLaunch& L, int dbytes, int n_max, int64_t cap_max);
 void batch_launch_rounds(const BatchArgs& b, const BatchLaunch& L, int rounds, int dbytes, cudaStream_t st);
+int batch_round_kernels(const BatchLaunch& L);   // kernels of a round
 // Prefix offsets over graphs of one kind of per-graph work (kb_plan), and the pair
 // corrections of round r (k_pair.cu).
 void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* out, int scan_unroll,

@@ -342,6 +342,10 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     batch_round_end(b, L, r, st);
 }
 
+// (round_launches, and the kernels of batch_pair_plan, batch_pair_launches, batch_walk_class,
+// batch_walk_launches and batch_round_end in it.)
+int batch_round_kernels(const BatchLaunch& L) { return 14 + (L.pairs & 1 ? 4 : 0) + (L.pairs & 2 ? 4 : 0); }
+
 void batch_plan(const BatchArgs& b, int r, int kind, int phase_active, int64_t* out, int scan_unroll,
                 cudaStream_t st) {
     kb_plan<<<1, 1024, 0, st>>>(b, r, kind, phase_active, out, scan_unroll);

@@ -329,7 +329,8 @@ static void round_launches(const BatchArgs& b, const BatchLaunch& L, int r, cuda
     if (L.pairs & 2) batch_walk_class(b, L, r, st);
     kb_plan<<<1, 1024, 0, st>>>(b, r, 2, 2, b.plan_acc, L.scan_unroll);
     // (disjoint dependency rows, the rest of the state only read: a branch each of the
-    // captured graph)
+    // captured graph.  A call of 8 rounds so and in one branch: 96 graphs of n < 2048 4.41 and
+    // 4.70 ms, 512 graphs 22.8 and 23.4, 24 graphs of n < 4000 with vertex updates 3.36 and 3.91)
     cudaEventRecord(L.fork, st);
     cudaStreamWaitEvent(L.side, L.fork, 0);
     if (L.acc_threads == 128) batch_accum<DT, 128>(b, L, r, L.side);

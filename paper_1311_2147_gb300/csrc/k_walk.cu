@@ -770,8 +770,9 @@ __global__ void __launch_bounds__(kLightWarps * 32, kLightPerSm) kb_walk_light(B
 
 // Rows with more targets (RETRY: rows that outgrew their table, in the dense arrays if
 // they outgrow this one too): a CTA each.  A light row has at most 16 targets (22 entries
-// in the mean, and up to 95 fit); one of more has some hundred entries, so 512 are enough
-// for most and leave eight CTAs an SM.
+// in the mean, and up to 95 fit); one of more has some hundred entries.  256 threads and 1024
+// entries, four CTAs an SM, took 421 us an update at n = 16384 where 512 entries and eight
+// CTAs took 432, and a CTA of 64 threads 475.
 template <bool RETRY>
 struct Cta {
     static_assert(4 * kPairCap <= 512 && 2 * kLightTargets < kLightH, "room for the targets");

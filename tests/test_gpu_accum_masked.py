@@ -34,6 +34,9 @@ GRAPHS = {
     "star": lambda: synth.star_graph(2500, 3),
     "hub-2000": lambda: _hub(3000, 2000, False, 5),
     "hub-directed": lambda: _hub(2200, 1500, True, 1 << 35),
+    "hub-255": lambda: _hub(900, 255, False, 4),
+    "hub-256": lambda: _hub(900, 256, False, 4),
+    "hub-700": lambda: _hub(2600, 700, False, 5),
     "equal-ba": lambda: synth.barabasi_albert(1500, 8, 4, 4, 3),
     "equal-er": lambda: synth.erdos_renyi(1100, 12000, 2, 2, 4, directed=True),
     "two-values": lambda: synth.complete_directed(150, 1, 2, 7),

@@ -353,20 +353,20 @@ def run_ours(args):
     dinfo = {k: infop1[k] - infop0[k] for k in infop1 if isinstance(infop1[k], int)}
     d_rows_acc, d_rows_scan = dinfo["rows_reaccumulated"], dinfo["rows_scanned"]
     d_low, d_tie = dinfo["pairs_lowered"], dinfo["pairs_tied"]
-    d_full, d_pair_rows, d_pair_tgts = dinfo["rows_full"], dinfo["pair_rows"], dinfo["pair_targets"]
+    d_pair_rows, d_pair_tgts = dinfo["pair_rows"], dinfo["pair_targets"]
+    # rows re-accumulated: those over the target cap, or without pair corrections every changed one
+    d_full = dinfo["rows_full"] if d_pair_rows else d_rows_acc
     d_walk_pairs, d_walk_vtx, d_walk_arcs = dinfo["walk_pairs"], dinfo["walk_vertices"], dinfo["walk_arcs"]
     # algorithmic HBM bytes per kernel class over the profiled steps
     alg_bytes = {
         # rank-1 pass: read d of every scanned pair, sigma read+write on ties, d+sigma
         # written where the distance drops
         "scan": d_rows_scan * n * sd + d_tie * 16 + d_low * (sd + 8),
-        # accumulation (the rows over the target cap): d row, sigma row, new delta row
-        "accumulate": d_full * n * (sd + 8 + 8),
-        # BC: the re-accumulated delta rows are read twice (before and after); with pair
-        # corrections only the full rows are, and per update the fixed-point column
-        # changes are read and BC (hi, lo) read and written (16 bytes each per column)
-        "bc_rows": (2 * d_full * n * 8 + len(prof_updates) * n * 48) if d_pair_rows
-        else 2 * d_rows_acc * n * 8,
+        # accumulation: d row, sigma row, old and new delta row
+        "accumulate": d_full * n * (sd + 8 + 8 + 8),
+        # end of an update: the fixed-point column changes read and BC (hi, lo) read and
+        # written (16 bytes each per column)
+        "bc_rows": len(prof_updates) * n * 48,
     }
     # pair corrections: per (row, changed target, column) one add and one compare for
     # each of the two states (integer ALU work; the rows come from L2)
@@ -374,10 +374,12 @@ def run_ours(args):
     peak, peak_kind = load_peaks()
     int_peak = int_alu_peak()
     if d_walk_pairs:
-        # pair corrections by DAG walks: per E* arc examined the arc (8 B) and d(s,x) (sd B);
-        # per vertex found its segment bounds (8 B), two path counts (16 B), its list entry
-        # written and read back (8 B) and its buffer entry written and read (8 B)
-        alg_bytes["pair_corrections"] = d_walk_arcs * (8 + sd) + d_walk_vtx * (8 + 16 + 8 + 8)
+        # pair corrections by DAG walks: per E* arc examined the arc (8 B; with 64-bit distances
+        # its weight, 8 B) and d(s,x) (sd B); per vertex found its segment bounds (8 B), its
+        # path count (8 B) and its dependency read and written (16 B); per changed target
+        # that and the distance and path count of both states
+        alg_bytes["pair_corrections"] = (d_walk_arcs * (8 + sd + (8 if sd == 8 else 0)) + d_walk_vtx * 32
+                                         + d_pair_tgts * (24 + 2 * (sd + 8)))
         alu_ops.pop("pair_corrections")
     dom = max(prof, key=lambda c: prof[c][0])
     dom_ms, dom_launches = prof[dom]
@@ -386,12 +388,12 @@ def run_ours(args):
         kl = len(prof_updates)
         achieved = alg_bytes[dom] / (dom_ms / 1e3) / 1e9
         roof = {"bound": "hbm", "kernel_class": dom,
-                "kernel": "k_walk_units + k_walk_rows_hash + k_walk_rows (DAG walks; with k_pair_plan, k_pair_weights)",
+                "kernel": "k_walk_light + k_walk_cta (DAG walks of a row; with k_walk_class)",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_kind": peak_kind,
                 "alg_bytes_per_launch": alg_bytes[dom] / kl,
-                "traffic": read_traffic("walks_ba8192", (d_walk_arcs + d_walk_vtx) / kl),
+                "traffic": read_traffic("walks_ba8192", (d_walk_arcs + d_walk_vtx + d_pair_tgts) / kl),
                 "launches": kl, "avg_launch_ms": dom_ms / kl,
-                "note": "latency-bound gathers along shortest-path DAGs; bytes counted per arc and vertex visited"}
+                "note": "latency-bound gathers along shortest-path DAGs; bytes counted per arc, vertex and target"}
     elif dom in alu_ops and dom_ms > 0 and dom_launches > 0:
         kl = dom_launches // 3 or 1   # k_pair_plan, k_pair_weights, k_pairdep per update
         achieved = alu_ops[dom] / (dom_ms / 1e3) / 1e12
@@ -562,7 +564,7 @@ def run_ours(args):
             C.close()
         gpu_full = {"ms": med, "runs": ms, "updates_per_s": 1e3 / med,
                     "incremental_speedup": value / world / (1e3 / med),
-                    "static": "searches restricted to E* as it becomes known (Algorithm 6 step 1)",
+                    "static": "of a dense graph, searches over a set of arcs that contains E* (Algorithm 6 step 1)",
                     "all_arcs_ms": statistics.median(ms_all),
                     "all_arcs_note": "the same static computation searching every arc (BC_STATIC_ALL_ARCS)"}
         if world == 1:
